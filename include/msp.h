@@ -182,8 +182,9 @@ msp_status msp_build_tree(msp_ctx *ctx, int64_t n, const float *x_dev, const flo
 msp_status msp_attraction(msp_ctx *ctx, float *u_dev, void *stream);
 
 /* The comparison path: Eq. 8 by all-pairs evaluation over every neuron, on
- * the tree's sorted copy (no cutoff, no expansion).  Same output convention
- * as msp_attraction.  Requires msp_build_tree.  Asynchronous. */
+ * the tree's sorted copy (no cutoff, no expansion; groups of sources whose
+ * every term is exactly zero in single precision, below 2^-126, are passed
+ * over).  Same output convention as msp_attraction.  Requires msp_build_tree.  Asynchronous. */
 msp_status msp_direct(msp_ctx *ctx, float *u_dev, void *stream);
 
 /* Steps a11-a12: Algorithm 1 with Algorithm 2's choice at every level, a

@@ -11,7 +11,7 @@
 // that array (MSP_NOALLOC_MAX_N * 24 bytes) until the process exits.
 #include <mutex>
 
-#include "msp_internal.cuh"
+#include "msp_direct.cuh"
 
 namespace msp {
 void set_last_error(const char* msg);
@@ -20,10 +20,15 @@ void set_last_error(const char* msg);
 namespace {
 
 constexpr size_t kNaPtsBytes = (size_t)MSP_NOALLOC_MAX_N * sizeof(float4);
-constexpr size_t kNaBytes = kNaPtsBytes + (size_t)MSP_NOALLOC_MAX_N * sizeof(float2);
+constexpr size_t kNaListBytes = (size_t)MSP_NOALLOC_MAX_N * sizeof(int32_t);
+constexpr size_t kNaBytes = (size_t)MSP_NOALLOC_MAX_N * 24;
+static_assert(kNaPtsBytes + kNaListBytes +
+                      msp::DirScratch::words(MSP_NOALLOC_MAX_N) * sizeof(int32_t) <= kNaBytes,
+              "the scratch holds the packed copy, the target lists, their counts and the boxes");
 
-// The scratch: packed positions (float4) followed by the dendrite weights
-// (float2) of up to MSP_NOALLOC_MAX_N neurons.  Shared by every call.
+// The scratch: the packed neurons (float4), the target lists (int32), their
+// counts and the source tiles' boxes of up to MSP_NOALLOC_MAX_N neurons.  Shared by every call; everything in it is rewritten before it is
+// read, so nothing left by an earlier call is ever used.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaBytes];
 
 // Device address of g_noalloc_scratch, looked up once per device and CUDA
@@ -89,67 +94,6 @@ bool on_device(const void* p, int dev) {
     return (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) && a.device == dev;
 }
 
-__device__ inline float na_ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// every entry [0, n) of the scratch is rewritten before it is read, so nothing
-// left by an earlier call is ever used
-__global__ void k_na_pack(int64_t n, const float* __restrict__ x, const float* __restrict__ y,
-                          const float* __restrict__ z, const uint8_t* __restrict__ type,
-                          const uint8_t* __restrict__ va, const uint8_t* __restrict__ vde,
-                          const uint8_t* __restrict__ vdi, float4* __restrict__ P,
-                          float2* __restrict__ Wt) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t packed = (uint32_t)(type[i] ? 1u : 0u) | ((uint32_t)va[i] << 8);
-        P[i] = make_float4(x[i], y[i], z[i], __uint_as_float(packed));
-        Wt[i] = make_float2((float)vde[i], (float)vdi[i]);
-    }
-}
-
-constexpr int kNaThreads = 256;
-
-// u(t) = sum_{s != t} w_s^{type t} 2^(-|t-s|^2 log2(e)/sigma^2), sources staged
-// through shared memory in tiles, in the caller's order; tile sums in single
-// precision, added across tiles with Kahan's compensated summation
-__global__ void __launch_bounds__(kNaThreads)
-k_na_direct(int64_t n, const float4* __restrict__ P, const float2* __restrict__ Wt, float k2,
-            float* __restrict__ u) {
-    __shared__ float4 sp[kNaThreads];
-    __shared__ float2 sw[kNaThreads];
-    for (int64_t tb = (int64_t)blockIdx.x * kNaThreads; tb < n; tb += (int64_t)gridDim.x * kNaThreads) {
-        const int64_t t = tb + threadIdx.x;
-        const bool active = t < n;
-        const float4 T = active ? P[t] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const uint32_t tw = __float_as_uint(T.w);
-        const bool inh = (tw & 0xffu) != 0;
-        float acc = 0.f, comp = 0.f;   // Kahan sum of the tile sums
-        for (int64_t sb = 0; sb < n; sb += kNaThreads) {
-            __syncthreads();
-            const int64_t s = sb + threadIdx.x;
-            sp[threadIdx.x] = s < n ? P[s] : make_float4(3e30f, 3e30f, 3e30f, 0.f);
-            sw[threadIdx.x] = s < n ? Wt[s] : make_float2(0.f, 0.f);
-            __syncthreads();
-            float part = 0.f;
-            for (int j = 0; j < kNaThreads; ++j) {
-                const float4 S = sp[j];
-                const float dx = T.x - S.x, dy = T.y - S.y, dz = T.z - S.z;
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                const float wj = sb + j == t ? 0.f : (inh ? sw[j].y : sw[j].x);
-                part = fmaf(wj, na_ex2(-r2 * k2), part);
-            }
-            const float y = __fsub_rn(part, comp);
-            const float t2 = __fadd_rn(acc, y);
-            comp = __fsub_rn(__fsub_rn(t2, acc), y);
-            acc = t2;
-        }
-        if (active) u[t] = ((tw >> 8) & 0xffu) > 0 ? acc : 0.f;
-    }
-}
-
 }  // namespace
 
 extern "C" msp_status msp_direct_noalloc(int64_t n, const float* x, const float* y, const float* z,
@@ -188,19 +132,27 @@ extern "C" msp_status msp_direct_noalloc(int64_t n, const float* x, const float*
                                 "current device");
             return MSP_ERR_INVALID_ARG;
         }
-    float4* P = static_cast<float4*>(base);
-    float2* Wt = reinterpret_cast<float2*>(static_cast<unsigned char*>(base) + kNaPtsBytes);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const float k2 = (float)(1.4426950408889634 / (sigma * sigma));
-    int g = (int)((n + kNaThreads - 1) / kNaThreads);
-    k_na_pack<<<g, kNaThreads, 0, s>>>(n, x, y, z, type, vac_axon, vac_dend_e, vac_dend_i, P, Wt);
-    k_na_direct<<<g, kNaThreads, 0, s>>>(n, P, Wt, k2, u);
+    const msp::DirRaw src{x, y, z, type, vac_axon, vac_dend_e, vac_dend_i};
+    int launches = 1;
+    if (n <= msp::kDirSmallN) {
+        msp::k_dir_small<false><<<(unsigned)((n + 31) / 32), msp::kDirSmallWarps * 32, 0, s>>>(
+            n, src, k2, nullptr, 0, nullptr, u);
+    } else {
+        unsigned char* sc = static_cast<unsigned char*>(base);
+        float4* P = reinterpret_cast<float4*>(sc);
+        int32_t* list = reinterpret_cast<int32_t*>(sc + kNaPtsBytes);
+        const msp::DirScratch t(reinterpret_cast<int32_t*>(sc + kNaPtsBytes + kNaListBytes), n);
+        msp::dir_launch_tiles<false>(n, src, P, P, list, t, k2, nullptr, 0, nullptr, u, s);
+        launches = 3;
+    }
     e = cudaGetLastError();
     if (e != cudaSuccess) {
         msp::set_last_error(cudaGetErrorString(e));
         return MSP_ERR_CUDA;
     }
-    msp::g_kernel_launches.fetch_add(2, std::memory_order_relaxed);
+    msp::g_kernel_launches.fetch_add(launches, std::memory_order_relaxed);
     msp::set_last_error("");
     return MSP_OK;
 }
