@@ -1224,7 +1224,7 @@ def run_profile_case(args):
         gv = torch.from_numpy(np.random.default_rng(6).normal(size=w.n)).float().cuda()
         for _ in range(steps):
             g.attraction_grad(typ, va, ve, vi, g=gv)
-        # then the synapse-length loss with its gradient (k_len_pairs)
+        # then the synapse-length loss with its gradient (k_len_forward, k_len_adjoint)
         for _ in range(steps):
             g.length_loss(typ, va, ve.float(), vi.float(), 1000.0)
     elif kind in ("graph", "graph_full"):

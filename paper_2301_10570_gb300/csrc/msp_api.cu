@@ -195,8 +195,8 @@ msp_status msp_destroy(msp_ctx* c) {
                          &c->gm_key1, &c->gm_q, &c->gm_q1, &c->gm_flag, &c->gm_gid,
                          &c->gm_gstart, &c->gm_ntile, &c->gm_toff, &c->gm_tiles, &c->gm_cnt,
                          &c->frame_off, &c->frame_cap, &c->frame_g2, &c->frame_rc2,
-                         &c->gr_w, &c->gr_tmp, &c->gr_key0, &c->gr_key1, &c->gr_val0,
-                         &c->gr_val1, &c->gr_flag, &c->gr_off, &c->gr_seg, &c->ln_sums,
+                         &c->gr_w, &c->gr_fl, &c->gr_tmp, &c->gr_pt, &c->gr_flag, &c->gr_off,
+                         &c->ln_sums,
                          &c->ln_part, &c->ln_coef,
                          &c->expA, &c->expM, &c->expB, &c->u_sorted, &c->items0, &c->items1,
                          &c->leaf_items, &c->rq_key0, &c->rq_val0,

@@ -15,511 +15,413 @@
 #include <algorithm>
 #include <cmath>
 
-#include "msp_internal.cuh"
+#include "msp_pairsum.cuh"
 
 namespace msp {
 
 namespace {
 
-__device__ inline float gr_ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// sorted-order weights: {w^E, w^I, g [a > 0], bit 0 type | bit 1 a > 0}
+// sorted-order inputs: the weights (w^E, w^I) and the targets' flags; grads of
+// points without terms stay zero (out of the pair sums)
 __global__ void k_grad_gather(int64_t n, const int32_t* __restrict__ perm,
                               const uint8_t* __restrict__ type, const uint8_t* __restrict__ va,
                               const uint8_t* __restrict__ vde, const uint8_t* __restrict__ vdi,
-                              const float* __restrict__ g, float4* __restrict__ gw) {
+                              float2* __restrict__ w, uint16_t* __restrict__ fl) {
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
          s += (int64_t)gridDim.x * blockDim.x) {
         const int32_t c = perm[s];
-        const bool act = va[c] > 0;
-        const uint32_t flags = (type[c] ? 1u : 0u) | (act ? 2u : 0u);
-        gw[s] = make_float4((float)vde[c], (float)vdi[c], (g && act) ? g[c] : 0.f,
-                            __uint_as_float(flags));
+        w[s] = make_float2((float)vde[c], (float)vdi[c]);
+        fl[s] = (uint16_t)((type[c] ? kPsInh : 0u) | (va[c] ? kPsAct : 0u) | ((uint32_t)va[c] << 8));
     }
 }
 
-constexpr int kGrWarps = 4;
-constexpr int kGrStage = 64;
-constexpr int kGrMaxR = 3;                // evaluation points per lane
-constexpr int kGrList = 32 * kGrMaxR;     // evaluation points per pass
-
-// A staged pair of sources against one evaluation point t, whose scaled
-// coordinates are broadcast into both halves of register pairs; every step is
-// a paired FP32 instruction (two results, one issue slot) with the
-// per-element rounding of the scalar form: dx = t - s (s is staged negated),
-// q = fma(dx, dx, fma(dy, dy, dz dz)), K = 2^-q.  Staged pair j (sources
-// 2j, 2j + 1): A = (-x0, -x1, -y0, -y1), B = (-z0, -z1, w0_0, w0_1),
-// C = (w1_0, w1_1, index0, index1); a padding source has zero weights and
-// index -1.  SELF: a source may be t itself (sorted index e); its term is zero.
-template <bool FORWARD, bool SELF>
-__device__ __forceinline__ void gr_term(const float4 A, const float4 B, const float4 C,
-                                        float2 tx, float2 ty, float2 tz, bool inh, int32_t e,
-                                        float2& a0, float2& a1) {
-    const float2 dx = __fadd2_rn(tx, make_float2(A.x, A.y));
-    const float2 dy = __fadd2_rn(ty, make_float2(A.z, A.w));
-    const float2 dz = __fadd2_rn(tz, make_float2(B.x, B.y));
-    const float2 q = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-    float2 ex = make_float2(gr_ex2(-q.x), gr_ex2(-q.y));
-    if (SELF) {
-        ex.x = __float_as_int(C.z) == e ? 0.f : ex.x;
-        ex.y = __float_as_int(C.w) == e ? 0.f : ex.y;
+// entries of the packed targets' scan: [0, n) excitatory, [n, 2n) inhibitory,
+// one zero after them
+__global__ void k_ps_flags(int64_t n, const uint16_t* __restrict__ fl, int32_t* __restrict__ flag,
+                           int64_t* __restrict__ scan_n) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *scan_n = 2 * n + 1;
+        flag[2 * n] = 0;
     }
-    if (FORWARD) {
-        const float2 wk = __fmul2_rn(inh ? make_float2(C.x, C.y) : make_float2(B.z, B.w), ex);
-        a0 = __fadd2_rn(a0, wk);
-        a1 = __ffma2_rn(wk, q, a1);
-    } else {
-        a0 = __ffma2_rn(make_float2(B.z, B.w), ex, a0);
-        a1 = __ffma2_rn(make_float2(C.x, C.y), ex, a1);
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
+         s += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t f = fl[s];
+        flag[s] = (f & kPsAct) && !(f & kPsInh);
+        flag[n + s] = (f & kPsAct) && (f & kPsInh);
     }
 }
 
-// The staged pairs j = ksl, ksl + slices, ... < mp against the lane's R points.
-template <bool FORWARD, bool SELF, int R>
-__device__ __forceinline__ void gr_eval(const float4* sA, const float4* sB, const float4* sC,
-                                        int mp, int ksl, int slices, const float2 (&tx)[R],
-                                        const float2 (&ty)[R], const float2 (&tz)[R],
-                                        const bool (&inh)[R], const int32_t (&e)[R],
-                                        float2 (&a0)[R], float2 (&a1)[R]) {
+// the packed targets with their g
+__global__ void k_grad_pack(int64_t n, const uint16_t* __restrict__ fl,
+                            const int32_t* __restrict__ off, const int32_t* __restrict__ perm,
+                            const float4* __restrict__ pts, const float* __restrict__ g,
+                            float4* __restrict__ pt, float* __restrict__ pg) {
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
+         s += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t f = fl[s];
+        if (!(f & kPsAct)) continue;
+        const int32_t k = off[((f & kPsInh) ? n : 0) + s];
+        const float4 P = pts[s];
+        pt[k] = make_float4(P.x, P.y, P.z, __int_as_float((int32_t)s));
+        pg[k] = g[perm[s]];
+    }
+}
+
+// FORWARD: u(t) = sum w K and sum w q K (times dscale: du/dsigma) for the
+// targets of the block's leaf.  The distance is formed as a difference: the
+// second sum needs q itself, which the expanded exponent gives only with an
+// absolute error that is large against q for the closest pairs.  Two terms:
+// dx = t - s (s staged negated), q = fma(dx, dx, fma(dy, dy, dz dz)), K =
+// 2^-q.  SELF: a source may be the target itself (sorted index); its term is
+// zero.
+constexpr int kGrFwdR = 4;
+
+template <int R, bool SELF>
+__device__ __forceinline__ void gr_fwd_eval(const float4* sA, const float4* sW, int mp, int ksl,
+                                            int slices, const float2 (&tx)[R],
+                                            const float2 (&ty)[R], const float2 (&tz)[R],
+                                            const int32_t (&e)[R], int32_t first, int32_t second,
+                                            float2 (&a0)[R], float2 (&a1)[R]) {
 #pragma unroll 2
     for (int j = ksl; j < mp; j += slices) {
-        const float4 A = sA[j], B = sB[j], C = sC[j];
+        const float4 A = sA[j], B = sW[j];
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-            gr_term<FORWARD, SELF>(A, B, C, tx[r], ty[r], tz[r], inh[r], e[r], a0[r], a1[r]);
+        for (int r = 0; r < R; ++r) {
+            const float2 dx = __fadd2_rn(tx[r], make_float2(A.x, A.y));
+            const float2 dy = __fadd2_rn(ty[r], make_float2(A.z, A.w));
+            const float2 dz = __fadd2_rn(tz[r], make_float2(B.x, B.y));
+            const float2 q = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+            float2 K = make_float2(ps_ex2(-q.x), ps_ex2(-q.y));
+            if (SELF) {
+                K.x = first + j == e[r] ? 0.f : K.x;
+                K.y = second + j == e[r] ? 0.f : K.y;
+            }
+            const float2 wk = __fmul2_rn(make_float2(B.z, B.w), K);
+            a0[r] = __fadd2_rn(a0[r], wk);
+            a1[r] = __ffma2_rn(wk, q, a1[r]);
+        }
     }
 }
 
-// The transposed sums in the expanded form: with the point s^ held as 2 s^ and
-// a staged partner t as (t^, -|t^|^2), E = 2 s^.t^ - |t^|^2 and
-// K(t,s) = 2^E 2^-|s^|^2 (the last factor applied once per point; E <= |s^|^2,
-// which the pass keeps at most kGrFastT2).  Staged pair j: A = (x0, x1, y0, y1),
-// B = (z0, z1, c0, c1), C = (gE0, gE1, gI0, gI1), D = (index0, index1).
-constexpr float kGrFastT2 = 20.f;
-
-template <bool SELF>
-__device__ __forceinline__ void gr_term_fast(const float4 A, const float4 B, const float4 C,
-                                             const int2 D, float2 tx, float2 ty, float2 tz,
-                                             int32_t e, float2& a0, float2& a1) {
-    const float2 E = __ffma2_rn(tx, make_float2(A.x, A.y),
-                                __ffma2_rn(ty, make_float2(A.z, A.w),
-                                           __ffma2_rn(tz, make_float2(B.x, B.y),
-                                                      make_float2(B.z, B.w))));
-    float2 k = make_float2(gr_ex2(E.x), gr_ex2(E.y));
-    if (SELF) {
-        k.x = D.x == e ? 0.f : k.x;
-        k.y = D.y == e ? 0.f : k.y;
-    }
-    a0 = __ffma2_rn(make_float2(C.x, C.y), k, a0);
-    a1 = __ffma2_rn(make_float2(C.z, C.w), k, a1);
-}
-
-template <bool SELF, int R>
-__device__ __forceinline__ void gr_eval_fast(const float4* sA, const float4* sB, const float4* sC,
-                                             const int2* sD, int mp, int ksl, int slices,
-                                             const float2 (&tx)[R], const float2 (&ty)[R],
-                                             const float2 (&tz)[R], const int32_t (&e)[R],
-                                             float2 (&a0)[R], float2 (&a1)[R]) {
-#pragma unroll 2
-    for (int j = ksl; j < mp; j += slices) {
-        const float4 A = sA[j], B = sB[j], C = sC[j];
-        const int2 D = SELF ? sD[j] : make_int2(0, 0);
-#pragma unroll
-        for (int r = 0; r < R; ++r) gr_term_fast<SELF>(A, B, C, D, tx[r], ty[r], tz[r], e[r], a0[r], a1[r]);
-    }
-}
-
-// One pass over the evaluation points plist[0, np) of leaf L against the
-// partner leaves of pairs [i0, i1).  A lane holds R points (slots R j .. R j
-// + R - 1 of its group j); when the groups fit in fewer lanes they take
-// npr = 2^k lanes and 32 / npr lanes share a group, each walking an
-// interleaved slice of the staged sources.  The 4 warps take the partner
-// leaves round-robin; each packs its partners' points into chunks of 64 in
-// shared memory, in pairs, as scaled positions sqrt(k2) (x - o) relative to a
-// point o of L, and two weights (L's own points last, in chunks of their own,
-// where a point skips itself).  The slices' sums are combined by a fixed butterfly
-// and the 4 warps' in a fixed order, so a point's sum does not depend on the
-// timing of the warps.
-template <bool FORWARD, int R, bool FAST>
-__device__ __forceinline__ void gr_pass(const int32_t* plist, int np, int32_t i0, int32_t i1,
-                                        int32_t L, const float4& O,
-                                        const int32_t* __restrict__ pairs,
-                                        const int32_t* __restrict__ pPart,
-                                        const int32_t* __restrict__ nfirst,
-                                        const int32_t* __restrict__ ncount,
-                                        const float4* __restrict__ pts,
-                                        const float4* __restrict__ gw, float sqk, float4* sAw,
-                                        float4* sBw, float4* sCw, int2* sDw,
-                                        float (*red)[2][kGrList]) {
-    static_assert(!(FAST && FORWARD), "the expanded form serves the transposed sums only");
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int lg = 0;
-    while ((1 << lg) < (np + R - 1) / R) ++lg;
-    const int npr = 1 << lg, slices = 32 >> lg;
-    const int j = lane & (npr - 1), ksl = lane >> lg;
-    const bool active = R * j < np;
+template <int R>
+__device__ __forceinline__ void gr_fwd_pass(const int32_t* list, int np, int32_t i0, int32_t i1,
+                                            int32_t lf, int32_t lc, const float4& O,
+                                            const int2* __restrict__ src,
+                                            const float4* __restrict__ pts,
+                                            const float2* __restrict__ wt,
+                                            const uint16_t* __restrict__ fl, float sqk,
+                                            PsFwdStage& st, int2* meta, float2* red) {
+    const int lane = threadIdx.x & 31;
+    const PsLanes ln(np, R);
     float2 tx[R], ty[R], tz[R], a0[R], a1[R];
-    bool inh[R];
     int32_t e[R];
-    float sc[R];   // FAST: 2^-|s^|^2 of the point
+    bool inh = false;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int slot = R * j + r;
-        const bool v = slot < np;
-        e[r] = v ? plist[slot] : -1;
-        const int32_t pi = v ? e[r] : plist[0];
-        const float4 T = pts[pi];
-        inh[r] = (__float_as_uint(gw[pi].w) & 1u) != 0;
+        const int slot = R * ln.j + r;
+        e[r] = slot < np ? list[slot] : -1;
+        const int32_t t = e[r] >= 0 ? e[r] : lf;
+        if (r == 0) inh = e[0] >= 0 && (fl[t] & kPsInh);
+        const float4 T = pts[t];
+        const float x = (T.x - O.x) * sqk, y = (T.y - O.y) * sqk, z = (T.z - O.z) * sqk;
+        tx[r] = make_float2(x, x);
+        ty[r] = make_float2(y, y);
+        tz[r] = make_float2(z, z);
+        a0[r] = a1[r] = make_float2(0.f, 0.f);
+    }
+    const float4* sW = inh ? st.I : st.E;
+    bool self = false;
+    ps_walk(
+        src, i0, i1, meta,
+        [&](int2 m) {
+            if (m.x == lf) {
+                self = true;
+                m.y = 0;
+            }
+            return m;
+        },
+        [&](int32_t a, int32_t b, bool two, int slot) {
+            ps_stage_fwd(st, pts, wt, a, b, two, slot, O, sqk);
+        },
+        [&](int mp) {
+            gr_fwd_eval<R, false>(st.A, sW, mp, ln.ksl, ln.slices, tx, ty, tz, e, 0, 0, a0, a1);
+        });
+    // L's own points, where a target skips itself
+    if (__any_sync(0xffffffffu, self))
+        for (int32_t p = 0; p < lc; p += kPsUnit) {
+            const int left = min(lc - p, kPsUnit), half = (left + 1) >> 1;
+            __syncwarp();
+            if (lane < half)
+                ps_stage_fwd(st, pts, wt, lf + p + lane, lf + p + half + lane, lane < left - half,
+                             lane, O, sqk);
+            __syncwarp();
+            gr_fwd_eval<R, true>(st.A, sW, half, ln.ksl, ln.slices, tx, ty, tz, e, lf + p,
+                                 lf + p + half, a0, a1);
+        }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float s0 = ln.sum(a0[r].x + a0[r].y), s1 = ln.sum(a1[r].x + a1[r].y);
+        if (ln.ksl == 0 && R * ln.j + r < np) red[R * ln.j + r] = make_float2(s0, s1);
+    }
+}
+
+__global__ void __launch_bounds__(kPsWarps * 32, 6)
+k_grad_forward(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nseg_dev,
+               const int32_t* __restrict__ order, const int32_t* __restrict__ pairs,
+               const int32_t* __restrict__ pX, const int2* __restrict__ src,
+               const int32_t* __restrict__ nfirst, const int32_t* __restrict__ ncount,
+               const float4* __restrict__ pts, const float2* __restrict__ wt,
+               const uint16_t* __restrict__ fl, const int32_t* __restrict__ perm, float sqk,
+               float dscale, float* __restrict__ u, float* __restrict__ du) {
+    __shared__ PsFwdStage st[kPsWarps];
+    __shared__ int2 meta[kPsWarps][32];
+    __shared__ float2 red[kPsWarps][kPsList];
+    __shared__ int32_t list[kPsList];
+    __shared__ int s_np, s_pos, s_R;
+    const int w = threadIdx.x >> 5;
+    const int64_t nseg = *nseg_dev;
+    for (int64_t b = blockIdx.x; b < nseg; b += gridDim.x) {
+        const int32_t sg = order[b], i0 = seg_first[sg], i1 = seg_first[sg + 1];
+        const int32_t L = pX[pairs[i0]], lf = nfirst[L], lc = ncount[L];
+        // positions relative to a point of L before scaling: small operands,
+        // so the differences keep their precision
+        const float4 O = pts[lf];
+        for (int32_t pos = 0; pos < lc;) {
+            // up to 4 R slots a pass; nine paired FP32 instructions a slot
+            // (18 quarter cycles an SM), two 16-byte loads a staged pair
+            if (w == 0)
+                ps_list_targets<kGrFwdR>(fl, lf, lc, pos, kPsList - kGrFwdR + 1, 18, 8, list,
+                                         &s_np, &s_pos, &s_R);
+            __syncthreads();
+            const int np = s_np, R = s_R;
+            pos = s_pos;
+            if (np > 0) {
+#define MSP_GR_FWD(RR)                                                                        \
+    gr_fwd_pass<RR>(list, np, i0, i1, lf, lc, O, src, pts, wt, fl, sqk, st[w], meta[w], red[w])
+                if (R == 1) MSP_GR_FWD(1);
+                else if (R == 2) MSP_GR_FWD(2);
+                else if (R == 3) MSP_GR_FWD(3);
+                else MSP_GR_FWD(4);
+#undef MSP_GR_FWD
+            }
+            __syncthreads();
+            for (int k = threadIdx.x; k < np; k += kPsWarps * 32) {
+                if (list[k] < 0) continue;
+                float2 v = red[0][k];
+#pragma unroll
+                for (int q = 1; q < kPsWarps; ++q) {
+                    v.x += red[q][k].x;
+                    v.y += red[q][k].y;
+                }
+                const int32_t c = perm[list[k]];
+                if (u) u[c] = v.x;
+                if (du) du[c] = v.y * dscale;
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// TRANSPOSED: for every point s of the block's leaf, sum_t g_t K(t,s) over the
+// partner leaves' targets of one channel after the other.  FAST, the expanded
+// form while every point of the pass has |s^|^2 <= kGrFastT2: with the point
+// held as 2 s^ and a staged target as (t^, -|t^|^2), E = 2 s^.t^ - |t^|^2 and
+// K = 2^E 2^-|s^|^2 (the last factor applied once per point; E <= |s^|^2).
+constexpr float kGrFastT2 = 20.f;
+constexpr int kGrAdjR = 5;
+
+template <int R, bool SELF, bool FAST>
+__device__ __forceinline__ void gr_adj_eval(const PsAdjStage& st, int mp, int ksl, int slices,
+                                            const float2 (&tx)[R], const float2 (&ty)[R],
+                                            const float2 (&tz)[R], const int32_t (&e)[R],
+                                            float2 (&acc)[R]) {
+#pragma unroll 2
+    for (int j = ksl; j < mp; j += slices) {
+        const float4 A = st.A[j], B = st.B[j];
+        const float2 C = FAST ? st.C[j] : make_float2(B.z, B.w);
+        const int2 D = SELF ? st.D[j] : make_int2(0, 0);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            float2 K;
+            if (FAST) {
+                const float2 E = __ffma2_rn(
+                    tx[r], make_float2(A.x, A.y),
+                    __ffma2_rn(ty[r], make_float2(A.z, A.w),
+                               __ffma2_rn(tz[r], make_float2(B.x, B.y), make_float2(B.z, B.w))));
+                K = make_float2(ps_ex2(E.x), ps_ex2(E.y));
+            } else {
+                const float2 dx = __fadd2_rn(tx[r], make_float2(A.x, A.y));
+                const float2 dy = __fadd2_rn(ty[r], make_float2(A.z, A.w));
+                const float2 dz = __fadd2_rn(tz[r], make_float2(B.x, B.y));
+                const float2 q = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+                K = make_float2(ps_ex2(-q.x), ps_ex2(-q.y));
+            }
+            if (SELF) {
+                K.x = D.x == e[r] ? 0.f : K.x;
+                K.y = D.y == e[r] ? 0.f : K.y;
+            }
+            acc[r] = __ffma2_rn(C, K, acc[r]);
+        }
+    }
+}
+
+template <int R, bool FAST>
+__device__ __forceinline__ void gr_adj_pass(int32_t first, int np, int32_t i0, int32_t i1,
+                                            int32_t lf, int32_t lc, int64_t n, const float4& O,
+                                            const int2* __restrict__ src,
+                                            const float4* __restrict__ pts, const PsPacked pk,
+                                            const float* __restrict__ pg, float sqk,
+                                            PsAdjStage& st, int2* meta, float2* red) {
+    const int lane = threadIdx.x & 31;
+    const PsLanes ln(np, R);
+    float2 tx[R], ty[R], tz[R], acc[R];
+    float sc[R], sE[R];
+    int32_t e[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int slot = R * ln.j + r;
+        e[r] = first + (slot < np ? slot : 0);
+        const float4 T = pts[e[r]];
         const float x = (T.x - O.x) * sqk, y = (T.y - O.y) * sqk, z = (T.z - O.z) * sqk;
         const float f = FAST ? 2.f : 1.f;
         tx[r] = make_float2(f * x, f * x);
         ty[r] = make_float2(f * y, f * y);
         tz[r] = make_float2(f * z, f * z);
-        sc[r] = FAST ? gr_ex2(-fmaf(x, x, fmaf(y, y, z * z))) : 1.f;
-        a0[r] = make_float2(0.f, 0.f);
-        a1[r] = make_float2(0.f, 0.f);
+        sc[r] = FAST ? ps_ex2(-fmaf(x, x, fmaf(y, y, z * z))) : 1.f;
+        sE[r] = 0.f;
     }
-    int* fD = reinterpret_cast<int*>(sDw);
-    float* fA = reinterpret_cast<float*>(sAw);
-    float* fB = reinterpret_cast<float*>(sBw);
-    float* fC = reinterpret_cast<float*>(sCw);
-    // stage sources [pf + sb, pf + sb + take) at chunk positions fill.. (two
-    // per staged pair); position m of an odd chunk is padded before use
-    auto stage = [&](int32_t pf, int32_t sb, int take, int fill) {
-        for (int k = lane; k < take; k += 32) {
-            const float4 S = pts[pf + sb + k];
-            const float4 W = gw[pf + sb + k];
-            float w0, w1;
-            if (FORWARD) {
-                w0 = W.x;
-                w1 = W.y;
-            } else {
-                const uint32_t f2 = __float_as_uint(W.w);
-                const float gv = (f2 & 2u) ? W.z : 0.f;
-                w0 = (f2 & 1u) ? 0.f : gv;
-                w1 = (f2 & 1u) ? gv : 0.f;
-            }
-            const int pos = fill + k, jj = pos >> 1, h = pos & 1;
-            if (FAST) {
-                const float sx = (S.x - O.x) * sqk, sy = (S.y - O.y) * sqk,
-                            sz = (S.z - O.z) * sqk;
-                fA[4 * jj + h] = sx;
-                fA[4 * jj + 2 + h] = sy;
-                fB[4 * jj + h] = sz;
-                fB[4 * jj + 2 + h] = -fmaf(sx, sx, fmaf(sy, sy, sz * sz));
-                fC[4 * jj + h] = w0;
-                fC[4 * jj + 2 + h] = w1;
-                fD[2 * jj + h] = pf + sb + k;
-            } else {
-                fA[4 * jj + h] = -(S.x - O.x) * sqk;
-                fA[4 * jj + 2 + h] = -(S.y - O.y) * sqk;
-                fB[4 * jj + h] = -(S.z - O.z) * sqk;
-                fB[4 * jj + 2 + h] = w0;
-                fC[4 * jj + h] = w1;
-                fC[4 * jj + 2 + h] = __int_as_float(pf + sb + k);
-            }
-        }
-    };
-    auto pad = [&](int m) {
-        if ((m & 1) && lane == 0) {
-            const int jj = m >> 1;
-            fA[4 * jj + 1] = 0.f;
-            fA[4 * jj + 3] = 0.f;
-            fB[4 * jj + 1] = 0.f;
-            fB[4 * jj + 3] = 0.f;
-            fC[4 * jj + 1] = 0.f;
-            fC[4 * jj + 3] = FAST ? 0.f : __int_as_float(-1);
-            if (FAST) fD[2 * jj + 1] = -1;
-        }
-    };
-    // the staged pairs [0, mp) against the lane's points
-    auto eval = [&](int mp, bool selfc) {
-        if (!active) return;
+    auto stage = [&](int32_t a, int32_t b, bool two, int slot) {
+        const float4 S0 = pk.pt[a], S1 = pk.pt[two ? b : a];
+        const float2 g = make_float2(pg[a], two ? pg[b] : 0.f);
+        const float2 k = make_float2(sqk, sqk);
+        float2 x = __fmul2_rn(__fadd2_rn(make_float2(S0.x, S1.x), make_float2(-O.x, -O.x)), k);
+        float2 y = __fmul2_rn(__fadd2_rn(make_float2(S0.y, S1.y), make_float2(-O.y, -O.y)), k);
+        float2 z = __fmul2_rn(__fadd2_rn(make_float2(S0.z, S1.z), make_float2(-O.z, -O.z)), k);
         if (FAST) {
-            if (selfc)
-                gr_eval_fast<true, R>(sAw, sBw, sCw, sDw, mp, ksl, slices, tx, ty, tz, e, a0, a1);
-            else
-                gr_eval_fast<false, R>(sAw, sBw, sCw, sDw, mp, ksl, slices, tx, ty, tz, e, a0,
-                                       a1);
+            const float2 q = __ffma2_rn(x, x, __ffma2_rn(y, y, __fmul2_rn(z, z)));
+            st.A[slot] = make_float4(x.x, x.y, y.x, y.y);
+            st.B[slot] = make_float4(z.x, z.y, -q.x, -q.y);
+            st.C[slot] = g;
         } else {
-            if (selfc)
-                gr_eval<FORWARD, true, R>(sAw, sBw, sCw, mp, ksl, slices, tx, ty, tz, inh, e, a0,
-                                          a1);
-            else
-                gr_eval<FORWARD, false, R>(sAw, sBw, sCw, mp, ksl, slices, tx, ty, tz, inh, e,
-                                           a0, a1);
+            st.A[slot] = make_float4(-x.x, -x.y, -y.x, -y.y);
+            st.B[slot] = make_float4(-z.x, -z.y, g.x, g.y);
         }
+        st.D[slot] = make_int2(__float_as_int(S0.w), two ? __float_as_int(S1.w) : -1);
     };
-    // the partner leaves other than L, packed into full chunks (the sums
-    // need no per-pair result); then L itself, whose terms skip t = s
-    int fill = 0;
-    bool self = false;
-    for (int32_t i = i0 + w; i < i1; i += kGrWarps) {
-        const int32_t P = pPart[pairs[i]];
-        if (P == L) {
-            self = true;
-            continue;
-        }
-        const int32_t pf = nfirst[P], pc = ncount[P];
-        for (int32_t sb = 0; sb < pc;) {
-            const int take = min(kGrStage - fill, pc - sb);
-            stage(pf, sb, take, fill);
-            fill += take;
-            sb += take;
-            if (fill == kGrStage) {
+#pragma unroll 1
+    for (int ch = 0; ch < 2; ++ch) {
+        const int32_t* off = pk.off + ch * n;
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = make_float2(0.f, 0.f);
+        bool self = false;
+        ps_walk(
+            src, i0, i1, meta,
+            [&](int2 m) {
+                if (m.x == lf) {
+                    self = true;
+                    return make_int2(0, 0);
+                }
+                const int32_t a = off[m.x];
+                return make_int2(a, off[m.x + m.y] - a);
+            },
+            stage,
+            [&](int mp) {
+                gr_adj_eval<R, false, FAST>(st, mp, ln.ksl, ln.slices, tx, ty, tz, e, acc);
+            });
+        // L's own targets, where a point skips itself
+        if (__any_sync(0xffffffffu, self)) {
+            const int32_t a0 = off[lf], a1 = off[lf + lc];
+            for (int32_t p = a0; p < a1; p += kPsUnit) {
+                const int left = min(a1 - p, kPsUnit), half = (left + 1) >> 1;
                 __syncwarp();
-                eval(kGrStage / 2, false);
+                if (lane < half) stage(p + lane, p + half + lane, lane < left - half, lane);
                 __syncwarp();
-                fill = 0;
+                gr_adj_eval<R, true, FAST>(st, half, ln.ksl, ln.slices, tx, ty, tz, e, acc);
             }
         }
-    }
-    if (fill > 0) {
-        pad(fill);
-        __syncwarp();
-        eval((fill + 1) >> 1, false);
-        __syncwarp();
-    }
-    if (self) {
-        const int32_t pf = nfirst[L], pc = ncount[L];
-        for (int32_t sb = 0; sb < pc; sb += kGrStage) {
-            const int m = min(kGrStage, pc - sb);
-            stage(pf, sb, m, 0);
-            pad(m);
-            __syncwarp();
-            eval((m + 1) >> 1, true);
-            __syncwarp();
-        }
-    }
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        float s0 = a0[r].x + a0[r].y, s1 = a1[r].x + a1[r].y;
-        for (int o = npr; o < 32; o <<= 1) {
-            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        }
-        if (FAST) {
-            s0 *= sc[r];
-            s1 *= sc[r];
-        }
-        const int slot = R * j + r;
-        if (ksl == 0 && slot < np) {
-            red[w][0][slot] = s0;
-            red[w][1][slot] = s1;
+        for (int r = 0; r < R; ++r) {
+            const float v = ln.sum(acc[r].x + acc[r].y) * sc[r];
+            if (ch == 0) {
+                sE[r] = v;
+            } else if (ln.ksl == 0 && R * ln.j + r < np) {
+                red[R * ln.j + r] = make_float2(sE[r], v);
+            }
         }
     }
 }
 
-// One block per leaf L of a segment list (the evaluation leaf; with `order`,
-// the segments longest first), its 4 warps taking the segment's partner
-// leaves P.  Warp 0 lists L's evaluation points, up to kGrList per pass
-// (FORWARD: the targets, a_t > 0; ADJOINT: every point), and the pass holds R
-// = 1..3 of them per lane, R the fewest evaluated slots per source (ties to
-// the larger R: fewer shared-memory loads per evaluation).
-//   FORWARD: evaluation points = targets t (a_t > 0), partner weights
-//            (w^E, w^I): u += w^{T(t)} 2^-q, d += w^{T(t)} q 2^-q.
-//   ADJOINT: evaluation points = sources s, partner weights
-//            (g_t [T(t) = E], g_t [T(t) = I]) (0 unless a_t > 0):
-//            gE += w0 2^-q, gI += w1 2^-q.
-// Points that are not evaluated keep the zero the caller wrote.
-template <bool FORWARD>
-__global__ void __launch_bounds__(kGrWarps * 32, 7)
-k_grad_pairs(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nseg_dev,
-             const int32_t* __restrict__ order, const int32_t* __restrict__ pairs,
-             const int32_t* __restrict__ pEval, const int32_t* __restrict__ pPart,
-             const int32_t* __restrict__ nfirst, const int32_t* __restrict__ ncount,
-             const float4* __restrict__ pts, const float4* __restrict__ gw,
-             const int32_t* __restrict__ perm, float sqk, float dscale, float* __restrict__ out0,
-             float* __restrict__ out1) {
-    __shared__ float4 sA[kGrWarps][kGrStage / 2], sB[kGrWarps][kGrStage / 2],
-        sC[kGrWarps][kGrStage / 2];
-    __shared__ int2 sD[kGrWarps][kGrStage / 2];
-    __shared__ float red[kGrWarps][2][kGrList];
-    __shared__ int32_t plist[kGrList];
-    __shared__ int s_np, s_pos;
+__global__ void __launch_bounds__(kPsWarps * 32, 6)
+k_grad_adjoint(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nseg_dev,
+               const int32_t* __restrict__ order, const int32_t* __restrict__ pairs,
+               const int32_t* __restrict__ pX, const int2* __restrict__ src,
+               const int32_t* __restrict__ nfirst, const int32_t* __restrict__ ncount, int64_t n,
+               const float4* __restrict__ pts, const PsPacked pk, const float* __restrict__ pg,
+               const int32_t* __restrict__ perm, float sqk, float* __restrict__ gE,
+               float* __restrict__ gI) {
+    __shared__ PsAdjStage st[kPsWarps];
+    __shared__ int2 meta[kPsWarps][32];
+    __shared__ float2 red[kPsWarps][kPsList];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nseg = *nseg_dev;
     for (int64_t b = blockIdx.x; b < nseg; b += gridDim.x) {
-        const int64_t sg = order ? order[b] : b;
-        const int32_t i0 = seg_first[sg], i1 = seg_first[sg + 1];
-        const int32_t L = pEval[pairs[i0]];
-        const int32_t lf = nfirst[L], lc = ncount[L];
-        // positions relative to a point of L before scaling: small operands,
-        // so the differences keep their precision
+        const int32_t sg = order[b], i0 = seg_first[sg], i1 = seg_first[sg + 1];
+        const int32_t L = pX[pairs[i0]], lf = nfirst[L], lc = ncount[L];
         const float4 O = pts[lf];
-        int32_t pos = 0;
-        for (;;) {
-            if (w == 0) {
-                // the next (at most) kGrList evaluation points from pos on
-                int np = 0;
-                int32_t p = pos;
-                while (p < lc && np < kGrList) {
-                    const int32_t idx = p + lane;
-                    bool ok = idx < lc;
-                    if (FORWARD && ok) ok = (__float_as_uint(gw[lf + idx].w) & 2u) != 0;
-                    const unsigned mk = __ballot_sync(0xffffffffu, ok);
-                    const int room = kGrList - np;
-                    const int rank = __popc(mk & ((1u << lane) - 1u));
-                    if (ok && rank < room) plist[np + rank] = lf + idx;
-                    if (__popc(mk) > room) {
-                        // the room-th point ends the pass: resume after it
-                        unsigned keep = mk;
-                        for (int k = 0; k < room; ++k) keep &= keep - 1u;
-                        p += __ffs(keep) - 1;
-                        np = kGrList;
-                        break;
-                    }
-                    np += __popc(mk);
-                    p += 32;
-                }
-                if (lane == 0) {
-                    s_np = np;
-                    s_pos = min(p, lc);
-                }
+        for (int32_t pos = 0; pos < lc; pos += kPsList) {
+            const int np = min(lc - pos, kPsList);
+            // expanded form: four paired FP32 instructions a slot, 40 bytes a
+            // staged pair; the same choice in every warp
+            const int R = ps_choose_r<kGrAdjR>([&](int) { return np; }, 8, 10);
+            float m2 = 0.f;
+            for (int k = lane; k < np; k += 32) {
+                const float4 T = pts[lf + pos + k];
+                const float x = (T.x - O.x) * sqk, y = (T.y - O.y) * sqk, z = (T.z - O.z) * sqk;
+                m2 = fmaxf(m2, fmaf(x, x, fmaf(y, y, z * z)));
             }
+            for (int o = 16; o > 0; o >>= 1) m2 = fmaxf(m2, __shfl_xor_sync(0xffffffffu, m2, o));
+            const bool fast = m2 <= kGrFastT2;
+#define MSP_GR_ADJ(RR, FF)                                                                      \
+    gr_adj_pass<RR, FF>(lf + pos, np, i0, i1, lf, lc, n, O, src, pts, pk, pg, sqk, st[w],       \
+                        meta[w], red[w])
+            if (!fast) {
+                // wide leaves: few, two points a lane up to 64, else four
+                if (np <= 64) MSP_GR_ADJ(2, false);
+                else MSP_GR_ADJ(4, false);
+            } else if (R == 1) MSP_GR_ADJ(1, true);
+            else if (R == 2) MSP_GR_ADJ(2, true);
+            else if (R == 3) MSP_GR_ADJ(3, true);
+            else if (R == 4) MSP_GR_ADJ(4, true);
+            else MSP_GR_ADJ(5, true);
+#undef MSP_GR_ADJ
             __syncthreads();
-            const int np = s_np;
-            pos = s_pos;
-            __syncthreads();
-            if (np == 0) break;
-            int R = 1, best = 1 << 30;
-            for (int rr = 1; rr <= kGrMaxR; ++rr) {
-                const int g = (np + rr - 1) / rr;
-                if (g > 32) continue;
-                int npr = 1;
-                while (npr < g) npr <<= 1;
-                if (npr * rr <= best) {
-                    best = npr * rr;
-                    R = rr;
-                }
-            }
-            // the transposed sums take the expanded form while every point of
-            // the pass has |s^|^2 <= kGrFastT2 (the same value in every warp)
-            bool fast = false;
-            if (!FORWARD) {
-                float m2 = 0.f;
-                for (int k = lane; k < np; k += 32) {
-                    const float4 T = pts[plist[k]];
-                    const float x = (T.x - O.x) * sqk, y = (T.y - O.y) * sqk,
-                                z = (T.z - O.z) * sqk;
-                    m2 = fmaxf(m2, fmaf(x, x, fmaf(y, y, z * z)));
-                }
-                for (int o = 16; o > 0; o >>= 1) m2 = fmaxf(m2, __shfl_xor_sync(0xffffffffu, m2, o));
-                fast = m2 <= kGrFastT2;
-            }
-#define MSP_GR_PASS(RR, FF)                                                                   \
-    gr_pass<FORWARD, RR, FF>(plist, np, i0, i1, L, O, pairs, pPart, nfirst, ncount, pts, gw, sqk, \
-                             sA[w], sB[w], sC[w], sD[w], red)
-            if (!FORWARD && fast) {
-                if (R == 1) MSP_GR_PASS(1, !FORWARD);
-                else if (R == 2) MSP_GR_PASS(2, !FORWARD);
-                else MSP_GR_PASS(3, !FORWARD);
-            } else {
-                if (R == 1) MSP_GR_PASS(1, false);
-                else if (R == 2) MSP_GR_PASS(2, false);
-                else MSP_GR_PASS(3, false);
-            }
-#undef MSP_GR_PASS
-            __syncthreads();
-            if (w == 0) {
+            for (int k = threadIdx.x; k < np; k += kPsWarps * 32) {
+                float2 v = red[0][k];
 #pragma unroll
-                for (int r = 0; r < kGrMaxR; ++r) {
-                    const int j = lane + 32 * r;
-                    if (j >= np) continue;
-                    float s0 = red[0][0][j], s1 = red[0][1][j];
-#pragma unroll
-                    for (int k = 1; k < kGrWarps; ++k) {
-                        s0 += red[k][0][j];
-                        s1 += red[k][1][j];
-                    }
-                    const int32_t c = perm[plist[j]];
-                    if (FORWARD) {
-                        if (out0) out0[c] = s0;
-                        if (out1) out1[c] = s1 * dscale;
-                    } else {
-                        out0[c] = s0;
-                        out1[c] = s1;
-                    }
+                for (int q = 1; q < kPsWarps; ++q) {
+                    v.x += red[q][k].x;
+                    v.y += red[q][k].y;
                 }
+                const int32_t c = perm[lf + pos + k];
+                if (gE) gE[c] = v.x;
+                if (gI) gI[c] = v.y;
             }
             __syncthreads();
-            if (pos >= lc) break;
         }
     }
-}
-
-// pair list regrouped by source leaf: key = source leaf, value = pair index
-__global__ void k_grad_keys(const int32_t* __restrict__ list_q, const int64_t* __restrict__ n_dev,
-                            const int32_t* __restrict__ pY, uint64_t* __restrict__ key,
-                            int32_t* __restrict__ val) {
-    const int64_t n = *n_dev;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t q = list_q[i];
-        key[i] = (uint64_t)pY[q];
-        val[i] = q;
-    }
-}
-
-__global__ void k_grad_seg_flags(const uint64_t* __restrict__ key, const int64_t* __restrict__ n_dev,
-                                 int32_t* __restrict__ flag) {
-    const int64_t n = *n_dev;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        flag[i] = i == 0 || key[i] != key[i - 1];
-}
-
-__global__ void k_grad_seg_first(const int32_t* __restrict__ flag, const int32_t* __restrict__ off,
-                                 const int64_t* __restrict__ n_dev,
-                                 const int64_t* __restrict__ nseg_dev,
-                                 int32_t* __restrict__ seg_first) {
-    const int64_t n = *n_dev;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        if (flag[i]) seg_first[off[i]] = (int32_t)i;
-    if (blockIdx.x == 0 && threadIdx.x == 0) seg_first[*nseg_dev] = (int32_t)n;
-}
-
-int bits_for_grad(int64_t v) {
-    int b = 1;
-    while (b < 63 && (1ll << b) <= v) ++b;
-    return b;
 }
 
 }  // namespace
 
-// The near-field pair list regrouped by source leaf (device radix sort of the
-// pair indices by Y): *list receives the pair indices, *segf the first list
-// entry of every source leaf's segment (segment count in dcounts(c)->scan_n).
-void pairs_by_source(msp_ctx& c, cudaStream_t s, const int32_t** segf_out,
-                     const int32_t** list_out) {
+const int32_t* ps_offsets(msp_ctx& c, const uint16_t* fl, cudaStream_t s) {
+    const int64_t n = c.n;
     DevCounts* dc = dcounts(c);
-    const int B = 256;
-    const int64_t nseg_cap = std::max<int64_t>(c.n_nodes, 1);
-    const int64_t cap = std::max<int64_t>(c.n_p2p, 1);
-    uint64_t* k0 = c.gr_key0.ensure<uint64_t>((size_t)cap);
-    uint64_t* k1 = c.gr_key1.ensure<uint64_t>((size_t)cap);
-    int32_t* v0 = c.gr_val0.ensure<int32_t>((size_t)cap);
-    int32_t* v1 = c.gr_val1.ensure<int32_t>((size_t)cap);
-    int32_t* flag = c.gr_flag.ensure<int32_t>((size_t)cap);
-    int32_t* off = c.gr_off.ensure<int32_t>((size_t)cap);
-    int32_t* segf = c.gr_seg.ensure<int32_t>((size_t)nseg_cap + 2);
-    const int Gp = grid_for(cap, B, (int64_t)c.sm_count * 16);
-    k_grad_keys<<<Gp, B, 0, s>>>(c.p2p_val0.get<int32_t>(), &dc->n_p2p, c.pr_Y.get<int32_t>(),
-                                 k0, v0);
-    MSP_LAUNCH("grad_keys");
-    radix_sort_dev(c, k0, v0, k1, v1, &dc->n_p2p, cap, bits_for_grad(c.n_nodes), s);
-    k_grad_seg_flags<<<Gp, B, 0, s>>>(k0, &dc->n_p2p, flag);
-    MSP_LAUNCH("grad_seg_flags");
-    scan_dev(c, flag, off, &dc->n_p2p, cap, &dc->scan_n, nullptr, s);
-    k_grad_seg_first<<<Gp, B, 0, s>>>(flag, off, &dc->n_p2p, &dc->scan_n, segf);
-    MSP_LAUNCH("grad_seg_first");
-    *segf_out = segf;
-    *list_out = v0;
+    int32_t* flag = c.gr_flag.ensure<int32_t>((size_t)2 * n + 1);
+    int32_t* off = c.gr_off.ensure<int32_t>((size_t)2 * n + 1);
+    k_ps_flags<<<grid_for(n, 256, (int64_t)c.sm_count * 16), 256, 0, s>>>(n, fl, flag, &dc->scan_n);
+    MSP_LAUNCH("ps_flags");
+    scan_dev(c, flag, off, &dc->scan_n, 2 * n + 1, nullptr, nullptr, s);
+    return off;
 }
 
 void attraction_grad(msp_ctx& c, const uint8_t* type, const uint8_t* va, const uint8_t* vde,
@@ -537,36 +439,39 @@ void attraction_grad(msp_ctx& c, const uint8_t* type, const uint8_t* va, const u
     const int B = 256;
     const int G = grid_for(n, B, (int64_t)c.sm_count * 16);
     DevCounts* dc = dcounts(c);
-    float4* gw = c.gr_w.ensure<float4>((size_t)n);
-    k_grad_gather<<<G, B, 0, s>>>(n, c.perm.get<int32_t>(), type, va, vde, vdi, g, gw);
+    float2* wt = c.gr_w.ensure<float2>((size_t)n);
+    uint16_t* fl = c.gr_fl.ensure<uint16_t>((size_t)n);
+    const int32_t* perm = c.perm.get<int32_t>();
+    k_grad_gather<<<G, B, 0, s>>>(n, perm, type, va, vde, vdi, wt, fl);
     MSP_LAUNCH("grad_gather");
     const float sqk = (float)std::sqrt(1.4426950408889634 / (cfg.sigma * cfg.sigma));
     const float dscale = (float)(2.0 / (cfg.sigma * 1.4426950408889634));
-    const int64_t nseg_cap = std::max<int64_t>(c.n_nodes, 1);
-    const int32_t* list_q = c.p2p_val0.get<int32_t>();
-    const int nb = (int)std::min<int64_t>(nseg_cap, 1 << 30);
+    // the segments in the near field's order (longest first) and its source
+    // ranges, kept with the lists
+    const int32_t *segf = c.seg_first.get<int32_t>(), *order = c.nf_oval0.get<int32_t>(),
+                  *list = c.p2p_val0.get<int32_t>(), *pX = c.pr_X.get<int32_t>(),
+                  *nfirst = c.nd_first.get<int32_t>(), *ncount = c.nd_count.get<int32_t>();
+    const int2* src = c.nf_src.get<int2>();
+    const float4* pts = c.pts.get<float4>();
+    const int nb = (int)std::min<int64_t>(std::max<int64_t>(c.n_nodes, 1), 1 << 30);
     if (u || dud) {
         if (u) MSP_CUDA(cudaMemsetAsync(u, 0, (size_t)n * sizeof(float), s));
         if (dud) MSP_CUDA(cudaMemsetAsync(dud, 0, (size_t)n * sizeof(float), s));
-        // the segments in the near field's order (longest first), kept with the lists
-        k_grad_pairs<true><<<nb, kGrWarps * 32, 0, s>>>(
-            c.seg_first.get<int32_t>(), &dc->nseg, c.nf_oval0.get<int32_t>(), list_q,
-            c.pr_X.get<int32_t>(),
-            c.pr_Y.get<int32_t>(), c.nd_first.get<int32_t>(), c.nd_count.get<int32_t>(),
-            c.pts.get<float4>(), gw, c.perm.get<int32_t>(), sqk, dscale, u, dud);
+        k_grad_forward<<<nb, kPsWarps * 32, 0, s>>>(segf, &dc->nseg, order, list, pX, src, nfirst,
+                                                    ncount, pts, wt, fl, perm, sqk, dscale, u, dud);
         MSP_LAUNCH("grad_forward");
     }
     if (gE || gI) {
-        float* oE = gE ? gE : c.gr_tmp.ensure<float>((size_t)n);
-        float* oI = gI ? gI : c.gr_tmp.ensure<float>((size_t)n);
-        MSP_CUDA(cudaMemsetAsync(oE, 0, (size_t)n * sizeof(float), s));
-        MSP_CUDA(cudaMemsetAsync(oI, 0, (size_t)n * sizeof(float), s));
-        const int32_t *segf = nullptr, *v0 = nullptr;
-        pairs_by_source(c, s, &segf, &v0);
-        k_grad_pairs<false><<<nb, kGrWarps * 32, 0, s>>>(
-            segf, &dc->scan_n, nullptr, v0, c.pr_Y.get<int32_t>(), c.pr_X.get<int32_t>(),
-            c.nd_first.get<int32_t>(), c.nd_count.get<int32_t>(), c.pts.get<float4>(), gw,
-            c.perm.get<int32_t>(), sqk, dscale, oE, oI);
+        if (gE) MSP_CUDA(cudaMemsetAsync(gE, 0, (size_t)n * sizeof(float), s));
+        if (gI) MSP_CUDA(cudaMemsetAsync(gI, 0, (size_t)n * sizeof(float), s));
+        const int32_t* off = ps_offsets(c, fl, s);
+        float4* pt = c.gr_pt.ensure<float4>((size_t)n);
+        float* pg = c.gr_tmp.ensure<float>((size_t)n);
+        k_grad_pack<<<G, B, 0, s>>>(n, fl, off, perm, pts, g, pt, pg);
+        MSP_LAUNCH("grad_pack");
+        k_grad_adjoint<<<nb, kPsWarps * 32, 0, s>>>(segf, &dc->nseg, order, list, pX, src, nfirst,
+                                                    ncount, n, pts, PsPacked{pt, off}, pg, perm,
+                                                    sqk, gE, gI);
         MSP_LAUNCH("grad_adjoint");
     }
 }

@@ -221,7 +221,7 @@ struct msp_ctx {
     msp::DBuf nd_gc, gm_key0, gm_key1, gm_q, gm_q1, gm_flag, gm_gid, gm_gstart, gm_ntile,
         gm_toff, gm_tiles, gm_cnt;
     // derivatives (msp_grad.cu)
-    msp::DBuf gr_w, gr_tmp, gr_key0, gr_key1, gr_val0, gr_val1, gr_flag, gr_off, gr_seg;
+    msp::DBuf gr_w, gr_fl, gr_tmp, gr_pt, gr_flag, gr_off;
     // expected synapse length (msp_length.cu): per-target sums, block
     // partials and results, per-target coefficients of the transposed sums
     msp::DBuf ln_sums, ln_part, ln_coef;

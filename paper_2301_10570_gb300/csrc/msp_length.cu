@@ -14,32 +14,34 @@
 //               alpha_t = a_t / (A u), beta_t = a_t v / (A u^2),
 // and every loss derivative is 2 (m - target) times m's.  The sums run over
 // the near-field leaf pairs of the last attraction (a plan without
-// translations: K r has no Hermite expansion), first grouped by target leaf
-// (u, v and their sigma derivatives), then by source leaf (the transposed
-// sums).  One block of 4 warps per leaf, 1-2 evaluation points per lane,
-// the warps taking the partner leaves; the partners' points are staged in
-// shared memory, and each staged chunk's sum is added with Kahan's
-// compensated summation.  Every sum has a fixed order, so
-// the results are reproducible; the scalar reductions run in double.
+// translations: K r has no Hermite expansion), u, v and their sigma
+// derivatives per target leaf, then the transposed sums per source leaf over
+// its partner leaves' targets of one channel after the other (both walks in
+// msp_pairsum.cuh).  Coordinates are scaled by sqk = sqrt(log2 e)/sigma
+// relative to the leaf's first point, so that q = |t^ - s^|^2 gives K = 2^-q
+// and r = rs sqrt(q), rs = sigma/sqrt(log2 e); rs is applied to the sums.
+// A lane's sums join its running totals by Kahan's compensated summation
+// after every 64 staged points (the transposed terms are signed: their partial
+// sums exceed their total; a fold per 32 partner leaves raised the error of
+// the weight gradients from 3.4e-7 to 4.7e-7).  Every sum has a fixed order, so the results are
+// reproducible; the scalar reductions run in double.
+//
+// Bound by the FP32 pipe, the special function unit (EX2 and SQRT per term)
+// and instruction issue.  131,072 clustered neurons (cutoff 5 sigma, leaf
+// capacity 128), against chunks of 32 with mixed channels per lane, in no order
+// of length, and a list sorted anew by source leaf: forward 1.51 -> 0.82 ms
+// (1.06 -> 0.60 G warp instructions), transposed 1.67 + 0.1 -> 0.64 + 0.02 ms;
+// the blocks' partials by one thread cost another 0.08 ms.
 #include <algorithm>
 #include <cmath>
 
-#include "msp_internal.cuh"
+#include "msp_pairsum.cuh"
 
 namespace msp {
-
-void pairs_by_source(msp_ctx& c, cudaStream_t s, const int32_t** segf_out,
-                     const int32_t** list_out);
 
 namespace {
 
 constexpr double kLog2e = 1.4426950408889634;
-
-__device__ inline float len_ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 __device__ inline float len_sqrt(float x) {
     float y;
@@ -54,361 +56,384 @@ __device__ inline void kahan_add(float& acc, float& cmp, float v) {
     acc = t;
 }
 
-// sorted-order inputs: {w^E, w^I, a, type}
+// sorted-order inputs: the weights, and the flags with a in the high byte
 __global__ void k_len_gather(int64_t n, const int32_t* __restrict__ perm,
                              const uint8_t* __restrict__ type, const uint8_t* __restrict__ va,
                              const float* __restrict__ we, const float* __restrict__ wi,
-                             float4* __restrict__ gw) {
+                             float2* __restrict__ w, uint16_t* __restrict__ fl) {
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
          s += (int64_t)gridDim.x * blockDim.x) {
         const int32_t c = perm[s];
-        gw[s] = make_float4(we[c], wi[c], (float)va[c], type[c] ? 1.f : 0.f);
+        w[s] = make_float2(we[c], wi[c]);
+        fl[s] = (uint16_t)((type[c] ? kPsInh : 0u) | (va[c] ? kPsAct : 0u) | ((uint32_t)va[c] << 8));
     }
 }
 
-constexpr int kLenWarps = 4;
-constexpr int kLenStage = 32;    // staged sources per warp and chunk
+__device__ __forceinline__ float len_count(uint16_t f) { return (float)(f >> 8); }
 
-// One block of 4 warps per leaf L of a segment list.  The leaf's points are
-// taken 32 at a time, one per lane, and every warp holds the same points; the
-// warps take the segment's partner leaves P round-robin, each packing its
-// partners' points into chunks of 32 in its own shared memory, and every
-// chunk's sum joins the lane's running sums by Kahan's compensated summation.
-// The 4 warps' compensated sums are added in a fixed order.  Coordinates are
-// scaled by sqk = sqrt(log2 e)/sigma relative to L's first point, so that
-// q = |t^ - s^|^2 gives K = 2^-q and r = rs sqrt(q), rs = sigma/sqrt(log2 e);
-// a point skips itself (by index).
-//   FORWARD (L = the target leaf): per target t with a_t > 0, the sums
-//     U = sum w K, V = sum w K r, QU = sum w K q, QV = sum w K q r
-//     (w: the staged source's weight of t's channel), written in sorted order.
-//   ADJOINT (L = the source leaf): per point s, for each channel T,
-//     G_T = sum_{t: T(t) = T} K (alpha_t r - beta_t)
-//     over the staged targets t (coefficients in cf), written in caller order.
-constexpr int kLenMaxR = 2;                 // evaluation points per lane
-constexpr int kLenList = 32 * kLenMaxR;     // evaluation points per pass
+// A lane's running totals with their compensations, N per slot, in shared
+// memory (touched once per unit; the registers are the loop's)
+template <int R, int N>
+struct LenTotals {
+    float* p;      // this thread's entry; entries lie kPsWarps * 32 floats apart
+    __device__ explicit LenTotals(float* base) : p(base + threadIdx.x) {
+        for (int k = 0; k < 2 * R * N; ++k) p[k * kPsWarps * 32] = 0.f;
+    }
+    __device__ void add(int k, float v) const {
+        float acc = p[2 * k * kPsWarps * 32], cmp = p[(2 * k + 1) * kPsWarps * 32];
+        kahan_add(acc, cmp, v);
+        p[2 * k * kPsWarps * 32] = acc;
+        p[(2 * k + 1) * kPsWarps * 32] = cmp;
+    }
+    __device__ float get(int k) const {
+        return __fsub_rn(p[2 * k * kPsWarps * 32], p[(2 * k + 1) * kPsWarps * 32]);
+    }
+};
 
-// The staged pairs j = ksl, ksl + slices, ... < mp of a chunk against the
-// lane's R points t[r], into their compensated running sums acc/cmp (4 each).
-// Staged pair j (sources 2j, 2j + 1):
-//   A = (-x0, -x1, -y0, -y1), B = (-z0, -z1, index0, index1),
-//   C = FORWARD: (w^E_0, w^E_1, w^I_0, w^I_1); ADJOINT: (alpha0, alpha1,
-//       beta0, beta1),
-//   D = ADJOINT: (I0, I1, E0, E1), the sources' channels as 0/1,
-// a padding source with zero weights; every step is a paired FP32
-// instruction over the two sources (two results, one issue slot) with the
-// per-element rounding of the scalar form.  SELF: a source may be t itself;
-// its term is zero.
-template <bool FORWARD, bool SELF, int R>
-__device__ __forceinline__ void len_eval(const float4* sA, const float4* sB, const float4* sC,
-                                         const float4* sD, int mp, int ksl, int slices,
-                                         const int32_t (&t)[R], const bool (&inh)[R],
-                                         const float2 (&tx)[R], const float2 (&ty)[R],
-                                         const float2 (&tz)[R], float rs, float (&acc)[R][4],
-                                         float (&cmp)[R][4]) {
-    const float2 rs2 = make_float2(rs, rs);
-    float2 p[R][4];
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) p[r][c] = make_float2(0.f, 0.f);
-    for (int j = ksl; j < mp; j += slices) {
-        const float4 A = sA[j], B = sB[j], C = sC[j];
-        float4 D = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (!FORWARD) D = sD[j];
+// FORWARD: per target t with a_t > 0, over the staged sources (w: the source's
+// weight of t's channel)
+//   U = sum w K, V = sum w K sqrt(q), QU = sum w K q, QV = sum w K q sqrt(q)
+// (V and QV in units of rs).  SELF: a source may be t itself; its
+// kernel is zero.
+constexpr int kLenFwdR = 3;
+
+template <int R, bool SELF>
+__device__ __forceinline__ void len_fwd_eval(const float4* sA, const float4* sW, int j0, int mp,
+                                             int slices, const float2 (&tx)[R],
+                                             const float2 (&ty)[R], const float2 (&tz)[R],
+                                             const int32_t (&e)[R], int32_t first, int32_t second,
+                                             float2 (&p)[R][4]) {
+    for (int j = j0; j < mp; j += slices) {
+        const float4 A = sA[j], B = sW[j];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const float2 dx = __fadd2_rn(tx[r], make_float2(A.x, A.y));
             const float2 dy = __fadd2_rn(ty[r], make_float2(A.z, A.w));
             const float2 dz = __fadd2_rn(tz[r], make_float2(B.x, B.y));
             const float2 q = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-            float2 K = make_float2(len_ex2(-q.x), len_ex2(-q.y));
+            float2 K = make_float2(ps_ex2(-q.x), ps_ex2(-q.y));
             if (SELF) {
-                K.x = __float_as_int(B.z) == t[r] ? 0.f : K.x;
-                K.y = __float_as_int(B.w) == t[r] ? 0.f : K.y;
+                K.x = first + j == e[r] ? 0.f : K.x;
+                K.y = second + j == e[r] ? 0.f : K.y;
             }
-            const float2 rr = __fmul2_rn(rs2, make_float2(len_sqrt(q.x), len_sqrt(q.y)));
-            if (FORWARD) {
-                const float2 wk =
-                    __fmul2_rn(inh[r] ? make_float2(C.z, C.w) : make_float2(C.x, C.y), K);
-                p[r][0] = __fadd2_rn(p[r][0], wk);
-                p[r][1] = __ffma2_rn(wk, rr, p[r][1]);
-                p[r][2] = __ffma2_rn(wk, q, p[r][2]);
-                p[r][3] = __ffma2_rn(__fmul2_rn(wk, q), rr, p[r][3]);
-            } else {
-                const float2 v = __fmul2_rn(K, __ffma2_rn(make_float2(C.x, C.y), rr,
-                                                          make_float2(-C.z, -C.w)));
-                p[r][1] = __ffma2_rn(make_float2(D.x, D.y), v, p[r][1]);
-                p[r][0] = __ffma2_rn(make_float2(D.z, D.w), v, p[r][0]);
-            }
+            const float2 wk = __fmul2_rn(make_float2(B.z, B.w), K);
+            const float2 wr = __fmul2_rn(wk, make_float2(len_sqrt(q.x), len_sqrt(q.y)));
+            p[r][0] = __fadd2_rn(p[r][0], wk);
+            p[r][1] = __fadd2_rn(p[r][1], wr);
+            p[r][2] = __ffma2_rn(wk, q, p[r][2]);
+            p[r][3] = __ffma2_rn(wr, q, p[r][3]);
         }
     }
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int c = 0; c < (FORWARD ? 4 : 2); ++c)
-            kahan_add(acc[r][c], cmp[r][c], p[r][c].x + p[r][c].y);
 }
 
-// One pass over the evaluation points plist[0, np) of leaf L (first point
-// lf, O its position) against the partner leaves of pairs [i0, i1).  A lane
-// holds R points (slots R j .. R j + R - 1 of its group j); when the groups
-// fit in fewer lanes they take npr = 2^k lanes and 32 / npr lanes share a
-// group, each walking an interleaved slice of the staged sources.  The 4
-// warps take the partner leaves round-robin, packing their points into
-// chunks of kLenStage in shared memory (L's own points last, in chunks of
-// their own); every chunk's sums join the lane's compensated running sums.
-// The slices' compensated sums are added by a fixed butterfly; the warps'
-// go to red for a fixed-order sum.
-template <bool FORWARD, int R>
-__device__ __forceinline__ void len_pass(const int32_t* plist, int np, int32_t i0, int32_t i1,
-                                         int32_t L, int32_t lf, int32_t lc, const float4& O,
-                                         const int32_t* __restrict__ pairs,
-                                         const int32_t* __restrict__ pPart,
-                                         const int32_t* __restrict__ nfirst,
-                                         const int32_t* __restrict__ ncount,
-                                         const float4* __restrict__ pts,
-                                         const float4* __restrict__ gw,
-                                         const float2* __restrict__ cf, float sqk, float rs,
-                                         float4* sA, float4* sB, float4* sC, float4* sD,
-                                         float4 (*red)[kLenList]) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int lg = 0;
-    while ((1 << lg) < (np + R - 1) / R) ++lg;
-    const int npr = 1 << lg, slices = 32 >> lg;
-    const int jg = lane & (npr - 1), ksl = lane >> lg;
-    const bool active = R * jg < np;
-    int32_t t[R];
-    bool inh[R];
-    float2 tx[R], ty[R], tz[R];
-    float acc[R][4], cmp[R][4];
+template <int R>
+__device__ __forceinline__ void len_fwd_pass(const int32_t* list, int np, int32_t i0, int32_t i1,
+                                             int32_t lf, int32_t lc, const float4& O,
+                                             const int2* __restrict__ src,
+                                             const float4* __restrict__ pts,
+                                             const float2* __restrict__ wt,
+                                             const uint16_t* __restrict__ fl, float sqk,
+                                             PsFwdStage& st, int2* meta, float* totals,
+                                             float4* red) {
+    const int lane = threadIdx.x & 31;
+    const PsLanes ln(np, R);
+    const LenTotals<R, 4> tot(totals);
+    float2 tx[R], ty[R], tz[R], p[R][4];
+    int32_t e[R];
+    bool inh = false;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int slot = R * jg + r;
-        t[r] = slot < np ? plist[slot] : -1;
-        const int32_t pi = slot < np ? t[r] : plist[0];
-        const float4 T = pts[pi];
-        inh[r] = gw[pi].w != 0.f;
+        const int slot = R * ln.j + r;
+        e[r] = slot < np ? list[slot] : -1;
+        const int32_t t = e[r] >= 0 ? e[r] : lf;
+        if (r == 0) inh = e[0] >= 0 && (fl[t] & kPsInh);
+        const float4 T = pts[t];
         const float x = (T.x - O.x) * sqk, y = (T.y - O.y) * sqk, z = (T.z - O.z) * sqk;
         tx[r] = make_float2(x, x);
         ty[r] = make_float2(y, y);
         tz[r] = make_float2(z, z);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = cmp[r][c] = 0.f;
+        for (int k = 0; k < 4; ++k) p[r][k] = make_float2(0.f, 0.f);
     }
-    float* fA = reinterpret_cast<float*>(sA);
-    float* fB = reinterpret_cast<float*>(sB);
-    float* fC = reinterpret_cast<float*>(sC);
-    float* fD = reinterpret_cast<float*>(sD);
-    // stage sources [pf + sb, pf + sb + take) at chunk positions fill..;
-    // position m of an odd chunk is padded before use
-    auto stage = [&](int32_t pf, int32_t sb, int take, int fill) {
-        if (lane < take) {
-            const int32_t j = pf + sb + lane;
-            const float4 S = pts[j];
-            const float4 SW = gw[j];
-            const int pos = fill + lane, jj = pos >> 1, h = pos & 1;
-            fA[4 * jj + h] = -(S.x - O.x) * sqk;
-            fA[4 * jj + 2 + h] = -(S.y - O.y) * sqk;
-            fB[4 * jj + h] = -(S.z - O.z) * sqk;
-            fB[4 * jj + 2 + h] = __int_as_float(j);
-            if (FORWARD) {
-                fC[4 * jj + h] = SW.x;
-                fC[4 * jj + 2 + h] = SW.y;
-            } else {
-                const float2 ab = SW.z > 0.f ? cf[j] : make_float2(0.f, 0.f);
-                fC[4 * jj + h] = ab.x;
-                fC[4 * jj + 2 + h] = ab.y;
-                fD[4 * jj + h] = SW.w != 0.f ? 1.f : 0.f;
-                fD[4 * jj + 2 + h] = SW.w != 0.f ? 0.f : 1.f;
+    auto fold = [&] {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                tot.add(4 * r + k, __fadd_rn(p[r][k].x, p[r][k].y));
+                p[r][k] = make_float2(0.f, 0.f);
             }
-        }
     };
-    auto pad = [&](int m) {
-        if ((m & 1) && lane == 0) {
-            const int jj = m >> 1;
-            fA[4 * jj + 1] = 0.f;
-            fA[4 * jj + 3] = 0.f;
-            fB[4 * jj + 1] = 0.f;
-            fB[4 * jj + 3] = __int_as_float(-1);
-            fC[4 * jj + 1] = 0.f;
-            fC[4 * jj + 3] = 0.f;
-            if (!FORWARD) {
-                fD[4 * jj + 1] = 0.f;
-                fD[4 * jj + 3] = 0.f;
-            }
-        }
-    };
-    int fill = 0;
+    const float4* sW = inh ? st.I : st.E;
     bool self = false;
-    for (int32_t i = i0 + w; i < i1; i += kLenWarps) {
-        const int32_t P = pPart[pairs[i]];
-        if (P == L) {
-            self = true;
-            continue;
-        }
-        const int32_t pf = nfirst[P], pc = ncount[P];
-        for (int32_t sb = 0; sb < pc;) {
-            const int take = min(kLenStage - fill, pc - sb);
-            stage(pf, sb, take, fill);
-            fill += take;
-            sb += take;
-            if (fill == kLenStage) {
-                __syncwarp();
-                if (active)
-                    len_eval<FORWARD, false, R>(sA, sB, sC, sD, kLenStage / 2, ksl, slices, t,
-                                                inh, tx, ty, tz, rs, acc, cmp);
-                __syncwarp();
-                fill = 0;
+    ps_walk(
+        src, i0, i1, meta,
+        [&](int2 m) {
+            if (m.x == lf) {
+                self = true;
+                m.y = 0;
             }
-        }
-    }
-    if (fill > 0) {
-        pad(fill);
-        __syncwarp();
-        if (active)
-            len_eval<FORWARD, false, R>(sA, sB, sC, sD, (fill + 1) >> 1, ksl, slices, t, inh, tx,
-                                        ty, tz, rs, acc, cmp);
-        __syncwarp();
-    }
-    if (self) {
-        for (int32_t sb = 0; sb < lc; sb += kLenStage) {
-            const int m = min(kLenStage, lc - sb);
-            stage(lf, sb, m, 0);
-            pad(m);
+            return m;
+        },
+        [&](int32_t a, int32_t b, bool two, int slot) {
+            ps_stage_fwd(st, pts, wt, a, b, two, slot, O, sqk);
+        },
+        [&](int mp) {
+            // a fold per unit of 64 sources
+            len_fwd_eval<R, false>(st.A, sW, ln.ksl, min(mp, kPsUnit / 2), ln.slices, tx, ty, tz, e,
+                                   0, 0, p);
+            fold();
+            if (mp > kPsUnit / 2) {
+                len_fwd_eval<R, false>(st.A, sW, kPsUnit / 2 + ln.ksl, mp, ln.slices, tx, ty, tz, e,
+                                       0, 0, p);
+                fold();
+            }
+        });
+    // L's own points, where a target skips itself
+    if (__any_sync(0xffffffffu, self)) {
+        for (int32_t q = 0; q < lc; q += kPsUnit) {
+            const int left = min(lc - q, kPsUnit), half = (left + 1) >> 1;
             __syncwarp();
-            if (active)
-                len_eval<FORWARD, true, R>(sA, sB, sC, sD, (m + 1) >> 1, ksl, slices, t, inh, tx,
-                                           ty, tz, rs, acc, cmp);
+            if (lane < half)
+                ps_stage_fwd(st, pts, wt, lf + q + lane, lf + q + half + lane, lane < left - half,
+                             lane, O, sqk);
             __syncwarp();
+            len_fwd_eval<R, true>(st.A, sW, ln.ksl, half, ln.slices, tx, ty, tz, e, lf + q,
+                                  lf + q + half, p);
+            fold();
         }
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         float v[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            v[c] = __fsub_rn(acc[r][c], cmp[r][c]);
-            for (int o = npr; o < 32; o <<= 1) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
-        }
-        const int slot = R * jg + r;
-        if (ksl == 0 && slot < np) red[w][slot] = make_float4(v[0], v[1], v[2], v[3]);
+        for (int k = 0; k < 4; ++k) v[k] = ln.sum(tot.get(4 * r + k));
+        if (ln.ksl == 0 && R * ln.j + r < np)
+            red[R * ln.j + r] = make_float4(v[0], v[1], v[2], v[3]);
     }
 }
 
-// One block of 4 warps per leaf L of a segment list.  Warp 0 lists L's
-// evaluation points (FORWARD: the targets, a_t > 0; ADJOINT: every point), up
-// to kLenList per pass, and the pass holds R = 1 or 2 of them per lane, R the
-// fewest evaluated slots per source (ties to the larger R).  Coordinates are
-// scaled by sqk = sqrt(log2 e)/sigma relative to L's first point, so that
-// q = |t^ - s^|^2 gives K = 2^-q and r = rs sqrt(q), rs = sigma/sqrt(log2 e).
-//   FORWARD (L = the target leaf): per target t with a_t > 0, the sums
-//     U = sum w K, V = sum w K r, QU = sum w K q, QV = sum w K q r
-//     (w: the staged source's weight of t's channel), written in sorted order.
-//   ADJOINT (L = the source leaf): per point s, for each channel T,
-//     G_T = sum_{t: T(t) = T} K (alpha_t r - beta_t)
-//     over the staged targets t (coefficients in cf), written in caller order.
-template <bool FORWARD>
-__global__ void __launch_bounds__(kLenWarps * 32, 6)
-k_len_pairs(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nseg_dev,
-            const int32_t* __restrict__ pairs, const int32_t* __restrict__ pEval,
-            const int32_t* __restrict__ pPart, const int32_t* __restrict__ nfirst,
-            const int32_t* __restrict__ ncount, const float4* __restrict__ pts,
-            const float4* __restrict__ gw, const float2* __restrict__ cf,
-            const int32_t* __restrict__ perm, float sqk, float rs, float4* __restrict__ sums,
-            float* __restrict__ gE, float* __restrict__ gI) {
-    __shared__ float4 sA_all[kLenWarps][kLenStage / 2], sB_all[kLenWarps][kLenStage / 2],
-        sC_all[kLenWarps][kLenStage / 2], sD_all[kLenWarps][FORWARD ? 1 : kLenStage / 2];
-    __shared__ float4 red[kLenWarps][kLenList];   // the warps' compensated sums per slot
-    __shared__ int32_t plist[kLenList];
-    __shared__ int s_np, s_pos;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(kPsWarps * 32, 5)
+k_len_forward(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nseg_dev,
+              const int32_t* __restrict__ order, const int32_t* __restrict__ pairs,
+              const int32_t* __restrict__ pX, const int2* __restrict__ src,
+              const int32_t* __restrict__ nfirst, const int32_t* __restrict__ ncount,
+              const float4* __restrict__ pts, const float2* __restrict__ wt,
+              const uint16_t* __restrict__ fl, float sqk, float4* __restrict__ sums) {
+    __shared__ PsFwdStage st[kPsWarps];
+    __shared__ int2 meta[kPsWarps][32];
+    __shared__ float totals[2 * kLenFwdR * 4 * kPsWarps * 32];
+    __shared__ float4 red[kPsWarps][32 * kLenFwdR];
+    __shared__ int32_t list[kPsList];
+    __shared__ int s_np, s_pos, s_R;
+    const int w = threadIdx.x >> 5;
     const int64_t nseg = *nseg_dev;
-    for (int64_t sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
-        const int32_t i0 = seg_first[sg], i1 = seg_first[sg + 1];
-        const int32_t L = pEval[pairs[i0]];
-        const int32_t lf = nfirst[L], lc = ncount[L];
+    for (int64_t b = blockIdx.x; b < nseg; b += gridDim.x) {
+        const int32_t sg = order[b], i0 = seg_first[sg], i1 = seg_first[sg + 1];
+        const int32_t L = pX[pairs[i0]], lf = nfirst[L], lc = ncount[L];
         const float4 O = pts[lf];
-        int32_t pos = 0;
-        for (;;) {
-            if (w == 0) {
-                // the next (at most) kLenList evaluation points from pos on
-                int np = 0;
-                int32_t p = pos;
-                while (p < lc && np < kLenList) {
-                    const int32_t idx = p + lane;
-                    bool ok = idx < lc;
-                    if (FORWARD && ok) ok = gw[lf + idx].z > 0.f;
-                    const unsigned mk = __ballot_sync(0xffffffffu, ok);
-                    const int room = kLenList - np;
-                    const int rank = __popc(mk & ((1u << lane) - 1u));
-                    if (ok && rank < room) plist[np + rank] = lf + idx;
-                    if (__popc(mk) > room) {
-                        // the room-th point ends the pass: resume after it
-                        unsigned keep = mk;
-                        for (int k = 0; k < room; ++k) keep &= keep - 1u;
-                        p += __ffs(keep) - 1;
-                        np = kLenList;
-                        break;
-                    }
-                    np += __popc(mk);
-                    p += 32;
-                }
-                if (lane == 0) {
-                    s_np = np;
-                    s_pos = min(p, lc);
-                }
-            }
+        for (int32_t pos = 0; pos < lc;) {
+            // twelve paired FP32 instructions a slot, two 16-byte loads a pair
+            if (w == 0)
+                ps_list_targets<kLenFwdR>(fl, lf, lc, pos, 32 * kLenFwdR - kLenFwdR + 1, 24, 8,
+                                          list, &s_np, &s_pos, &s_R);
             __syncthreads();
-            const int np = s_np;
+            const int np = s_np, R = s_R;
             pos = s_pos;
-            __syncthreads();
-            if (np == 0) break;
-            int R = 1, best = 1 << 30;
-            for (int rr = 1; rr <= kLenMaxR; ++rr) {
-                const int g = (np + rr - 1) / rr;
-                if (g > 32) continue;
-                int npr = 1;
-                while (npr < g) npr <<= 1;
-                if (npr * rr <= best) {
-                    best = npr * rr;
-                    R = rr;
-                }
-            }
-            if (R == 1)
-                len_pass<FORWARD, 1>(plist, np, i0, i1, L, lf, lc, O, pairs, pPart, nfirst,
-                                     ncount, pts, gw, cf, sqk, rs, sA_all[w], sB_all[w],
-                                     sC_all[w], sD_all[w], red);
-            else
-                len_pass<FORWARD, 2>(plist, np, i0, i1, L, lf, lc, O, pairs, pPart, nfirst,
-                                     ncount, pts, gw, cf, sqk, rs, sA_all[w], sB_all[w],
-                                     sC_all[w], sD_all[w], red);
-            __syncthreads();
-            if (w == 0) {
-#pragma unroll
-                for (int rr = 0; rr < kLenMaxR; ++rr) {
-                    const int j = lane + 32 * rr;
-                    if (j >= np) continue;
-                    float4 v = red[0][j];
-#pragma unroll
-                    for (int k = 1; k < kLenWarps; ++k) {
-                        const float4 x = red[k][j];
-                        v.x += x.x;
-                        v.y += x.y;
-                        v.z += x.z;
-                        v.w += x.w;
-                    }
-                    const int32_t t = plist[j];
-                    if (FORWARD) {
-                        sums[t] = v;
-                    } else {
-                        const int32_t o = perm[t];
-                        if (gE) gE[o] = v.x;
-                        if (gI) gI[o] = v.y;
-                    }
-                }
+            if (np > 0) {
+#define MSP_LEN_FWD(RR)                                                                        \
+    len_fwd_pass<RR>(list, np, i0, i1, lf, lc, O, src, pts, wt, fl, sqk, st[w], meta[w], totals, \
+                     red[w])
+                if (R == 1) MSP_LEN_FWD(1);
+                else if (R == 2) MSP_LEN_FWD(2);
+                else MSP_LEN_FWD(3);
+#undef MSP_LEN_FWD
             }
             __syncthreads();
-            if (pos >= lc) break;
+            for (int k = threadIdx.x; k < np; k += kPsWarps * 32) {
+                if (list[k] < 0) continue;
+                float4 v = red[0][k];
+#pragma unroll
+                for (int q = 1; q < kPsWarps; ++q) {
+                    const float4 x = red[q][k];
+                    v.x += x.x;
+                    v.y += x.y;
+                    v.z += x.z;
+                    v.w += x.w;
+                }
+                sums[list[k]] = v;
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// TRANSPOSED: for every point s of the block's leaf and each channel T,
+//   G_T = sum_{t: T(t) = T} K (alpha_t r - beta_t)
+// over the partner leaves' targets of the channel, staged as A = (-x0, -x1,
+// -y0, -y1), B = (-z0, -z1, alpha0, alpha1), C = (-beta0, -beta1) (alpha times
+// rs), D = the sorted indices.
+constexpr int kLenAdjR = 4;
+
+template <int R, bool SELF>
+__device__ __forceinline__ void len_adj_eval(const PsAdjStage& st, int j0, int mp, int slices,
+                                             const float2 (&tx)[R], const float2 (&ty)[R],
+                                             const float2 (&tz)[R], const int32_t (&e)[R],
+                                             float2 (&p)[R]) {
+    for (int j = j0; j < mp; j += slices) {
+        const float4 A = st.A[j], B = st.B[j];
+        const float2 C = st.C[j];
+        const int2 D = SELF ? st.D[j] : make_int2(0, 0);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float2 dx = __fadd2_rn(tx[r], make_float2(A.x, A.y));
+            const float2 dy = __fadd2_rn(ty[r], make_float2(A.z, A.w));
+            const float2 dz = __fadd2_rn(tz[r], make_float2(B.x, B.y));
+            const float2 q = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+            float2 K = make_float2(ps_ex2(-q.x), ps_ex2(-q.y));
+            if (SELF) {
+                K.x = D.x == e[r] ? 0.f : K.x;
+                K.y = D.y == e[r] ? 0.f : K.y;
+            }
+            const float2 f =
+                __ffma2_rn(make_float2(B.z, B.w), make_float2(len_sqrt(q.x), len_sqrt(q.y)), C);
+            p[r] = __ffma2_rn(K, f, p[r]);
+        }
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void len_adj_pass(int32_t first, int np, int32_t i0, int32_t i1,
+                                             int32_t lf, int32_t lc, int64_t n, const float4& O,
+                                             const int2* __restrict__ src,
+                                             const float4* __restrict__ pts, const PsPacked pk,
+                                             const float2* __restrict__ cf, float sqk,
+                                             PsAdjStage& st, int2* meta, float* totals,
+                                             float2* red) {
+    const int lane = threadIdx.x & 31;
+    const PsLanes ln(np, R);
+    const LenTotals<R, 2> tot(totals);
+    float2 tx[R], ty[R], tz[R], p[R];
+    int32_t e[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int slot = R * ln.j + r;
+        e[r] = first + (slot < np ? slot : 0);
+        const float4 T = pts[e[r]];
+        const float x = (T.x - O.x) * sqk, y = (T.y - O.y) * sqk, z = (T.z - O.z) * sqk;
+        tx[r] = make_float2(x, x);
+        ty[r] = make_float2(y, y);
+        tz[r] = make_float2(z, z);
+        p[r] = make_float2(0.f, 0.f);
+    }
+    auto stage = [&](int32_t a, int32_t b, bool two, int slot) {
+        const float4 S0 = pk.pt[a], S1 = pk.pt[two ? b : a];
+        const float2 c0 = cf[a], c1 = two ? cf[b] : make_float2(0.f, 0.f);
+        const float2 k = make_float2(sqk, sqk);
+        const float2 x = __fmul2_rn(__fadd2_rn(make_float2(O.x, O.x), make_float2(-S0.x, -S1.x)), k);
+        const float2 y = __fmul2_rn(__fadd2_rn(make_float2(O.y, O.y), make_float2(-S0.y, -S1.y)), k);
+        const float2 z = __fmul2_rn(__fadd2_rn(make_float2(O.z, O.z), make_float2(-S0.z, -S1.z)), k);
+        st.A[slot] = make_float4(x.x, x.y, y.x, y.y);
+        st.B[slot] = make_float4(z.x, z.y, c0.x, c1.x);
+        st.C[slot] = make_float2(c0.y, c1.y);
+        st.D[slot] = make_int2(__float_as_int(S0.w), two ? __float_as_int(S1.w) : -1);
+    };
+#pragma unroll 1
+    for (int ch = 0; ch < 2; ++ch) {
+        const int32_t* off = pk.off + ch * n;
+        auto fold = [&] {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                tot.add(2 * r + ch, __fadd_rn(p[r].x, p[r].y));
+                p[r] = make_float2(0.f, 0.f);
+            }
+        };
+        bool self = false;
+        ps_walk(
+            src, i0, i1, meta,
+            [&](int2 m) {
+                if (m.x == lf) {
+                    self = true;
+                    return make_int2(0, 0);
+                }
+                const int32_t a = off[m.x];
+                return make_int2(a, off[m.x + m.y] - a);
+            },
+            stage,
+            [&](int mp) {
+                // a fold per unit of 64 targets
+                len_adj_eval<R, false>(st, ln.ksl, min(mp, kPsUnit / 2), ln.slices, tx, ty, tz, e, p);
+                fold();
+                if (mp > kPsUnit / 2) {
+                    len_adj_eval<R, false>(st, kPsUnit / 2 + ln.ksl, mp, ln.slices, tx, ty, tz, e,
+                                           p);
+                    fold();
+                }
+            });
+        // L's own targets, where a point skips itself
+        if (__any_sync(0xffffffffu, self)) {
+            const int32_t a0 = off[lf], a1 = off[lf + lc];
+            for (int32_t q = a0; q < a1; q += kPsUnit) {
+                const int left = min(a1 - q, kPsUnit), half = (left + 1) >> 1;
+                __syncwarp();
+                if (lane < half) stage(q + lane, q + half + lane, lane < left - half, lane);
+                __syncwarp();
+                len_adj_eval<R, true>(st, ln.ksl, half, ln.slices, tx, ty, tz, e, p);
+                fold();
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float vE = ln.sum(tot.get(2 * r)), vI = ln.sum(tot.get(2 * r + 1));
+        if (ln.ksl == 0 && R * ln.j + r < np) red[R * ln.j + r] = make_float2(vE, vI);
+    }
+}
+
+__global__ void __launch_bounds__(kPsWarps * 32, 6)
+k_len_adjoint(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nseg_dev,
+              const int32_t* __restrict__ order, const int32_t* __restrict__ pairs,
+              const int32_t* __restrict__ pX, const int2* __restrict__ src,
+              const int32_t* __restrict__ nfirst, const int32_t* __restrict__ ncount, int64_t n,
+              const float4* __restrict__ pts, const PsPacked pk, const float2* __restrict__ cf,
+              const int32_t* __restrict__ perm, float sqk, float* __restrict__ gE,
+              float* __restrict__ gI) {
+    __shared__ PsAdjStage st[kPsWarps];
+    __shared__ int2 meta[kPsWarps][32];
+    __shared__ float totals[2 * kLenAdjR * 2 * kPsWarps * 32];
+    __shared__ float2 red[kPsWarps][kPsList];
+    const int w = threadIdx.x >> 5;
+    const int64_t nseg = *nseg_dev;
+    for (int64_t b = blockIdx.x; b < nseg; b += gridDim.x) {
+        const int32_t sg = order[b], i0 = seg_first[sg], i1 = seg_first[sg + 1];
+        const int32_t L = pX[pairs[i0]], lf = nfirst[L], lc = ncount[L];
+        const float4 O = pts[lf];
+        for (int32_t pos = 0; pos < lc; pos += kPsList) {
+            const int np = min(lc - pos, kPsList);
+            // EX2 and SQRT for two sources a slot (the special function unit's
+            // 17 quarter cycles), 40 bytes a staged pair
+            const int R = ps_choose_r<kLenAdjR>([&](int) { return np; }, 17, 10);
+#define MSP_LEN_ADJ(RR)                                                                        \
+    len_adj_pass<RR>(lf + pos, np, i0, i1, lf, lc, n, O, src, pts, pk, cf, sqk, st[w], meta[w], \
+                     totals, red[w])
+            if (R == 1) MSP_LEN_ADJ(1);
+            else if (R == 2) MSP_LEN_ADJ(2);
+            else if (R == 3) MSP_LEN_ADJ(3);
+            else MSP_LEN_ADJ(4);
+#undef MSP_LEN_ADJ
+            __syncthreads();
+            for (int k = threadIdx.x; k < np; k += kPsWarps * 32) {
+                float2 v = red[0][k];
+#pragma unroll
+                for (int q = 1; q < kPsWarps; ++q) {
+                    v.x += red[q][k].x;
+                    v.y += red[q][k].y;
+                }
+                const int32_t c = perm[lf + pos + k];
+                if (gE) gE[c] = v.x;
+                if (gI) gI[c] = v.y;
+            }
+            __syncthreads();
         }
     }
 }
@@ -419,18 +444,18 @@ constexpr int kLenRedThreads = 256;
 // over the targets it takes (a > 0, U > 0), in double, reduced in a fixed
 // order; V' / U' are QV / QU times dscale = 2 / (sigma log2 e)
 __global__ void __launch_bounds__(kLenRedThreads)
-k_len_reduce(int64_t n, const float4* __restrict__ gw, const float4* __restrict__ sums,
-             double dscale, double* __restrict__ part) {
+k_len_reduce(int64_t n, const uint16_t* __restrict__ fl, const float4* __restrict__ sums,
+             double rs, double dscale, double* __restrict__ part) {
     __shared__ double red[3][kLenRedThreads];
     double A = 0.0, S = 0.0, D = 0.0;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
          t += (int64_t)gridDim.x * blockDim.x) {
-        const float a = gw[t].z;
+        const float a = len_count(fl[t]);
         if (!(a > 0.f)) continue;
         const float4 s4 = sums[t];
-        const double U = s4.x, V = s4.y;
+        const double U = s4.x, V = rs * s4.y;
         if (!(U > 0.0)) continue;
-        const double dU = dscale * s4.z, dV = dscale * s4.w;
+        const double dU = dscale * s4.z, dV = dscale * rs * s4.w;
         A += a;
         S += a * V / U;
         D += a * (dV * U - V * dU) / (U * U);
@@ -448,15 +473,23 @@ k_len_reduce(int64_t n, const float4* __restrict__ gw, const float4* __restrict_
         for (int k = 0; k < 3; ++k) part[3 * blockIdx.x + k] = red[k][0];
 }
 
-// the blocks' partials in order; res = {loss, m, dloss/dsigma, dm/dsigma, A, f}
-__global__ void k_len_final(const double* __restrict__ part, int nblocks, double target,
-                            double* __restrict__ res) {
-    double A = 0.0, S = 0.0, D = 0.0;
-    for (int b = 0; b < nblocks; ++b) {
-        A += part[3 * b];
-        S += part[3 * b + 1];
-        D += part[3 * b + 2];
+// the blocks' partials, added in a fixed order by one block; res = {loss, m,
+// dloss/dsigma, dm/dsigma, A, f}
+__global__ void __launch_bounds__(kLenRedThreads)
+k_len_final(const double* __restrict__ part, int nblocks, double target, double* __restrict__ res) {
+    __shared__ double red[3][kLenRedThreads];
+    double v[3] = {0.0, 0.0, 0.0};
+    for (int b = threadIdx.x; b < nblocks; b += kLenRedThreads)
+        for (int k = 0; k < 3; ++k) v[k] += part[3 * b + k];
+    for (int k = 0; k < 3; ++k) red[k][threadIdx.x] = v[k];
+    __syncthreads();
+    for (int o = kLenRedThreads / 2; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o)
+            for (int k = 0; k < 3; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + o];
+        __syncthreads();
     }
+    if (threadIdx.x) return;
+    const double A = red[0][0], S = red[1][0], D = red[2][0];
     const double m = A > 0.0 ? S / A : 0.0;
     const double dm = A > 0.0 ? D / A : 0.0;
     const double f = 2.0 * (m - target);
@@ -468,20 +501,26 @@ __global__ void k_len_final(const double* __restrict__ part, int nblocks, double
     res[5] = f;
 }
 
-// per target: (f alpha_t, f beta_t), f = 2 (m - target), sorted order
-__global__ void k_len_coef(int64_t n, const float4* __restrict__ gw,
+// the packed targets: point, and (f alpha_t rs, -f beta_t), f = 2 (m - target)
+__global__ void k_len_pack(int64_t n, const uint16_t* __restrict__ fl,
+                           const int32_t* __restrict__ off, const float4* __restrict__ pts,
                            const float4* __restrict__ sums, const double* __restrict__ res,
-                           float2* __restrict__ cf) {
+                           double rs, float4* __restrict__ pt, float2* __restrict__ cf) {
     const double A = res[4], f = res[5];
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
          t += (int64_t)gridDim.x * blockDim.x) {
-        const float a = gw[t].z;
+        const uint32_t fw = fl[t];
+        if (!(fw & kPsAct)) continue;
+        const float a = len_count((uint16_t)fw);
         const float4 s4 = sums[t];
-        const double U = s4.x, V = s4.y;
+        const double U = s4.x, V = rs * s4.y;
         float2 c = make_float2(0.f, 0.f);
-        if (a > 0.f && U > 0.0 && A > 0.0)
-            c = make_float2((float)(f * a / (A * U)), (float)(f * a * V / (A * U * U)));
-        cf[t] = c;
+        if (U > 0.0 && A > 0.0)
+            c = make_float2((float)(rs * (f * a / (A * U))), (float)(-(f * a * V / (A * U * U))));
+        const int32_t k = off[((fw & kPsInh) ? n : 0) + t];
+        const float4 P = pts[t];
+        pt[k] = make_float4(P.x, P.y, P.z, __int_as_float((int32_t)t));
+        cf[k] = c;
     }
 }
 
@@ -502,41 +541,45 @@ void length_loss(msp_ctx& c, const uint8_t* type, const uint8_t* va, const float
     const int B = 256;
     const int G = grid_for(n, B, (int64_t)c.sm_count * 16);
     DevCounts* dc = dcounts(c);
-    float4* gw = c.gr_w.ensure<float4>((size_t)n);
-    k_len_gather<<<G, B, 0, s>>>(n, c.perm.get<int32_t>(), type, va, we, wi, gw);
+    float2* wt = c.gr_w.ensure<float2>((size_t)n);
+    uint16_t* fl = c.gr_fl.ensure<uint16_t>((size_t)n);
+    const int32_t* perm = c.perm.get<int32_t>();
+    k_len_gather<<<G, B, 0, s>>>(n, perm, type, va, we, wi, wt, fl);
     MSP_LAUNCH("len_gather");
     const float sqk = (float)std::sqrt(kLog2e / (cfg.sigma * cfg.sigma));
-    const float rs = (float)(cfg.sigma / std::sqrt(kLog2e));
+    const double rs = cfg.sigma / std::sqrt(kLog2e);
     const double dscale = 2.0 / (cfg.sigma * kLog2e);
-    const int64_t nseg_cap = std::max<int64_t>(c.n_nodes, 1);
-    const int nb = (int)std::min<int64_t>(nseg_cap, 1 << 30);
+    // the segments in the near field's order (longest first) and its source
+    // ranges, kept with the lists
+    const int32_t *segf = c.seg_first.get<int32_t>(), *order = c.nf_oval0.get<int32_t>(),
+                  *list = c.p2p_val0.get<int32_t>(), *pX = c.pr_X.get<int32_t>(),
+                  *nfirst = c.nd_first.get<int32_t>(), *ncount = c.nd_count.get<int32_t>();
+    const int2* src = c.nf_src.get<int2>();
+    const float4* pts = c.pts.get<float4>();
+    const int nb = (int)std::min<int64_t>(std::max<int64_t>(c.n_nodes, 1), 1 << 30);
     float4* sums = c.ln_sums.ensure<float4>((size_t)n);
     MSP_CUDA(cudaMemsetAsync(sums, 0, (size_t)n * sizeof(float4), s));
-    k_len_pairs<true><<<nb, kLenWarps * 32, 0, s>>>(
-        c.seg_first.get<int32_t>(), &dc->nseg, c.p2p_val0.get<int32_t>(), c.pr_X.get<int32_t>(),
-        c.pr_Y.get<int32_t>(), c.nd_first.get<int32_t>(), c.nd_count.get<int32_t>(),
-        c.pts.get<float4>(), gw, nullptr, c.perm.get<int32_t>(), sqk, rs, sums, nullptr,
-        nullptr);
+    k_len_forward<<<nb, kPsWarps * 32, 0, s>>>(segf, &dc->nseg, order, list, pX, src, nfirst, ncount,
+                                               pts, wt, fl, sqk, sums);
     MSP_LAUNCH("len_forward");
     const int Gr = (int)std::min<int64_t>(grid_for(n, kLenRedThreads), (int64_t)c.sm_count * 4);
     double* part = c.ln_part.ensure<double>((size_t)3 * Gr + 8);
-    k_len_reduce<<<Gr, kLenRedThreads, 0, s>>>(n, gw, sums, dscale, part);
+    k_len_reduce<<<Gr, kLenRedThreads, 0, s>>>(n, fl, sums, rs, dscale, part);
     MSP_LAUNCH("len_reduce");
     double* res = part + 3 * Gr;
-    k_len_final<<<1, 1, 0, s>>>(part, Gr, target, res);
+    k_len_final<<<1, kLenRedThreads, 0, s>>>(part, Gr, target, res);
     MSP_LAUNCH("len_final");
     if (gE || gI) {
-        float2* cf = c.ln_coef.ensure<float2>((size_t)n);
-        k_len_coef<<<G, B, 0, s>>>(n, gw, sums, res, cf);
-        MSP_LAUNCH("len_coef");
         if (gE) MSP_CUDA(cudaMemsetAsync(gE, 0, (size_t)n * sizeof(float), s));
         if (gI) MSP_CUDA(cudaMemsetAsync(gI, 0, (size_t)n * sizeof(float), s));
-        const int32_t *segf = nullptr, *list = nullptr;
-        pairs_by_source(c, s, &segf, &list);
-        k_len_pairs<false><<<nb, kLenWarps * 32, 0, s>>>(
-            segf, &dc->scan_n, list, c.pr_Y.get<int32_t>(), c.pr_X.get<int32_t>(),
-            c.nd_first.get<int32_t>(), c.nd_count.get<int32_t>(), c.pts.get<float4>(), gw, cf,
-            c.perm.get<int32_t>(), sqk, rs, nullptr, gE, gI);
+        const int32_t* off = ps_offsets(c, fl, s);
+        float4* pt = c.gr_pt.ensure<float4>((size_t)n);
+        float2* cf = c.ln_coef.ensure<float2>((size_t)n);
+        k_len_pack<<<G, B, 0, s>>>(n, fl, off, pts, sums, res, rs, pt, cf);
+        MSP_LAUNCH("len_pack");
+        k_len_adjoint<<<nb, kPsWarps * 32, 0, s>>>(segf, &dc->nseg, order, list, pX, src, nfirst,
+                                                   ncount, n, pts, PsPacked{pt, off}, cf, perm, sqk,
+                                                   gE, gI);
         MSP_LAUNCH("len_adjoint");
     }
     MSP_CUDA(cudaMemcpyAsync(out4, res, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
