@@ -200,7 +200,7 @@ msp_status msp_destroy(msp_ctx* c) {
                          &c->ln_part, &c->ln_coef,
                          &c->expA, &c->expM, &c->expB, &c->u_sorted, &c->items0, &c->items1,
                          &c->leaf_items, &c->rq_key0, &c->rq_val0,
-                         &c->accepted, &c->acc_off, &c->rq_gcnt, &c->rq_goff, &c->cnt, &c->off, &c->scan_tmp,
+                         &c->accepted, &c->acc_off, &c->rq_gcnt, &c->rq_goff, &c->cnt, &c->off, &c->rs_status,
                          &c->rs_hist, &c->h_u, &c->h_partner, &c->h_pre,
                          &c->h_post, &c->h_type, &c->h_nsyn, &c->hs_u, &c->hs_partner,
                          &c->hs_pre, &c->hs_post, &c->hs_type, &c->hs_nsyn, &c->c_type,

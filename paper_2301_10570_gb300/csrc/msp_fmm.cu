@@ -765,9 +765,12 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
     uint64_t* pk0 = c.p2p_key0.ensure<uint64_t>((size_t)cap);
     uint64_t* pk1 = c.p2p_key1.ensure<uint64_t>((size_t)cap);
     int32_t* pv1 = c.p2p_val1.ensure<int32_t>((size_t)cap);
-    k_compact_kind<<<Gt, B, 0, s>>>(kind, n_pairs_dev, kP2P, off, c.pr_X.get<int32_t>(), pv0, pk0);
+    const int xbits = bits_for(c.n_nodes);
+    const bool odd = radix_from_tmp(cap, xbits);
+    k_compact_kind<<<Gt, B, 0, s>>>(kind, n_pairs_dev, kP2P, off, c.pr_X.get<int32_t>(),
+                                    odd ? pv1 : pv0, odd ? pk1 : pk0);
     MSP_LAUNCH("compact_p2p");
-    radix_sort_dev(c, pk0, pv0, pk1, pv1, &dc->n_p2p, cap, bits_for(c.n_nodes), s);
+    radix_sort_dev(c, pk0, pv0, pk1, pv1, &dc->n_p2p, cap, xbits, s);
     int32_t* sflag = c.seg_flag.ensure<int32_t>((size_t)cap);
     int32_t* soff = cnt;
     k_seg_flags<<<Gt, B, 0, s>>>(pk0, &dc->n_p2p, sflag);
@@ -820,10 +823,12 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
         int32_t* moff = c.m2_off.ensure<int32_t>((size_t)cap);
         int32_t* mseg = c.m2_seg.ensure<int32_t>((size_t)c.n_nodes + 2);
         if (!reuse_lists || geo) {
-            k_m2l_keys<<<Gt, B, 0, s>>>(mq, &dc->n_far, first, c.pr_X.get<int32_t>(), mk0, mv0,
-                                        &dc->m2l_n);
+            const int xbits = bits_for(c.n_nodes);
+            const bool odd = radix_from_tmp(cap, xbits);
+            k_m2l_keys<<<Gt, B, 0, s>>>(mq, &dc->n_far, first, c.pr_X.get<int32_t>(),
+                                        odd ? mk1 : mk0, odd ? mv1 : mv0, &dc->m2l_n);
             MSP_LAUNCH("m2l_keys");
-            radix_sort_dev(c, mk0, mv0, mk1, mv1, &dc->m2l_n, cap, bits_for(c.n_nodes), s);
+            radix_sort_dev(c, mk0, mv0, mk1, mv1, &dc->m2l_n, cap, xbits, s);
             k_seg_flags<<<Gt, B, 0, s>>>(mk0, &dc->m2l_n, mflag);
             MSP_LAUNCH("m2l_seg_flags");
             scan_dev(c, mflag, moff, &dc->m2l_n, cap, &dc->m2l_nseg, nullptr, s);

@@ -232,7 +232,7 @@ struct msp_ctx {
     msp::DBuf items0, items1, leaf_items, rq_key0, rq_val0, accepted, acc_off;
     msp::DBuf rq_gcnt, rq_goff;                          // requests per (channel, dendrite)
     // generic scratch
-    msp::DBuf cnt, off, scan_tmp, rs_hist, sd_tmp;
+    msp::DBuf cnt, off, rs_hist, rs_status, sd_tmp;
     // device-resident sizes and their pinned host mirror
     msp::DBuf dcount;
     msp::DevCounts* hcount = nullptr;
@@ -305,10 +305,6 @@ namespace msp {
 // ---------------------------------------------------------------------------
 // primitives (msp_prims.cu)
 // ---------------------------------------------------------------------------
-// Stable LSD radix sort of (key, value) by the low `bits` bits of key.  The
-// result ends in (keys, vals); (keys_tmp, vals_tmp) are scratch of n entries.
-void radix_sort(msp_ctx& c, uint64_t* keys, int32_t* vals, uint64_t* keys_tmp,
-                int32_t* vals_tmp, int64_t n, int bits, cudaStream_t s);
 // Step a9, the near field over the leaf pairs grouped by target leaf
 // (msp_nearfield.cu); accumulates into u_sorted and the pair table.
 // Segment and list counts live in device memory (*nseg_dev <= nseg_cap,
@@ -330,7 +326,11 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
 void scan_dev(msp_ctx& c, const int32_t* in, int32_t* out, const int64_t* n_dev, int64_t n_cap,
               int64_t* total_dst, const int64_t* base, cudaStream_t s, int64_t clamp_cap = 0,
               int64_t* overflow = nullptr, int64_t* need = nullptr, int64_t overflow_bit = 1);
-// Stable radix sort of the first *n_dev (<= n_cap) pairs.  No host sync.
+// Stable radix sort of the first *n_dev (n_dev null: n_cap) of at most n_cap
+// pairs by the low `bits` bits of the key.  No host sync.  The result ends in
+// (keys, vals); the input is read from there, or from (keys_tmp, vals_tmp)
+// when radix_from_tmp says so (an odd number of passes).
+bool radix_from_tmp(int64_t n_cap, int bits);
 void radix_sort_dev(msp_ctx& c, uint64_t* keys, int32_t* vals, uint64_t* keys_tmp,
                     int32_t* vals_tmp, const int64_t* n_dev, int64_t n_cap, int bits,
                     cudaStream_t s);

@@ -638,9 +638,11 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
     // the order and the source ranges depend on the lists only: kept when
     // the lists are (keep_order)
     if (!keep_order) {
+        const bool odd = radix_from_tmp(nseg_cap, 16);
         k_seg_order_keys<<<(int)std::max<int64_t>(1, (int64_t)c.sm_count * 16), 128, 0, s>>>(
             seg_first, nseg_dev, list_q, c.pr_X.get<int32_t>(), c.pr_Y.get<int32_t>(),
-            c.nd_first.get<int32_t>(), c.nd_count.get<int32_t>(), ok0, ov0, src);
+            c.nd_first.get<int32_t>(), c.nd_count.get<int32_t>(), odd ? ok1 : ok0, odd ? ov1 : ov0,
+            src);
         MSP_LAUNCH("seg_order_keys");
         radix_sort_dev(c, ok0, ov0, ok1, ov1, nseg_dev, nseg_cap, 16, s);
     }

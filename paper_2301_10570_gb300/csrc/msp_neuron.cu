@@ -467,14 +467,18 @@ void update_synapses(msp_ctx& c, int64_t n, uint64_t step, const float* za, cons
     scan_dev(c, bin, sin, cnt + 1, 2 * n, cnt + 3, nullptr, s);
     const uint64_t seed = c.cfg.seed;
     // the axon side, then the dendrite side
-    k_del_keys<<<ge, 256, 0, s>>>(n_edges, pre, post, typ, 0, seed, step, k0, v0);
+    const int abits = 32 + bits_for_neuron(n), dbits = 32 + bits_for_neuron(2 * n);
+    const bool aodd = radix_from_tmp(cap, abits), dodd = radix_from_tmp(cap, dbits);
+    k_del_keys<<<ge, 256, 0, s>>>(n_edges, pre, post, typ, 0, seed, step, aodd ? k1 : k0,
+                                  aodd ? v1 : v0);
     MSP_LAUNCH("del_keys");
-    radix_sort_dev(c, k0, v0, k1, v1, n_edges, cap, 32 + bits_for_neuron(n), s);
+    radix_sort_dev(c, k0, v0, k1, v1, n_edges, cap, abits, s);
     k_del_mark<<<ge, 256, 0, s>>>(n_edges, k0, v0, sout, xout, del);
     MSP_LAUNCH("del_mark");
-    k_del_keys<<<ge, 256, 0, s>>>(n_edges, pre, post, typ, 1, seed, step, k0, v0);
+    k_del_keys<<<ge, 256, 0, s>>>(n_edges, pre, post, typ, 1, seed, step, dodd ? k1 : k0,
+                                  dodd ? v1 : v0);
     MSP_LAUNCH("del_keys");
-    radix_sort_dev(c, k0, v0, k1, v1, n_edges, cap, 32 + bits_for_neuron(2 * n), s);
+    radix_sort_dev(c, k0, v0, k1, v1, n_edges, cap, dbits, s);
     k_del_mark<<<ge, 256, 0, s>>>(n_edges, k0, v0, sin, xin, del);
     MSP_LAUNCH("del_mark");
     // compaction, order kept

@@ -525,18 +525,21 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
 
     // a1 + a2: keys, stable sort, gather into Morton order
     if (n > 0) {
+        const bool odd = radix_from_tmp(n, 3 * kMortonBits);
+        uint64_t* mk = odd ? k1 : k0;
+        int32_t* mv = odd ? v1 : v0;
         if (framed) {
             k_morton_frames<<<G, B, 0, s>>>(x, y, z, n, c.frame_off.get<int64_t>(),
                                             (int64_t)c.frame_off_host.size() - 1, c.frame_level,
-                                            ldexpf(cfg.side, -c.frame_level), c.morton_scale, k0,
-                                            v0, &dc->bad_pos);
+                                            ldexpf(cfg.side, -c.frame_level), c.morton_scale, mk,
+                                            mv, &dc->bad_pos);
             MSP_LAUNCH("morton_frames");
         } else {
             k_morton<<<G, B, 0, s>>>(x, y, z, n, cfg.origin[0], cfg.origin[1], cfg.origin[2],
-                                     cfg.side, c.morton_scale, k0, v0, &dc->bad_pos);
+                                     cfg.side, c.morton_scale, mk, mv, &dc->bad_pos);
             MSP_LAUNCH("morton");
         }
-        radix_sort(c, k0, v0, k1, v1, n, 3 * kMortonBits, s);
+        radix_sort_dev(c, k0, v0, k1, v1, nullptr, n, 3 * kMortonBits, s);
         k_gather<<<G, B, 0, s>>>(v0, n, x, y, z, type, va, vde, vdi, perm, inv, pts, wts, lw);
         MSP_LAUNCH("gather");
         // element offsets: exclusive prefix of the vacant axonal counts
