@@ -184,9 +184,9 @@ msp_status msp_destroy(msp_ctx* c) {
                          &c->nd_first, &c->nd_count, &c->nd_parent, &c->nd_child_first,
                          &c->nd_nchild, &c->nd_sums, &c->nd_ca, &c->nd_cd, &c->nd_arrive, &c->pr_X, &c->pr_Y,
                          &c->pr_kind, &c->pr_cf, &c->pr_nb, &c->pr_w, &c->far_q, &c->split_q, &c->m2_key0,
-                         &c->m2_key1, &c->m2_val0, &c->m2_val1, &c->m2_flag, &c->m2_off,
+                         &c->m2_key1, &c->m2_val0, &c->m2_val1, 
                          &c->m2_seg, &c->p2p_key0,
-                         &c->p2p_key1, &c->p2p_val0, &c->p2p_val1, &c->seg_first, &c->seg_flag,
+                         &c->p2p_key1, &c->p2p_val0, &c->p2p_val1, &c->seg_first,
                          &c->nf_w32, &c->nf_okey0, &c->nf_okey1, &c->nf_oval0, &c->nf_oval1, &c->nf_src,
                          &c->nr_inp, &c->nr_bout, &c->nr_bin, &c->nr_xout, &c->nr_xin,
                          &c->nr_sout, &c->nr_sin, &c->nr_cnt, &c->nr_key0, &c->nr_key1,
@@ -200,7 +200,7 @@ msp_status msp_destroy(msp_ctx* c) {
                          &c->ln_part, &c->ln_coef,
                          &c->expA, &c->expM, &c->expB, &c->u_sorted, &c->items0, &c->items1,
                          &c->leaf_items, &c->rq_key0, &c->rq_val0,
-                         &c->accepted, &c->acc_off, &c->rq_gcnt, &c->rq_goff, &c->cnt, &c->off, &c->rs_status,
+                         &c->accepted, &c->acc_off, &c->rq_gcnt, &c->rq_goff, &c->cnt, &c->off, &c->rs_status, &c->lv_status, &c->tv_status,
                          &c->rs_hist, &c->h_u, &c->h_partner, &c->h_pre,
                          &c->h_post, &c->h_type, &c->h_nsyn, &c->hs_u, &c->hs_partner,
                          &c->hs_pre, &c->hs_post, &c->hs_type, &c->hs_nsyn, &c->c_type,

@@ -2,9 +2,10 @@
 // rule, Hermite coefficients (Eq. 7), Hermite-to-Taylor translation (Eq. 7
 // composed with the Taylor expansion of Eq. 6), Taylor evaluation (Eq. 6), the
 // exact near field (Eq. 8) and the box-pair attraction table.
+#include <algorithm>
 #include <cmath>
 
-#include "msp_internal.cuh"
+#include "msp_scan.cuh"
 
 namespace msp {
 
@@ -91,140 +92,234 @@ __device__ inline uint8_t classify(const NodeView& nv, const Geo& geo, int32_t X
     return kSplit;
 }
 
-__device__ inline int block_size(const NodeView& nv, int32_t X, int32_t Y) {
-    bool lx = nv.child_first[X] < 0, ly = nv.child_first[Y] < 0;
-    return (lx ? 1 : nv.nchild[X]) * (ly ? 1 : nv.nchild[Y]);
-}
-
-// the root pair (root, root) at depth 0
-__global__ void k_init_pairs(int64_t n, int32_t* pX, int32_t* pY, DevCounts* dc) {
-    dc->depth_start[0] = 0;
-    dc->depth_start[1] = n > 0 ? 1 : 0;
-    dc->overflow &= ~1ll;       // the traversal's bit; the build's (16) stays for the step check
-    dc->need_pairs = 0;
-    dc->interactions = 0;
-    if (n > 0) {
-        pX[0] = 0;
-        pY[0] = 0;
-    }
-}
-
 // a replay that keeps the lists: only the near field's work counter restarts
 __global__ void k_reuse_init(DevCounts* dc) {
     dc->overflow &= ~1ll;
     dc->interactions = 0;
 }
 
-// pairs of one depth: [db[0], db[1]); their count goes to *scan_n
-__global__ void k_classify(const int64_t* __restrict__ db, NodeView nv, Geo geo,
-                           const int32_t* __restrict__ pX, const int32_t* __restrict__ pY,
-                           uint8_t* __restrict__ kind, int32_t* __restrict__ cnt,
-                           int64_t* __restrict__ scan_n) {
-    const int64_t q0 = db[0], nq = db[1] - db[0];
-    if (blockIdx.x == 0 && threadIdx.x == 0) *scan_n = nq;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nq;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        int64_t q = q0 + k;
-        int32_t X = pX[q], Y = pY[q];
-        uint8_t kd = classify(nv, geo, X, Y);
-        kind[q] = kd;
-        cnt[k] = kd == kSplit ? block_size(nv, X, Y) : 0;
-    }
-}
+// The traversal's tables and lists: the pair table, and as the pairs are
+// classified, in pair order, the split pairs (pair, first child, child count,
+// 0), the near-field pairs with their target leaf as the key of the sort that
+// groups them, and the far pairs.
+struct TravArgs {
+    NodeView nv;
+    Geo geo;
+    int32_t *pX, *pY, *pcf;
+    uint8_t *kind, *pnb;
+    float4* pw;
+    int64_t cap;
+    int4* split;
+    uint64_t* p2p_key;
+    int32_t *p2p_q, *far_q;
+    DevCounts* dc;
+};
 
-// Children of the split pairs of one depth, one contiguous block per pair,
-// axon-child major, from db[1] on.  When the children do not fit in the table
-// (overflow bit 0, set by the scan that also left the next depth empty) no
-// child is written and the traversal ends here; the caller grows the table
-// and redoes it.
-__global__ void k_emit_pairs(const int64_t* __restrict__ db, NodeView nv,
-                             const uint8_t* __restrict__ kind, const int32_t* __restrict__ off,
-                             int32_t* __restrict__ pX, int32_t* __restrict__ pY,
-                             int32_t* __restrict__ pcf, uint8_t* __restrict__ pnb,
-                             float4* __restrict__ pw, int64_t cap,
-                             const int64_t* __restrict__ overflow) {
-    const int64_t q0 = db[0], nq = db[1] - db[0], next0 = db[1];
-    const bool full = (*overflow & 1) != 0;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nq;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        int64_t q = q0 + k;
-        pw[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (kind[q] != kSplit) {
-            pcf[q] = -1;
-            continue;
+// Tile t of depth d (pairs q0 + 256 t ..., one per thread): classifies them
+// and counts their children and the kinds; with the sums of the tiles before
+// (excl(own, ex) gives them to every thread) writes the children, one
+// contiguous block per pair, axon-child major, from next0 on, and the list
+// entries.  A pair's children are written by its warp, 32 at a time.  Bound by
+// latency at the sizes of one network; the step of a rebuilding replay at
+// 262,144 neurons (five depths) went from 732 to 608 us with this and the
+// octree's one-launch levels (classification, scan, writing and the three
+// lists' flags, scans and compactions were 24 launches).
+//
+// Children that do not fit in the table (overflow bit 0) are not written and
+// their pair has none; the fitting ones are a prefix of the depth's children,
+// and the next depth ends there.  The caller grows the table and redoes the
+// traversal.
+constexpr int kTravTile = 256;
+
+template <class Excl>
+__device__ __forceinline__ void trav_tile(const TravArgs& a, int d, int64_t t, int64_t q0,
+                                          int64_t nq, int64_t next0, bool last, Excl exclusive) {
+    __shared__ int s_w[4][kTravTile / 32];
+    __shared__ int s_tot[4];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t k = t * kTravTile + threadIdx.x, q = q0 + k;
+    const bool in = k < nq;
+    int32_t X = 0, Y = 0;
+    uint8_t kd = kPruned;
+    int nb = 0;
+    int2 child = make_int2(0, 0);      // the first child of X (X if a leaf), of Y (Y if a leaf)
+    int ny = 1;
+    if (in) {
+        X = a.pX[q];
+        Y = a.pY[q];
+        kd = classify(a.nv, a.geo, X, Y);
+        a.kind[q] = kd;
+        a.pw[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (kd == kSplit) {
+            const int32_t cx = a.nv.child_first[X], cy = a.nv.child_first[Y];
+            const int nx = cx < 0 ? 1 : a.nv.nchild[X];
+            ny = cy < 0 ? 1 : a.nv.nchild[Y];
+            nb = nx * ny;
+            child = make_int2(cx < 0 ? X : cx, cy < 0 ? Y : cy);
         }
-        int32_t X = pX[q], Y = pY[q];
-        int64_t cf = next0 + off[k];
-        const int nb = block_size(nv, X, Y);
-        if (full || cf + nb > cap) {
-            pcf[q] = -1;
-            continue;
+    }
+    // offsets inside the tile
+    int inc = nb;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += u;
+    }
+    const unsigned mS = __ballot_sync(0xffffffffu, in && kd == kSplit);
+    const unsigned mP = __ballot_sync(0xffffffffu, in && kd == kP2P);
+    const unsigned mF = __ballot_sync(0xffffffffu, in && kd == kFar);
+    if (lane == 31) s_w[0][w] = inc;
+    if (lane == 0) {
+        s_w[1][w] = __popc(mS);
+        s_w[2][w] = __popc(mP);
+        s_w[3][w] = __popc(mF);
+    }
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        int run = 0;
+#pragma unroll
+        for (int j = 0; j < kTravTile / 32; ++j) {
+            const int v = s_w[threadIdx.x][j];
+            s_w[threadIdx.x][j] = run;
+            run += v;
         }
-        pcf[q] = (int32_t)cf;
-        pnb[q] = (uint8_t)nb;
-        int32_t cx = nv.child_first[X], cy = nv.child_first[Y];
-        if (cx >= 0 && cy >= 0) {
-            int nx = nv.nchild[X], ny = nv.nchild[Y];
-            for (int i = 0; i < nx; ++i)
-                for (int j = 0; j < ny; ++j) {
-                    pX[cf + i * ny + j] = cx + i;
-                    pY[cf + i * ny + j] = cy + j;
-                }
-        } else if (cx < 0) {
-            int ny = nv.nchild[Y];
-            for (int j = 0; j < ny; ++j) {
-                pX[cf + j] = X;
-                pY[cf + j] = cy + j;
-            }
+        s_tot[threadIdx.x] = run;
+    }
+    __syncthreads();
+    const unsigned lt = (1u << lane) - 1u;
+    const int pre = s_w[0][w] + inc - nb;
+    long long ex[4];
+    exclusive(s_tot, ex);             // a block barrier
+    const int64_t c0 = next0 + ex[0];
+    if (in) {
+        const int64_t cf = c0 + pre;
+        const bool stored = kd == kSplit && cf + nb <= a.cap;
+        a.pcf[q] = stored ? (int32_t)cf : -1;
+        if (stored) a.pnb[q] = (uint8_t)nb;
+        if (kd == kSplit) {
+            a.split[a.dc->split_start[d] + ex[1] + s_w[1][w] + __popc(mS & lt)] =
+                make_int4((int32_t)q, stored ? (int32_t)cf : -1, nb, 0);
+            // the first pair whose children do not fit
+            if (!stored && cf <= a.cap) a.dc->depth_start[d + 2] = cf;
+        } else if (kd == kP2P) {
+            const int64_t r = a.dc->p2p_start[d] + ex[2] + s_w[2][w] + __popc(mP & lt);
+            a.p2p_key[r] = (uint64_t)X;
+            a.p2p_q[r] = (int32_t)q;
+        } else if (kd == kFar) {
+            a.far_q[a.dc->far_start[d] + ex[3] + s_w[3][w] + __popc(mF & lt)] = (int32_t)q;
+        }
+    }
+    // a split pair's children by the whole warp, 32 at a time
+    const int rcp = (2048 + ny - 1) / ny;         // floor(c / ny) = c rcp >> 11 for c < 64, ny <= 8
+    for (unsigned todo = mS; todo; todo &= todo - 1) {
+        const int l = __ffs(todo) - 1;
+        const int lnb = __shfl_sync(0xffffffffu, nb, l), lpre = __shfl_sync(0xffffffffu, pre, l);
+        const int lny = __shfl_sync(0xffffffffu, ny, l), lrcp = __shfl_sync(0xffffffffu, rcp, l);
+        const int2 lc = make_int2(__shfl_sync(0xffffffffu, child.x, l),
+                                  __shfl_sync(0xffffffffu, child.y, l));
+        const int64_t f = c0 + lpre;
+        if (f + lnb > a.cap) break;                // nor do the ones after it fit
+        for (int k2 = lane; k2 < lnb; k2 += 32) {
+            const int i = k2 * lrcp >> 11;
+            a.pX[f + k2] = lc.x + i;
+            a.pY[f + k2] = lc.y + k2 - i * lny;
+        }
+    }
+    if (last && threadIdx.x == 0) {
+        DevCounts* dc = a.dc;
+        const int64_t end = c0 + s_tot[0];
+        if (end <= a.cap) {
+            dc->depth_start[d + 2] = end;
         } else {
-            int nx = nv.nchild[X];
-            for (int i = 0; i < nx; ++i) {
-                pX[cf + i] = cx + i;
-                pY[cf + i] = Y;
-            }
+            atomicOr(reinterpret_cast<unsigned long long*>(&dc->overflow), 1ull);
+            atomicMax(reinterpret_cast<unsigned long long*>(&dc->need_pairs),
+                      (unsigned long long)end);
+        }
+        dc->n_split = dc->split_start[d + 1] = dc->split_start[d] + ex[1] + s_tot[1];
+        dc->n_p2p = dc->p2p_start[d + 1] = dc->p2p_start[d] + ex[2] + s_tot[2];
+        dc->n_far = dc->far_start[d + 1] = dc->far_start[d] + ex[3] + s_tot[3];
+    }
+}
+
+// a depth without pairs: its lists and the next depth are empty
+__device__ __forceinline__ void trav_empty(DevCounts* dc, int d) {
+    dc->depth_start[d + 2] = dc->depth_start[d + 1];
+    dc->n_split = dc->split_start[d + 1] = dc->split_start[d];
+    dc->n_p2p = dc->p2p_start[d + 1] = dc->p2p_start[d];
+    dc->n_far = dc->far_start[d + 1] = dc->far_start[d];
+}
+
+// the root pair (root, root) and the depths before kTopDepths (1 and at most
+// 64 pairs: one tile each) by one block
+constexpr int kTopDepths = 2;
+
+__global__ void __launch_bounds__(kTravTile) k_trav_top(TravArgs a, int64_t n, int depths) {
+    DevCounts* dc = a.dc;
+    if (threadIdx.x == 0) {
+        dc->depth_start[0] = 0;
+        dc->depth_start[1] = n > 0 ? 1 : 0;
+        dc->split_start[0] = dc->p2p_start[0] = dc->far_start[0] = 0;
+        dc->overflow &= ~1ll;       // the traversal's bit; the build's (16) stays for the step check
+        dc->need_pairs = 0;
+        dc->interactions = 0;
+        if (n > 0) {
+            a.pX[0] = 0;
+            a.pY[0] = 0;
+        }
+    }
+    for (int d = 0; d < depths; ++d) {
+        __syncthreads();
+        const int64_t q0 = dc->depth_start[d], next0 = dc->depth_start[d + 1], nq = next0 - q0;
+        __syncthreads();
+        if (nq == 0) {
+            if (threadIdx.x == 0) trav_empty(dc, d);
+        } else {
+            trav_tile(a, d, 0, q0, nq, next0, true, [](const int*, long long (&ex)[4]) {
+                ex[0] = ex[1] = ex[2] = ex[3] = 0;
+                __syncthreads();
+            });
         }
     }
 }
 
-__global__ void k_flag_kind(const uint8_t* __restrict__ kind, const int64_t* __restrict__ n_dev,
-                            uint8_t K, int32_t* __restrict__ flag) {
-    const int64_t n = *n_dev;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        flag[i] = kind[i] == K;
-}
-
-__global__ void k_compact_kind(const uint8_t* __restrict__ kind, const int64_t* __restrict__ n_dev,
-                               uint8_t K, const int32_t* __restrict__ off,
-                               const int32_t* __restrict__ pX, int32_t* __restrict__ out_q,
-                               uint64_t* __restrict__ out_key) {
-    const int64_t n = *n_dev;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        if (kind[i] == K) {
-            int32_t o = off[i];
-            out_q[o] = (int32_t)i;
-            if (out_key) out_key[o] = (uint64_t)pX[i];
-        }
-}
-
-__global__ void k_seg_flags(const uint64_t* __restrict__ key, const int64_t* __restrict__ n_dev,
-                            int32_t* __restrict__ flag) {
-    const int64_t n = *n_dev;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        flag[i] = (i == 0 || key[i] != key[i - 1]) ? 1 : 0;
-}
-
-// segment starts, and seg_first[nseg] = n
-__global__ void k_seg_first(const int32_t* __restrict__ flag, const int32_t* __restrict__ off,
-                            const int64_t* __restrict__ n_dev, const int64_t* __restrict__ nseg_dev,
-                            int32_t* __restrict__ seg_first) {
-    const int64_t n = *n_dev;
-    if (blockIdx.x == 0 && threadIdx.x == 0) seg_first[*nseg_dev] = (int32_t)n;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        if (flag[i]) seg_first[off[i]] = (int32_t)i;
+// one depth; status: a tile counter and two words per tile (children and
+// split pairs, near-field and far pairs, 31 bits each), zero on entry
+__global__ void __launch_bounds__(kTravTile)
+k_trav_depth(TravArgs a, int d, unsigned long long* status, int64_t timeout_bit) {
+    __shared__ int64_t s_tile;
+    __shared__ long long s_ex[2];
+    DevCounts* dc = a.dc;
+    const int64_t q0 = dc->depth_start[d], next0 = dc->depth_start[d + 1], nq = next0 - q0;
+    const int64_t ntiles = (nq + kTravTile - 1) / kTravTile;
+    if (ntiles == 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) trav_empty(dc, d);
+        return;
+    }
+    for (;;) {
+        if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
+        __syncthreads();
+        const int64_t t = s_tile;
+        if (t >= ntiles) break;
+        trav_tile(a, d, t, q0, nq, next0, t == ntiles - 1, [&](const int* tot, long long (&ex)[4]) {
+            if (threadIdx.x < 32) {
+                const long long own[2] = {(long long)tot[0] << 31 | tot[1],
+                                          (long long)tot[2] << 31 | tot[3]};
+                long long e[2];
+                look_back<2>(status + 1, t, own, e, &dc->overflow, timeout_bit, kSpinLimit);
+                if (threadIdx.x == 0) {
+                    s_ex[0] = e[0];
+                    s_ex[1] = e[1];
+                }
+            }
+            __syncthreads();
+            const long long m = (1ll << 31) - 1;
+            ex[0] = s_ex[0] >> 31;
+            ex[1] = s_ex[0] & m;
+            ex[2] = s_ex[1] >> 31;
+            ex[3] = s_ex[1] & m;
+        });
+        __syncthreads();
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -601,26 +696,6 @@ __global__ void k_reduce_split(const int64_t* __restrict__ sb, const int4* __res
     }
 }
 
-// the split pairs in pair order (off: exclusive scan of their flags), each
-// with its child block
-__global__ void k_compact_split(const uint8_t* __restrict__ kind, const int64_t* __restrict__ n_dev,
-                                const int32_t* __restrict__ off, const int32_t* __restrict__ pcf,
-                                const uint8_t* __restrict__ pnb, int4* __restrict__ split) {
-    const int64_t n = *n_dev;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        if (kind[i] == kSplit) split[off[i]] = make_int4((int32_t)i, pcf[i], (int)pnb[i], 0);
-}
-
-// the split pairs' range of every depth d <= D in split: the exclusive scan
-// of the split flags at the depth's first pair
-__global__ void k_split_starts(DevCounts* dc, const int32_t* __restrict__ off, int D) {
-    const int d = threadIdx.x;
-    if (d > D) return;
-    const int64_t q = dc->depth_start[d], n = dc->depth_start[D];
-    dc->split_start[d] = q < n ? (int64_t)off[q] : dc->n_split;
-}
-
 __global__ void k_scatter_u(const float* __restrict__ us, const int32_t* __restrict__ perm,
                             int64_t n, float* __restrict__ u) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
@@ -711,15 +786,12 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
     c.pr_cf.ensure<int32_t>((size_t)cap);
     c.pr_nb.ensure<uint8_t>((size_t)cap);
     c.pr_w.ensure<float4>((size_t)cap);
-    int32_t* cnt = c.cnt.ensure<int32_t>((size_t)cap);
-    int32_t* off = c.off.ensure<int32_t>((size_t)cap);
     uint8_t* kind = c.pr_kind.get<uint8_t>();
 
     int32_t* far_q = c.far_q.ensure<int32_t>((size_t)cap);
     int4* split = c.split_q.ensure<int4>((size_t)cap);
     int32_t* pv0 = c.p2p_val0.ensure<int32_t>((size_t)cap);
     int32_t* seg_first = c.seg_first.ensure<int32_t>((size_t)c.n_nodes + 2);
-    const int64_t* n_pairs_dev = &dc->depth_start[D];
     if (reuse_lists) {
         // the step graph's replays keep the traversal and the lists of the
         // eager attraction of the same positions (guarded by the build's
@@ -727,58 +799,52 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
         k_reuse_init<<<1, 1, 0, s>>>(dc);
         MSP_LAUNCH("reuse_init");
     } else {
-    // a5: breadth-first dual traversal from (root, root)
-    k_init_pairs<<<1, 1, 0, s>>>(n, c.pr_X.get<int32_t>(), c.pr_Y.get<int32_t>(), dc);
-    MSP_LAUNCH("init_pairs");
-    for (int d = 0; d < D; ++d) {
-        k_classify<<<Gt, B, 0, s>>>(&dc->depth_start[d], nv, geo, c.pr_X.get<int32_t>(),
-                                    c.pr_Y.get<int32_t>(), kind, cnt, &dc->scan_n);
-        MSP_LAUNCH("classify");
-        scan_dev(c, cnt, off, &dc->scan_n, cap, &dc->depth_start[d + 2], &dc->depth_start[d + 1], s,
-                 cap, &dc->overflow, &dc->need_pairs);
-        k_emit_pairs<<<Gt, B, 0, s>>>(&dc->depth_start[d], nv, kind, off, c.pr_X.get<int32_t>(),
-                                      c.pr_Y.get<int32_t>(), c.pr_cf.get<int32_t>(),
-                                      c.pr_nb.get<uint8_t>(), c.pr_w.get<float4>(), cap,
-                                      &dc->overflow);
-        MSP_LAUNCH("emit_pairs");
-    }
-
-    // far and near-field lists
-    int32_t* flag = cnt;
-    k_flag_kind<<<Gt, B, 0, s>>>(kind, n_pairs_dev, kSplit, flag);
-    MSP_LAUNCH("flag_split");
-    scan_dev(c, flag, off, n_pairs_dev, cap, &dc->n_split, nullptr, s);
-    k_compact_split<<<Gt, B, 0, s>>>(kind, n_pairs_dev, off, c.pr_cf.get<int32_t>(),
-                                     c.pr_nb.get<uint8_t>(), split);
-    MSP_LAUNCH("compact_split");
-    k_split_starts<<<1, 32, 0, s>>>(dc, off, D);
-    MSP_LAUNCH("split_starts");
-    k_flag_kind<<<Gt, B, 0, s>>>(kind, n_pairs_dev, kFar, flag);
-    MSP_LAUNCH("flag_far");
-    scan_dev(c, flag, off, n_pairs_dev, cap, &dc->n_far, nullptr, s);
-    k_compact_kind<<<Gt, B, 0, s>>>(kind, n_pairs_dev, kFar, off, c.pr_X.get<int32_t>(), far_q,
-                                    nullptr);
-    MSP_LAUNCH("compact_far");
-    k_flag_kind<<<Gt, B, 0, s>>>(kind, n_pairs_dev, kP2P, flag);
-    MSP_LAUNCH("flag_p2p");
-    scan_dev(c, flag, off, n_pairs_dev, cap, &dc->n_p2p, nullptr, s);
+    // a5: breadth-first dual traversal from (root, root): the first depths in
+    // one launch, then one per depth (status words cleared together; depth d
+    // holds at most 64^d pairs), each writing its part of the lists
+    const int xbits = bits_for(c.n_nodes);
+    const bool odd = radix_from_tmp(cap, xbits);
     uint64_t* pk0 = c.p2p_key0.ensure<uint64_t>((size_t)cap);
     uint64_t* pk1 = c.p2p_key1.ensure<uint64_t>((size_t)cap);
     int32_t* pv1 = c.p2p_val1.ensure<int32_t>((size_t)cap);
-    const int xbits = bits_for(c.n_nodes);
-    const bool odd = radix_from_tmp(cap, xbits);
-    k_compact_kind<<<Gt, B, 0, s>>>(kind, n_pairs_dev, kP2P, off, c.pr_X.get<int32_t>(),
-                                    odd ? pv1 : pv0, odd ? pk1 : pk0);
-    MSP_LAUNCH("compact_p2p");
+    TravArgs ta;
+    ta.nv = nv;
+    ta.geo = geo;
+    ta.pX = c.pr_X.get<int32_t>();
+    ta.pY = c.pr_Y.get<int32_t>();
+    ta.pcf = c.pr_cf.get<int32_t>();
+    ta.kind = kind;
+    ta.pnb = c.pr_nb.get<uint8_t>();
+    ta.pw = c.pr_w.get<float4>();
+    ta.cap = cap;
+    ta.split = split;
+    ta.p2p_key = odd ? pk1 : pk0;
+    ta.p2p_q = odd ? pv1 : pv0;
+    ta.far_q = far_q;
+    ta.dc = dc;
+    auto tiles_at = [&](int d) {
+        const int64_t pairs = d < 5 ? std::min<int64_t>((int64_t)1 << (6 * d), cap) : cap;
+        return (pairs + kTravTile - 1) / kTravTile;
+    };
+    const int dtop = std::min(D, kTopDepths);
+    int64_t nw = 0;
+    for (int d = dtop; d < D; ++d) nw += 1 + 2 * tiles_at(d);
+    unsigned long long* st = c.tv_status.ensure<unsigned long long>((size_t)std::max<int64_t>(nw, 1));
+    if (nw > 0) MSP_CUDA(cudaMemsetAsync(st, 0, (size_t)nw * sizeof(unsigned long long), s));
+    k_trav_top<<<1, kTravTile, 0, s>>>(ta, n, dtop);
+    MSP_LAUNCH("trav_top");
+    for (int d = dtop; d < D; ++d) {
+        const int64_t tiles = tiles_at(d);
+        k_trav_depth<<<(unsigned)std::min<int64_t>(tiles, (int64_t)c.sm_count * 6), kTravTile, 0, s>>>(
+            ta, d, st, kScanTimeoutBit);
+        MSP_LAUNCH("trav_depth");
+        st += 1 + 2 * tiles;
+    }
+    // the near-field list grouped by target leaf (at most one segment per box)
     radix_sort_dev(c, pk0, pv0, pk1, pv1, &dc->n_p2p, cap, xbits, s);
-    int32_t* sflag = c.seg_flag.ensure<int32_t>((size_t)cap);
-    int32_t* soff = cnt;
-    k_seg_flags<<<Gt, B, 0, s>>>(pk0, &dc->n_p2p, sflag);
-    MSP_LAUNCH("seg_flags");
-    scan_dev(c, sflag, soff, &dc->n_p2p, cap, &dc->nseg, nullptr, s);
-    // at most one segment per box
-    k_seg_first<<<Gt, B, 0, s>>>(sflag, soff, &dc->n_p2p, &dc->nseg, seg_first);
-    MSP_LAUNCH("seg_first");
+    const ScanHeads head{pk0};
+    scan_launch(c, head, ScanFirsts{head, seg_first}, ScanSegments{&dc->nseg, seg_first, &dc->n_p2p},
+                &dc->n_p2p, cap, s);
     }
 
     // a6: expansions of every box at level >= l_far
@@ -819,8 +885,6 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
         uint64_t* mk1 = c.m2_key1.ensure<uint64_t>((size_t)cap);
         int32_t* mv0 = c.m2_val0.ensure<int32_t>((size_t)cap);
         int32_t* mv1 = c.m2_val1.ensure<int32_t>((size_t)cap);
-        int32_t* mflag = c.m2_flag.ensure<int32_t>((size_t)cap);
-        int32_t* moff = c.m2_off.ensure<int32_t>((size_t)cap);
         int32_t* mseg = c.m2_seg.ensure<int32_t>((size_t)c.n_nodes + 2);
         if (!reuse_lists || geo) {
             const int xbits = bits_for(c.n_nodes);
@@ -829,11 +893,9 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
                                         odd ? mk1 : mk0, odd ? mv1 : mv0, &dc->m2l_n);
             MSP_LAUNCH("m2l_keys");
             radix_sort_dev(c, mk0, mv0, mk1, mv1, &dc->m2l_n, cap, xbits, s);
-            k_seg_flags<<<Gt, B, 0, s>>>(mk0, &dc->m2l_n, mflag);
-            MSP_LAUNCH("m2l_seg_flags");
-            scan_dev(c, mflag, moff, &dc->m2l_n, cap, &dc->m2l_nseg, nullptr, s);
-            k_seg_first<<<Gt, B, 0, s>>>(mflag, moff, &dc->m2l_n, &dc->m2l_nseg, mseg);
-            MSP_LAUNCH("m2l_seg_first");
+            const ScanHeads head{mk0};
+            scan_launch(c, head, ScanFirsts{head, mseg}, ScanSegments{&dc->m2l_nseg, mseg, &dc->m2l_n},
+                        &dc->m2l_n, cap, s);
         }
         const int gm = (int)c.sm_count * 8;
 #define MSP_M2L_CASE(PP)                                                                       \

@@ -420,7 +420,7 @@ const int32_t* ps_offsets(msp_ctx& c, const uint16_t* fl, cudaStream_t s) {
     int32_t* off = c.gr_off.ensure<int32_t>((size_t)2 * n + 1);
     k_ps_flags<<<grid_for(n, 256, (int64_t)c.sm_count * 16), 256, 0, s>>>(n, fl, flag, &dc->scan_n);
     MSP_LAUNCH("ps_flags");
-    scan_dev(c, flag, off, &dc->scan_n, 2 * n + 1, nullptr, nullptr, s);
+    scan_dev(c, flag, off, &dc->scan_n, 2 * n + 1, nullptr, s);
     return off;
 }
 

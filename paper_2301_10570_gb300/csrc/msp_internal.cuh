@@ -139,7 +139,9 @@ struct DevCounts {
     int64_t m2l_n, m2l_nseg;                 // far pairs translated pair by pair, their targets
     int64_t n_split;                         // split pairs of the last traversal
     int64_t n_groups;                        // request groups (channel, dendrite): 2 n
-    int64_t split_start[kMaxLevels + 3];     // depth d split pairs: split_q[split_start[d], [d+1])
+    // depth d's split, near-field and far pairs: entries [start[d], start[d+1])
+    // of split_q, of the near-field list before its sort and of far_q
+    int64_t split_start[kMaxLevels + 3], p2p_start[kMaxLevels + 3], far_start[kMaxLevels + 3];
 };
 
 // DevCounts::overflow bit set when a bounded wait of the single-pass scan
@@ -206,8 +208,8 @@ struct msp_ctx {
     // dual traversal
     msp::DBuf pr_X, pr_Y, pr_kind, pr_cf, pr_nb, pr_w;
     // lists
-    msp::DBuf m2_key0, m2_key1, m2_val0, m2_val1, m2_flag, m2_off, m2_seg;   // far pairs by X
-    msp::DBuf far_q, p2p_key0, p2p_key1, p2p_val0, p2p_val1, seg_first, seg_flag, nf_w32;
+    msp::DBuf m2_key0, m2_key1, m2_val0, m2_val1, m2_seg;   // far pairs by X
+    msp::DBuf far_q, p2p_key0, p2p_key1, p2p_val0, p2p_val1, seg_first, nf_w32;
     msp::DBuf split_q;                                   // split pairs, by depth (int4 entries)
     msp::DBuf nf_okey0, nf_okey1, nf_oval0, nf_oval1;   // near-field segment order
     msp::DBuf nf_src;                                    // per near-field pair: (first, count) of Y
@@ -232,7 +234,7 @@ struct msp_ctx {
     msp::DBuf items0, items1, leaf_items, rq_key0, rq_val0, accepted, acc_off;
     msp::DBuf rq_gcnt, rq_goff;                          // requests per (channel, dendrite)
     // generic scratch
-    msp::DBuf cnt, off, rs_hist, rs_status, sd_tmp;
+    msp::DBuf cnt, off, rs_hist, rs_status, sd_tmp, lv_status, tv_status;
     // device-resident sizes and their pinned host mirror
     msp::DBuf dcount;
     msp::DevCounts* hcount = nullptr;
@@ -320,12 +322,10 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
                        int64_t nlist_cap, float* u_sorted, unsigned long long* work,
                        bool keep_order, cudaStream_t s);
 // Exclusive scan of in[0, *n_dev) (n_dev in device memory, at most n_cap)
-// into out; *total_dst = total (+ *base if base).  No host synchronisation.
-// With overflow given, an end above clamp_cap sets overflow_bit in *overflow,
-// raises *need to it and stores *base instead.
+// into out; *total_dst = total (may be null).  No host synchronisation.
+// (msp_scan.cuh holds the kernel, for scans of values computed on the way.)
 void scan_dev(msp_ctx& c, const int32_t* in, int32_t* out, const int64_t* n_dev, int64_t n_cap,
-              int64_t* total_dst, const int64_t* base, cudaStream_t s, int64_t clamp_cap = 0,
-              int64_t* overflow = nullptr, int64_t* need = nullptr, int64_t overflow_bit = 1);
+              int64_t* total_dst, cudaStream_t s);
 // Stable radix sort of the first *n_dev (n_dev null: n_cap) of at most n_cap
 // pairs by the low `bits` bits of the key.  No host sync.  The result ends in
 // (keys, vals); the input is read from there, or from (keys_tmp, vals_tmp)
@@ -336,7 +336,6 @@ void radix_sort_dev(msp_ctx& c, uint64_t* keys, int32_t* vals, uint64_t* keys_tm
                     cudaStream_t s);
 // small device-side bookkeeping (msp_prims.cu)
 void dev_set(int64_t* dst, int64_t v, cudaStream_t s);
-void dev_store_i32(int32_t* dst, const int64_t* src, cudaStream_t s);
 // device counts of a context and their host mirror (synchronous)
 inline DevCounts* dcounts(msp_ctx& c) { return c.dcount.get<DevCounts>(); }
 void pull_counts(msp_ctx& c, cudaStream_t s);

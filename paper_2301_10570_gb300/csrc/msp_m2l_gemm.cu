@@ -300,13 +300,13 @@ const int32_t* m2l_gemm(msp_ctx& c, const int32_t* far_q, const int64_t* nfar, i
     MSP_CUDA(cudaMemcpyAsync(cnt + 2, nfar, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
     k_group_flags<<<ge, 256, 0, s>>>(k0, nfar, flag, cnt + 2);
     MSP_LAUNCH("group_flags");
-    scan_dev(c, flag, gid, nfar, cap, cnt, nullptr, s);
+    scan_dev(c, flag, gid, nfar, cap, cnt, s);
     // gid holds the exclusive count: a group's index is gid at its flag
     k_group_starts<<<ge, 256, 0, s>>>(flag, gid, nfar, gstart);
     MSP_LAUNCH("group_starts");
     k_group_tiles<<<ge, 256, 0, s>>>(gstart, cnt, cnt + 2, ntile);
     MSP_LAUNCH("group_tiles");
-    scan_dev(c, ntile, toff, cnt, cap, cnt + 1, nullptr, s);
+    scan_dev(c, ntile, toff, cnt, cap, cnt + 1, s);
     k_tile_list<<<ge, 256, 0, s>>>(gstart, ntile, toff, cnt, tiles);
     MSP_LAUNCH("tile_list");
     const int p = c.cfg.p, p3 = p * p * p;

@@ -396,7 +396,7 @@ void neuron_steps(msp_ctx& c, int64_t n, uint64_t first_step, int n_steps,
     k_out_degree<<<ge, 256, 0, s>>>(n_edges, cap, n, pre, post, deg);
     MSP_LAUNCH("out_degree");
     dev_set(cnt, n, s);
-    scan_dev(c, deg, off, cnt, n, cnt + 2, nullptr, s);
+    scan_dev(c, deg, off, cnt, n, cnt + 2, s);
     k_out_fill<<<ge, 256, 0, s>>>(n_edges, cap, n, pre, post, off, cursor, targets);
     MSP_LAUNCH("out_fill");
     k_seed_input<<<gn, 256, 0, s>>>(n, spiked, off, deg, targets, inp);
@@ -463,8 +463,8 @@ void update_synapses(msp_ctx& c, int64_t n, uint64_t step, const float* za, cons
     k_excess<<<gn, 256, 0, s>>>(n, za, ze, zi, bout, bin, xout, xin);
     MSP_LAUNCH("excess");
     // group starts in (group, priority) order
-    scan_dev(c, bout, sout, cnt, n, cnt + 2, nullptr, s);
-    scan_dev(c, bin, sin, cnt + 1, 2 * n, cnt + 3, nullptr, s);
+    scan_dev(c, bout, sout, cnt, n, cnt + 2, s);
+    scan_dev(c, bin, sin, cnt + 1, 2 * n, cnt + 3, s);
     const uint64_t seed = c.cfg.seed;
     // the axon side, then the dendrite side
     const int abits = 32 + bits_for_neuron(n), dbits = 32 + bits_for_neuron(2 * n);
@@ -484,7 +484,7 @@ void update_synapses(msp_ctx& c, int64_t n, uint64_t step, const float* za, cons
     // compaction, order kept
     k_keep_flags<<<ge, 256, 0, s>>>(n_edges, del, keep);
     MSP_LAUNCH("keep_flags");
-    scan_dev(c, keep, pos, n_edges, cap, cnt + 2, nullptr, s);
+    scan_dev(c, keep, pos, n_edges, cap, cnt + 2, s);
     k_compact<<<ge, 256, 0, s>>>(n_edges, keep, pos, pre, post, typ, pre2, post2, typ2);
     MSP_LAUNCH("compact");
     MSP_CUDA(cudaMemcpyAsync(n_edges, cnt + 2, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));

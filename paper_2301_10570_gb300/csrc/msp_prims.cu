@@ -1,172 +1,10 @@
 // msp_prims.cu -- device-wide exclusive scan and stable LSD radix sort used by
 // the tree build, the pair lists, the descent and the request resolution.
-#include "msp_internal.cuh"
+#include "msp_scan.cuh"
 
 namespace msp {
 
 namespace {
-
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 8;
-constexpr int kScanTile = kScanThreads * kScanItems;
-
-__device__ inline long long warp_incl_scan(long long v) {
-    int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        long long t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
-    }
-    return v;
-}
-
-// exclusive scan over the block of one value per thread; returns the block total
-__device__ inline long long block_excl_scan(long long v, long long* total) {
-    __shared__ long long warp_sums[kScanThreads / 32];
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    long long inc = warp_incl_scan(v);
-    if (lane == 31) warp_sums[w] = inc;
-    __syncthreads();
-    if (w == 0) {
-        long long s = lane < kScanThreads / 32 ? warp_sums[lane] : 0;
-        long long si = warp_incl_scan(s);
-        if (lane < kScanThreads / 32) warp_sums[lane] = si - s;
-        if (lane == kScanThreads / 32 - 1) *total = si;
-    }
-    __syncthreads();
-    long long r = inc - v + warp_sums[w];
-    __syncthreads();
-    return r;
-}
-
-}  // namespace
-
-// ---------------------------------------------------------------------------
-// the element count is in device memory (no host sync; launch shapes come from
-// a host-side capacity bound)
-// ---------------------------------------------------------------------------
-namespace {
-
-// Single-pass exclusive scan of in[0, *n_dev) with a decoupled look-back.
-// Blocks take tiles in order from a counter (status[0]), so every tile's
-// predecessors have started; a tile publishes its sum (flag 1) before it
-// looks back, then its inclusive prefix (flag 2), in status[1 + tile] as one
-// 64-bit word (flag in the top two bits).  The look-back reads 32
-// predecessors per step with a warp, waiting on each for at most kSpinLimit
-// polls; a wait that gives up sets bit kScanTimeoutBit in *overflow and
-// counts the tile as 0 (the result is then wrong and the host reports it).
-// The last tile writes the total (+ *base) to *dst; with a clamp, an end
-// beyond clamp_cap is recorded (overflow_bit, need = the largest end asked
-// for) and *dst gets *base instead: the next range is empty.
-constexpr unsigned long long kFlagAgg = 1ull << 62, kFlagPre = 2ull << 62;
-constexpr unsigned long long kValMask = (1ull << 62) - 1;
-constexpr int kSpinLimit = 1 << 22;
-
-__global__ void __launch_bounds__(kScanThreads)
-k_scan_1p(const int32_t* in, int32_t* out, const int64_t* __restrict__ n_dev,
-          unsigned long long* status, int64_t* __restrict__ dst,
-          const int64_t* __restrict__ base, int64_t clamp_cap, int64_t* __restrict__ overflow,
-          int64_t* __restrict__ need, int64_t overflow_bit, int64_t timeout_bit, int spin_limit) {
-    __shared__ int32_t s_v[kScanTile + kScanTile / 32];
-    __shared__ long long s_tot, s_excl;
-    __shared__ int64_t s_tile;
-    const int64_t n = *n_dev;
-    const int64_t ntiles = (n + kScanTile - 1) / kScanTile;
-    volatile unsigned long long* st = status;
-    if (ntiles == 0) {
-        if (blockIdx.x == 0 && threadIdx.x == 0 && dst) *dst = base ? *base : 0;
-        return;
-    }
-    for (;;) {
-        if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
-        __syncthreads();
-        const int64_t t = s_tile;
-        __syncthreads();
-        if (t >= ntiles) break;
-        const int64_t t0 = t * kScanTile;
-        // coalesced load into shared memory (one padding word per 32)
-        for (int j = threadIdx.x; j < kScanTile; j += kScanThreads) {
-            const int64_t i = t0 + j;
-            s_v[j + (j >> 5)] = i < n ? in[i] : 0;
-        }
-        __syncthreads();
-        // each thread: kScanItems consecutive values
-        long long v[kScanItems];
-        long long sum = 0;
-#pragma unroll
-        for (int k = 0; k < kScanItems; ++k) {
-            const int j = threadIdx.x * kScanItems + k;
-            v[k] = s_v[j + (j >> 5)];
-            sum += v[k];
-        }
-        const long long pre = block_excl_scan(sum, &s_tot);
-        const long long agg = s_tot;
-        // publish the sum, then look back
-        if (threadIdx.x == 0)
-            st[1 + t] = (t == 0 ? kFlagPre : kFlagAgg) | ((unsigned long long)agg & kValMask);
-        if (threadIdx.x < 32) {
-            long long excl = 0;
-            int64_t j = t - 1;
-            const int lane = threadIdx.x;
-            while (j >= 0) {
-                const int64_t jj = j - lane;
-                unsigned long long w = kFlagPre;     // lanes past tile 0 count as a prefix of 0
-                if (jj >= 0) {
-                    int spin = 0;
-                    w = st[1 + jj];
-                    while ((w >> 62) == 0 && spin < spin_limit) {
-                        ++spin;
-                        w = st[1 + jj];
-                    }
-                    if ((w >> 62) == 0) {
-                        atomicOr(reinterpret_cast<unsigned long long*>(overflow),
-                                 (unsigned long long)timeout_bit);
-                        w = kFlagPre;
-                    }
-                }
-                const unsigned pmask = __ballot_sync(0xffffffffu, (w >> 62) == 2);
-                const int stop = pmask ? __ffs(pmask) - 1 : 31;   // first prefix, else all 32
-                long long val = lane <= stop ? (long long)(w & kValMask) : 0;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) val += __shfl_xor_sync(0xffffffffu, val, o);
-                excl += val;
-                if (pmask) break;
-                j -= 32;
-            }
-            if (lane == 0) {
-                s_excl = excl;
-                if (t > 0) st[1 + t] = kFlagPre | ((unsigned long long)(excl + agg) & kValMask);
-            }
-        }
-        __syncthreads();
-        const long long excl = s_excl;
-        // offsets through shared memory, stored coalesced
-        long long run = excl + pre;
-#pragma unroll
-        for (int k = 0; k < kScanItems; ++k) {
-            const int j = threadIdx.x * kScanItems + k;
-            s_v[j + (j >> 5)] = (int32_t)run;
-            run += v[k];
-        }
-        __syncthreads();
-        for (int j = threadIdx.x; j < kScanTile; j += kScanThreads) {
-            const int64_t i = t0 + j;
-            if (i < n) out[i] = s_v[j + (j >> 5)];
-        }
-        if (t == ntiles - 1 && threadIdx.x == 0 && dst) {
-            const int64_t b = base ? *base : 0;
-            int64_t end = excl + agg + b;
-            if (overflow && end > clamp_cap && clamp_cap > 0) {
-                atomicOr(reinterpret_cast<unsigned long long*>(overflow),
-                         (unsigned long long)overflow_bit);
-                atomicMax(reinterpret_cast<unsigned long long*>(need), (unsigned long long)end);
-                end = b;
-            }
-            *dst = end;
-        }
-        __syncthreads();
-    }
-}
 
 // ---------------------------------------------------------------------------
 // Stable LSD radix sort, one kernel per digit.  A first kernel counts the
@@ -387,16 +225,11 @@ k_rs_pass(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin,
 
 namespace {
 __global__ void k_dev_set(int64_t* dst, int64_t v) { *dst = v; }
-__global__ void k_dev_store_i32(int32_t* dst, const int64_t* src) { *dst = (int32_t)*src; }
 }  // namespace
 
 void dev_set(int64_t* dst, int64_t v, cudaStream_t s) {
     k_dev_set<<<1, 1, 0, s>>>(dst, v);
     MSP_LAUNCH("dev_set");
-}
-void dev_store_i32(int32_t* dst, const int64_t* src, cudaStream_t s) {
-    k_dev_store_i32<<<1, 1, 0, s>>>(dst, src);
-    MSP_LAUNCH("dev_store_i32");
 }
 void pull_counts(msp_ctx& c, cudaStream_t s) {
     MSP_CUDA(cudaMemcpyAsync(c.hcount, c.dcount.p, sizeof(DevCounts), cudaMemcpyDeviceToHost, s));
@@ -409,18 +242,8 @@ void pull_counts(msp_ctx& c, cudaStream_t s) {
 }
 
 void scan_dev(msp_ctx& c, const int32_t* in, int32_t* out, const int64_t* n_dev, int64_t n_cap,
-              int64_t* total_dst, const int64_t* base, cudaStream_t s, int64_t clamp_cap,
-              int64_t* overflow, int64_t* need, int64_t overflow_bit) {
-    const int64_t tiles_cap = std::max<int64_t>((n_cap + kScanTile - 1) / kScanTile, 1);
-    // single pass: a tile counter and one status word per tile, cleared first
-    unsigned long long* status = c.sd_tmp.ensure<unsigned long long>((size_t)tiles_cap + 1);
-    MSP_CUDA(cudaMemsetAsync(status, 0, ((size_t)tiles_cap + 1) * sizeof(unsigned long long), s));
-    const int G = (int)std::min<int64_t>(tiles_cap, (int64_t)c.sm_count * 4);
-    DevCounts* dc = dcounts(c);
-    k_scan_1p<<<G, kScanThreads, 0, s>>>(in, out, n_dev, status, total_dst, base,
-                                         overflow ? clamp_cap : 0, overflow ? overflow : &dc->overflow,
-                                         need, overflow_bit, kScanTimeoutBit, kSpinLimit);
-    MSP_LAUNCH("scan_dev");
+              int64_t* total_dst, cudaStream_t s) {
+    scan_launch(c, ScanI32{in}, ScanStore{out}, ScanTotal{total_dst}, n_dev, n_cap, s);
 }
 
 // The scan's bounded wait, exercised: the tile counter starts at 1, so tile
@@ -437,9 +260,8 @@ void scan_wait_selftest(msp_ctx& c, cudaStream_t s) {
     MSP_CUDA(cudaMemsetAsync(status, 0, 5 * sizeof(unsigned long long), s));
     dev_set(reinterpret_cast<int64_t*>(status), 1, s);       // tile 0 is skipped
     dev_set(nd, n, s);
-    k_scan_1p<<<3, kScanThreads, 0, s>>>(in, out, nd, status, nd + 1, nullptr, 0,
-                                         &dcounts(c)->overflow, nullptr, 0, kScanTimeoutBit,
-                                         1 << 12);
+    k_scan_1p<<<3, kScanThreads, 0, s>>>(ScanI32{in}, ScanStore{out}, ScanTotal{nd + 1}, nd, status,
+                                         &dcounts(c)->overflow, kScanTimeoutBit, 1 << 12);
     MSP_LAUNCH("scan_wait_selftest");
     pull_counts(c, s);
 }

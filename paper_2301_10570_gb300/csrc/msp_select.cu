@@ -6,7 +6,7 @@
 // consumption of formed synapses.
 #include <algorithm>
 
-#include "msp_internal.cuh"
+#include "msp_scan.cuh"
 
 namespace msp {
 
@@ -659,14 +659,6 @@ __global__ void k_accept(const uint64_t* __restrict__ key, const int32_t* __rest
     }
 }
 
-__global__ void k_acc_flags(const uint8_t* __restrict__ acc, const int64_t* __restrict__ n_dev,
-                            int32_t* __restrict__ flag) {
-    const int64_t n_elem = *n_dev;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n_elem;
-         e += (int64_t)gridDim.x * blockDim.x)
-        flag[e] = acc[e];
-}
-
 __global__ void k_emit_synapses(int64_t n, const uint8_t* __restrict__ type,
                                 const uint8_t* __restrict__ va, const int32_t* __restrict__ eoff,
                                 const int32_t* __restrict__ partner,
@@ -827,7 +819,6 @@ void select_partners(msp_ctx& c, uint64_t step, const uint8_t* type_dev, const u
     MSP_LAUNCH("leaf_draw");
 
     // a12: requests grouped by (channel, dendrite), ranked by (priority, element)
-    int32_t* flag = c.cnt.ensure<int32_t>((size_t)ne);
     const int gn = grid_for(n, B, (int64_t)c.sm_count * 16);
     const size_t ng = (size_t)std::max<int64_t>(2 * n, 1);
     // the group counts: cleared before an eager selection and whenever the
@@ -844,7 +835,7 @@ void select_partners(msp_ctx& c, uint64_t step, const uint8_t* type_dev, const u
     k_req_count<<<gn, B, 0, s>>>(n, type_dev, va_dev, c.elem_off.get<int32_t>(), partner, gcnt,
                                  &dc->n_elem, &dc->n_groups);
     MSP_LAUNCH("req_count");
-    scan_dev(c, gcnt, goff, &dc->n_groups, (int64_t)ng, &dc->n_req, nullptr, s);
+    scan_dev(c, gcnt, goff, &dc->n_groups, (int64_t)ng, &dc->n_req, s);
     k_req_scatter<<<gn, B, 0, s>>>(n, type_dev, va_dev, c.elem_off.get<int32_t>(), partner, goff,
                                    gcnt, cfg.seed, stp, k0, v0, &dc->n_elem, (int64_t)ne,
                                    &dc->overflow);
@@ -852,10 +843,8 @@ void select_partners(msp_ctx& c, uint64_t step, const uint8_t* type_dev, const u
     k_accept<<<ge, B, 0, s>>>(k0, v0, goff, gcnt, &dc->n_req, n, vde_dev, vdi_dev, acc,
                               &dc->overflow);
     MSP_LAUNCH("accept");
-    k_acc_flags<<<ge, B, 0, s>>>(acc, &dc->n_elem, flag);
-    MSP_LAUNCH("acc_flags");
     int32_t* soff = c.acc_off.ensure<int32_t>((size_t)ne);
-    scan_dev(c, flag, soff, &dc->n_elem, ne, &dc->n_syn, nullptr, s);
+    scan_launch(c, ScanU8{acc}, ScanStore{soff}, ScanTotal{&dc->n_syn}, &dc->n_elem, ne, s);
     k_emit_synapses<<<gn, B, 0, s>>>(n, type_dev, va_dev, c.elem_off.get<int32_t>(), partner, acc,
                                      soff, syn_pre, syn_post, syn_type, &dc->n_elem);
     MSP_LAUNCH("emit_synapses");

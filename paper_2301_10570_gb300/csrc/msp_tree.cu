@@ -1,7 +1,7 @@
 // msp_tree.cu -- steps a1-a4: Morton keys, stable sort + gather into a
 // Morton-ordered float4 array, the adaptive octree (Section 3.2) built level
 // by level, and the per-box sums of vacant elements and centroids.
-#include "msp_internal.cuh"
+#include "msp_scan.cuh"
 
 namespace msp {
 
@@ -143,151 +143,250 @@ __global__ void k_gather(const int32_t* __restrict__ order, int64_t n, const flo
     }
 }
 
-__global__ void k_u8_to_i32(const uint8_t* __restrict__ a, int64_t n, int32_t* __restrict__ out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = a[i];
+// The octree arrays and the split rule of a build.  Per-network leaf
+// capacities (cap non-null, points in frames): a box at or below the frame
+// level splits above its network's capacity, a box above it (several
+// networks' cells) always splits.
+struct LevelArgs {
+    int64_t n;
+    const uint64_t* keys;
+    uint8_t* level;
+    uint64_t* prefix;
+    int32_t *first, *count, *parent, *child_first;
+    uint8_t* nchild;
+    int leaf_capacity, max_depth;
+    const int32_t* cap;
+    int frame_level;
+    int64_t nf;
+    int64_t node_cap;
+};
+
+__device__ __forceinline__ bool splits(const LevelArgs& a, int64_t i, int level, int32_t c) {
+    int cap = a.leaf_capacity;
+    if (a.cap)
+        cap = level >= a.frame_level ? a.cap[box_frame(a.prefix[i], level, a.frame_level, a.nf)] : -1;
+    return c > cap && level < a.max_depth;
 }
 
-__global__ void k_init_root(int64_t n, uint8_t* level, uint64_t* prefix, int32_t* first,
-                            int32_t* count, int32_t* parent, int32_t* child_first,
-                            uint8_t* nchild, int64_t* level_start, int64_t* overflow) {
-    level_start[0] = 0;
-    level_start[1] = 1;
-    *overflow &= ~16ll;
-    level[0] = 0;
-    prefix[0] = 0;
-    first[0] = 0;
-    count[0] = (int32_t)n;
-    parent[0] = -1;
-    child_first[0] = -1;
-    nchild[0] = 0;
-}
-
-// first index in [lo, hi) whose octant (at shift) is >= o; octants are
-// non-decreasing inside a box because the higher bits are the box prefix
-__device__ inline int32_t octant_lower_bound(const uint64_t* __restrict__ keys, int32_t lo,
-                                             int32_t hi, int shift, uint32_t o) {
+// First index in [lo, hi) whose octant (at shift) is at least o; octants are
+// non-decreasing inside a box because the higher bits are the box prefix.
+// Seven probes at once leave an eighth of the range: a chain of 6 reads
+// instead of 18 in a box of 262,144 points.
+__device__ __forceinline__ int32_t octant_lower_bound(const uint64_t* __restrict__ keys, int32_t lo,
+                                                      int32_t hi, int shift, uint32_t o) {
     while (lo < hi) {
-        int32_t mid = lo + ((hi - lo) >> 1);
-        if (((keys[mid] >> shift) & 7u) < o)
-            lo = mid + 1;
-        else
-            hi = mid;
+        const int64_t len = hi - lo;
+        uint64_t k[7];
+#pragma unroll
+        for (int p = 0; p < 7; ++p) k[p] = keys[lo + (int32_t)(len * (p + 1) >> 3)];
+        int below = 0;
+#pragma unroll
+        for (int p = 0; p < 7; ++p) below += ((k[p] >> shift) & 7u) < o;
+        const int32_t l0 = lo;
+        if (below > 0) lo = l0 + (int32_t)(len * below >> 3) + 1;
+        if (below < 7) hi = l0 + (int32_t)(len * (below + 1) >> 3);
     }
     return lo;
 }
 
-// Octant boundaries of the boxes of one level, 8 lanes per box (one binary
-// search per octant): lane o of a box's group returns the end of octant o and
-// the start of octant o (its neighbour's end, or the box start for o = 0).
-// Whole warps take part (4 boxes per warp per round).
-struct OctantSplit {
-    int64_t k;         // box index within the level (valid if < nl)
-    bool valid, split;
-    int32_t lo, end, start;
-};
-
-// Per-network leaf capacities (Caps.cap non-null, points in frames): a box at
-// or below the frame level splits above its network's capacity, a box above
-// it (several networks' cells) always splits.
-struct Caps {
-    const int32_t* cap;        // per network, or null: leaf_capacity for every box
-    const uint64_t* prefix;    // box prefixes (with cap)
-    int frame_level;
-    int64_t nf;
-};
-
-__device__ inline OctantSplit octant_split(int64_t base, int64_t l0, int64_t nl, int level,
-                                           int leaf_capacity, int max_depth, Caps cp,
-                                           const uint64_t* __restrict__ keys,
-                                           const int32_t* __restrict__ first,
-                                           const int32_t* __restrict__ count) {
-    const int lane = threadIdx.x & 31, o = lane & 7;
-    OctantSplit r;
-    r.k = base + (lane >> 3);
-    r.valid = r.k < nl;
-    r.split = false;
-    r.lo = 0;
-    int32_t e = 0;
-    if (r.valid) {
-        const int64_t i = l0 + r.k;
-        const int32_t c = count[i];
-        r.lo = first[i];
-        int cap = leaf_capacity;
-        if (cp.cap)
-            cap = level >= cp.frame_level
-                      ? cp.cap[box_frame(cp.prefix[i], level, cp.frame_level, cp.nf)]
-                      : -1;
-        r.split = c > cap && level < max_depth;
-        if (r.split)
-            e = octant_lower_bound(keys, r.lo, r.lo + c, 3 * (kMortonBits - (level + 1)),
+// Octant boundaries of box i (level `level`), 8 lanes per box: lane o returns
+// the start and end of octant o (empty unless the box splits).  Whole warps
+// take part (4 boxes per warp).
+__device__ __forceinline__ void octant_split(const LevelArgs& a, bool valid, int64_t i, int level,
+                                             int32_t& start, int32_t& end) {
+    const int o = threadIdx.x & 7;
+    int32_t lo = 0, e = 0;
+    if (valid) {
+        const int32_t c = a.count[i];
+        lo = e = a.first[i];
+        if (splits(a, i, level, c))
+            e = octant_lower_bound(a.keys, lo, lo + c, 3 * (kMortonBits - (level + 1)),
                                    (uint32_t)o + 1);
     }
-    int32_t prev = __shfl_up_sync(0xffffffffu, e, 1);
-    r.end = e;
-    r.start = o == 0 ? r.lo : prev;
-    return r;
+    const int32_t prev = __shfl_up_sync(0xffffffffu, e, 1);
+    end = e;
+    start = o == 0 ? lo : prev;
 }
 
-// number of non-empty octants of every box at this level that is split; the
-// level's boxes are [lb[0], lb[1]), their count goes to *scan_n for the scan
-__global__ void k_count_children(const int64_t* __restrict__ lb, int level, int leaf_capacity,
-                                 int max_depth, Caps cp, const uint64_t* __restrict__ keys,
-                                 const int32_t* __restrict__ first, const int32_t* __restrict__ count,
-                                 int32_t* __restrict__ cnt, int64_t* __restrict__ scan_n) {
-    const int lane = threadIdx.x & 31;
-    const int64_t l0 = lb[0], nl = lb[1] - lb[0];
-    if (blockIdx.x == 0 && threadIdx.x == 0) *scan_n = nl;
-    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t base = wid * 4; base < nl; base += nw * 4) {
-        OctantSplit r =
-            octant_split(base, l0, nl, level, leaf_capacity, max_depth, cp, keys, first, count);
-        const unsigned m = __ballot_sync(0xffffffffu, r.split && r.end > r.start);
-        if (r.valid && (lane & 7) == 0) cnt[r.k] = __popc((m >> (lane & ~7)) & 0xffu);
+// The children of box i, one per lane with a non-empty octant: first child at
+// cf, this lane's child at ci; grp: the box's non-empty octants.
+__device__ __forceinline__ void emit_children(const LevelArgs& a, int64_t i, int level,
+                                              unsigned grp, int64_t cf, int64_t ci, int32_t start,
+                                              int32_t end) {
+    const int o = threadIdx.x & 7;
+    if (o == 0) {
+        a.child_first[i] = (int32_t)cf;
+        a.nchild[i] = (uint8_t)__popc(grp);
+    }
+    if (end > start) {
+        a.level[ci] = (uint8_t)(level + 1);
+        a.prefix[ci] = (a.prefix[i] << 3) | (uint64_t)o;
+        a.first[ci] = start;
+        a.count[ci] = end - start;
+        a.parent[ci] = (int32_t)i;
+        a.child_first[ci] = -1;
+        a.nchild[ci] = 0;
     }
 }
 
-// children of the level's boxes [lb[0], lb[1]); the next level starts at lb[1]
-__global__ void k_emit_children(const int64_t* __restrict__ lb, int level, int leaf_capacity,
-                                int max_depth, Caps cp, const uint64_t* __restrict__ keys,
-                                const int32_t* __restrict__ off, uint8_t* __restrict__ nd_level,
-                                uint64_t* __restrict__ nd_prefix, int32_t* __restrict__ nd_first,
-                                int32_t* __restrict__ nd_count, int32_t* __restrict__ nd_parent,
-                                int32_t* __restrict__ nd_child_first,
-                                uint8_t* __restrict__ nd_nchild,
-                                const int64_t* __restrict__ overflow) {
-    const int lane = threadIdx.x & 31, o = lane & 7;
-    const int64_t l0 = lb[0], nl = lb[1] - lb[0], next0 = lb[1];
-    // the node arrays could not hold the next level (a bound that cannot be
-    // exceeded; guarded all the same): no children are written
-    if (*overflow & 16) return;
-    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t base = wid * 4; base < nl; base += nw * 4) {
-        OctantSplit r = octant_split(base, l0, nl, level, leaf_capacity, max_depth, cp, keys,
-                                     nd_first, nd_count);
-        const bool ne = r.split && r.end > r.start;
-        const unsigned m = __ballot_sync(0xffffffffu, ne);
-        const unsigned grp = (m >> (lane & ~7)) & 0xffu;
-        if (!r.valid || grp == 0) continue;
-        const int64_t i = l0 + r.k;
-        const int64_t cf = next0 + off[r.k];
-        if (o == 0) {
-            nd_child_first[i] = (int32_t)cf;
-            nd_nchild[i] = (uint8_t)__popc(grp);
+// The root and the levels below it down to level `levels` (at most kTopLevels:
+// one round of at most 64 boxes per level) by one block, a block barrier
+// between levels instead of a launch each.  (A fourth level, four rounds of
+// dependent reads on one SM, took longer than a launch over several.)
+constexpr int kTopLevels = 3;
+
+__global__ void __launch_bounds__(1024) k_tree_top(LevelArgs a, int levels, DevCounts* dc) {
+    __shared__ int s_off[32];
+    __shared__ int s_tot;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        dc->level_start[0] = 0;
+        dc->level_start[1] = 1;
+        dc->overflow &= ~16ll;
+        dc->more_levels = 0;
+        a.level[0] = 0;
+        a.prefix[0] = 0;
+        a.first[0] = 0;
+        a.count[0] = (int32_t)a.n;
+        a.parent[0] = -1;
+        a.child_first[0] = -1;
+        a.nchild[0] = 0;
+    }
+    int64_t l0 = 0, nl = 1;
+    for (int l = 0; l < levels; ++l) {
+        __syncthreads();
+        const int64_t next0 = l0 + nl;
+        int64_t run = 0;
+        for (int64_t base = 0; base < nl; base += 128) {
+            const int64_t k = base + 4 * w + (lane >> 3), i = l0 + k;
+            const bool valid = k < nl;
+            int32_t start, end;
+            octant_split(a, valid, i, l, start, end);
+            const unsigned m = __ballot_sync(0xffffffffu, end > start);
+            if (lane == 0) s_off[w] = __popc(m);
+            __syncthreads();
+            if (w == 0) {
+                const int v = s_off[lane];
+                int inc = v;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int u = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += u;
+                }
+                s_off[lane] = inc - v;
+                if (lane == 31) s_tot = inc;
+            }
+            __syncthreads();
+            const int64_t at = next0 + run + s_off[w];
+            const unsigned grp = (m >> (lane & ~7)) & 0xffu;
+            const bool fits = next0 + run + s_tot <= a.node_cap;
+            if (valid && grp && fits)
+                emit_children(a, i, l, grp, at + __popc(m & ((1u << (lane & ~7)) - 1u)),
+                              at + __popc(m & ((1u << lane) - 1u)), start, end);
+            // the node arrays could not hold the level (a bound that cannot
+            // be exceeded; guarded all the same)
+            if (!fits && threadIdx.x == 0) {
+                dc->overflow |= 16;
+                dc->need_nodes = next0 + run + s_tot;
+            }
+            if (fits) run += s_tot;
+            __syncthreads();
         }
-        if (ne) {
-            const int64_t ci = cf + __popc(grp & ((1u << o) - 1u));
-            nd_level[ci] = (uint8_t)(level + 1);
-            nd_prefix[ci] = (nd_prefix[i] << 3) | (uint64_t)o;
-            nd_first[ci] = r.start;
-            nd_count[ci] = r.end - r.start;
-            nd_parent[ci] = (int32_t)i;
-            nd_child_first[ci] = -1;
-            nd_nchild[ci] = 0;
+        if (threadIdx.x == 0) dc->level_start[l + 2] = next0 + run;
+        l0 = next0;
+        nl = run;
+    }
+}
+
+// One level: the children of the boxes [level_start[l], level_start[l+1]),
+// appended in box order.  A tile of 128 boxes finds its octant boundaries,
+// publishes its number of children, looks back and writes them: one launch
+// (the count, its scan and the writing with a second search took 24 us a
+// level; serialised, cold).  COUNT_ONLY: whether a box of the level would
+// split (more_levels).
+constexpr int kLevelRounds = 4;
+constexpr int kLevelTile = 32 * kLevelRounds;
+
+template <bool COUNT_ONLY>
+__global__ void __launch_bounds__(256)
+k_tree_level(LevelArgs a, int level, DevCounts* dc, unsigned long long* status,
+             int64_t timeout_bit) {
+    __shared__ int s_off[8 * kLevelRounds];
+    __shared__ int s_tot;
+    __shared__ long long s_excl;
+    __shared__ int64_t s_tile;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t l0 = dc->level_start[level], nl = dc->level_start[level + 1] - l0;
+    const int64_t next0 = l0 + nl;
+    if (COUNT_ONLY) {
+        bool any = false;
+        for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nl;
+             k += (int64_t)gridDim.x * blockDim.x)
+            any |= splits(a, l0 + k, level, a.count[l0 + k]);
+        if (__any_sync(0xffffffffu, any) && lane == 0)
+            atomicOr(reinterpret_cast<unsigned long long*>(&dc->more_levels), 1ull);
+        return;
+    }
+    const int64_t ntiles = (nl + kLevelTile - 1) / kLevelTile;
+    if (ntiles == 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) dc->level_start[level + 2] = next0;
+        return;
+    }
+    for (;;) {
+        if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
+        __syncthreads();
+        const int64_t t = s_tile;
+        if (t >= ntiles) break;
+        int32_t start[kLevelRounds], end[kLevelRounds];
+        unsigned m[kLevelRounds];
+#pragma unroll
+        for (int r = 0; r < kLevelRounds; ++r) {
+            const int64_t k = t * kLevelTile + 32 * r + 4 * w + (lane >> 3);
+            octant_split(a, k < nl, l0 + k, level, start[r], end[r]);
+            m[r] = __ballot_sync(0xffffffffu, end[r] > start[r]);
+            if (lane == 0) s_off[8 * r + w] = __popc(m[r]);
         }
+        __syncthreads();
+        if (w == 0) {
+            const int v = s_off[lane];
+            int inc = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += u;
+            }
+            s_off[lane] = inc - v;
+            const long long own[1] = {(long long)__shfl_sync(0xffffffffu, inc, 31)};
+            long long excl[1];
+            look_back<1>(status + 1, t, own, excl, &dc->overflow, timeout_bit, kSpinLimit);
+            if (lane == 0) {
+                s_excl = excl[0];
+                s_tot = (int)own[0];
+            }
+        }
+        __syncthreads();
+        const int64_t at0 = next0 + s_excl;
+        const bool fits = at0 + s_tot <= a.node_cap;
+#pragma unroll
+        for (int r = 0; r < kLevelRounds; ++r) {
+            const int64_t k = t * kLevelTile + 32 * r + 4 * w + (lane >> 3);
+            const int64_t at = at0 + s_off[8 * r + w];
+            const unsigned grp = (m[r] >> (lane & ~7)) & 0xffu;
+            if (k < nl && grp && fits)
+                emit_children(a, l0 + k, level, grp,
+                              at + __popc(m[r] & ((1u << (lane & ~7)) - 1u)),
+                              at + __popc(m[r] & ((1u << lane) - 1u)), start[r], end[r]);
+        }
+        if (t == ntiles - 1 && threadIdx.x == 0) {
+            int64_t e = at0 + s_tot;
+            if (e > a.node_cap) {
+                atomicOr(reinterpret_cast<unsigned long long*>(&dc->overflow), 16ull);
+                dc->need_nodes = e;
+                e = next0;
+            }
+            dc->level_start[level + 2] = e;
+        }
+        __syncthreads();
     }
 }
 
@@ -497,11 +596,8 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
         if (n > 0) {
             k_gather<<<G, B, 0, s>>>(v0, n, x, y, z, type, va, vde, vdi, perm, inv, pts, wts, lw);
             MSP_LAUNCH("gather");
-            int32_t* tmp = c.cnt.ensure<int32_t>(nn);
-            k_u8_to_i32<<<G, B, 0, s>>>(va, n, tmp);
-            MSP_LAUNCH("u8_to_i32");
-            scan_dev(c, tmp, eoff, &dc->n, n, &dc->n_elem, nullptr, s);
-            dev_store_i32(eoff + n, &dc->n_elem, s);
+            scan_launch(c, ScanU8{va}, ScanStore{eoff}, ScanTotalAfter{&dc->n_elem, eoff, &dc->n},
+                        &dc->n, n, s);
         } else {
             dev_set(&dc->n_elem, 0, s);
         }
@@ -543,11 +639,8 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
         k_gather<<<G, B, 0, s>>>(v0, n, x, y, z, type, va, vde, vdi, perm, inv, pts, wts, lw);
         MSP_LAUNCH("gather");
         // element offsets: exclusive prefix of the vacant axonal counts
-        int32_t* tmp = c.cnt.ensure<int32_t>(nn);
-        k_u8_to_i32<<<G, B, 0, s>>>(va, n, tmp);
-        MSP_LAUNCH("u8_to_i32");
-        scan_dev(c, tmp, eoff, &dc->n, n, &dc->n_elem, nullptr, s);
-        dev_store_i32(eoff + n, &dc->n_elem, s);
+        scan_launch(c, ScanU8{va}, ScanStore{eoff}, ScanTotalAfter{&dc->n_elem, eoff, &dc->n},
+                    &dc->n, n, s);
     } else {
         dev_set(&dc->n_elem, 0, s);
     }
@@ -565,12 +658,12 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
     }
     L = std::min(std::max(L, 0), cfg.max_depth);
     const int Gt = (int)std::max<int64_t>(1, (int64_t)c.sm_count * 8);
-    Caps cp{nullptr, nullptr, c.frame_level, (int64_t)c.frame_off_host.size() - 1};
     int min_cap = cfg.leaf_capacity;
     if (framed && c.frame_plans)
         for (int32_t v : c.frame_cap_host) min_cap = std::min(min_cap, (int)v);
-    int32_t* cnt = c.cnt.ensure<int32_t>(nn + 8);
-    int32_t* off = c.off.ensure<int32_t>(nn + 8);
+    // scratch of later steps (msp_direct's lists among them), sized here
+    c.cnt.ensure<int32_t>(nn + 8);
+    c.off.ensure<int32_t>(nn + 8);
     // boxes at level l: at most min(8^l, n), and (l >= 1) at most 8 children
     // of each box of level l-1 that splits, i.e. holds more than C neurons
     const int64_t splitters = (int64_t)nn / ((int64_t)min_cap + 1);
@@ -591,10 +684,6 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
         c.nd_child_first.ensure<int32_t>((size_t)cap);
         c.nd_nchild.ensure<uint8_t>((size_t)cap);
         int4* sums = c.nd_sums.ensure<int4>((size_t)cap);
-        if (framed && c.frame_plans) {
-            cp.cap = c.frame_cap.get<int32_t>();
-            cp.prefix = c.nd_prefix.get<uint64_t>();
-        }
         float4* ca = c.nd_ca.ensure<float4>((size_t)cap);
         float4* cd = c.nd_cd.ensure<float4>((size_t)cap);
         // the arrival counters: cleared before an eager build and whenever
@@ -605,35 +694,43 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
         int32_t* arrive = c.nd_arrive.ensure<int32_t>((size_t)cap);
         if (!c.graph_mode || c.nd_arrive.bytes != arrive_bytes)
             MSP_CUDA(cudaMemsetAsync(arrive, 0, c.nd_arrive.bytes, s));
-        k_init_root<<<1, 1, 0, s>>>(n, c.nd_level.get<uint8_t>(), c.nd_prefix.get<uint64_t>(),
-                                    c.nd_first.get<int32_t>(), c.nd_count.get<int32_t>(),
-                                    c.nd_parent.get<int32_t>(), c.nd_child_first.get<int32_t>(),
-                                    c.nd_nchild.get<uint8_t>(), dc->level_start, &dc->overflow);
-        MSP_LAUNCH("init_root");
-        for (int l = 0; l < L; ++l) {
-            const int64_t lcap = level_cap(l);
-            k_count_children<<<Gt, B, 0, s>>>(&dc->level_start[l], l, cfg.leaf_capacity,
-                                              cfg.max_depth, cp, k0, c.nd_first.get<int32_t>(),
-                                              c.nd_count.get<int32_t>(), cnt, &dc->scan_n);
-            MSP_LAUNCH("count_children");
-            scan_dev(c, cnt, off, &dc->scan_n, lcap, &dc->level_start[l + 2],
-                     &dc->level_start[l + 1], s, cap, &dc->overflow, &dc->need_nodes, 16);
-            k_emit_children<<<Gt, B, 0, s>>>(
-                &dc->level_start[l], l, cfg.leaf_capacity, cfg.max_depth, cp, k0, off,
-                c.nd_level.get<uint8_t>(), c.nd_prefix.get<uint64_t>(), c.nd_first.get<int32_t>(),
-                c.nd_count.get<int32_t>(), c.nd_parent.get<int32_t>(),
-                c.nd_child_first.get<int32_t>(), c.nd_nchild.get<uint8_t>(), &dc->overflow);
-            MSP_LAUNCH("emit_children");
+        LevelArgs la;
+        la.n = n;
+        la.keys = k0;
+        la.level = c.nd_level.get<uint8_t>();
+        la.prefix = c.nd_prefix.get<uint64_t>();
+        la.first = c.nd_first.get<int32_t>();
+        la.count = c.nd_count.get<int32_t>();
+        la.parent = c.nd_parent.get<int32_t>();
+        la.child_first = c.nd_child_first.get<int32_t>();
+        la.nchild = c.nd_nchild.get<uint8_t>();
+        la.leaf_capacity = cfg.leaf_capacity;
+        la.max_depth = cfg.max_depth;
+        la.cap = framed && c.frame_plans ? c.frame_cap.get<int32_t>() : nullptr;
+        la.frame_level = c.frame_level;
+        la.nf = (int64_t)c.frame_off_host.size() - 1;
+        la.node_cap = cap;
+        // the top levels in one block, then a launch per level; per level a
+        // tile counter and one status word per tile, cleared together
+        const int top = std::min(L, kTopLevels);
+        auto words = [&](int l) { return 1 + (level_cap(l) + kLevelTile - 1) / kLevelTile; };
+        int64_t nw = 0;
+        for (int l = top; l < L; ++l) nw += words(l);
+        unsigned long long* st = c.lv_status.ensure<unsigned long long>((size_t)std::max<int64_t>(nw, 1));
+        if (nw > 0) MSP_CUDA(cudaMemsetAsync(st, 0, (size_t)nw * sizeof(unsigned long long), s));
+        k_tree_top<<<1, 1024, 0, s>>>(la, top, dc);
+        MSP_LAUNCH("tree_top");
+        for (int l = top; l < L; ++l) {
+            const int64_t tiles = words(l) - 1;
+            k_tree_level<false><<<(unsigned)std::min<int64_t>(tiles, (int64_t)c.sm_count * 4), 256, 0,
+                                  s>>>(la, l, dc, st, kScanTimeoutBit);
+            MSP_LAUNCH("tree_level");
+            st += words(l);
         }
         // would a box of the last built level still split?
         if (L < cfg.max_depth) {
-            k_count_children<<<Gt, B, 0, s>>>(&dc->level_start[L], L, cfg.leaf_capacity,
-                                              cfg.max_depth, cp, k0, c.nd_first.get<int32_t>(),
-                                              c.nd_count.get<int32_t>(), cnt, &dc->scan_n);
-            MSP_LAUNCH("count_children");
-            scan_dev(c, cnt, off, &dc->scan_n, (int64_t)nn, &dc->more_levels, nullptr, s);
-        } else {
-            dev_set(&dc->more_levels, 0, s);
+            k_tree_level<true><<<grid_for(level_cap(L), 256, Gt), 256, 0, s>>>(la, L, dc, nullptr, 0);
+            MSP_LAUNCH("tree_more");
         }
         // a4: aggregates, leaves up to the root in one launch
         k_aggregate_tree<<<agg_grid(cap, c.sm_count), 128, 0, s>>>(
