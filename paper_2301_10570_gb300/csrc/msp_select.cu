@@ -278,25 +278,34 @@ k_descend(const Item* __restrict__ in, Tree tr, Exps ex,
 }
 
 // Per-element draw inside the chosen dendrite leaf, one warp per leaf pair
-// (X, Y, channel) taken from a device work counter: the warp stages Y's
-// points with their weights of the channel in shared memory, collects X's
-// neurons of that channel with vacant axons, and gives each lane one of them.
-// A lane forms the weights w_s K(t,s) of the sources s != t of Y, truncated at
-// the cutoff, their total and then the inclusive prefix sums in exact 64-bit
+// (X, Y, channel), or per part of X's neurons where there are few leaf pairs,
+// taken from a device work counter: the warp stages Y's points with their
+// weights of the channel in shared memory and takes X's neurons of that
+// channel with vacant axons up to 32 at a time.  Their weights w_s K(t,s) of
+// the sources s != t of Y, truncated at the cutoff, are summed in exact 64-bit
 // fixed point (scale 2^shift; a weight is at most 255: integer adds are exact
 // and full rate, where double precision adds are scarce on this GPU; weights
 // below 2^-shift, far below exp(-cutoff^2) for the cutoffs the library
-// accepts, count as zero).  The element draws r_e = floor(U_e tot) (U_e with
-// 53 bits) go in groups of up to 8 sorted thresholds; one prefix walk serves
-// a group: the first source whose inclusive prefix exceeds r_e.  Leaves of
-// more than kLdStage points (possible only where coincident points overfill a
-// leaf at the deepest level) read their points from global memory.
+// accepts, count as zero).  A lane sums a neuron's sources, or with at most 16
+// neurons a slice of them, and keeps the prefix sums of kLdBlocks blocks.  The
+// element draws r_e = floor(U_e tot) (U_e with 53 bits) are then handed out to
+// the lanes evenly, whatever each neuron's number of elements: the slice and
+// the block by the prefix sums, the source (the first one whose inclusive
+// prefix exceeds r_e) by evaluating that one block again.
+//
+// Bound by instruction issue: about 17 instructions per weight.  Against a
+// walk over blocks of 32 sources by each lane for its own neuron's elements
+// (the warp waited for its slowest lane) and one warp for a leaf pair whatever
+// their number (serialised, cold): 1,048,576 neurons 322 -> 155 us, 262,144 in
+// clusters 305 -> 95, 21,013 (some 700 leaf pairs) 223 -> 30 us.
 constexpr int kLdWarps = 4;
 constexpr int kLdStage = 256;
-constexpr int kLdBlocks = kLdStage / 32;   // blocks of 32 sources per lane slice
+constexpr int kLdBlocks = 16;              // prefix sums per lane
 
+// weight of source j: the staged point {x, y, z, w} or, for leaves of more
+// than kLdStage points, global memory
 struct LdSrc {
-    const float4* sp;      // staged points {x, y, z, w} or null (global memory)
+    const float4* sp;
     const float4* pts;
     const float2* wts;
     int32_t sf;
@@ -308,30 +317,21 @@ struct LdSrc {
     }
 };
 
-// floor(v * 2^shift) for a finite 0 <= v < 2^24 (shift <= 40), exact, from the
-// bits of v on the integer pipe: a float to 64-bit integer conversion runs on
-// the FP64 unit, which is scarce on this GPU
+// floor(v * 2^shift) for a finite 0 <= v < 2^8 (shift <= 40), exact, from the
+// bits of v on the integer pipe (a float to 64-bit integer conversion runs on
+// the FP64 unit, which is scarce on this GPU): the mantissa at the place of
+// the largest exponent, 2^47, shifted down by what the exponent lacks; v = 0
+// (and anything below 2^-shift) shifts out
 __device__ __forceinline__ uint64_t fixed_point(float v, int shift) {
     const uint32_t b = __float_as_uint(v);
-    const int e = (int)(b >> 23);                  // biased exponent (v >= 0)
-    if (e == 0) return 0ull;                       // zero or subnormal: below 2^-126
-    const uint64_t m = (uint64_t)((b & 0x7fffffu) | 0x800000u);
-    const int sh = e - 150 + shift;                // v * 2^shift = m * 2^sh
-    if (sh >= 0) return m << sh;
-    return sh > -24 ? m >> -sh : 0ull;
+    const uint32_t m = (b & 0x7fffffu) | 0x800000u;
+    const int s = min(174 - shift - (int)(b >> 23), 63);
+    return ((uint64_t)m << 24) >> s;
 }
 
-__device__ __forceinline__ uint64_t ld_weight(const float4& T, const float4& S, float k2,
-                                              float rc2, int shift) {
-    const float dx = T.x - S.x, dy = T.y - S.y, dz = T.z - S.z;
-    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    const float ws = r2 < rc2 ? S.w * ex2_approx_sel(-r2 * k2) : 0.f;
-    return fixed_point(ws, shift);
-}
-
-// the weights of two sources at once: the distance, the exponent's argument
-// and the scale in paired FP32 (each element rounded as in ld_weight, so the
-// totals and the walk see the same values)
+// the weights of two sources at once (paired FP32: each element rounded as in
+// the scalar form); a source at position self (relative to the leaf) is t
+// itself
 __device__ __forceinline__ void ld_weight2(const float4& T, const float4& S0, const float4& S1,
                                            float k2, float rc2, int shift, uint64_t& v0,
                                            uint64_t& v1) {
@@ -366,25 +366,35 @@ k_leaf_draw_w(const Item* __restrict__ items, const int64_t* __restrict__ n_leaf
               int32_t* __restrict__ partner, unsigned long long* __restrict__ draw_ctr,
               const int64_t* __restrict__ n_elem) {
     __shared__ float4 s_pts[kLdWarps][kLdStage];
-    __shared__ int32_t s_tl[kLdWarps][32];
-    __shared__ uint64_t s_bsum[kLdWarps][kLdBlocks][32];   // per lane: sums of 32 sources
+    __shared__ uint64_t s_pre[kLdWarps][kLdBlocks][32];   // inclusive prefix per block and lane
+    __shared__ float4 s_T[kLdWarps][32];                  // a round's neurons
+    __shared__ int32_t s_tl[kLdWarps][32], s_a[kLdWarps][32];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t step = stp.get();
     const int64_t ne = *n_elem;
     const int64_t n_items = min(*n_leaf, cap_leaf);
+    // parts per leaf pair: a few thousand units keep the chip's warps busy
+    // (a leaf pair alone is one long chain)
+    const int lgK = n_items >= 8192 ? 0 : (n_items >= 4096 ? 1 : (n_items >= 2048 ? 2 : 3));
     unsigned long long draws = 0;
     for (;;) {
         unsigned long long k = 0;
         if (lane == 0) k = atomicAdd(next, 1ull);
         k = __shfl_sync(0xffffffffu, k, 0);
-        if ((int64_t)k >= n_items) break;
-        const Item it = items[k];
+        if ((int64_t)(k >> lgK) >= n_items) break;
+        const Item it = items[k >> lgK];
+        const int part = (int)(k & ((1u << lgK) - 1u));
+        const int32_t tf = nfirst[it.X], tc = ncount[it.X];
+        const int parts = min(1 << lgK, (tc + 47) / 48);
+        if (part >= parts) continue;
+        const int32_t tend = (int32_t)((int64_t)tc * (part + 1) / parts);
+        int32_t pos = (int32_t)((int64_t)tc * part / parts);
         const int ch = it.ch;
         const float rc2 =
             fr.rc2 ? fr.rc2[box_frame(fr.prefix[it.X], fr.level[it.X], fr.frame_level, fr.nf)]
                    : rc2_all;
-        const int32_t tf = nfirst[it.X], tc = ncount[it.X];
         const int32_t sf = nfirst[it.Y], sc = ncount[it.Y];
+        const bool own = it.X == it.Y;         // a neuron may meet itself
         // fixed-point scale: sc weights of at most 2^8 must stay below 2^63
         int lg = 0;
         while ((1 << lg) < sc + 1 && lg < 30) ++lg;
@@ -399,21 +409,24 @@ k_leaf_draw_w(const Item* __restrict__ items, const int64_t* __restrict__ n_leaf
             __syncwarp();
             src.sp = s_pts[w];
         }
-        int32_t pos = 0;
-        while (pos < tc) {
+        while (pos < tend) {
             // up to 32 of X's neurons of the channel with vacant axons, from pos on
             int nt = 0;
-            while (pos < tc && nt < 32) {
+            while (pos < tend && nt < 32) {
                 const int32_t tt = tf + pos + lane;
-                uint32_t tw = 0;
-                if (pos + lane < tc) tw = __float_as_uint(pts[tt].w);
+                float4 P = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (pos + lane < tend) P = pts[tt];
+                const uint32_t tw = __float_as_uint(P.w);
                 const bool mine =
-                    pos + lane < tc && pk_axon(tw) > 0 && (pk_type(tw) ? 1 : 0) == ch;
+                    pos + lane < tend && pk_axon(tw) > 0 && (pk_type(tw) ? 1 : 0) == ch;
                 const unsigned mask = __ballot_sync(0xffffffffu, mine);
                 const int room = 32 - nt, cnt = __popc(mask);
                 const int take = min(cnt, room);
                 const int rank = __popc(mask & ((1u << lane) - 1u));
-                if (mine && rank < take) s_tl[w][nt + rank] = tt;
+                if (mine && rank < take) {
+                    s_tl[w][nt + rank] = tt;
+                    s_T[w][nt + rank] = P;
+                }
                 nt += take;
                 if (take < cnt) {
                     // continue after the lane of the last target taken
@@ -423,146 +436,124 @@ k_leaf_draw_w(const Item* __restrict__ items, const int64_t* __restrict__ n_leaf
                 pos += 32;
             }
             __syncwarp();
+            if (nt == 0) continue;
             // S lanes per target when the round has few targets (S = 32 / nt,
             // at most 8; TS = nt lanes per slice, the last 32 - S TS lanes idle):
             // lane = q * TS + ti takes target ti and slice q of the sources
-            const int TS = nt <= 16 ? max(nt, 1) : 32;
+            const int TS = nt <= 16 ? nt : 32;
             const int S = nt <= 16 ? min(8, 32 / TS) : 1;
             const int ti = lane % TS, q = lane / TS;
             const bool act = ti < nt && q < S;
-            const int32_t t = act ? s_tl[w][ti] : tf;
-            __syncwarp();
-            const float4 T = pts[t];
-            const int a = act ? (int)pk_axon(__float_as_uint(T.w)) : 0;
             const int L = (sc + S - 1) / S;
+            // blocks of bs sources (an even number), kLdBlocks per slice
+            const int bs = max(2, ((L + kLdBlocks - 1) / kLdBlocks + 1) & ~1);
+            const float4 T = s_T[w][act ? ti : 0];
+            const int32_t t = s_tl[w][act ? ti : 0];
             const int j0 = min(q * L, sc), j1 = min(j0 + L, sc);
-            // the slice's sum, the target's total and the slice's offset
-            // (integer sums: exact, the same as one walk over all sources);
-            // with at most kLdBlocks blocks of 32 sources per slice the block
-            // sums are kept too, so that the walk can skip whole blocks
-            const bool use_blocks = L <= 32 * kLdBlocks;
-            uint64_t part = 0;
-            if (nt > 0) {
-                // the sum over sources [ja, jb), two at a time
-                auto span = [&](int ja, int jb) {
-                    uint64_t sum = 0;
+            // the slice's block sums (integer sums: exact, the same as one
+            // walk over all sources)
+            uint64_t part_sum = 0;
+            if (act) {
+                const int self = own ? t - sf : -1;
+                for (int b = 0; b < kLdBlocks; ++b) {
+                    const int ja = j0 + b * bs, jb = min(ja + bs, j1);
                     int j = ja;
                     for (; j + 1 < jb; j += 2) {
                         uint64_t v0, v1;
                         ld_weight2(T, src.get(j), src.get(j + 1), k2, rc2, shift, v0, v1);
-                        sum += (sf + j == t ? 0ull : v0) + (sf + j + 1 == t ? 0ull : v1);
+                        if (own) {
+                            v0 = j == self ? 0ull : v0;
+                            v1 = j + 1 == self ? 0ull : v1;
+                        }
+                        part_sum += v0 + v1;
                     }
                     if (j < jb) {
-                        const uint64_t v = ld_weight(T, src.get(j), k2, rc2, shift);
-                        sum += sf + j == t ? 0ull : v;
+                        uint64_t v0, v1;
+                        const float4 Sj = src.get(j);
+                        ld_weight2(T, Sj, Sj, k2, rc2, shift, v0, v1);
+                        part_sum += own && j == self ? 0ull : v0;
                     }
-                    return sum;
-                };
-                if (use_blocks) {
-                    for (int b = 0; j0 + 32 * b < j1; ++b) {
-                        const uint64_t bsum = span(j0 + 32 * b, min(j1, j0 + 32 * b + 32));
-                        s_bsum[w][b][lane] = bsum;
-                        part += bsum;
-                    }
-                } else {
-                    part = span(j0, j1);
+                    s_pre[w][b][lane] = part_sum;
                 }
             }
-            // inclusive scan of the slices' sums over q (offsets TS, 2 TS, ...;
-            // a lane reads only from lanes of the same target below it), the
-            // target's total from its last slice
-            uint64_t incl = part;
+            // the slices' offsets (an inclusive scan over q; a lane reads only
+            // from lanes of the same target below it), added to the prefix sums
+            uint64_t incl = part_sum;
             for (int o = TS; o < S * TS; o <<= 1) {
                 const uint64_t up = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += up;
             }
-            const uint64_t tot = __shfl_sync(0xffffffffu, incl, (S - 1) * TS + ti);
-            const uint64_t off = incl - part;
-            const int32_t to = perm[t];
-            const bool draw = act && tot != 0 && (int64_t)eoff[to] + a <= ne;
-            constexpr int kGroup = 8;
-            const int groups = draw ? (a + kGroup - 1) / kGroup : 0;
-            const int gmax = __reduce_max_sync(0xffffffffu, groups);
-            for (int gi = 0; gi < gmax; ++gi) {
-                const int e0 = gi * kGroup;
-                const int ng = gi < groups ? min(kGroup, a - e0) : 0;
-                uint64_t r[kGroup];
-                int ord[kGroup];
-                for (int e = 0; e < ng; ++e) {
-                    uint32_t c1 = (uint32_t)(e0 + e) | ((uint32_t)ch << 8) | (kTagLeaf << 16);
-                    uint32_t o4[4];
-                    philox_draw(seed, (uint32_t)to, c1, step, o4);
-                    uint64_t u53 = (((uint64_t)o4[0] << 32) | o4[1]) >> 11;
-                    uint64_t v = __umul64hi(u53 << 11, tot);     // floor(u53 * tot / 2^53)
-                    int jj = e;
-                    while (jj > 0 && r[jj - 1] > v) {
-                        r[jj] = r[jj - 1];
-                        ord[jj] = ord[jj - 1];
-                        --jj;
-                    }
-                    r[jj] = v;
-                    ord[jj] = e;
-                }
-                // this slice owns the thresholds in [off, off + part): the
-                // first source whose inclusive prefix exceeds a threshold
-                // lies in the slice whose prefix range contains it
-                int nx = 0;
-                while (nx < ng && r[nx] < off) ++nx;
-                int nend = nx;
-                while (nend < ng && r[nend] < off + part) ++nend;
-                uint64_t pre = off;
-                if (use_blocks) {
-                    // from the block holding the next threshold (the blocks
-                    // before it are skipped by their sums), source by source;
-                    // at most L evaluations, the warp voting in each
-                    int b = 0, j = j0;
-                    uint64_t cb = off;          // prefix before block b
-                    bool placed = false;
-                    for (int it = 0; it < L; ++it) {
-                        if (!__any_sync(0xffffffffu, nx < nend)) break;
-                        if (nx < nend) {
-                            if (!placed) {
-                                while (cb + s_bsum[w][b][lane] <= r[nx]) {
-                                    cb += s_bsum[w][b][lane];
-                                    ++b;
-                                }
-                                j = j0 + 32 * b;
-                                pre = cb;
-                                placed = true;
-                            }
-                            const uint64_t v = ld_weight(T, src.get(j), k2, rc2, shift);
-                            pre += sf + j == t ? 0ull : v;
-                            while (nx < nend && pre > r[nx]) {
-                                partner[eoff[to] + e0 + ord[nx]] = perm[sf + j];
-                                ++draws;
-                                ++nx;
-                            }
-                            ++j;
-                            // the next threshold beyond this block: skip again
-                            if (nx < nend && r[nx] >= cb + s_bsum[w][b][lane]) {
-                                cb += s_bsum[w][b][lane];
-                                ++b;
-                                placed = false;
-                            }
-                        }
-                    }
-                } else {
-                    // every lane runs the same L iterations (the warp votes in each)
-                    for (int jj = 0; jj < L; ++jj) {
-                        const int j = j0 + jj;
-                        if (!__any_sync(0xffffffffu, nx < nend && j < j1)) break;
-                        if (nx < nend && j < j1) {
-                            const uint64_t v = ld_weight(T, src.get(j), k2, rc2, shift);
-                            pre += sf + j == t ? 0ull : v;
-                            while (nx < nend && pre > r[nx]) {
-                                partner[eoff[to] + e0 + ord[nx]] = perm[sf + j];
-                                ++draws;
-                                ++nx;
-                            }
-                        }
-                    }
-                }
+            if (S > 1 && act && q > 0) {
+                const uint64_t off = incl - part_sum;
+                for (int b = 0; b < kLdBlocks; ++b) s_pre[w][b][lane] += off;
             }
+            // the neurons' numbers of draws, and their running sum
+            const uint64_t tot = __shfl_sync(0xffffffffu, incl, (S - 1) * TS + ti);
+            int a = 0;
+            if (lane < nt) {
+                const int32_t to = perm[t];
+                a = (int)pk_axon(__float_as_uint(T.w));
+                if (tot == 0 || (int64_t)eoff[to] + a > ne) a = 0;
+            }
+            int run = a;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, run, o);
+                if (lane >= o) run += up;
+            }
+            s_a[w][lane] = run - a;
+            const int total = __shfl_sync(0xffffffffu, run, 31);
+            __syncwarp();
+            for (int d0 = 0; d0 < total; d0 += 32) {
+                const int d = d0 + lane;
+                if (d >= total) continue;
+                // the drawing neuron: the last one whose draws start at or
+                // before d (neurons without draws share the next one's start)
+                int u = 0;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    if (s_a[w][u + o] <= d) u += o;
+                const int e = d - s_a[w][u];
+                const int32_t tu = s_tl[w][u], to = perm[tu];
+                const float4 Tu = s_T[w][u];
+                uint32_t o4[4];
+                philox_draw(seed, (uint32_t)to, (uint32_t)e | ((uint32_t)ch << 8) | (kTagLeaf << 16),
+                            step, o4);
+                const uint64_t u53 = (((uint64_t)o4[0] << 32) | o4[1]) >> 11;
+                const uint64_t r =
+                    __umul64hi(u53 << 11, s_pre[w][kLdBlocks - 1][(S - 1) * TS + u]);   // floor(U tot)
+                int sq = 0;
+                while (sq + 1 < S && s_pre[w][kLdBlocks - 1][sq * TS + u] <= r) ++sq;
+                const int ln = sq * TS + u;
+                int b = 0;                     // the first block whose prefix exceeds r
+#pragma unroll
+                for (int o = kLdBlocks / 2; o > 0; o >>= 1)
+                    if (s_pre[w][b + o - 1][ln] <= r) b += o;
+                uint64_t pre = b > 0 ? s_pre[w][b - 1][ln]
+                                     : (sq > 0 ? s_pre[w][kLdBlocks - 1][ln - TS] : 0ull);
+                const int self = own ? tu - sf : -1;
+                int j = sq * L + b * bs;
+                const int je = min(min(sq * L + (b + 1) * bs, (sq + 1) * L), sc);
+                int hit = -1;
+                for (; j + 1 < je; j += 2) {
+                    uint64_t v0, v1;
+                    ld_weight2(Tu, src.get(j), src.get(j + 1), k2, rc2, shift, v0, v1);
+                    pre += j == self ? 0ull : v0;
+                    if (pre > r) {
+                        hit = j;
+                        break;
+                    }
+                    pre += j + 1 == self ? 0ull : v1;
+                    if (pre > r) {
+                        hit = j + 1;
+                        break;
+                    }
+                }
+                if (hit < 0) hit = je - 1;     // the block's sum exceeds r
+                partner[eoff[to] + e] = perm[sf + hit];
+                ++draws;
+            }
+            __syncwarp();
         }
     }
     for (int o = 16; o > 0; o >>= 1) draws += __shfl_xor_sync(0xffffffffu, draws, o);
