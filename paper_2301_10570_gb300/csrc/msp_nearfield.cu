@@ -1,12 +1,13 @@
 // msp_nearfield.cu -- step a9: the exact near field (Eq. 8) over the
 // near-field leaf pairs of the dual traversal, which dominates the step.
 //
-// Work unit: one target leaf X (one block of 4 warps) and all its partner
-// leaves Y (a contiguous segment of the pair list sorted by X).  Blocks take
-// the segments longest first (the order comes from an estimate of each
-// segment's work), so the last wave of blocks is short.  The block collects
-// the targets of X with vacant axons, up to 125 at a time, and evaluates them
-// in one pass; the warps take the partner pairs round-robin.  A lane holds R
+// Work unit: one target leaf X (one block of NW = 4, 8 or 16 warps, by the
+// number of boxes) and all its partner leaves Y (a contiguous segment of the
+// pair list sorted by X).  Blocks take the segments longest first (the order
+// comes from an estimate of each segment's work), so the last wave of blocks
+// is short.  The block collects the targets of X with vacant axons, up to 125
+// at a time, and evaluates them in one pass; the warps take the partner pairs
+// round-robin.  A lane holds R
 // targets of one channel, R = 3 or 4 chosen per round (below; excitatory
 // targets first, their count padded with empty slots to a multiple of R when
 // inhibitory ones follow).  Each warp stages the sources of its current pair
@@ -15,7 +16,7 @@
 // serves 2R evaluations; when the round's target groups fit in fewer lanes
 // they are padded to P = 2^k lanes and 32/P lanes share a group, walking
 // interleaved slices of the sources (small leaves still fill the warp).
-// The per-target sums of the 4 warps are added in a fixed order, so u is
+// The per-target sums of the warps are added in a fixed order, so u is
 // reproducible run to run.  Per pair, the warp reduces the box-pair
 // attraction W(X,Y) = sum_t a_t sum_s w_s K(t,s) of each channel in single
 // precision into a per-pair slot; a second kernel widens it into the double
@@ -40,13 +41,6 @@ namespace msp {
 
 namespace {
 
-// the block's transposed per-pair W buffer (16 pairs x 32 lanes per warp, one
-// padding column), set by the kernel before use
-__shared__ float* s_wt;
-__shared__ int32_t* s_wii;
-
-constexpr int kNFWarps = 4;
-constexpr int kNFThreads = kNFWarps * 32;
 constexpr int kNFStage = 128;
 constexpr int kNFMaxT = 32 * 4;    // targets per pass (3 or 4 per lane)
 constexpr int kNFList = 128;       // target slots per round (one pass)
@@ -89,19 +83,6 @@ struct Tgts {
     int slot0;                // slot of target 0 (targets r at slot0 + r)
 };
 
-// per slot of the current pass: 2^(-|t^|^2) (or 1), a_t times it (0 for
-// padding) and the target list (sorted index, -1 for padding; slots past the
-// pass hold stale entries whose results are discarded), set by the kernel
-// before use
-__shared__ float* s_scale;
-__shared__ float* s_fa;
-__shared__ const int32_t* s_tl;
-// per thread and target r: the compensation of the Kahan sum of the target's
-// per-pair sums, targets 2i and 2i+1 as one float2 at [i * kNFThreads +
-// thread] (kept in shared memory: the kernel's registers are taken by the
-// evaluation loop)
-__shared__ float* s_cmp;
-
 // A warp's staged sources, in pairs: pair j (sources 2j, 2j+1) is the float4
 // (x0, x1, y0, y1) at [j] and (z0, z1, c0, c1) at [kNFZE + j] for the
 // excitatory and at [kNFZI + j] for the inhibitory channel (one float4 apart
@@ -111,6 +92,32 @@ __shared__ float* s_cmp;
 constexpr int kNFZE = kNFStage / 2, kNFZI = kNFStage + 1;
 constexpr int kNFStageFloats = 4 * (kNFZI + kNFStage / 2);
 
+// A block's shared memory, NW warps.
+template <int NW>
+struct NFShared {
+    float4 st[NW][kNFStageFloats / 4];   // each warp's staged sources
+    float cmp[4 * NW * 32];              // per thread and target r: the compensation of the Kahan
+                                         // sum of the target's per-pair sums, targets 2i and 2i+1
+                                         // as one float2 at [i * threads + thread] (the kernel's
+                                         // registers are taken by the evaluation loop)
+    float wt[NW][16][33];                // transposed per-pair W (16 pairs x 32 lanes)
+    int32_t wii[NW][16];
+    float red[NW][kNFMaxT];
+    // per slot of the current pass: 2^(-|t^|^2) (or 1), a_t times it (0 for
+    // padding) and the target list (sorted index, -1 for padding; slots past
+    // the pass hold stale entries whose results are discarded)
+    float scale[kNFMaxT], fa[kNFMaxT];
+    int32_t tl[kNFList];
+    int nt, nreal, pos, R;
+};
+
+extern __shared__ float4 nf_shared[];
+
+template <int NW>
+__device__ __forceinline__ NFShared<NW>& nf_sm() {
+    return *reinterpret_cast<NFShared<NW>*>(nf_shared);
+}
+
 // Evaluate the staged source pairs [0, mp) (lane slice ksl of `slices`)
 // against the lane's R targets.  MODE 0: expanded form; 1: expanded, skipping
 // the target itself; 2: difference form; 3: difference form, skipping the
@@ -118,7 +125,7 @@ constexpr int kNFStageFloats = 4 * (kNFZI + kNFStage / 2);
 // FMAs, two EX2 and one paired add (the paired FP32 instructions take one
 // issue slot for two results); the difference form stages -s^ and takes
 // t^ - s^ first.  In MODE 1 and 3 target r sits at position
-// s_tl[slot0 + r] - base among the staged sources (out of range when it is not
+// tl[slot0 + r] - base among the staged sources (out of range when it is not
 // among them).
 template <int R, int MODE>
 __device__ __forceinline__ float2 nf_term(const Tgts<R>& tg, int r, const float4& A,
@@ -143,7 +150,8 @@ __device__ __forceinline__ float2 nf_term(const Tgts<R>& tg, int r, const float4
 
 template <int R, int MODE>
 __device__ __forceinline__ void nf_eval(const float4* st, int mp, int ksl, int slices,
-                                        const Tgts<R>& tg, int32_t base, float (&part)[R]) {
+                                        const Tgts<R>& tg, const int32_t* tl, int32_t base,
+                                        float (&part)[R]) {
     constexpr bool kSkip = MODE == 1 || MODE == 3;
     constexpr int NA = R == 2 ? 2 : 1;   // accumulator pairs per target
     float2 P[R][NA];
@@ -170,7 +178,7 @@ __device__ __forceinline__ void nf_eval(const float4* st, int mp, int ksl, int s
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             float2 X = nf_term<R, MODE>(tg, r, A, B);
-            const int d = s_tl[tg.slot0 + r] - base - 2 * j;
+            const int d = tl[tg.slot0 + r] - base - 2 * j;
             X.x = d == 0 ? 0.f : X.x;
             X.y = d == 1 ? 0.f : X.y;
             P[r][0] = __fadd2_rn(P[r][0], X);
@@ -228,24 +236,25 @@ __device__ __forceinline__ void nf_eval_unit(const float4* st, int mp, const Tgt
 }
 
 // the pairs of segment [i0, i1) that belong to warp w, for a lane holding R targets
-template <int R>
+template <int R, int NW>
 __device__ __forceinline__ void nf_pairs(const NFArgs& a, int32_t i0, int32_t i1, int32_t tf,
                                          bool fast, float cx, float cy, float cz, int ksl,
                                          int slices, const Tgts<R>& tg, float (&acc)[R],
                                          float4* stw, unsigned long long& evals, int nreal) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float (*wt)[33] = reinterpret_cast<float (*)[33]>(s_wt + w * 16 * 33);
-    int32_t* wii = s_wii + w * 16;
+    NFShared<NW>& sm = nf_sm<NW>();
+    float (*wt)[33] = sm.wt[w];
+    int32_t* wii = sm.wii[w];
     const unsigned imask = __ballot_sync(0xffffffffu, tg.ch != 0);   // inhibitory lanes
-    for (int32_t cb = i0 + w; cb < i1; cb += 32 * kNFWarps) {
+    for (int32_t cb = i0 + w; cb < i1; cb += 32 * NW) {
         // metadata of the warp's next 32 pairs, one per lane
-        int32_t mi = cb + kNFWarps * lane, msf = 0, msc = 0;
+        int32_t mi = cb + NW * lane, msf = 0, msc = 0;
         if (mi < i1) {
             const int2 m = a.src[mi];
             msf = m.x;
             msc = m.y;
         }
-        const int nb = min(32, (i1 - cb + kNFWarps - 1) / kNFWarps);
+        const int nb = min(32, (i1 - cb + NW - 1) / NW);
         for (int r = 0; r < nb; ++r) {
             const int32_t ii = __shfl_sync(0xffffffffu, mi, r);
             const int32_t sf = __shfl_sync(0xffffffffu, msf, r);
@@ -296,12 +305,12 @@ __device__ __forceinline__ void nf_pairs(const NFArgs& a, int32_t i0, int32_t i1
                 }
                 __syncwarp();
                 if (fast) {
-                    if (self)             nf_eval<R, 1>(stw, mp, ksl, slices, tg, sf + sb, part);
+                    if (self)             nf_eval<R, 1>(stw, mp, ksl, slices, tg, sm.tl, sf + sb, part);
                     else if (slices == 1) nf_eval_unit<R>(stw, mp, tg, part);
-                    else                  nf_eval<R, 0>(stw, mp, ksl, slices, tg, sf + sb, part);
+                    else                  nf_eval<R, 0>(stw, mp, ksl, slices, tg, sm.tl, sf + sb, part);
                 } else {
-                    if (self) nf_eval<R, 3>(stw, mp, ksl, slices, tg, sf + sb, part);
-                    else      nf_eval<R, 2>(stw, mp, ksl, slices, tg, sf + sb, part);
+                    if (self) nf_eval<R, 3>(stw, mp, ksl, slices, tg, sm.tl, sf + sb, part);
+                    else      nf_eval<R, 2>(stw, mp, ksl, slices, tg, sm.tl, sf + sb, part);
                 }
             }
             // the pair's sum joins the target's total by Kahan's compensated
@@ -312,7 +321,7 @@ __device__ __forceinline__ void nf_pairs(const NFArgs& a, int32_t i0, int32_t i1
             // target); the compensations of targets k, k+1 as one float2
 #pragma unroll
             for (int k = 0; k < R; k += 2) {
-                float2* cp = reinterpret_cast<float2*>(s_cmp) + (k >> 1) * kNFThreads + threadIdx.x;
+                float2* cp = reinterpret_cast<float2*>(sm.cmp) + (k >> 1) * NW * 32 + threadIdx.x;
                 if (k + 1 < R) {
                     const float2 c2 = *cp, p2 = make_float2(part[k], part[k + 1]);
                     const float2 a2 = make_float2(acc[k], acc[k + 1]);
@@ -331,7 +340,7 @@ __device__ __forceinline__ void nf_pairs(const NFArgs& a, int32_t i0, int32_t i1
                 }
             }
 #pragma unroll
-            for (int k = 0; k < R; ++k) v = fmaf(s_fa[tg.slot0 + k], part[k], v);
+            for (int k = 0; k < R; ++k) v = fmaf(sm.fa[tg.slot0 + k], part[k], v);
             // W(X,Y) of each channel: every lane's term goes into a transposed
             // buffer; every 16 pairs the warp sums the rows (half a row per
             // lane, then one shuffle) and adds them to the pairs' slots
@@ -365,13 +374,14 @@ __device__ __forceinline__ void nf_pairs(const NFArgs& a, int32_t i0, int32_t i1
 // (one channel); when they fit in fewer lanes the target groups are padded to
 // a power of two P and 32/P lanes share a group, each walking an interleaved
 // slice of the sources.
-template <int R>
-__device__ __forceinline__ void nf_targets(const NFArgs& a, const int32_t* tl, int nt, int nreal,
-                                           int32_t i0, int32_t i1, int32_t tf, bool fast, float cx,
-                                           float cy, float cz, float4* stw,
-                                           float (*red)[kNFMaxT], unsigned long long& evals) {
+template <int R, int NW>
+__device__ __forceinline__ void nf_targets(const NFArgs& a, int nt, int nreal, int32_t i0, int32_t i1,
+                                           int32_t tf, bool fast, float cx, float cy, float cz,
+                                           unsigned long long& evals) {
     static_assert(R >= 2 && R <= 4, "two to four targets per lane (the compensation buffer holds four)");
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    NFShared<NW>& sm = nf_sm<NW>();
+    const int32_t* tl = sm.tl;
     int lg = 0;
     while ((1 << lg) < (nt + R - 1) / R) ++lg;
     const int npr = 1 << lg;                // lanes per slice (target groups)
@@ -400,28 +410,25 @@ __device__ __forceinline__ void nf_targets(const NFArgs& a, const int32_t* tl, i
         tg.y[r] = make_float2(f2 * hy, f2 * hy);
         tg.z[r] = make_float2(f2 * hz, f2 * hz);
         acc[r] = 0.f;
-        reinterpret_cast<float*>(reinterpret_cast<float2*>(s_cmp) + (r >> 1) * kNFThreads +
-                                 threadIdx.x)[r & 1] = 0.f;
+        sm.cmp[2 * ((r >> 1) * NW * 32 + threadIdx.x) + (r & 1)] = 0.f;
         if (w == 0 && ksl == 0) {
             const float sc = fast ? nf_ex2(-fmaf(hx, hx, fmaf(hy, hy, hz * hz))) : 1.f;
-            s_scale[slot] = sc;
-            s_fa[slot] = valid ? (float)pk_axon(tw) * sc : 0.f;
+            sm.scale[slot] = sc;
+            sm.fa[slot] = valid ? (float)pk_axon(tw) * sc : 0.f;
         }
     }
     __syncthreads();
-    nf_pairs<R>(a, i0, i1, tf, fast, cx, cy, cz, ksl, slices, tg, acc, stw, evals, nreal);
-    // the compensated totals, then the slices of a target group and the 4
+    nf_pairs<R, NW>(a, i0, i1, tf, fast, cx, cy, cz, ksl, slices, tg, acc, sm.st[w], evals, nreal);
+    // the compensated totals, then the slices of a target group and the
     // warps in a fixed order
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        acc[r] = __fsub_rn(acc[r], reinterpret_cast<float*>(reinterpret_cast<float2*>(s_cmp) +
-                                                             (r >> 1) * kNFThreads +
-                                                             threadIdx.x)[r & 1]);
+        acc[r] = __fsub_rn(acc[r], sm.cmp[2 * ((r >> 1) * NW * 32 + threadIdx.x) + (r & 1)]);
         for (int o = npr; o < 32; o <<= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
     }
     if (ksl == 0) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) red[w][tg.slot0 + r] = acc[r];
+        for (int r = 0; r < R; ++r) sm.red[w][tg.slot0 + r] = acc[r];
     }
     __syncthreads();
     if (w == 0 && ksl == 0) {
@@ -430,33 +437,21 @@ __device__ __forceinline__ void nf_targets(const NFArgs& a, const int32_t* tl, i
             const int slot = tg.slot0 + r;
             const int32_t t = slot < nt ? tl[slot] : -1;
             if (t >= 0) {
-                float sacc = red[0][slot];
+                float sacc = sm.red[0][slot];
 #pragma unroll
-                for (int k = 1; k < kNFWarps; ++k) sacc += red[k][slot];
-                a.u[t] += sacc * s_scale[slot];
+                for (int k = 1; k < NW; ++k) sacc += sm.red[k][slot];
+                a.u[t] += sacc * sm.scale[slot];
             }
         }
     }
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kNFWarps * 32, 7) k_near_field(NFArgs a) {
-    __shared__ float4 st[kNFWarps][kNFStageFloats / 4];
-    __shared__ float red[kNFWarps][kNFMaxT];
-    __shared__ int32_t tl[kNFList];
-    __shared__ int s_nt, s_nreal, s_pos, s_R;
-    __shared__ float wt_all[kNFWarps][16][33];
-    __shared__ int32_t wii_all[kNFWarps][16];
-    __shared__ float scale_all[kNFMaxT], fa_all[kNFMaxT];
-    __shared__ __align__(16) float cmp_all[4 * kNFThreads];
-    s_cmp = cmp_all;
-    s_wt = &wt_all[0][0][0];
-    s_wii = &wii_all[0][0];
-    s_scale = scale_all;
-    s_fa = fa_all;
-    s_tl = tl;
+template <int NW>
+__global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : (NW == 8 ? 3 : 1)) k_near_field(NFArgs a) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float4* stw = st[w];
+    NFShared<NW>& sm = nf_sm<NW>();
+    int32_t* tl = sm.tl;
     const int64_t nseg = *a.nseg;
     for (int64_t b = blockIdx.x; b < nseg; b += gridDim.x) {
         const int32_t sg = a.order[b];
@@ -542,21 +537,21 @@ __global__ void __launch_bounds__(kNFWarps * 32, 7) k_near_field(NFArgs a) {
                 }
                 if (lane < pad) tl[nE + lane] = -1;
                 if (lane == 0) {
-                    s_nt = nt + pad;
-                    s_nreal = nt;
-                    s_R = R;
-                    s_pos = pend;
+                    sm.nt = nt + pad;
+                    sm.nreal = nt;
+                    sm.R = R;
+                    sm.pos = pend;
                 }
             }
             __syncthreads();
-            const int ntl = s_nt, R = s_R, nreal = s_nreal;
-            pos = s_pos;
+            const int ntl = sm.nt, R = sm.R, nreal = sm.nreal;
+            pos = sm.pos;
             __syncthreads();
             if (ntl == 0) break;
             if (R == 4)
-                nf_targets<4>(a, tl, ntl, nreal, i0, i1, tf, fast, cx, cy, cz, stw, red, evals);
+                nf_targets<4, NW>(a, ntl, nreal, i0, i1, tf, fast, cx, cy, cz, evals);
             else
-                nf_targets<3>(a, tl, ntl, nreal, i0, i1, tf, fast, cx, cy, cz, stw, red, evals);
+                nf_targets<3, NW>(a, ntl, nreal, i0, i1, tf, fast, cx, cy, cz, evals);
             if (pos >= tc) break;
         }
         if (lane == 0 && evals) atomicAdd(a.work, evals);
@@ -670,8 +665,25 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
     a.w32 = w32;
     a.work = work;
     // one block per segment; blocks past the device count return at once
-    int grid = (int)std::min<int64_t>(nseg_cap, 1 << 30);
-    k_near_field<<<grid, kNFWarps * 32, 0, s>>>(a);
+    const int grid = (int)std::min<int64_t>(nseg_cap, 1 << 30);
+    auto launch = [&](auto kernel, int nw, size_t smem) {
+        if (smem > 48 * 1024)
+            MSP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)smem));
+        kernel<<<grid, nw * 32, smem, s>>>(a);
+    };
+    // Warps per segment by the number of boxes (a bound on the segments): 4
+    // where the segments fill the chip several times (7 blocks an SM), 8 below
+    // 16 boxes an SM and 16 below 3, where the longest segment's chain is the
+    // time.  Measured, steps of clustered networks with 4 / 8 / 16 warps: 262,144
+    // neurons (27 boxes an SM) 1043 / 1093 / 1276 us, 131,072 (14) 831 / 771 /
+    // 873, 32,768 (4) 716 / 589 / 521, two of 21,013 (2.6) 1661 / 1554 / 1443.
+    if (c.n_nodes > 16 * (int64_t)c.sm_count)
+        launch(k_near_field<4>, 4, sizeof(NFShared<4>));
+    else if (c.n_nodes > 3 * (int64_t)c.sm_count)
+        launch(k_near_field<8>, 8, sizeof(NFShared<8>));
+    else
+        launch(k_near_field<16>, 16, sizeof(NFShared<16>));
     MSP_LAUNCH("near_field");
     k_widen_w<<<gl, 256, 0, s>>>(list_q, w32, nlist_dev, c.pr_w.get<float4>());
     MSP_LAUNCH("widen_w");
