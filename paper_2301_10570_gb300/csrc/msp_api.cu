@@ -188,10 +188,9 @@ msp_status msp_destroy(msp_ctx* c) {
                          &c->m2_seg, &c->p2p_key0,
                          &c->p2p_key1, &c->p2p_val0, &c->p2p_val1, &c->seg_first,
                          &c->nf_w32, &c->nf_okey0, &c->nf_okey1, &c->nf_oval0, &c->nf_oval1, &c->nf_src,
-                         &c->nr_inp, &c->nr_bout, &c->nr_bin, &c->nr_xout, &c->nr_xin,
-                         &c->nr_sout, &c->nr_sin, &c->nr_cnt, &c->nr_key0, &c->nr_key1,
-                         &c->nr_val0, &c->nr_val1, &c->nr_del, &c->nr_keep, &c->nr_pos,
-                         &c->nr_pre2, &c->nr_post2, &c->nr_typ2, &c->nd_gc, &c->gm_key0,
+                         &c->nr_inp, &c->nr_bout, &c->nr_xout, &c->nr_sout, &c->nr_pos, &c->nr_cnt,
+                         &c->nr_bin, &c->nr_xin, &c->nr_sin, &c->nr_key0, &c->nr_key1, &c->nr_val0,
+                         &c->nr_val1, &c->nr_del, &c->nr_upd, &c->nd_gc, &c->gm_key0,
                          &c->gm_key1, &c->gm_q, &c->gm_q1, &c->gm_flag, &c->gm_gid,
                          &c->gm_gstart, &c->gm_ntile, &c->gm_toff, &c->gm_tiles, &c->gm_cnt,
                          &c->frame_off, &c->frame_cap, &c->frame_g2, &c->frame_rc2,

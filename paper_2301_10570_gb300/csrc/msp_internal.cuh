@@ -213,11 +213,10 @@ struct msp_ctx {
     msp::DBuf split_q;                                   // split pairs, by depth (int4 entries)
     msp::DBuf nf_okey0, nf_okey1, nf_oval0, nf_oval1;   // near-field segment order
     msp::DBuf nf_src;                                    // per near-field pair: (first, count) of Y
-    // neuron side (msp_neuron.cu): input counts, bound synapses, excess, group
-    // starts, deletion sort keys, flags and the compacted edge copy
-    msp::DBuf nr_inp, nr_bout, nr_bin, nr_xout, nr_xin, nr_sout, nr_sin, nr_cnt;
-    msp::DBuf nr_key0, nr_key1, nr_val0, nr_val1, nr_del, nr_keep, nr_pos;
-    msp::DBuf nr_pre2, nr_post2, nr_typ2;
+    // neuron side (msp_neuron.cu): input counts, outgoing-edge lists; bound
+    // synapses, excess and starts per group, deletion sort keys and flags
+    msp::DBuf nr_inp, nr_bout, nr_xout, nr_sout, nr_pos, nr_cnt;
+    msp::DBuf nr_bin, nr_xin, nr_sin, nr_key0, nr_key1, nr_val0, nr_val1, nr_del, nr_upd;
     // geometric expansion centres and the grouped translations (msp_m2l_gemm.cu)
     int gm_smem_set = 0;   // dynamic shared memory opted in for the grouped translations
     msp::DBuf nd_gc, gm_key0, gm_key1, gm_q, gm_q1, gm_flag, gm_gid, gm_gstart, gm_ntile,
