@@ -187,7 +187,7 @@ msp_status msp_destroy(msp_ctx* c) {
                          &c->m2_key1, &c->m2_val0, &c->m2_val1, 
                          &c->m2_seg, &c->p2p_key0,
                          &c->p2p_key1, &c->p2p_val0, &c->p2p_val1, &c->seg_first,
-                         &c->nf_w32, &c->nf_okey0, &c->nf_okey1, &c->nf_oval0, &c->nf_oval1, &c->nf_src,
+                         &c->nf_w32, &c->nf_okey0, &c->nf_okey1, &c->nf_oval0, &c->nf_oval1, &c->nf_src, &c->nf_small,
                          &c->nr_inp, &c->nr_bout, &c->nr_xout, &c->nr_sout, &c->nr_pos, &c->nr_cnt,
                          &c->nr_bin, &c->nr_xin, &c->nr_sin, &c->nr_key0, &c->nr_key1, &c->nr_val0,
                          &c->nr_val1, &c->nr_del, &c->nr_upd, &c->nd_gc, &c->gm_key0,

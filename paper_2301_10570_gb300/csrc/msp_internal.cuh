@@ -213,6 +213,7 @@ struct msp_ctx {
     msp::DBuf split_q;                                   // split pairs, by depth (int4 entries)
     msp::DBuf nf_okey0, nf_okey1, nf_oval0, nf_oval1;   // near-field segment order
     msp::DBuf nf_src;                                    // per near-field pair: (first, count) of Y
+    msp::DBuf nf_small;                                  // per segment: every leaf is small
     // neuron side (msp_neuron.cu): input counts, outgoing-edge lists; bound
     // synapses, excess and starts per group, deletion sort keys and flags
     msp::DBuf nr_inp, nr_bout, nr_xout, nr_sout, nr_pos, nr_cnt;

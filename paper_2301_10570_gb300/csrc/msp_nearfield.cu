@@ -71,6 +71,8 @@ struct NFArgs {
     float* u;
     float2* w32;                 // per near-field pair (list order): W of E and I
     unsigned long long* work;
+    const uint8_t* small;        // segments that k_near_small takes, or null: none
+    float4* pw;                  // the pair table (k_near_small's results)
 };
 
 // the targets of a lane (R of them, one channel), each coordinate broadcast
@@ -447,6 +449,25 @@ __device__ __forceinline__ void nf_targets(const NFArgs& a, int nt, int nreal, i
     __syncthreads();
 }
 
+// R targets per lane (3 or 4), by the cost of a pass per staged source pair:
+// the iterations of a lane (npr / 32 with npr lanes per slice, a power of two)
+// times the cost of one iteration, the larger of the shared-memory delivery
+// (two 16-byte loads per lane: 8 cycles) and the EX2 unit (2 R results per lane
+// at ~30 per SM per clock)
+__device__ __forceinline__ int nf_pad(int nE, int nI, int R) {
+    return nI > 0 ? (R - nE % R) % R : 0;
+}
+__device__ __forceinline__ int nf_choose_r(int nE, int nI) {
+    auto cost_for = [&](int R) {
+        const int g = (nE + nI + nf_pad(nE, nI, R) + R - 1) / R;
+        if (g > 32) return 1 << 30;
+        int npr = 1;
+        while (npr < g) npr <<= 1;
+        return npr * max(53 * R, 200);
+    };
+    return cost_for(3) <= cost_for(4) ? 3 : 4;
+}
+
 template <int NW>
 __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : (NW == 8 ? 3 : 1)) k_near_field(NFArgs a) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -455,6 +476,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : (NW == 8 ? 3 : 1)) k_ne
     const int64_t nseg = *a.nseg;
     for (int64_t b = blockIdx.x; b < nseg; b += gridDim.x) {
         const int32_t sg = a.order[b];
+        if (a.small && a.small[sg]) continue;
         const int32_t i0 = a.seg_first[sg], i1 = a.seg_first[sg + 1];
         const int32_t X = a.pX[a.list_q[i0]];
         const int32_t tf = a.nfirst[X], tc = a.ncount[X];
@@ -504,22 +526,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : (NW == 8 ? 3 : 1)) k_ne
                 }
                 const int32_t pend = min(p, tc);
                 const int nI = nt - nE;
-                // R targets per lane (3 or 4), by the cost of a pass per
-                // staged source pair: the iterations of a lane (npr / 32 with
-                // npr lanes per slice, a power of two) times the cost of one
-                // iteration, the larger of the shared-memory delivery (two
-                // 16-byte loads per lane: 8 cycles) and the EX2 unit (2 R
-                // results per lane at ~30 per SM per clock)
-                auto pad_for = [&](int R) { return nI > 0 ? (R - nE % R) % R : 0; };
-                auto cost_for = [&](int R) {
-                    const int g = (nt + pad_for(R) + R - 1) / R;
-                    if (g > 32) return 1 << 30;
-                    int npr = 1;
-                    while (npr < g) npr <<= 1;
-                    return npr * max(53 * R, 200);
-                };
-                const int R = cost_for(3) <= cost_for(4) ? 3 : 4;
-                const int pad = pad_for(R);
+                const int R = nf_choose_r(nE, nI), pad = nf_pad(nE, nI, R);
                 int we = 0, wi = nE + pad;
                 for (int32_t q = pos; q < pend; q += 32) {
                     const int32_t t = tf + q + lane;
@@ -558,17 +565,193 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : (NW == 8 ? 3 : 1)) k_ne
     }
 }
 
+// Segments of small leaves (at most kNFSmall points in X and in every Y: the
+// plans with translated pairs, leaf capacity 8).  A pair is then 10 evaluations
+// or so, and a warp per pair spends nearly all its time on staging, shuffles
+// and the pair's W.  Here a warp takes a segment and its lanes take pairs: the
+// targets of X form g <= 3 groups of R slots, as in the general kernel, and a
+// pair is g neighbouring lanes, each evaluating its group against Y's points
+// read straight from memory.  W(X,Y) adds the same terms in the same order as
+// the general kernel does (source pair by source pair, group by group), so it
+// is the same bit for bit.  Bound by the latency of the points' reads.  65,536
+// neurons with translated pairs (4.2 M near-field pairs of 2.6 points a leaf):
+// 1020 us and 58 for the pair slots in the general kernel, 234 and 22 here
+// (the latter for the few segments that are not small).
+constexpr int kNFSmall = 8;
+constexpr int kNFSmallWarps = 8;
+
+template <int R>
+__device__ __forceinline__ void nf_small_segment(const NFArgs& a, const int32_t* tl, int nt, int g,
+                                                 unsigned imask, int nreal, int32_t i0, int32_t i1,
+                                                 int32_t tf, bool fast, float cx, float cy, float cz,
+                                                 unsigned long long& evals) {
+    constexpr int kPairs = kNFSmall / 2;       // staged source pairs of a leaf
+    const int lane = threadIdx.x & 31;
+    const int per = 32 / g;                    // pairs at a time
+    const int pl = lane / g, j = lane - pl * g;
+    Tgts<R> tg;
+    tg.slot0 = R * j;
+    tg.ch = (imask >> j) & 1u;
+    float fa[R], scale[R], acc[R], cmp[R];
+    int32_t t[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int slot = tg.slot0 + r;
+        t[r] = slot < nt ? tl[slot] : -1;
+        const float4 T = a.pts[t[r] >= 0 ? t[r] : tl[0]];
+        const float hx = (T.x - cx) * a.sqk, hy = (T.y - cy) * a.sqk, hz = (T.z - cz) * a.sqk;
+        const float f2 = fast ? 2.f : 1.f;
+        tg.x[r] = make_float2(f2 * hx, f2 * hx);
+        tg.y[r] = make_float2(f2 * hy, f2 * hy);
+        tg.z[r] = make_float2(f2 * hz, f2 * hz);
+        scale[r] = fast ? nf_ex2(-fmaf(hx, hx, fmaf(hy, hy, hz * hz))) : 1.f;
+        fa[r] = t[r] >= 0 ? (float)pk_axon(__float_as_uint(T.w)) * scale[r] : 0.f;
+        acc[r] = cmp[r] = 0.f;
+    }
+    const float2 nc = make_float2(-cx, -cx), ncy = make_float2(-cy, -cy), ncz = make_float2(-cz, -cz),
+                 k2 = make_float2(a.sqk, a.sqk);
+    for (int32_t ib = i0; ib < i1; ib += per) {
+        const int32_t ii = ib + pl;
+        const bool in = pl < per && ii < i1;
+        const int2 m = in ? a.src[ii] : make_int2(tf, 0);
+        const bool self = m.x == tf;
+        float part[R], v[kPairs];
+#pragma unroll
+        for (int r = 0; r < R; ++r) part[r] = 0.f;
+#pragma unroll
+        for (int q = 0; q < kPairs; ++q) {
+            v[q] = 0.f;
+            const int e = 2 * q;
+            if (e >= m.y) continue;
+            // stage as the general kernel does
+            const bool two = e + 1 < m.y;
+            const float4 S0 = a.pts[m.x + e], S1 = a.pts[m.x + (two ? e + 1 : e)];
+            const float2 L0 = a.lw[m.x + e], L1 = a.lw[m.x + (two ? e + 1 : e)];
+            float2 sx = __fmul2_rn(__fadd2_rn(make_float2(S0.x, S1.x), nc), k2);
+            float2 sy = __fmul2_rn(__fadd2_rn(make_float2(S0.y, S1.y), ncy), k2);
+            float2 sz = __fmul2_rn(__fadd2_rn(make_float2(S0.z, S1.z), ncz), k2);
+            float2 n2 = make_float2(0.f, 0.f);
+            if (fast) {
+                const float2 qq = __ffma2_rn(sx, sx, __ffma2_rn(sy, sy, __fmul2_rn(sz, sz)));
+                n2 = make_float2(-qq.x, -qq.y);
+            }
+            float2 c = __fadd2_rn(n2, tg.ch ? make_float2(L0.y, L1.y) : make_float2(L0.x, L1.x));
+            if (!fast) {
+                sx = make_float2(-sx.x, -sx.y);
+                sy = make_float2(-sy.x, -sy.y);
+                sz = make_float2(-sz.x, -sz.y);
+            }
+            if (!two) {
+                sx.y = sy.y = sz.y = 0.f;
+                c.y = -INFINITY;
+            }
+            const float4 A = make_float4(sx.x, sx.y, sy.x, sy.y), B = make_float4(sz.x, sz.y, c.x, c.y);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                float2 K = fast ? nf_term<R, 0>(tg, r, A, B) : nf_term<R, 2>(tg, r, A, B);
+                if (self) {
+                    const int d = t[r] - m.x - e;
+                    K.x = d == 0 ? 0.f : K.x;
+                    K.y = d == 1 ? 0.f : K.y;
+                }
+                const float p = K.x + K.y;
+                part[r] += p;
+                v[q] = fmaf(fa[r], p, v[q]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float y = __fsub_rn(part[r], cmp[r]);
+            const float t2 = __fadd_rn(acc[r], y);
+            cmp[r] = __fsub_rn(__fsub_rn(t2, acc[r]), y);
+            acc[r] = t2;
+        }
+        // W(X,Y) of each channel: source pairs in order, a source pair's
+        // groups in order
+        float sE = 0.f, sI = 0.f;
+#pragma unroll
+        for (int q = 0; q < kPairs; ++q)
+            for (int k = 0; k < g; ++k) {
+                const float x = __shfl_sync(0xffffffffu, v[q], pl * g + k);
+                if ((imask >> k) & 1u) sI += x; else sE += x;
+            }
+        if (in && j == 0) a.pw[a.list_q[ii]] = make_float4(sE, 0.f, sI, 0.f);
+        if (in && j == 0) evals += (unsigned long long)m.y * (unsigned long long)nreal;
+    }
+    // a group's sums over its lanes (one per pair at a time), in a fixed order
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float mine = __fsub_rn(acc[r], cmp[r]);
+        float total = 0.f;
+        for (int k = 0; k < per; ++k)
+            total += __shfl_sync(0xffffffffu, mine, k * g + j < 32 ? k * g + j : lane);
+        if (pl == 0 && t[r] >= 0) a.u[t[r]] += total * scale[r];
+    }
+}
+
+__global__ void __launch_bounds__(kNFSmallWarps * 32, 3) k_near_small(NFArgs a) {
+    __shared__ int32_t s_tl[kNFSmallWarps][kNFSmall + 4];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t nseg = *a.nseg;
+    unsigned long long evals = 0;
+    for (int64_t b = blockIdx.x * (int64_t)kNFSmallWarps + w; b < nseg;
+         b += (int64_t)gridDim.x * kNFSmallWarps) {
+        const int32_t sg = a.order[b];
+        if (!a.small[sg]) continue;
+        const int32_t i0 = a.seg_first[sg], i1 = a.seg_first[sg + 1];
+        const int32_t X = a.pX[a.list_q[i0]];
+        const int32_t tf = a.nfirst[X], tc = a.ncount[X];
+        const uint64_t pre = a.nprefix[X];
+        const int lX = (int)a.nlevel[X];
+        const float bs = ldexpf(a.side, -lX);
+        const float cx = a.ox + ((float)box_axis(pre, 0, lX, a.frame_level) + 0.5f) * bs;
+        const float cy = a.oy + ((float)box_axis(pre, 1, lX, a.frame_level) + 0.5f) * bs;
+        const float cz = a.oz + ((float)box_axis(pre, 2, lX, a.frame_level) + 0.5f) * bs;
+        const bool fast = 0.75f * a.sqk * a.sqk * bs * bs <= kNFFastT2;
+        // the targets by channel, padded, and R as the general kernel chooses
+        const uint32_t tw = lane < tc ? __float_as_uint(a.pts[tf + lane].w) : 0u;
+        const bool act = pk_axon(tw) > 0;
+        const unsigned mE = __ballot_sync(0xffffffffu, act && !pk_type(tw));
+        const unsigned mI = __ballot_sync(0xffffffffu, act && pk_type(tw));
+        const int nE = __popc(mE), nI = __popc(mI), nt = nE + nI;
+        if (nt == 0) {
+            // no target: the attractions are zero
+            for (int32_t i = i0 + lane; i < i1; i += 32)
+                a.pw[a.list_q[i]] = make_float4(0.f, 0.f, 0.f, 0.f);
+            continue;
+        }
+        const int R = nf_choose_r(nE, nI), pad = nf_pad(nE, nI, R);
+        const unsigned lt = (1u << lane) - 1u;
+        __syncwarp();
+        if ((mE >> lane) & 1u) s_tl[w][__popc(mE & lt)] = tf + lane;
+        if ((mI >> lane) & 1u) s_tl[w][nE + pad + __popc(mI & lt)] = tf + lane;
+        if (lane < pad) s_tl[w][nE + lane] = -1;
+        __syncwarp();
+        const int slots = nt + pad, g = (slots + R - 1) / R;
+        // the groups of inhibitory targets
+        const unsigned imask = nI > 0 ? ~((1u << ((nE + pad) / R)) - 1u) : 0u;
+        if (R == 4)
+            nf_small_segment<4>(a, s_tl[w], slots, g, imask, nt, i0, i1, tf, fast, cx, cy, cz, evals);
+        else
+            nf_small_segment<3>(a, s_tl[w], slots, g, imask, nt, i0, i1, tf, fast, cx, cy, cz, evals);
+    }
+    for (int o = 16; o > 0; o >>= 1) evals += __shfl_xor_sync(0xffffffffu, evals, o);
+    if (lane == 0 && evals) atomicAdd(a.work, evals);
+}
+
 // Segment order, longest first: key = 16-bit complement of 1024 log2(work),
 // work = targets of X times the sources of its partner leaves (an estimate:
 // every neuron of X counts as a target).  Also the source range of every
-// pair in list order, so the near field reads one int2 per pair.
+// pair in list order, so the near field reads one int2 per pair, and (small
+// given) whether every leaf of the segment has at most kNFSmall points.
 __global__ void k_seg_order_keys(const int32_t* __restrict__ seg_first,
                                  const int64_t* __restrict__ nseg_dev,
                                  const int32_t* __restrict__ list_q,
                                  const int32_t* __restrict__ pX, const int32_t* __restrict__ pY,
                                  const int32_t* __restrict__ nfirst,
                                  const int32_t* __restrict__ ncount, uint64_t* __restrict__ key,
-                                 int32_t* __restrict__ val, int2* __restrict__ src) {
+                                 int32_t* __restrict__ val, int2* __restrict__ src,
+                                 uint8_t* __restrict__ small) {
     // one warp per segment, lanes over its pairs
     const int64_t nseg = *nseg_dev;
     const int lane = threadIdx.x & 31;
@@ -577,11 +760,17 @@ __global__ void k_seg_order_keys(const int32_t* __restrict__ seg_first,
          sg += nw) {
         const int32_t i0 = seg_first[sg], i1 = seg_first[sg + 1];
         float srcs = 0.f;
+        int32_t most = ncount[pX[list_q[i0]]];
         for (int32_t i = i0 + lane; i < i1; i += 32) {
             const int32_t Y = pY[list_q[i]];
             const int32_t cnt = ncount[Y];
             src[i] = make_int2(nfirst[Y], cnt);
             srcs += (float)cnt;
+            most = max(most, cnt);
+        }
+        if (small) {
+            most = __reduce_max_sync(0xffffffffu, most);
+            if (lane == 0) small[sg] = most <= kNFSmall;
         }
         for (int o = 16; o > 0; o >>= 1) srcs += __shfl_xor_sync(0xffffffffu, srcs, o);
         if (lane == 0) {
@@ -599,6 +788,33 @@ __global__ void k_zero_w(float2* __restrict__ w32, const int64_t* __restrict__ n
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
         w32[i] = make_float2(0.f, 0.f);
+}
+
+// the single precision per-pair attractions of the segments that are not small
+// into the pair table
+__global__ void k_widen_big(const NFArgs a) {
+    const int64_t nseg = *a.nseg;
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t sg = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); sg < nseg;
+         sg += nw) {
+        if (a.small[sg]) continue;
+        for (int32_t i = a.seg_first[sg] + lane; i < a.seg_first[sg + 1]; i += 32) {
+            const float2 v = a.w32[i];
+            a.pw[a.list_q[i]] = make_float4(v.x, 0.f, v.y, 0.f);
+        }
+    }
+}
+__global__ void k_zero_big(const NFArgs a) {
+    const int64_t nseg = *a.nseg;
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t sg = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); sg < nseg;
+         sg += nw) {
+        if (a.small[sg]) continue;
+        for (int32_t i = a.seg_first[sg] + lane; i < a.seg_first[sg + 1]; i += 32)
+            a.w32[i] = make_float2(0.f, 0.f);
+    }
 }
 
 // the single precision per-pair attractions into the pair table (double-FP32)
@@ -622,8 +838,11 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
     const msp_config& cfg = c.cfg;
     float2* w32 = c.nf_w32.ensure<float2>((size_t)nlist_cap);
     const int gl = (int)std::max<int64_t>(1, (int64_t)c.sm_count * 8);
-    k_zero_w<<<gl, 256, 0, s>>>(w32, nlist_dev);
-    MSP_LAUNCH("zero_w");
+    // small leaves: most segments go to k_near_small
+    int max_cap = cfg.leaf_capacity;
+    if (c.frame_level > 0 && c.frame_plans)
+        for (int32_t v : c.frame_cap_host) max_cap = std::max(max_cap, (int)v);
+    uint8_t* small = max_cap <= kNFSmall ? c.nf_small.ensure<uint8_t>((size_t)nseg_cap) : nullptr;
     // longest segments first
     uint64_t* ok0 = c.nf_okey0.ensure<uint64_t>((size_t)nseg_cap);
     uint64_t* ok1 = c.nf_okey1.ensure<uint64_t>((size_t)nseg_cap);
@@ -637,7 +856,7 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
         k_seg_order_keys<<<(int)std::max<int64_t>(1, (int64_t)c.sm_count * 16), 128, 0, s>>>(
             seg_first, nseg_dev, list_q, c.pr_X.get<int32_t>(), c.pr_Y.get<int32_t>(),
             c.nd_first.get<int32_t>(), c.nd_count.get<int32_t>(), odd ? ok1 : ok0, odd ? ov1 : ov0,
-            src);
+            src, small);
         MSP_LAUNCH("seg_order_keys");
         radix_sort_dev(c, ok0, ov0, ok1, ov1, nseg_dev, nseg_cap, 16, s);
     }
@@ -664,8 +883,21 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
     a.u = u_sorted;
     a.w32 = w32;
     a.work = work;
-    // one block per segment; blocks past the device count return at once
-    const int grid = (int)std::min<int64_t>(nseg_cap, 1 << 30);
+    a.small = small;
+    a.pw = c.pr_w.get<float4>();
+    if (small) {
+        k_zero_big<<<gl, 256, 0, s>>>(a);
+        MSP_LAUNCH("zero_big");
+        k_near_small<<<gl, kNFSmallWarps * 32, 0, s>>>(a);
+        MSP_LAUNCH("near_small");
+    } else {
+        k_zero_w<<<gl, 256, 0, s>>>(w32, nlist_dev);
+        MSP_LAUNCH("zero_w");
+    }
+    // one block per segment (blocks past the device count return at once), or
+    // as many as are resident where few segments are left
+    const int64_t segs = small ? std::min<int64_t>(nseg_cap, 7 * (int64_t)c.sm_count) : nseg_cap;
+    const int grid = (int)std::min<int64_t>(segs, 1 << 30);
     auto launch = [&](auto kernel, int nw, size_t smem) {
         if (smem > 48 * 1024)
             MSP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -685,7 +917,10 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
     else
         launch(k_near_field<16>, 16, sizeof(NFShared<16>));
     MSP_LAUNCH("near_field");
-    k_widen_w<<<gl, 256, 0, s>>>(list_q, w32, nlist_dev, c.pr_w.get<float4>());
+    if (small)
+        k_widen_big<<<gl, 256, 0, s>>>(a);
+    else
+        k_widen_w<<<gl, 256, 0, s>>>(list_q, w32, nlist_dev, a.pw);
     MSP_LAUNCH("widen_w");
 }
 
