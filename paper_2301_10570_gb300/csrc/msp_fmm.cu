@@ -329,42 +329,47 @@ k_trav_depth(TravArgs a, int d, unsigned long long* status, int64_t timeout_bit)
 constexpr int kP2MThreads = 128;
 constexpr int kP2MChunk = 32;
 
+// The order is a template parameter: with it in a register the divisions of
+// every index by p and the loops over powers were most of the instructions.
+// 20 k boxes of at most 20 points, order 4: 76 us before, 20 us.  Bound by the
+// chain of a block's few steps (load, powers, sums), not by its 1 KB a box.
+template <int P>
 __global__ void __launch_bounds__(kP2MThreads)
-k_p2m(int64_t first_node, int p, float inv_sigma, const float4* __restrict__ pts,
+k_p2m(int64_t first_node, float inv_sigma, const float4* __restrict__ pts,
       const int32_t* __restrict__ nfirst, const int32_t* __restrict__ ncount,
       const float4* __restrict__ ca, const float4* __restrict__ cd, float* __restrict__ A,
       float* __restrict__ M) {
-    __shared__ float ypow[kP2MChunk][3][kMaxP];
-    __shared__ float xpow[kP2MChunk][3][kMaxP];
+    constexpr int P2 = P * P, P3 = P2 * P;
+    // powers of a point's offset from the dendritic [0] and axonal [1] centre
+    __shared__ float pow_[2][kP2MChunk][3][P];
     __shared__ float wgt[kP2MChunk][4];
     const int64_t node = first_node + blockIdx.x;
-    const int p3 = p * p * p;
     const float4 cD = cd[node], cA = ca[node];
     const int32_t f = nfirst[node], c = ncount[node];
-    constexpr int kMaxAcc = (4 * kMaxP * kMaxP * kMaxP + kP2MThreads - 1) / kP2MThreads;
-    float acc[kMaxAcc];
+    constexpr int NACC = (4 * P3 + kP2MThreads - 1) / kP2MThreads;
+    float acc[NACC];
 #pragma unroll
-    for (int r = 0; r < kMaxAcc; ++r) acc[r] = 0.f;
+    for (int r = 0; r < NACC; ++r) acc[r] = 0.f;
     for (int base = 0; base < c; base += kP2MChunk) {
-        int m = min(kP2MChunk, c - base);
-        __syncthreads();
-        for (int t = threadIdx.x; t < m * 3; t += kP2MThreads) {
-            int j = t / 3, d = t % 3;
-            float4 P = pts[f + base + j];
-            float pv = d == 0 ? P.x : (d == 1 ? P.y : P.z);
-            float yv = (pv - (d == 0 ? cD.x : (d == 1 ? cD.y : cD.z))) * inv_sigma;
-            float xv = (pv - (d == 0 ? cA.x : (d == 1 ? cA.y : cA.z))) * inv_sigma;
-            float py = 1.f, px = 1.f;
-            for (int k = 0; k < p; ++k) {
-                ypow[j][d][k] = py;
-                xpow[j][d][k] = px;
-                py *= yv;
-                px *= xv;
+        const int m = min(kP2MChunk, c - base);
+        if (base) __syncthreads();
+        // thread (point, centre, dimension)
+        for (int t = threadIdx.x; t < m * 6; t += kP2MThreads) {
+            const int j = t / 6, g = (t % 6) / 3, d = t % 3;
+            const float4 pt = pts[f + base + j];
+            const float4 c4 = g ? cA : cD;
+            const float v = ((d == 0 ? pt.x : (d == 1 ? pt.y : pt.z)) -
+                             (d == 0 ? c4.x : (d == 1 ? c4.y : c4.z))) * inv_sigma;
+            float pv = 1.f;
+#pragma unroll
+            for (int k = 0; k < P; ++k) {
+                pow_[g][j][d][k] = pv;
+                pv *= v;
             }
-            if (d == 0) {
-                uint32_t w = __float_as_uint(P.w);
-                float a = (float)pk_axon(w);
-                bool inh = pk_type(w) != 0;
+            if (t % 6 == 0) {
+                const uint32_t w = __float_as_uint(pt.w);
+                const float a = (float)pk_axon(w);
+                const bool inh = pk_type(w) != 0;
                 wgt[j][0] = (float)pk_de(w);
                 wgt[j][1] = (float)pk_di(w);
                 wgt[j][2] = inh ? 0.f : a;
@@ -373,33 +378,29 @@ k_p2m(int64_t first_node, int p, float inv_sigma, const float4* __restrict__ pts
         }
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < kMaxAcc; ++r) {
-            int idx = threadIdx.x + r * kP2MThreads;
-            if (idx >= 4 * p3) continue;
-            int which = idx / p3, a = idx - which * p3;
-            int a0 = a / (p * p), a1 = (a / p) % p, a2 = a % p;
+        for (int r = 0; r < NACC; ++r) {
+            const int idx = threadIdx.x + r * kP2MThreads;
+            if (idx >= 4 * P3) continue;
+            const int which = idx / P3, a = idx % P3;
+            const int a0 = a / P2, a1 = (a / P) % P, a2 = a % P;
+            const float(*pw)[3][P] = pow_[which >> 1];
             float s = acc[r];
-            if (which < 2) {
-                for (int j = 0; j < m; ++j)
-                    s = fmaf(wgt[j][which] * ypow[j][0][a0], ypow[j][1][a1] * ypow[j][2][a2], s);
-            } else {
-                for (int j = 0; j < m; ++j)
-                    s = fmaf(wgt[j][which] * xpow[j][0][a0], xpow[j][1][a1] * xpow[j][2][a2], s);
-            }
+            for (int j = 0; j < m; ++j)
+                s = fmaf(wgt[j][which] * pw[j][0][a0], pw[j][1][a1] * pw[j][2][a2], s);
             acc[r] = s;
         }
     }
     const int64_t e = (int64_t)blockIdx.x;
 #pragma unroll
-    for (int r = 0; r < kMaxAcc; ++r) {
-        int idx = threadIdx.x + r * kP2MThreads;
-        if (idx >= 4 * p3) continue;
-        int which = idx / p3, a = idx - which * p3;
-        int a0 = a / (p * p), a1 = (a / p) % p, a2 = a % p;
+    for (int r = 0; r < NACC; ++r) {
+        const int idx = threadIdx.x + r * kP2MThreads;
+        if (idx >= 4 * P3) continue;
+        const int which = idx / P3, a = idx % P3;
         if (which < 2)
-            A[(e * 2 + which) * p3 + a] = acc[r] * c_inv_fact[a0] * c_inv_fact[a1] * c_inv_fact[a2];
+            A[(e * 2 + which) * P3 + a] = acc[r] * c_inv_fact[a / P2] *
+                                          c_inv_fact[(a / P) % P] * c_inv_fact[a % P];
         else
-            M[(e * 2 + which - 2) * p3 + a] = acc[r];
+            M[(e * 2 + which - 2) * P3 + a] = acc[r];
     }
 }
 
@@ -989,9 +990,18 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
     }
     if (c.exp_nodes > 0) {
         MSP_CUDA(cudaMemsetAsync(eB, 0, ecount * sizeof(float), s));
-        k_p2m<<<(unsigned)c.exp_nodes, kP2MThreads, 0, s>>>(
-            c.exp_first, p, inv_sigma, c.pts.get<float4>(), c.nd_first.get<int32_t>(),
-            c.nd_count.get<int32_t>(), eca, ecd, eA, eM);
+#define MSP_P2M_CASE(PP)                                                                    \
+    case PP:                                                                                \
+        k_p2m<PP><<<(unsigned)c.exp_nodes, kP2MThreads, 0, s>>>(                            \
+            c.exp_first, inv_sigma, c.pts.get<float4>(), c.nd_first.get<int32_t>(),         \
+            c.nd_count.get<int32_t>(), eca, ecd, eA, eM);                                   \
+        break;
+        switch (p) {
+            MSP_P2M_CASE(1) MSP_P2M_CASE(2) MSP_P2M_CASE(3) MSP_P2M_CASE(4)
+            MSP_P2M_CASE(5) MSP_P2M_CASE(6) MSP_P2M_CASE(7) MSP_P2M_CASE(8)
+            default: throw Error(MSP_ERR_INVALID_ARG, "expansion order out of range");
+        }
+#undef MSP_P2M_CASE
         MSP_LAUNCH("p2m");
     }
     // a7: translations, accumulating B(X) and W(X,Y); with geometric centres
