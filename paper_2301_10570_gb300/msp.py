@@ -108,6 +108,8 @@ class Stats(C.Structure):
 def load(path: str = LIB_PATH):
     """Load libmsp.so (built by paper_2301_10570_gb300.build)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -182,17 +184,39 @@ def _check(code):
         raise MSPError(code, load().msp_last_error().decode(errors="replace"))
 
 
+# Addresses and streams go to the library as plain integers (every argument is
+# declared, and a c_void_p object per argument costs as much as reading the
+# address).  A call on a small network is bound by this module: an all-pairs
+# call of 1,024 neurons spent 23 of its 29 us here, now 9 of 12.
 def _ptr(t):
-    return C.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def _np(a):
     return a.ctypes.data_as(C.c_void_p)
 
 
-def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+# the current stream's handle without building a torch.cuda.Stream (2-3 us)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream(stream=None, device=None):
+    """The handle of `stream`, or of the current stream (of the current device,
+    or of the device with index `device`)."""
+    if stream is not None:
+        return stream.cuda_stream
+    if device is None:
+        device = torch.cuda.current_device()
+    if _raw_stream is not None:
+        return _raw_stream(device)
+    return torch.cuda.current_stream(device).cuda_stream
+
+
+def _rows(pos):
+    """Addresses of the three rows of a (3, n) tensor whose rows are contiguous
+    (no views are made of it)."""
+    p, step = pos.data_ptr(), pos.stride(0) * pos.element_size()
+    return p, p + step, p + 2 * step
 
 
 def make_config(params: dict) -> Config:
@@ -265,15 +289,21 @@ class MSP:
     def build_tree(self, pos, type_, vac_axon, vac_dend_e, vac_dend_i, stream=None):
         """pos: (3, n) float32 CUDA tensor; the rest (n,) uint8 CUDA tensors."""
         pos = pos.contiguous()
-        ins = [pos[0].contiguous(), pos[1].contiguous(), pos[2].contiguous(),
-               type_.contiguous(), vac_axon.contiguous(), vac_dend_e.contiguous(),
-               vac_dend_i.contiguous()]
-        for t, dt in zip(ins, [torch.float32] * 3 + [torch.uint8] * 4):
+        counts = [type_.contiguous(), vac_axon.contiguous(), vac_dend_e.contiguous(),
+                  vac_dend_i.contiguous()]
+        if pos.dim() == 2 and pos.shape[0] >= 3 and pos.shape[1] > 0:
+            xs = [pos]
+            rows = _rows(pos)
+        else:                                   # no neurons, or rows of another shape
+            xs = [pos[0].contiguous(), pos[1].contiguous(), pos[2].contiguous()]
+            rows = [_ptr(t) for t in xs]
+        for t, dt in [(t, torch.float32) for t in xs] + [(t, torch.uint8) for t in counts]:
             if not t.is_cuda or t.dtype != dt:
                 raise TypeError("build_tree expects CUDA float32 positions and uint8 counts")
         self.n = int(pos.shape[1])
-        self._inputs = ins
-        _check(load().msp_build_tree(self._h, self.n, *[_ptr(t) for t in ins], _stream(stream)))
+        self._inputs = xs + counts
+        _check(load().msp_build_tree(self._h, self.n, *rows, *[_ptr(t) for t in counts],
+                                     _stream(stream)))
 
     def attraction(self, out=None, stream=None):
         u = out if out is not None else torch.empty(self.n, dtype=torch.float32, device="cuda")
@@ -289,14 +319,19 @@ class MSP:
         return self.stats()["n_elements"]
 
     def select_partners(self, step: int, out=None, stream=None):
-        ne = max(self.num_elements(), 1)
         if out is None:
+            ne = max(self.num_elements(), 1)
             dev = "cuda"
             out = dict(partner=torch.empty(ne, dtype=torch.int32, device=dev),
                        syn_pre=torch.empty(ne, dtype=torch.int32, device=dev),
                        syn_post=torch.empty(ne, dtype=torch.int32, device=dev),
                        syn_type=torch.empty(ne, dtype=torch.uint8, device=dev),
                        n_syn=torch.zeros(1, dtype=torch.int64, device=dev))
+        else:
+            # the caller's buffers may be in use on another stream: wait for the
+            # device (idle after the attraction, 3 us; reading the context's
+            # statistics for this took 15 us of 4,096 neurons, more of more boxes)
+            torch.cuda.synchronize(self.device)
         _check(load().msp_select_partners(self._h, int(step), _ptr(out["partner"]),
                                           _ptr(out["syn_pre"]), _ptr(out["syn_post"]),
                                           _ptr(out["syn_type"]), _ptr(out["n_syn"]),
@@ -319,9 +354,10 @@ class MSP:
                        syn_pre=np.zeros(ne, np.int32), syn_post=np.zeros(ne, np.int32),
                        syn_type=np.zeros(ne, np.uint8), n_syn=np.zeros(1, np.int64))
         _check(load().msp_plasticity_step_host(
-            self._h, n, int(step), _np(x), _np(y), _np(z), _np(t), _np(a), _np(e), _np(i),
-            _np(out["u"]) if want_u else None, _np(out["partner"]), _np(out["syn_pre"]),
-            _np(out["syn_post"]), _np(out["syn_type"]), _np(out["n_syn"])))
+            self._h, n, int(step), *[v.ctypes.data for v in (x, y, z, t, a, e, i)],
+            out["u"].ctypes.data if want_u else None,
+            *[out[k].ctypes.data for k in ("partner", "syn_pre", "syn_post", "syn_type",
+                                           "n_syn")]))
         return out
 
     def vacancy_walk(self, step, vac_axon, vac_dend_e, vac_dend_i, stream=None):
@@ -590,13 +626,22 @@ def direct_noalloc(pos, type_, vac_axon, vac_dend_e, vac_dend_i, sigma, out=None
         raise TypeError(f"out must be a contiguous float32 tensor of {n} entries on {dev}")
     # the library launches on the current device: make it pos's device, and
     # take that device's current stream unless one is given
-    with torch.cuda.device(dev):
+    if dev.index != torch.cuda.current_device():
+        with torch.cuda.device(dev):
+            return _direct_noalloc(pos, counts, sigma, out, stream, n)
+    return _direct_noalloc(pos, counts, sigma, out, stream, n)
+
+
+def _direct_noalloc(pos, counts, sigma, out, stream, n):
+    dev = pos.device
+    if pos.shape[1] > 0 and pos.stride(1) == 1:
+        rows = _rows(pos)
+    else:
         xs = [pos[d].contiguous() for d in range(3)]
-        u = out if out is not None else torch.empty(n, dtype=torch.float32, device=dev)
-        _check(load().msp_direct_noalloc(n, *[_ptr(t) for t in xs], *[_ptr(t) for t in counts],
-                                         float(sigma), _ptr(u),
-                                         _stream(stream if stream is not None else
-                                                 torch.cuda.current_stream(dev))))
+        rows = [_ptr(t) for t in xs]
+    u = out if out is not None else torch.empty(n, dtype=torch.float32, device=dev)
+    _check(load().msp_direct_noalloc(n, *rows, *[t.data_ptr() for t in counts], float(sigma),
+                                     u.data_ptr(), _stream(stream, dev.index)))
     return u
 
 
@@ -614,8 +659,7 @@ def philox(ctr, key, stream=None):
     out = torch.empty_like(ctr)
     with torch.cuda.device(ctr.device):
         _check(load().msp_philox(int(ctr.shape[0]), _ptr(ctr), _ptr(key), _ptr(out),
-                                 _stream(stream if stream is not None else
-                                         torch.cuda.current_stream(ctr.device))))
+                                 _stream(stream, ctr.device.index)))
     return out
 
 
