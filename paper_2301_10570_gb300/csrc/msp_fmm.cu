@@ -92,12 +92,6 @@ __device__ inline uint8_t classify(const NodeView& nv, const Geo& geo, int32_t X
     return kSplit;
 }
 
-// a replay that keeps the lists: only the near field's work counter restarts
-__global__ void k_reuse_init(DevCounts* dc) {
-    dc->overflow &= ~1ll;
-    dc->interactions = 0;
-}
-
 // The traversal's tables and lists: the pair table, and as the pairs are
 // classified, in pair order, the split pairs (pair, first child, child count,
 // 0), the near-field pairs with their target leaf as the key of the sort that
@@ -728,12 +722,19 @@ __global__ void k_m2l_keys(const int32_t* __restrict__ list, const int64_t* __re
 
 // ---------------------------------------------------------------------------
 // a8: Taylor evaluation (Eq. 6) at every target from each of its boxes that
-// carries an expansion; initialises u_sorted.
+// carries an expansion; initialises u_sorted and (uo not null) the caller's u.
+// reuse not null: first launch of an attraction that keeps its lists; clears
+// the counters that the traversal would have cleared.
 // ---------------------------------------------------------------------------
 __global__ void k_l2p(int64_t n, int64_t exp_first, int p, float inv_sigma,
                       const float4* __restrict__ pts, const int32_t* __restrict__ leaf_of,
                       const int32_t* __restrict__ parent, const float4* __restrict__ ca,
-                      const float* __restrict__ B, float* __restrict__ u) {
+                      const float* __restrict__ B, const int32_t* __restrict__ perm,
+                      float* __restrict__ u, float* __restrict__ uo, DevCounts* reuse) {
+    if (reuse && blockIdx.x == 0 && threadIdx.x == 0) {
+        reuse->overflow &= ~1ll;
+        reuse->interactions = 0;
+    }
     const int p3 = p * p * p;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
          j += (int64_t)gridDim.x * blockDim.x) {
@@ -768,6 +769,7 @@ __global__ void k_l2p(int64_t n, int64_t exp_first, int p, float inv_sigma,
             }
         }
         u[j] = acc;
+        if (uo) uo[perm[j]] = acc;
     }
 }
 
@@ -820,13 +822,6 @@ __global__ void k_reduce_split(const int64_t* __restrict__ sb, const int4* __res
             pw[q] = make_float4(e.x, e.y, i.x, i.y);
         }
     }
-}
-
-__global__ void k_scatter_u(const float* __restrict__ us, const int32_t* __restrict__ perm,
-                            int64_t n, float* __restrict__ u) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
-         j += (int64_t)gridDim.x * blockDim.x)
-        u[perm[j]] = us[j];
 }
 
 }  // namespace
@@ -918,13 +913,10 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
     int4* split = c.split_q.ensure<int4>((size_t)cap);
     int32_t* pv0 = c.p2p_val0.ensure<int32_t>((size_t)cap);
     int32_t* seg_first = c.seg_first.ensure<int32_t>((size_t)c.n_nodes + 2);
-    if (reuse_lists) {
-        // the step graph's replays keep the traversal and the lists of the
-        // eager attraction of the same positions (guarded by the build's
-        // checksum and generation stamp)
-        k_reuse_init<<<1, 1, 0, s>>>(dc);
-        MSP_LAUNCH("reuse_init");
-    } else {
+    // the step graph's replays keep the traversal and the lists of the eager
+    // attraction of the same positions (guarded by the build's checksum and
+    // generation stamp); k_l2p restarts the near field's work counter
+    if (!reuse_lists) {
     // a5: breadth-first dual traversal from (root, root): the first depths in
     // one launch, then one per depth (status words cleared together; depth d
     // holds at most 64^d pairs), each writing its part of the lists
@@ -1060,10 +1052,11 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
     if (n > 0) {
         k_l2p<<<grid_for(n, B, (int64_t)c.sm_count * 16), B, 0, s>>>(
             n, c.exp_first, p, inv_sigma, c.pts.get<float4>(), c.leaf_of.get<int32_t>(),
-            c.nd_parent.get<int32_t>(), eca, eB, us);
+            c.nd_parent.get<int32_t>(), eca, eB, c.perm.get<int32_t>(), us, u_dev,
+            reuse_lists ? dc : nullptr);
         MSP_LAUNCH("l2p");
         MSP_CUDA(cudaEventRecordWithFlags(c.ev_nf0, s, ev_flags));
-        launch_near_field(c, seg_first, &dc->nseg, c.n_nodes, pv0, &dc->n_p2p, cap, us, work,
+        launch_near_field(c, seg_first, &dc->nseg, c.n_nodes, pv0, cap, us, u_dev, work,
                           reuse_lists, s);
         MSP_CUDA(cudaEventRecordWithFlags(c.ev_nf1, s, ev_flags));
     }
@@ -1072,11 +1065,6 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
     for (int dd = D - 1; dd >= 0; --dd) {
         k_reduce_split<<<Gt, B, 0, s>>>(&dc->split_start[dd], split, c.pr_w.get<float4>());
         MSP_LAUNCH("reduce_split");
-    }
-    if (u_dev && n > 0) {
-        k_scatter_u<<<grid_for(n, B, (int64_t)c.sm_count * 16), B, 0, s>>>(
-            us, c.perm.get<int32_t>(), n, u_dev);
-        MSP_LAUNCH("scatter_u");
     }
     // inside the whole-step graph the table does not grow: an overflow halts
     // the graph (checked on the device after the selection)

@@ -308,9 +308,10 @@ namespace msp {
 // primitives (msp_prims.cu)
 // ---------------------------------------------------------------------------
 // Step a9, the near field over the leaf pairs grouped by target leaf
-// (msp_nearfield.cu); accumulates into u_sorted and the pair table.
-// Segment and list counts live in device memory (*nseg_dev <= nseg_cap,
-// *nlist_dev <= nlist_cap); no host synchronisation.
+// (msp_nearfield.cu); adds to u_sorted (and u_out, in the caller's order, unless
+// null: it holds the same values) and writes the list's pairs of the pair table.
+// The segment count lives in device memory (*nseg_dev <= nseg_cap); no host
+// synchronisation.
 // expansions about the geometric centres (msp_m2l_gemm.cu)
 void geo_centres(msp_ctx& c, cudaStream_t s);
 bool m2l_gemm_fits(int p);
@@ -318,9 +319,9 @@ const int32_t* m2l_gemm(msp_ctx& c, const int32_t* far_q, const int64_t* nfar, i
                         const float* A, const float* M, float* B, float4* pw,
                         int64_t** first_fallback, cudaStream_t s);
 void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg_dev,
-                       int64_t nseg_cap, const int32_t* list_q, const int64_t* nlist_dev,
-                       int64_t nlist_cap, float* u_sorted, unsigned long long* work,
-                       bool keep_order, cudaStream_t s);
+                       int64_t nseg_cap, const int32_t* list_q, int64_t nlist_cap,
+                       float* u_sorted, float* u_out, unsigned long long* work, bool keep_order,
+                       cudaStream_t s);
 // Exclusive scan of in[0, *n_dev) (n_dev in device memory, at most n_cap)
 // into out; *total_dst = total (may be null).  No host synchronisation.
 // (msp_scan.cuh holds the kernel, for scans of values computed on the way.)

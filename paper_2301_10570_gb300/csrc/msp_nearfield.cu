@@ -68,12 +68,20 @@ struct NFArgs {
     const float2* lw;
     float sqk, ox, oy, oz, side;
     int frame_level;             // > 0: box centres in each network's own frame
-    float* u;
+    float* u;                    // in sorted order, and (uo not null) also in the caller's
+    float* uo;
+    const int32_t* perm;
     float2* w32;                 // per near-field pair (list order): W of E and I
     unsigned long long* work;
     const uint8_t* small;        // segments that k_near_small takes, or null: none
     float4* pw;                  // the pair table (k_near_small's results)
 };
+
+__device__ __forceinline__ void nf_add_u(const NFArgs& a, int32_t t, float v) {
+    const float u = a.u[t] + v;
+    a.u[t] = u;
+    if (a.uo) a.uo[a.perm[t]] = u;
+}
 
 // the targets of a lane (R of them, one channel), each coordinate broadcast
 // into both halves of a register pair; their scale factors and axon weights
@@ -442,7 +450,7 @@ __device__ __forceinline__ void nf_targets(const NFArgs& a, int nt, int nreal, i
                 float sacc = sm.red[0][slot];
 #pragma unroll
                 for (int k = 1; k < NW; ++k) sacc += sm.red[k][slot];
-                a.u[t] += sacc * sm.scale[slot];
+                nf_add_u(a, t, sacc * sm.scale[slot]);
             }
         }
     }
@@ -490,6 +498,10 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : (NW == 8 ? 3 : 1)) k_ne
         const bool fast = 0.75f * a.sqk * a.sqk * bs * bs <= kNFFastT2;
         unsigned long long evals = 0;
         int32_t pos = 0;
+        // the segment's attractions of a pair start at zero (ordered before
+        // the first addition by the barriers below)
+        for (int32_t i = i0 + (int32_t)threadIdx.x; i < i1; i += NW * 32)
+            a.w32[i] = make_float2(0.f, 0.f);
         for (;;) {
             // warp 0 collects up to kNFList - 3 targets with vacant axons from
             // pos on: first walk counts them per channel and finds where the
@@ -561,6 +573,15 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : (NW == 8 ? 3 : 1)) k_ne
                 nf_targets<3, NW>(a, ntl, nreal, i0, i1, tf, fast, cx, cy, cz, evals);
             if (pos >= tc) break;
         }
+        // ... and, complete here (a barrier closes every round), go to the pair
+        // table in double-FP32; read from L2, where the additions were made.
+        // (As passes of their own, the clearing and this cost two launches and
+        // 24 us of a 1,000,000 neurons' 2.4 ms step, 7 of 4,096 neurons' 163.)
+        const int32_t e1 = a.seg_first[sg + 1];
+        for (int32_t i = a.seg_first[sg] + (int32_t)threadIdx.x; i < e1; i += NW * 32) {
+            const float2 v = __ldcg(&a.w32[i]);
+            a.pw[a.list_q[i]] = make_float4(v.x, 0.f, v.y, 0.f);
+        }
         if (lane == 0 && evals) atomicAdd(a.work, evals);
     }
 }
@@ -575,8 +596,8 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : (NW == 8 ? 3 : 1)) k_ne
 // the general kernel does (source pair by source pair, group by group), so it
 // is the same bit for bit.  Bound by the latency of the points' reads.  65,536
 // neurons with translated pairs (4.2 M near-field pairs of 2.6 points a leaf):
-// 1020 us and 58 for the pair slots in the general kernel, 234 and 22 here
-// (the latter for the few segments that are not small).
+// 1020 us and 58 for the pair slots in the general kernel, 234 us here and 14 in
+// the general kernel for the few segments that are not small.
 constexpr int kNFSmall = 8;
 constexpr int kNFSmallWarps = 8;
 
@@ -685,7 +706,7 @@ __device__ __forceinline__ void nf_small_segment(const NFArgs& a, const int32_t*
         float total = 0.f;
         for (int k = 0; k < per; ++k)
             total += __shfl_sync(0xffffffffu, mine, k * g + j < 32 ? k * g + j : lane);
-        if (pl == 0 && t[r] >= 0) a.u[t[r]] += total * scale[r];
+        if (pl == 0 && t[r] >= 0) nf_add_u(a, t[r], total * scale[r]);
     }
 }
 
@@ -783,57 +804,12 @@ __global__ void k_seg_order_keys(const int32_t* __restrict__ seg_first,
     }
 }
 
-__global__ void k_zero_w(float2* __restrict__ w32, const int64_t* __restrict__ n_dev) {
-    const int64_t n = *n_dev;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        w32[i] = make_float2(0.f, 0.f);
-}
-
-// the single precision per-pair attractions of the segments that are not small
-// into the pair table
-__global__ void k_widen_big(const NFArgs a) {
-    const int64_t nseg = *a.nseg;
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t sg = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); sg < nseg;
-         sg += nw) {
-        if (a.small[sg]) continue;
-        for (int32_t i = a.seg_first[sg] + lane; i < a.seg_first[sg + 1]; i += 32) {
-            const float2 v = a.w32[i];
-            a.pw[a.list_q[i]] = make_float4(v.x, 0.f, v.y, 0.f);
-        }
-    }
-}
-__global__ void k_zero_big(const NFArgs a) {
-    const int64_t nseg = *a.nseg;
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t sg = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); sg < nseg;
-         sg += nw) {
-        if (a.small[sg]) continue;
-        for (int32_t i = a.seg_first[sg] + lane; i < a.seg_first[sg + 1]; i += 32)
-            a.w32[i] = make_float2(0.f, 0.f);
-    }
-}
-
-// the single precision per-pair attractions into the pair table (double-FP32)
-__global__ void k_widen_w(const int32_t* __restrict__ list_q, const float2* __restrict__ w32,
-                          const int64_t* __restrict__ n_dev, float4* __restrict__ pw) {
-    const int64_t n = *n_dev;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        float2 v = w32[i];
-        pw[list_q[i]] = make_float4(v.x, 0.f, v.y, 0.f);
-    }
-}
-
 }  // namespace
 
 void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg_dev,
-                       int64_t nseg_cap, const int32_t* list_q, const int64_t* nlist_dev,
-                       int64_t nlist_cap, float* u_sorted, unsigned long long* work,
-                       bool keep_order, cudaStream_t s) {
+                       int64_t nseg_cap, const int32_t* list_q, int64_t nlist_cap,
+                       float* u_sorted, float* u_out, unsigned long long* work, bool keep_order,
+                       cudaStream_t s) {
     if (nseg_cap <= 0 || nlist_cap <= 0) return;
     const msp_config& cfg = c.cfg;
     float2* w32 = c.nf_w32.ensure<float2>((size_t)nlist_cap);
@@ -881,18 +857,15 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
     a.side = cfg.side;
     a.frame_level = c.frame_level;
     a.u = u_sorted;
+    a.uo = u_out;
+    a.perm = c.perm.get<int32_t>();
     a.w32 = w32;
     a.work = work;
     a.small = small;
     a.pw = c.pr_w.get<float4>();
     if (small) {
-        k_zero_big<<<gl, 256, 0, s>>>(a);
-        MSP_LAUNCH("zero_big");
         k_near_small<<<gl, kNFSmallWarps * 32, 0, s>>>(a);
         MSP_LAUNCH("near_small");
-    } else {
-        k_zero_w<<<gl, 256, 0, s>>>(w32, nlist_dev);
-        MSP_LAUNCH("zero_w");
     }
     // one block per segment (blocks past the device count return at once), or
     // as many as are resident where few segments are left
@@ -917,11 +890,6 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
     else
         launch(k_near_field<16>, 16, sizeof(NFShared<16>));
     MSP_LAUNCH("near_field");
-    if (small)
-        k_widen_big<<<gl, 256, 0, s>>>(a);
-    else
-        k_widen_w<<<gl, 256, 0, s>>>(list_q, w32, nlist_dev, a.pw);
-    MSP_LAUNCH("widen_w");
 }
 
 }  // namespace msp
