@@ -39,24 +39,11 @@ void commit_synapses(msp_ctx& c, const int64_t* n_syn, int64_t capacity, const i
 
 namespace {
 
-// halt bits
-constexpr int64_t kHaltPairs = 1, kHaltItems = 2, kHaltLevels = 4, kHaltDescent = 8,
-                  kHaltElements = 16;
-
 __global__ void k_graph_init(DevCounts* dc, uint64_t step, int64_t halt) {
     dc->step = step;
     dc->halt = halt;
     dc->steps_run = 0;
     dc->interactions_run = 0;
-}
-
-// after the build: more elements than the selection's buffers hold leave the
-// step with no element (every element kernel is bounded by the count)
-__global__ void k_graph_guard(DevCounts* dc, int64_t elem_cap) {
-    if (dc->n_elem > elem_cap) {
-        dc->halt |= kHaltElements;
-        dc->n_elem = 0;
-    }
 }
 
 // after the selection, before the commit
@@ -97,8 +84,6 @@ void record_step(msp_ctx& c, const msp_ctx::GraphArgs& g, cudaStream_t s) {
     DevCounts* dc = dcounts(c);
     if (g.walk) vacancy_walk(c, g.n, 0, g.va, g.vde, g.vdi, s);
     build_tree(c, g.n, g.x, g.y, g.z, g.type, g.va, g.vde, g.vdi, s);
-    k_graph_guard<<<1, 1, 0, s>>>(dc, g.elem_cap);
-    MSP_LAUNCH("graph_guard");
     attraction(c, g.u, s);
     select_partners(c, 0, g.type, g.va, g.vde, g.vdi, g.partner, g.pre, g.post, g.styp, g.n_syn,
                     s);

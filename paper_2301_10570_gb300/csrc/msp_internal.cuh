@@ -135,7 +135,8 @@ struct DevCounts {
     int64_t steps_run;
     int64_t interactions_run;                // near-field interactions over the replays
     uint64_t pos_sum;                        // checksum of the positions of the last build
-    uint64_t tree_gen;                       // generation stamp of the last eager build
+    uint64_t tree_gen;                       // generation stamp of the last eager build (after
+                                             // pos_sum: the two are read together)
     int64_t m2l_n, m2l_nseg;                 // far pairs translated pair by pair, their targets
     int64_t n_split;                         // split pairs of the last traversal
     int64_t n_groups;                        // request groups (channel, dendrite): 2 n
@@ -147,6 +148,10 @@ struct DevCounts {
 // DevCounts::overflow bit set when a bounded wait of the single-pass scan
 // gave up (its result is then wrong; the host reports MSP_ERR_TIMEOUT)
 constexpr int64_t kScanTimeoutBit = 1ll << 40;
+
+// DevCounts::halt bits of a graph step
+constexpr int64_t kHaltPairs = 1, kHaltItems = 2, kHaltLevels = 4, kHaltDescent = 8,
+                  kHaltElements = 16;
 
 // the vacancy walk keeps every vacant count in [0, kMaxVacancy]
 constexpr int kMaxVacancy = 5;
@@ -200,7 +205,7 @@ struct msp_ctx {
     msp::DBuf frame_cap, frame_g2, frame_rc2;
     // sorted points
     msp::DBuf keys0, keys1, vals0, vals1;
-    msp::DBuf perm, inv, pts, wts, lw, elem_off, leaf_of;
+    msp::DBuf perm, pts, wts, lw, elem_off, leaf_of;
     // octree (SoA)
     msp::DBuf nd_level, nd_prefix, nd_first, nd_count, nd_parent, nd_child_first, nd_nchild;
     msp::DBuf nd_sums, nd_ca, nd_cd;

@@ -224,13 +224,23 @@ struct ScanSegments {
     }
 };
 
+// a tile counter and one status word per tile
+inline int64_t scan_status_words(int64_t n_cap) {
+    return std::max<int64_t>((n_cap + kScanTile - 1) / kScanTile, 1) + 1;
+}
+inline unsigned long long* scan_status(msp_ctx& c, int64_t n_cap) {
+    return c.sd_tmp.ensure<unsigned long long>((size_t)scan_status_words(n_cap));
+}
+
+// cleared: the scan's status words, if an earlier kernel has cleared them (no
+// other scan in between); otherwise they are cleared here
 template <class In, class Out, class Fin>
 inline void scan_launch(msp_ctx& c, In in, Out out, Fin fin, const int64_t* n_dev, int64_t n_cap,
-                        cudaStream_t s) {
-    const int64_t tiles_cap = std::max<int64_t>((n_cap + kScanTile - 1) / kScanTile, 1);
-    // a tile counter and one status word per tile, cleared first
-    unsigned long long* status = c.sd_tmp.ensure<unsigned long long>((size_t)tiles_cap + 1);
-    MSP_CUDA(cudaMemsetAsync(status, 0, ((size_t)tiles_cap + 1) * sizeof(unsigned long long), s));
+                        cudaStream_t s, unsigned long long* cleared = nullptr) {
+    const int64_t tiles_cap = scan_status_words(n_cap) - 1;
+    unsigned long long* status = cleared ? cleared : scan_status(c, n_cap);
+    if (!cleared)
+        MSP_CUDA(cudaMemsetAsync(status, 0, ((size_t)tiles_cap + 1) * sizeof(unsigned long long), s));
     const int G = (int)std::min<int64_t>(tiles_cap, (int64_t)c.sm_count * 4);
     k_scan_1p<<<G, kScanThreads, 0, s>>>(in, out, fin, n_dev, status, &dcounts(c)->overflow,
                                          kScanTimeoutBit, kSpinLimit);

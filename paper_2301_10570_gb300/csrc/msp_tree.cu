@@ -16,10 +16,19 @@ __device__ inline uint32_t quantise(float v, float o, float scale) {
     return (uint32_t)f;
 }
 
-__global__ void k_build_init(DevCounts* dc, int64_t n) {
-    dc->n = n;
-    dc->bad_pos = 0;
-    dc->pos_sum = 0;
+// start of a build; also clears the status words of its element scan and
+// (n_arrive > 0) the arrival counters of the aggregation
+__global__ void k_build_init(DevCounts* dc, int64_t n, unsigned long long* __restrict__ status,
+                             int64_t n_status, int32_t* __restrict__ arrive, int64_t n_arrive) {
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    if (i0 == 0) {
+        dc->n = n;
+        dc->bad_pos = 0;
+        dc->pos_sum = 0;
+    }
+    for (int64_t i = i0; i < n_status; i += step) status[i] = 0;
+    for (int64_t i = i0; i < n_arrive; i += step) arrive[i] = 0;
 }
 
 // order-independent checksum of the positions: the sum over i (modulo 2^64)
@@ -35,32 +44,57 @@ __device__ inline unsigned long long pos_mix(unsigned long long h) {
     return h;
 }
 
+__device__ inline unsigned long long pos_hash(int64_t i, float x, float y, float z) {
+    const unsigned long long xy = ((unsigned long long)__float_as_uint(x) << 32) |
+                                  __float_as_uint(y);
+    const unsigned long long h = pos_mix(xy ^ ((unsigned long long)i * 0x9E3779B97F4A7C15ull));
+    return pos_mix(h ^ ((unsigned long long)__float_as_uint(z) * 0xD6E8FEB86659FD93ull));
+}
+
+// adds the block's sum to *out (one atomic per block: one per warp, at
+// 1,000,000 neurons, took longer than reading the positions)
+__device__ inline void add_pos_sum(unsigned long long acc, unsigned long long* out) {
+    __shared__ unsigned long long s_sum;
+    if (threadIdx.x == 0) s_sum = 0;
+    __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&s_sum, acc);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(out, s_sum);
+}
+
 __global__ void k_pos_sum(const float* __restrict__ x, const float* __restrict__ y,
                           const float* __restrict__ z, int64_t n,
                           unsigned long long* __restrict__ out) {
     unsigned long long acc = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long xy = ((unsigned long long)__float_as_uint(x[i]) << 32) |
-                                      __float_as_uint(y[i]);
-        unsigned long long h = pos_mix(xy ^ ((unsigned long long)i * 0x9E3779B97F4A7C15ull));
-        h = pos_mix(h ^ ((unsigned long long)__float_as_uint(z[i]) * 0xD6E8FEB86659FD93ull));
-        acc += h;
+         i += (int64_t)gridDim.x * blockDim.x)
+        acc += pos_hash(i, x[i], y[i], z[i]);
+    add_pos_sum(acc, out);
+}
+
+// End of a graph step's build, in its last kernel (k_aggregate_tree).
+struct BuildEnd {
+    DevCounts* dc;
+    bool graph;              // otherwise nothing to do (the host looks)
+    // octree kept: the positions must be those of the build that made it
+    // (checksum ref) and the arrays that build's (stamp gen), or the step halts;
+    // octree built anew: no capture holds the stamp it leaves
+    bool keep;
+    uint64_t ref, gen;
+    // more elements than the selection's buffers hold leave the step with no
+    // element (every element kernel is bounded by the count)
+    int64_t elem_cap;
+    __device__ void operator()() const {
+        if (!graph) return;
+        if (!keep) dc->tree_gen = ~0ull;
+        else if (dc->pos_sum != ref || dc->tree_gen != gen) dc->bad_pos = 1;
+        if (dc->n_elem > elem_cap) {
+            dc->halt |= kHaltElements;
+            dc->n_elem = 0;
+        }
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0 && acc) atomicAdd(out, acc);
-}
-
-// the positions of a graph step must be those its octree was built from
-// a replay that reuses the octree: the positions must be those of the build
-// (checksum) and the octree arrays those of that build (generation stamp)
-__global__ void k_pos_check(DevCounts* dc, uint64_t ref, uint64_t gen) {
-    if (dc->pos_sum != ref || dc->tree_gen != gen) dc->bad_pos = 1;
-}
-
-// a graph replay that rebuilt the octree: no capture holds this stamp, so a
-// replay of another graph that reuses the octree halts instead
-__global__ void k_mark_graph_tree(DevCounts* dc) { dc->tree_gen = ~0ull; }
+};
 
 // keys; a position outside [origin, origin + side) or not finite is counted
 // (the build then fails: the tree's boxes must contain their points)
@@ -121,26 +155,54 @@ __global__ void k_morton_frames(const float* __restrict__ x, const float* __rest
         atomicAdd(reinterpret_cast<unsigned long long*>(bad), 1ull);
 }
 
+__device__ __forceinline__ uint32_t pack_counts(uint8_t type, uint8_t va, uint8_t vde, uint8_t vdi) {
+    return (uint32_t)(type ? 1u : 0u) | ((uint32_t)va << 8) | ((uint32_t)vde << 16) |
+           ((uint32_t)vdi << 24);
+}
+// the dendrite weights, and their log2 (-inf for none), added in the exponent
+__device__ __forceinline__ void put_weights(int64_t j, uint8_t vde, uint8_t vdi, float2* wts,
+                                            float2* lw) {
+    wts[j] = make_float2((float)vde, (float)vdi);
+    lw[j] = make_float2(vde ? log2f((float)vde) : -INFINITY, vdi ? log2f((float)vdi) : -INFINITY);
+}
+
 __global__ void k_gather(const int32_t* __restrict__ order, int64_t n, const float* __restrict__ x,
                          const float* __restrict__ y, const float* __restrict__ z,
                          const uint8_t* __restrict__ type, const uint8_t* __restrict__ va,
                          const uint8_t* __restrict__ vde, const uint8_t* __restrict__ vdi,
-                         int32_t* __restrict__ perm, int32_t* __restrict__ inv,
-                         float4* __restrict__ pts, float2* __restrict__ wts,
-                         float2* __restrict__ lw) {
+                         int32_t* __restrict__ perm, float4* __restrict__ pts,
+                         float2* __restrict__ wts, float2* __restrict__ lw) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
          j += (int64_t)gridDim.x * blockDim.x) {
-        int32_t i = order[j];
+        const int32_t i = order[j];
         perm[j] = i;
-        inv[i] = (int32_t)j;
-        uint32_t packed = (uint32_t)(type[i] ? 1u : 0u) | ((uint32_t)va[i] << 8) |
-                          ((uint32_t)vde[i] << 16) | ((uint32_t)vdi[i] << 24);
-        pts[j] = make_float4(x[i], y[i], z[i], __uint_as_float(packed));
-        wts[j] = make_float2((float)vde[i], (float)vdi[i]);
-        // log2 of the dendrite weights (-inf for none), added in the exponent
-        lw[j] = make_float2(vde[i] ? log2f((float)vde[i]) : -INFINITY,
-                            vdi[i] ? log2f((float)vdi[i]) : -INFINITY);
+        pts[j] = make_float4(x[i], y[i], z[i],
+                             __uint_as_float(pack_counts(type[i], va[i], vde[i], vdi[i])));
+        put_weights(j, vde[i], vdi[i], wts, lw);
     }
+}
+
+// A build that keeps the sorted order: the positions' checksum (read in the
+// caller's order, coalesced) and the counts gathered again; the sorted
+// positions are those of the build that made the order, or the checksum tells
+// and the octree is built anew.  Bound by the gather's 32-byte sectors.
+// 1,000,000 neurons: 33 us for a full gather and 18 for the checksum before, 21 now.
+__global__ void k_gather_counts(int64_t n, const float* __restrict__ x,
+                                const float* __restrict__ y, const float* __restrict__ z,
+                                const uint8_t* __restrict__ type, const uint8_t* __restrict__ va,
+                                const uint8_t* __restrict__ vde, const uint8_t* __restrict__ vdi,
+                                const int32_t* __restrict__ perm, float4* __restrict__ pts,
+                                float2* __restrict__ wts, float2* __restrict__ lw,
+                                unsigned long long* __restrict__ sum) {
+    unsigned long long acc = 0;
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
+         j += (int64_t)gridDim.x * blockDim.x) {
+        acc += pos_hash(j, x[j], y[j], z[j]);
+        const int32_t i = perm[j];
+        pts[j].w = __uint_as_float(pack_counts(type[i], va[i], vde[i], vdi[i]));
+        put_weights(j, vde[i], vdi[i], wts, lw);
+    }
+    add_pos_sum(acc, sum);
 }
 
 // The octree arrays and the split rule of a build.  Per-network leaf
@@ -483,7 +545,7 @@ __device__ __forceinline__ int arrive_acq_rel(int32_t* p) {
 }
 
 // nodes_end: the node count (device memory); one warp per leaf
-__global__ void k_aggregate_tree(const int64_t* __restrict__ nodes_end, int frame_level, float ox,
+__global__ void k_aggregate_tree(const BuildEnd end, const int64_t* __restrict__ nodes_end, int frame_level, float ox,
                                  float oy, float oz, float side, const float4* __restrict__ pts,
                                  const uint8_t* __restrict__ level,
                                  const uint64_t* __restrict__ prefix,
@@ -494,6 +556,7 @@ __global__ void k_aggregate_tree(const int64_t* __restrict__ nodes_end, int fram
                                  const uint8_t* __restrict__ nchild, int4* __restrict__ sums,
                                  float4* __restrict__ ca, float4* __restrict__ cd,
                                  int32_t* __restrict__ leaf_of, int32_t* __restrict__ arrive) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) end();
     const int64_t nn = *nodes_end;
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -530,7 +593,7 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
                 const uint8_t* type, const uint8_t* va, const uint8_t* vde, const uint8_t* vdi,
                 cudaStream_t s) {
     NvtxRange nv_("msp build_tree");
-    const bool was_built = c.tree_built;
+    const bool was_built = c.tree_built, prev_kept = c.tree_reused;
     const int64_t prev_n = c.n;
     if (!c.graph_mode) {
         c.tree_built = false;
@@ -540,15 +603,12 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
     c.n = n;
     const msp_config& cfg = c.cfg;
     DevCounts* dc = dcounts(c);
-    k_build_init<<<1, 1, 0, s>>>(dc, n);
-    MSP_LAUNCH("build_init");
     size_t nn = (size_t)(n > 0 ? n : 1);
     uint64_t* k0 = c.keys0.ensure<uint64_t>(nn);
     uint64_t* k1 = c.keys1.ensure<uint64_t>(nn);
     int32_t* v0 = c.vals0.ensure<int32_t>(nn);
     int32_t* v1 = c.vals1.ensure<int32_t>(nn);
     int32_t* perm = c.perm.ensure<int32_t>(nn);
-    int32_t* inv = c.inv.ensure<int32_t>(nn);
     float4* pts = c.pts.ensure<float4>(nn);
     float2* wts = c.wts.ensure<float2>(nn);
     float2* lw = c.lw.ensure<float2>(nn);
@@ -563,61 +623,70 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
     if (framed && n != c.frame_off_host.back())
         throw Error(MSP_ERR_INVALID_ARG, "the frames (msp_set_frames) hold a different number "
                                          "of neurons");
-    if (n > 0) {
+    unsigned long long* scan_st = scan_status(c, n);
+    const int64_t n_scan_st = scan_status_words(n);
+
+    // An eager build on the positions of the last build keeps its sorted order
+    // and octree, which depend on the positions only: their checksum tells.
+    // After a build that kept them the next one is expected to as well and goes
+    // ahead, its checksum read with its counts (a step of 4,096 neurons spends
+    // 20 us on a second synchronisation); otherwise the checksum is read first.
+    // Inside the whole-step graph the positions are those of the last eager
+    // build, or the graph halts.  A full-build replay may have built another
+    // octree since: the arrays' generation stamp tells.
+    auto kept = [&] {
+        return c.hcount->pos_sum == c.pos_sum_ref && c.hcount->tree_gen == c.tree_gen;
+    };
+    const bool may_keep = !c.graph_mode && was_built && n == prev_n && n > 0;
+    const bool graph_keep = c.graph_mode && c.tree_built && !c.graph_full_build;
+    const bool expect = may_keep && prev_kept;
+    const int64_t n_arrive = may_keep ? (int64_t)(c.nd_arrive.bytes / sizeof(int32_t)) : 0;
+    k_build_init<<<grid_for(std::max(n_scan_st, n_arrive), B, (int64_t)c.sm_count * 2), B, 0, s>>>(
+        dc, n, scan_st, n_scan_st, c.nd_arrive.get<int32_t>(), n_arrive);
+    MSP_LAUNCH("build_init");
+    bool keep = graph_keep || expect;
+    const BuildEnd end{dc, c.graph_mode, graph_keep, c.pos_sum_ref, c.tree_gen, c.graph_elem_cap};
+    if (!keep && n > 0 && !c.graph_mode) {
         k_pos_sum<<<G, B, 0, s>>>(x, y, z, n, reinterpret_cast<unsigned long long*>(&dc->pos_sum));
         MSP_LAUNCH("pos_sum");
-    }
-
-    // An eager build on the positions of the last build (their checksum,
-    // read back: one more synchronisation) keeps its sorted order and octree,
-    // which depend on the positions only.
-    bool eager_reuse = false;
-    if (!c.graph_mode && was_built && n == prev_n && n > 0) {
-        unsigned long long ps = 0;
-        MSP_CUDA(cudaMemcpyAsync(&ps, &dc->pos_sum, sizeof(ps), cudaMemcpyDeviceToHost, s));
-        MSP_CUDA(cudaStreamSynchronize(s));
-        eager_reuse = ps == c.pos_sum_ref;
-    }
-    if (!eager_reuse && !c.graph_mode) c.lists_valid = false;
-
-    // Inside the whole-step graph the positions are those of the last eager
-    // build (checked: a different checksum halts the graph), so its sorted
-    // order and octree are reused; the counts are gathered again and the
-    // aggregates recomputed.  The same for an eager build on those positions.
-    if ((c.graph_mode && c.tree_built && !c.graph_full_build) || eager_reuse) {
-        if (c.graph_mode) {
-            k_pos_check<<<1, 1, 0, s>>>(dc, c.pos_sum_ref, c.tree_gen);
-            MSP_LAUNCH("pos_check");
-        } else {
-            // the octree arrays are those of generation tree_gen (a graph
-            // replay that rebuilt them for the same positions left its mark)
-            dev_set(reinterpret_cast<int64_t*>(&dc->tree_gen), (int64_t)c.tree_gen, s);
+        if (may_keep) {
+            MSP_CUDA(cudaMemcpyAsync(&c.hcount->pos_sum, &dc->pos_sum, 2 * sizeof(uint64_t),
+                                     cudaMemcpyDeviceToHost, s));   // and tree_gen
+            MSP_CUDA(cudaStreamSynchronize(s));
+            keep = kept();
+            if (keep) MSP_CUDA(cudaMemsetAsync(&dc->pos_sum, 0, sizeof(uint64_t), s));
         }
+    }
+
+    // the octree kept: the counts are gathered again and the aggregates recomputed
+    if (keep) {
         if (n > 0) {
-            k_gather<<<G, B, 0, s>>>(v0, n, x, y, z, type, va, vde, vdi, perm, inv, pts, wts, lw);
-            MSP_LAUNCH("gather");
+            k_gather_counts<<<G, B, 0, s>>>(n, x, y, z, type, va, vde, vdi, perm, pts, wts, lw,
+                                            reinterpret_cast<unsigned long long*>(&dc->pos_sum));
+            MSP_LAUNCH("gather_counts");
             scan_launch(c, ScanU8{va}, ScanStore{eoff}, ScanTotalAfter{&dc->n_elem, eoff, &dc->n},
-                        &dc->n, n, s);
+                        &dc->n, n, s, scan_st);
         } else {
             dev_set(&dc->n_elem, 0, s);
         }
-        const int Gt = (int)std::max<int64_t>(1, (int64_t)c.sm_count * 8);
-        if (!c.graph_mode) MSP_CUDA(cudaMemsetAsync(c.nd_arrive.p, 0, c.nd_arrive.bytes, s));
         k_aggregate_tree<<<agg_grid(c.n_nodes, c.sm_count), 128, 0, s>>>(
-            &dc->level_start[c.tree_levels + 1], c.frame_level, o3[0], o3[1], o3[2], cfg.side, pts,
-            c.nd_level.get<uint8_t>(), c.nd_prefix.get<uint64_t>(), c.nd_first.get<int32_t>(),
+            end, &dc->level_start[c.tree_levels + 1], c.frame_level, o3[0], o3[1], o3[2], cfg.side,
+            pts, c.nd_level.get<uint8_t>(), c.nd_prefix.get<uint64_t>(), c.nd_first.get<int32_t>(),
             c.nd_count.get<int32_t>(), c.nd_parent.get<int32_t>(), c.nd_child_first.get<int32_t>(),
             c.nd_nchild.get<uint8_t>(), c.nd_sums.get<int4>(), c.nd_ca.get<float4>(),
             c.nd_cd.get<float4>(), leaf_of, c.nd_arrive.get<int32_t>());
         MSP_LAUNCH("aggregate");
-        if (eager_reuse) {
-            pull_counts(c, s);          // the one synchronisation of the build
+        if (c.graph_mode) return;
+        pull_counts(c, s);              // the one synchronisation of the build
+        if (kept()) {
             c.n_elem = c.hcount->n_elem;
             c.tree_built = true;
             c.tree_reused = true;
+            return;
         }
-        return;
+        // the positions changed after all (dc->pos_sum is their checksum)
     }
+    if (!c.graph_mode) c.lists_valid = false;
 
     // a1 + a2: keys, stable sort, gather into Morton order
     if (n > 0) {
@@ -636,11 +705,11 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
             MSP_LAUNCH("morton");
         }
         radix_sort_dev(c, k0, v0, k1, v1, nullptr, n, 3 * kMortonBits, s);
-        k_gather<<<G, B, 0, s>>>(v0, n, x, y, z, type, va, vde, vdi, perm, inv, pts, wts, lw);
+        k_gather<<<G, B, 0, s>>>(v0, n, x, y, z, type, va, vde, vdi, perm, pts, wts, lw);
         MSP_LAUNCH("gather");
         // element offsets: exclusive prefix of the vacant axonal counts
         scan_launch(c, ScanU8{va}, ScanStore{eoff}, ScanTotalAfter{&dc->n_elem, eoff, &dc->n},
-                    &dc->n, n, s);
+                    &dc->n, n, s, keep ? nullptr : scan_st);
     } else {
         dev_set(&dc->n_elem, 0, s);
     }
@@ -734,18 +803,14 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
         }
         // a4: aggregates, leaves up to the root in one launch
         k_aggregate_tree<<<agg_grid(cap, c.sm_count), 128, 0, s>>>(
-            &dc->level_start[L + 1], c.frame_level, o3[0], o3[1], o3[2], cfg.side, pts,
+            end, &dc->level_start[L + 1], c.frame_level, o3[0], o3[1], o3[2], cfg.side, pts,
             c.nd_level.get<uint8_t>(), c.nd_prefix.get<uint64_t>(), c.nd_first.get<int32_t>(),
             c.nd_count.get<int32_t>(), c.nd_parent.get<int32_t>(), c.nd_child_first.get<int32_t>(),
             c.nd_nchild.get<uint8_t>(), sums, ca, cd, leaf_of, arrive);
         MSP_LAUNCH("aggregate");
         // inside the whole-step graph the tree of the same positions has the
         // same levels; a deeper one sets more_levels, which halts the graph
-        if (c.graph_mode) {
-            k_mark_graph_tree<<<1, 1, 0, s>>>(dc);
-            MSP_LAUNCH("mark_graph_tree");
-            return;
-        }
+        if (c.graph_mode) return;
         pull_counts(c, s);          // the one synchronisation of the build
         if (c.hcount->bad_pos)
             throw Error(MSP_ERR_INVALID_ARG,
