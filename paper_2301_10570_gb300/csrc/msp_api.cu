@@ -8,7 +8,7 @@
 namespace msp {
 void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const float* z,
                 const uint8_t* type, const uint8_t* va, const uint8_t* vde, const uint8_t* vdi,
-                cudaStream_t s);
+                cudaStream_t s, const CountCopy* copy = nullptr);
 void attraction(msp_ctx& c, float* u_dev, cudaStream_t s);
 void direct(msp_ctx& c, float* u_dev, cudaStream_t s);
 void select_partners(msp_ctx& c, uint64_t step, const uint8_t* type_dev, const uint8_t* va_dev,
@@ -199,7 +199,7 @@ msp_status msp_destroy(msp_ctx* c) {
                          &c->ln_part, &c->ln_coef,
                          &c->expA, &c->expM, &c->expB, &c->u_sorted, &c->items0, &c->items1,
                          &c->leaf_items, &c->rq_key0, &c->rq_val0,
-                         &c->accepted, &c->acc_off, &c->rq_gcnt, &c->rq_goff, &c->cnt, &c->off, &c->rs_status, &c->lv_status, &c->tv_status,
+                         &c->accepted, &c->rq_owner, &c->rq_gcnt, &c->rq_goff, &c->cnt, &c->off, &c->rs_status, &c->lv_status, &c->tv_status,
                          &c->rs_hist, &c->h_u, &c->h_partner, &c->h_pre,
                          &c->h_post, &c->h_type, &c->h_nsyn, &c->hs_u, &c->hs_partner,
                          &c->hs_pre, &c->hs_post, &c->hs_type, &c->hs_nsyn, &c->c_type,
@@ -229,14 +229,9 @@ msp_status msp_build_tree(msp_ctx* c, int64_t n, const float* x, const float* y,
         uint8_t* ca = c->c_va.ensure<uint8_t>(nn);
         uint8_t* ce = c->c_vde.ensure<uint8_t>(nn);
         uint8_t* ci = c->c_vdi.ensure<uint8_t>(nn);
-        if (n > 0) {
-            MSP_CUDA(cudaMemcpyAsync(ct, type, n, cudaMemcpyDeviceToDevice, s));
-            MSP_CUDA(cudaMemcpyAsync(ca, va, n, cudaMemcpyDeviceToDevice, s));
-            MSP_CUDA(cudaMemcpyAsync(ce, vde, n, cudaMemcpyDeviceToDevice, s));
-            MSP_CUDA(cudaMemcpyAsync(ci, vdi, n, cudaMemcpyDeviceToDevice, s));
-        }
         c->in_type = ct; c->in_va = ca; c->in_vde = ce; c->in_vdi = ci;
-        msp::build_tree(*c, n, x, y, z, ct, ca, ce, ci, s);
+        const msp::CountCopy cp{{type, va, vde, vdi}, {ct, ca, ce, ci}, n};
+        msp::build_tree(*c, n, x, y, z, ct, ca, ce, ci, s, &cp);
     });
 }
 

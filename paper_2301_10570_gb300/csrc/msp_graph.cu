@@ -25,7 +25,7 @@ namespace msp {
 
 void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const float* z,
                 const uint8_t* type, const uint8_t* va, const uint8_t* vde, const uint8_t* vdi,
-                cudaStream_t s);
+                cudaStream_t s, const CountCopy* copy = nullptr);
 void attraction(msp_ctx& c, float* u_dev, cudaStream_t s);
 void select_partners(msp_ctx& c, uint64_t step, const uint8_t* type_dev, const uint8_t* va_dev,
                      const uint8_t* vde_dev, const uint8_t* vdi_dev, int32_t* partner,
@@ -46,24 +46,8 @@ __global__ void k_graph_init(DevCounts* dc, uint64_t step, int64_t halt) {
     dc->interactions_run = 0;
 }
 
-// after the selection, before the commit
-__global__ void k_graph_check(DevCounts* dc, int left_slot) {
-    int64_t bad = 0;
-    if (dc->overflow & 1) bad |= kHaltPairs;
-    if (dc->overflow & 38) bad |= kHaltItems;
-    if (dc->more_levels > 0 || (dc->overflow & 16) || dc->bad_pos) bad |= kHaltLevels;
-    if (dc->items[left_slot] != 0) bad |= kHaltDescent;
-    dc->halt |= bad;
-}
-
-__global__ void k_graph_step_end(DevCounts* dc, int64_t* history, int64_t len, uint64_t first) {
-    dc->interactions_run += dc->interactions;   // the near field runs in every replay
-    if (dc->halt) return;
-    const uint64_t k = dc->step - first;
-    if (history && k < (uint64_t)len) history[k] = dc->n_syn;
-    dc->step += 1;
-    dc->steps_run += 1;
-}
+// a step without neurons has no selection to end it
+__global__ void k_graph_end(DevCounts* dc, GraphEnd end) { end(dc); }
 
 // graph mode for the dry run and the capture, with the graph's options
 struct GraphModeScope {
@@ -72,6 +56,7 @@ struct GraphModeScope {
         c.graph_mode = true;
         c.graph_elem_cap = g.elem_cap;
         c.graph_full_build = g.full_build;
+        c.graph_end = GraphEnd{true, 0, g.history, g.history_len, g.first_step};
     }
     ~GraphModeScope() {
         c.graph_mode = false;
@@ -87,12 +72,12 @@ void record_step(msp_ctx& c, const msp_ctx::GraphArgs& g, cudaStream_t s) {
     attraction(c, g.u, s);
     select_partners(c, 0, g.type, g.va, g.vde, g.vdi, g.partner, g.pre, g.post, g.styp, g.n_syn,
                     s);
-    k_graph_check<<<1, 1, 0, s>>>(dc, c.cap_left_slot);
-    MSP_LAUNCH("graph_check");
+    if (g.elem_cap <= 0) {
+        k_graph_end<<<1, 1, 0, s>>>(dc, c.graph_end);
+        MSP_LAUNCH("graph_end");
+    }
     if (g.commit)
         commit_synapses(c, g.n_syn, g.capacity, g.pre, g.post, g.styp, g.va, g.vde, g.vdi, s);
-    k_graph_step_end<<<1, 1, 0, s>>>(dc, g.history, g.history_len, g.first_step);
-    MSP_LAUNCH("graph_step_end");
 }
 
 void release(msp_ctx::StepGraph& G) {
@@ -160,7 +145,6 @@ void capture(msp_ctx& c, msp_ctx::StepGraph& G, const msp_ctx::GraphArgs& args, 
             throw;
         }
         MSP_CUDA(cudaStreamEndCapture(cs, &graph));
-        G.left_slot = c.cap_left_slot;
         // kernels were only recorded, not run
         G.kernels = g_kernel_launches.load() - k0;
         g_kernel_launches -= G.kernels;

@@ -145,6 +145,14 @@ struct DevCounts {
     int64_t split_start[kMaxLevels + 3], p2p_start[kMaxLevels + 3], far_start[kMaxLevels + 3];
 };
 
+// The caller's type and vacant counts (src, on the device) that a build copies
+// to dst first: the selection reads what the build read.
+struct CountCopy {
+    const uint8_t* src[4] = {};
+    uint8_t* dst[4] = {};        // 16-byte aligned
+    int64_t n = 0;
+};
+
 // DevCounts::overflow bit set when a bounded wait of the single-pass scan
 // gave up (its result is then wrong; the host reports MSP_ERR_TIMEOUT)
 constexpr int64_t kScanTimeoutBit = 1ll << 40;
@@ -152,6 +160,32 @@ constexpr int64_t kScanTimeoutBit = 1ll << 40;
 // DevCounts::halt bits of a graph step
 constexpr int64_t kHaltPairs = 1, kHaltItems = 2, kHaltLevels = 4, kHaltDescent = 8,
                   kHaltElements = 16;
+
+// End of a graph step's selection, before its commit (which, like the walk, does
+// nothing once the step has halted): what exceeded a capacity, the step's entry
+// of the history, the next step's index.
+struct GraphEnd {
+    bool on = false;              // otherwise nothing to do (the host looks)
+    int left_slot = 0;            // the descent's items after its last step
+    int64_t* history = nullptr;
+    int64_t len = 0;
+    uint64_t first = 0;
+    __device__ __forceinline__ void operator()(DevCounts* dc) const {
+        if (!on) return;
+        int64_t bad = 0;
+        if (dc->overflow & 1) bad |= kHaltPairs;
+        if (dc->overflow & 38) bad |= kHaltItems;
+        if (dc->more_levels > 0 || (dc->overflow & 16) || dc->bad_pos) bad |= kHaltLevels;
+        if (dc->items[left_slot] != 0) bad |= kHaltDescent;
+        dc->halt |= bad;
+        dc->interactions_run += dc->interactions;   // the near field runs in every replay
+        if (dc->halt) return;
+        const uint64_t k = dc->step - first;
+        if (history && k < (uint64_t)len) history[k] = dc->n_syn;
+        dc->step += 1;
+        dc->steps_run += 1;
+    }
+};
 
 // the vacancy walk keeps every vacant count in [0, kMaxVacancy]
 constexpr int kMaxVacancy = 5;
@@ -236,7 +270,7 @@ struct msp_ctx {
     msp::DBuf expA, expM, expB;
     msp::DBuf u_sorted;
     // descent
-    msp::DBuf items0, items1, leaf_items, rq_key0, rq_val0, accepted, acc_off;
+    msp::DBuf items0, items1, leaf_items, rq_key0, rq_val0, accepted, rq_owner;
     msp::DBuf rq_gcnt, rq_goff;                          // requests per (channel, dendrite)
     // generic scratch
     msp::DBuf cnt, off, rs_hist, rs_status, sd_tmp, lv_status, tv_status;
@@ -262,7 +296,7 @@ struct msp_ctx {
     bool graph_mode = false;
     int64_t graph_elem_cap = 0;                // element capacity in graph mode
     bool graph_full_build = false;             // graph mode rebuilds the whole octree
-    int cap_left_slot = 0;                     // set by the selection while recording
+    msp::GraphEnd graph_end;                   // the end of a step in graph mode
     // every eager build stamps a new tree generation (also in device memory);
     // a replay that reuses the octree checks the stamp it was captured with
     uint64_t tree_gen = 0;
@@ -289,7 +323,6 @@ struct msp_ctx {
         cudaGraph_t tmpl = nullptr;
         int64_t kernels = 0;                      // kernel launches per replay
         cudaGraphNode_t nf0 = nullptr, nf1 = nullptr;   // event records around the near field
-        int left_slot = 0;                        // descent counter slot that must end empty
         long long epoch = -1;                     // allocation epoch at capture
         GraphArgs args;
     };

@@ -599,10 +599,16 @@ struct DelKeys {
     uint64_t seed, step;
     uint64_t* key;
     int32_t* val;
-    __device__ void operator()(int64_t i, int32_t at) const {
+    using Read = int64_t;                       // the group, or -1: not kept
+    __device__ Read read(int64_t i) const {
         int side;
         const int64_t e = in.edge(i, side), g = in.group(e, side);
-        if (in.excess[g] <= 0) return;
+        return in.excess[g] > 0 ? g : -1;
+    }
+    __device__ void operator()(int64_t i, int32_t at, Read g) const {
+        if (g < 0) return;
+        int side;
+        const int64_t e = in.edge(i, side);
         const uint32_t tag = (side ? kTagDelDend : kTagDelAxon) << 16;
         key[at] = ((uint64_t)g << 32) | nr_draw(seed, (uint32_t)e, tag, step);
         val[at] = (int32_t)e;

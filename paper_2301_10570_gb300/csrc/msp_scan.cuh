@@ -105,7 +105,8 @@ __device__ __forceinline__ void look_back(volatile unsigned long long* st, int64
             st[W * t + k] = 2ull << 62 | ((unsigned long long)(excl[k] + own[k]) & kValMask);
 }
 
-// Exclusive scan of in(i), i < *n_dev: out(i, sum before i) for every i, then
+// Exclusive scan of in(i), i < *n_dev: out(i, sum before i, out.read(i)) for every
+// i (nothing that read reads is written by the scan), then
 // fin(total) once (also for no element).  status[0]: the tile counter,
 // status[1 + tile]: the tiles' words, zero on entry.
 template <class In, class Out, class Fin>
@@ -128,10 +129,15 @@ k_scan_1p(In in, Out out, Fin fin, const int64_t* __restrict__ n_dev, unsigned l
         __syncthreads();
         if (t >= ntiles) break;
         const int64_t t0 = t * kScanTile;
-        // coalesced load into shared memory (one padding word per 32)
-        for (int j = threadIdx.x; j < kScanTile; j += kScanThreads) {
+        // coalesced load into shared memory (one padding word per 32), and what
+        // the output will read: all loads of a thread in flight at once
+        typename Out::Read rd[kScanItems];
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            const int j = threadIdx.x + k * kScanThreads;
             const int64_t i = t0 + j;
             s_v[j + (j >> 5)] = i < n ? in(i) : 0;
+            if (i < n) rd[k] = out.read(i);
         }
         __syncthreads();
         // each thread: kScanItems consecutive values
@@ -162,9 +168,11 @@ k_scan_1p(In in, Out out, Fin fin, const int64_t* __restrict__ n_dev, unsigned l
             run += v[k];
         }
         __syncthreads();
-        for (int j = threadIdx.x; j < kScanTile; j += kScanThreads) {
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            const int j = threadIdx.x + k * kScanThreads;
             const int64_t i = t0 + j;
-            if (i < n) out(i, s_v[j + (j >> 5)]);
+            if (i < n) out(i, s_v[j + (j >> 5)], rd[k]);
         }
         if (t == ntiles - 1 && threadIdx.x == 0) fin((int64_t)(excl + agg));
         __syncthreads();
@@ -187,14 +195,18 @@ struct ScanHeads {
 };
 struct ScanStore {
     int32_t* out;
-    __device__ void operator()(int64_t i, int32_t v) const { out[i] = v; }
+    struct Read {};
+    __device__ Read read(int64_t) const { return Read{}; }
+    __device__ void operator()(int64_t i, int32_t v, const Read&) const { out[i] = v; }
 };
 // first[k] = the first entry of segment k
 struct ScanFirsts {
     ScanHeads head;
     int32_t* first;
-    __device__ void operator()(int64_t i, int32_t v) const {
-        if (head(i)) first[v] = (int32_t)i;
+    using Read = int32_t;
+    __device__ Read read(int64_t i) const { return head(i); }
+    __device__ void operator()(int64_t i, int32_t v, Read h) const {
+        if (h) first[v] = (int32_t)i;
     }
 };
 struct ScanTotal {

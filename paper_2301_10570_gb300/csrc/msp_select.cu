@@ -127,19 +127,39 @@ struct DescCtr {
 
 // the items of both channels start at (root, root) where the root has
 // vacancies and attraction in that channel
-__global__ void k_init_items(const int4* __restrict__ sums, const float4* __restrict__ pw,
-                             Item* __restrict__ items, DevCounts* dc) {
-    const int4 rs = sums[0];
-    const float4 rw = pw[0];
-    int64_t k = 0;
-    if (rs.x > 0 && rw.x > kMinAttractionF) items[k++] = Item{0, 0, 0, 0};
-    if (rs.y > 0 && rw.z > kMinAttractionF) items[k++] = Item{0, 0, 0, 1};
-    dc->items[0] = k;
-    dc->items[1] = 0;
-    dc->n_leaf = 0;
-    dc->leaf_next = 0;
-    dc->draws = 0;
-    dc->overflow &= ~38ll;      // the selection's bits; bit 0 (pair table) stays
+// Start of a selection: the root's items and the counters by one thread; no
+// partner and nothing accepted yet, empty request groups (ng > 0: unless the last
+// selection left them empty), the status words of its scans.  One launch instead
+// of two and four clears (a clear of 2 us each and a gap: a selection of 4,096
+// neurons is bound by its launches).
+__global__ void k_select_init(const int4* __restrict__ sums, const float4* __restrict__ pw,
+                              Item* __restrict__ items, DevCounts* dc, int64_t n,
+                              int32_t* __restrict__ partner, uint8_t* __restrict__ acc,
+                              int32_t* __restrict__ gcnt, int64_t ng,
+                              unsigned long long* __restrict__ status, int64_t n_status) {
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    if (i0 == 0) {
+        const int4 rs = sums[0];
+        const float4 rw = pw[0];
+        int64_t k = 0;
+        if (rs.x > 0 && rw.x > kMinAttractionF) items[k++] = Item{0, 0, 0, 0};
+        if (rs.y > 0 && rw.z > kMinAttractionF) items[k++] = Item{0, 0, 0, 1};
+        dc->items[0] = k;
+        dc->items[1] = 0;
+        dc->n_leaf = 0;
+        dc->leaf_next = 0;
+        dc->draws = 0;
+        dc->n_groups = 2 * n;
+        dc->overflow &= ~38ll;      // the selection's bits; bit 0 (pair table) stays
+    }
+    const int64_t ne = dc->n_elem;
+    for (int64_t i = i0; i < ne; i += stride) {
+        partner[i] = -1;
+        acc[i] = 0;
+    }
+    for (int64_t i = i0; i < ng; i += stride) gcnt[i] = 0;
+    for (int64_t i = i0; i < n_status; i += stride) status[i] = 0;
 }
 
 // One level step of the descent.  A warp takes four items, 8 lanes each
@@ -363,8 +383,8 @@ k_leaf_draw_w(const Item* __restrict__ items, const int64_t* __restrict__ n_leaf
               const float2* __restrict__ wts, const int32_t* __restrict__ perm,
               const int32_t* __restrict__ eoff, float k2, float rc2_all, FrameRc2 fr,
               uint64_t seed, StepRef stp,
-              int32_t* __restrict__ partner, unsigned long long* __restrict__ draw_ctr,
-              const int64_t* __restrict__ n_elem) {
+              int32_t* __restrict__ partner, int32_t* __restrict__ gcnt, int64_t n,
+              unsigned long long* __restrict__ draw_ctr, const int64_t* __restrict__ n_elem) {
     __shared__ float4 s_pts[kLdWarps][kLdStage];
     __shared__ uint64_t s_pre[kLdWarps][kLdBlocks][32];   // inclusive prefix per block and lane
     __shared__ float4 s_T[kLdWarps][32];                  // a round's neurons
@@ -550,7 +570,9 @@ k_leaf_draw_w(const Item* __restrict__ items, const int64_t* __restrict__ n_leaf
                     }
                 }
                 if (hit < 0) hit = je - 1;     // the block's sum exceeds r
-                partner[eoff[to] + e] = perm[sf + hit];
+                const int32_t dend = perm[sf + hit];
+                partner[eoff[to] + e] = dend;
+                atomicAdd(&gcnt[(ch ? n : 0) + dend], 1);    // the request's group
                 ++draws;
             }
             __syncwarp();
@@ -561,29 +583,10 @@ k_leaf_draw_w(const Item* __restrict__ items, const int64_t* __restrict__ n_leaf
 }
 
 // a12: the requests grouped by (channel, dendrite), group g = channel * n +
-// dendrite, by a counting sort: counts per group, their exclusive scan, and a
-// scatter that takes each request's slot from its group's count (counting it
-// back down to zero).  The order inside a group is left to the atomics; the
-// ranking below does not depend on it.
-__global__ void k_req_count(int64_t n, const uint8_t* __restrict__ type,
-                            const uint8_t* __restrict__ va, const int32_t* __restrict__ eoff,
-                            const int32_t* __restrict__ partner, int32_t* __restrict__ gcnt,
-                            const int64_t* __restrict__ n_elem, int64_t* __restrict__ n_groups) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) *n_groups = 2 * n;
-    const int64_t ne = *n_elem;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int a = va[t];
-        const int32_t e0 = eoff[t];
-        if ((int64_t)e0 + a > ne) continue;
-        const int64_t base = type[t] ? n : 0;
-        for (int k = 0; k < a; ++k) {
-            const int32_t s = partner[e0 + k];
-            if (s >= 0) atomicAdd(&gcnt[base + s], 1);
-        }
-    }
-}
-
+// dendrite, by a counting sort: counts per group (added by the leaf draw), their
+// exclusive scan, and a scatter that takes each request's slot from its group's
+// count (counting it back down to zero).  The order inside a group is left to the
+// atomics; the ranking below does not depend on it.
 // key = priority << 32 | group, val = element; cap bounds the slots (the
 // buffers' length): a slot outside it (counts that do not match) is not
 // written and sets bit 5 of *overflow
@@ -592,6 +595,7 @@ __global__ void k_req_scatter(int64_t n, const uint8_t* __restrict__ type,
                               const int32_t* __restrict__ partner, const int32_t* __restrict__ goff,
                               int32_t* __restrict__ gcnt, uint64_t seed, StepRef stp,
                               uint64_t* __restrict__ key, int32_t* __restrict__ val,
+                              int32_t* __restrict__ owner,
                               const int64_t* __restrict__ n_elem, int64_t cap,
                               int64_t* __restrict__ overflow) {
     const uint64_t step = stp.get();
@@ -615,6 +619,7 @@ __global__ void k_req_scatter(int64_t n, const uint8_t* __restrict__ type,
             }
             key[r] = ((uint64_t)o[0] << 32) | (uint32_t)g;
             val[r] = e0 + k;
+            owner[e0 + k] = (int32_t)t;
         }
     }
 }
@@ -622,8 +627,9 @@ __global__ void k_req_scatter(int64_t n, const uint8_t* __restrict__ type,
 // A dendrite neuron accepts, per channel, its first `capacity` requests in
 // (priority, element) order: the rank of request i is the number of requests
 // of its group before it in that order.  Groups are small (the requests one
-// neuron receives), so each request counts over its group directly.  A group
-// whose count the scatter did not bring back to zero sets bit 5 of *overflow.
+// neuron receives), so each request counts over its group directly, unless the
+// group fits.  accepted: 0, or 1 + the channel.  A group whose count the scatter
+// did not bring back to zero sets bit 5 of *overflow.
 __global__ void k_accept(const uint64_t* __restrict__ key, const int32_t* __restrict__ val,
                          const int32_t* __restrict__ goff, const int32_t* __restrict__ gcnt,
                          const int64_t* __restrict__ nr_dev, int64_t n,
@@ -642,35 +648,51 @@ __global__ void k_accept(const uint64_t* __restrict__ key, const int32_t* __rest
         if (gcnt[g] != 0) atomicOr(reinterpret_cast<unsigned long long*>(overflow), 32ull);
         const int64_t j0 = goff[g], j1 = g + 1 < 2 * n ? (int64_t)goff[g + 1] : nr;
         int rank = 0;
-        for (int64_t j = j0; j < j1 && rank < cap; ++j) {
-            const uint32_t pj = (uint32_t)(key[j] >> 32);
-            rank += pj < pr || (pj == pr && val[j] < ei);
-        }
-        accepted[ei] = rank < cap ? 1 : 0;
+        if (j1 - j0 > cap)
+            for (int64_t j = j0; j < j1 && rank < cap; ++j) {
+                const uint32_t pj = (uint32_t)(key[j] >> 32);
+                rank += pj < pr || (pj == pr && val[j] < ei);
+            }
+        accepted[ei] = rank < cap ? (inh ? 2 : 1) : 0;
     }
 }
 
-__global__ void k_emit_synapses(int64_t n, const uint8_t* __restrict__ type,
-                                const uint8_t* __restrict__ va, const int32_t* __restrict__ eoff,
-                                const int32_t* __restrict__ partner,
-                                const uint8_t* __restrict__ acc, const int32_t* __restrict__ soff,
-                                int32_t* __restrict__ pre, int32_t* __restrict__ post,
-                                uint8_t* __restrict__ styp, const int64_t* __restrict__ n_elem) {
-    const int64_t ne = *n_elem;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        int a = va[t];
-        int32_t e0 = eoff[t];
-        if ((int64_t)e0 + a > ne) continue;
-        for (int k = 0; k < a; ++k) {
-            if (!acc[e0 + k]) continue;
-            int32_t r = soff[e0 + k];
-            pre[r] = (int32_t)t;
-            post[r] = partner[e0 + k];
-            styp[r] = type[t] ? 1 : 0;
-        }
+// The scan over the elements that writes the synapses, in element order: an
+// accepted element's prefix is its synapse's index.  (A scan and a pass over the
+// neurons took 22 us of 1,000,000 neurons, this takes 13; bound by the latency of
+// its reads, so k_scan_1p has all of a thread's in flight at once.)
+struct ScanAccepted {
+    const uint8_t* acc;
+    __device__ int32_t operator()(int64_t i) const { return acc[i] != 0; }
+};
+struct ScanEmit {
+    const uint8_t* acc;
+    const int32_t *owner, *partner;
+    int32_t *pre, *post;
+    uint8_t* type;
+    struct Read {
+        int32_t owner, partner;
+        uint8_t acc;
+    };
+    __device__ Read read(int64_t i) const { return Read{owner[i], partner[i], acc[i]}; }
+    __device__ void operator()(int64_t, int32_t v, const Read& e) const {
+        if (!e.acc) return;
+        pre[v] = e.owner;
+        post[v] = e.partner;
+        type[v] = e.acc - 1;
     }
-}
+};
+// the number of synapses, and in a graph step the step's end
+struct ScanSynapses {
+    DevCounts* dc;
+    int64_t* n_syn;
+    GraphEnd end;
+    __device__ void operator()(int64_t total) const {
+        dc->n_syn = total;
+        if (n_syn) *n_syn = total;
+        end(dc);
+    }
+};
 
 __global__ void k_walk(int64_t n, uint64_t seed, StepRef stp, uint8_t* __restrict__ va,
                        uint8_t* __restrict__ vde, uint8_t* __restrict__ vdi,
@@ -718,13 +740,6 @@ __global__ void k_commit(const int64_t* __restrict__ n_syn, int64_t capacity,
     }
 }
 
-__global__ void k_fill_i32(int32_t* __restrict__ p, const int64_t* __restrict__ n_dev, int32_t v) {
-    const int64_t n = *n_dev;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = v;
-}
-
 }  // namespace
 
 void select_partners(msp_ctx& c, uint64_t step, const uint8_t* type_dev, const uint8_t* va_dev,
@@ -752,9 +767,6 @@ void select_partners(msp_ctx& c, uint64_t step, const uint8_t* type_dev, const u
     DevCounts* dc = dcounts(c);
     const StepRef stp{step, c.graph_mode ? &dc->step : nullptr};
     const int ge = grid_for(ne, B, (int64_t)c.sm_count * 16);
-    k_fill_i32<<<ge, B, 0, s>>>(partner, &dc->n_elem, -1);
-    MSP_LAUNCH("fill_partner");
-
     Tree tr;
     tr.level = c.nd_level.get<uint8_t>();
     tr.first = c.nd_first.get<int32_t>();
@@ -779,8 +791,25 @@ void select_partners(msp_ctx& c, uint64_t step, const uint8_t* type_dev, const u
     const int64_t cap_items = 2 * c.n_nodes + 64, cap_leaf = 2 * c.n_nodes + 64;
     Item* ib[2] = {c.items0.ensure<Item>((size_t)cap_items), c.items1.ensure<Item>((size_t)cap_items)};
     Item* lit = c.leaf_items.ensure<Item>((size_t)cap_leaf);
-    k_init_items<<<1, 1, 0, s>>>(c.nd_sums.get<int4>(), c.pr_w.get<float4>(), ib[0], dc);
-    MSP_LAUNCH("init_items");
+    // the group counts: cleared before an eager selection and whenever the
+    // buffer is new; every complete scatter counts them back down to zero
+    const size_t ng = (size_t)std::max<int64_t>(2 * n, 1);
+    const size_t gcnt_bytes = c.rq_gcnt.bytes;
+    int32_t* gcnt = c.rq_gcnt.ensure<int32_t>(ng);
+    const bool clear_gcnt = !c.graph_mode || c.rq_gcnt.bytes != gcnt_bytes;
+    int32_t* goff = c.rq_goff.ensure<int32_t>(ng);
+    uint8_t* acc = c.accepted.ensure<uint8_t>((size_t)ne);
+    uint64_t* k0 = c.rq_key0.ensure<uint64_t>((size_t)ne);
+    int32_t* v0 = c.rq_val0.ensure<int32_t>((size_t)ne);
+    int32_t* owner = c.rq_owner.ensure<int32_t>((size_t)ne);
+    // status words of the two scans, one after the other
+    const int64_t n_st0 = scan_status_words((int64_t)ng), n_st1 = scan_status_words(ne);
+    unsigned long long* st0 = c.sd_tmp.ensure<unsigned long long>((size_t)(n_st0 + n_st1));
+    k_select_init<<<grid_for(std::max<int64_t>(ne, clear_gcnt ? (int64_t)ng : 0), B,
+                             (int64_t)c.sm_count * 8), B, 0, s>>>(
+        c.nd_sums.get<int4>(), c.pr_w.get<float4>(), ib[0], dc, n, partner, acc, gcnt,
+        clear_gcnt ? (int64_t)(c.rq_gcnt.bytes / sizeof(int32_t)) : 0, st0, n_st0 + n_st1);
+    MSP_LAUNCH("select_init");
     auto ull = [](int64_t* p) { return reinterpret_cast<unsigned long long*>(p); };
     const int n_steps = c.tree_depth + 1;
     const int gd = (int)std::max<int64_t>(1, (int64_t)c.sm_count * 16);
@@ -806,45 +835,29 @@ void select_partners(msp_ctx& c, uint64_t step, const uint8_t* type_dev, const u
         lit, &dc->n_leaf, cap_leaf, ull(&dc->leaf_next), c.nd_first.get<int32_t>(),
         c.nd_count.get<int32_t>(), c.pts.get<float4>(), c.wts.get<float2>(),
         c.perm.get<int32_t>(), c.elem_off.get<int32_t>(), k2, rc2, frc, cfg.seed, stp, partner,
-        ull(&dc->draws), &dc->n_elem);
+        gcnt, n, ull(&dc->draws), &dc->n_elem);
     MSP_LAUNCH("leaf_draw");
 
     // a12: requests grouped by (channel, dendrite), ranked by (priority, element)
     const int gn = grid_for(n, B, (int64_t)c.sm_count * 16);
-    const size_t ng = (size_t)std::max<int64_t>(2 * n, 1);
-    // the group counts: cleared before an eager selection and whenever the
-    // buffer is new; every complete scatter counts them back down to zero
-    const size_t gcnt_bytes = c.rq_gcnt.bytes;
-    int32_t* gcnt = c.rq_gcnt.ensure<int32_t>(ng);
-    if (!c.graph_mode || c.rq_gcnt.bytes != gcnt_bytes)
-        MSP_CUDA(cudaMemsetAsync(gcnt, 0, c.rq_gcnt.bytes, s));
-    int32_t* goff = c.rq_goff.ensure<int32_t>(ng);
-    uint8_t* acc = c.accepted.ensure<uint8_t>((size_t)ne);
-    MSP_CUDA(cudaMemsetAsync(acc, 0, (size_t)ne, s));
-    uint64_t* k0 = c.rq_key0.ensure<uint64_t>((size_t)ne);
-    int32_t* v0 = c.rq_val0.ensure<int32_t>((size_t)ne);
-    k_req_count<<<gn, B, 0, s>>>(n, type_dev, va_dev, c.elem_off.get<int32_t>(), partner, gcnt,
-                                 &dc->n_elem, &dc->n_groups);
-    MSP_LAUNCH("req_count");
-    scan_dev(c, gcnt, goff, &dc->n_groups, (int64_t)ng, &dc->n_req, s);
+    scan_launch(c, ScanI32{gcnt}, ScanStore{goff}, ScanTotal{&dc->n_req}, &dc->n_groups, (int64_t)ng,
+                s, st0);
     k_req_scatter<<<gn, B, 0, s>>>(n, type_dev, va_dev, c.elem_off.get<int32_t>(), partner, goff,
-                                   gcnt, cfg.seed, stp, k0, v0, &dc->n_elem, (int64_t)ne,
+                                   gcnt, cfg.seed, stp, k0, v0, owner, &dc->n_elem, (int64_t)ne,
                                    &dc->overflow);
     MSP_LAUNCH("req_scatter");
     k_accept<<<ge, B, 0, s>>>(k0, v0, goff, gcnt, &dc->n_req, n, vde_dev, vdi_dev, acc,
                               &dc->overflow);
     MSP_LAUNCH("accept");
-    int32_t* soff = c.acc_off.ensure<int32_t>((size_t)ne);
-    scan_launch(c, ScanU8{acc}, ScanStore{soff}, ScanTotal{&dc->n_syn}, &dc->n_elem, ne, s);
-    k_emit_synapses<<<gn, B, 0, s>>>(n, type_dev, va_dev, c.elem_off.get<int32_t>(), partner, acc,
-                                     soff, syn_pre, syn_post, syn_type, &dc->n_elem);
-    MSP_LAUNCH("emit_synapses");
-    MSP_CUDA(cudaMemcpyAsync(n_syn, &dc->n_syn, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    if (c.graph_mode) {
-        // checked on the device at the end of the graph's step
-        c.cap_left_slot = n_steps % 3;
-        return;
-    }
+    const bool aligned = reinterpret_cast<uintptr_t>(n_syn) % sizeof(int64_t) == 0;
+    GraphEnd end = c.graph_end;
+    end.on = c.graph_mode;
+    end.left_slot = n_steps % 3;
+    scan_launch(c, ScanAccepted{acc}, ScanEmit{acc, owner, partner, syn_pre, syn_post, syn_type},
+                ScanSynapses{dc, aligned ? n_syn : nullptr, end}, &dc->n_elem, ne, s, st0 + n_st0);
+    if (!aligned)
+        MSP_CUDA(cudaMemcpyAsync(n_syn, &dc->n_syn, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+    if (c.graph_mode) return;       // checked on the device (GraphEnd)
     pull_counts(c, s);              // the one synchronisation of the selection
     const DevCounts& hc = *c.hcount;
     if (hc.overflow & 6) throw Error(MSP_ERR_CHECK, "descent item capacity exceeded");

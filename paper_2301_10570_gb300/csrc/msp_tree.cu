@@ -16,10 +16,12 @@ __device__ inline uint32_t quantise(float v, float o, float scale) {
     return (uint32_t)f;
 }
 
-// start of a build; also clears the status words of its element scan and
-// (n_arrive > 0) the arrival counters of the aggregation
+// start of a build; also copies the caller's counts (cp.n > 0) and clears the
+// status words of the element scan and (n_arrive > 0) the arrival counters of the
+// aggregation
 __global__ void k_build_init(DevCounts* dc, int64_t n, unsigned long long* __restrict__ status,
-                             int64_t n_status, int32_t* __restrict__ arrive, int64_t n_arrive) {
+                             int64_t n_status, int32_t* __restrict__ arrive, int64_t n_arrive,
+                             CountCopy cp) {
     const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
     if (i0 == 0) {
@@ -29,6 +31,13 @@ __global__ void k_build_init(DevCounts* dc, int64_t n, unsigned long long* __res
     }
     for (int64_t i = i0; i < n_status; i += step) status[i] = 0;
     for (int64_t i = i0; i < n_arrive; i += step) arrive[i] = 0;
+    for (int k = 0; k < 4; ++k) {
+        // 16 bytes at a time where the caller's array allows it
+        const int64_t nv = reinterpret_cast<uintptr_t>(cp.src[k]) % 16 == 0 ? cp.n / 16 : 0;
+        for (int64_t i = i0; i < nv; i += step)
+            reinterpret_cast<uint4*>(cp.dst[k])[i] = reinterpret_cast<const uint4*>(cp.src[k])[i];
+        for (int64_t i = 16 * nv + i0; i < cp.n; i += step) cp.dst[k][i] = cp.src[k][i];
+    }
 }
 
 // order-independent checksum of the positions: the sum over i (modulo 2^64)
@@ -591,7 +600,7 @@ int agg_grid(int64_t nodes, int64_t sm_count) {
 
 void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const float* z,
                 const uint8_t* type, const uint8_t* va, const uint8_t* vde, const uint8_t* vdi,
-                cudaStream_t s) {
+                cudaStream_t s, const CountCopy* copy) {
     NvtxRange nv_("msp build_tree");
     const bool was_built = c.tree_built, prev_kept = c.tree_reused;
     const int64_t prev_n = c.n;
@@ -641,8 +650,9 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
     const bool graph_keep = c.graph_mode && c.tree_built && !c.graph_full_build;
     const bool expect = may_keep && prev_kept;
     const int64_t n_arrive = may_keep ? (int64_t)(c.nd_arrive.bytes / sizeof(int32_t)) : 0;
-    k_build_init<<<grid_for(std::max(n_scan_st, n_arrive), B, (int64_t)c.sm_count * 2), B, 0, s>>>(
-        dc, n, scan_st, n_scan_st, c.nd_arrive.get<int32_t>(), n_arrive);
+    k_build_init<<<grid_for(std::max({n_scan_st, n_arrive, copy ? n / 8 : 0}), B,
+                            (int64_t)c.sm_count * 2), B, 0, s>>>(
+        dc, n, scan_st, n_scan_st, c.nd_arrive.get<int32_t>(), n_arrive, copy ? *copy : CountCopy{});
     MSP_LAUNCH("build_init");
     bool keep = graph_keep || expect;
     const BuildEnd end{dc, c.graph_mode, graph_keep, c.pos_sum_ref, c.tree_gen, c.graph_elem_cap};
