@@ -95,39 +95,35 @@ __device__ float warp_far_w(const Tree& tr, const Exps& ex, int32_t X, int32_t Y
 // prefix sums, and the last positive candidate when rounding puts r at the
 // total.  The candidates, their prefix sums and r = U * total are double-FP32
 // values (hi + lo; the sign of a value is that of hi).
-__device__ inline int draw_index(const float2* w, int k, uint64_t bits53) {
+// (All loops have the constant bound of 8 candidates, so nothing is indexed at run
+// time and the candidates stay in registers.)
+__device__ __forceinline__ int draw_index(const float2 (&w)[8], int k, uint64_t bits53) {
     float2 pre[8];
     float2 tot = make_float2(0.f, 0.f);
-    for (int i = 0; i < k; ++i) {
-        tot = ff_add(tot, w[i].x > 0.f ? w[i] : make_float2(0.f, 0.f));
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        if (i < k) tot = ff_add(tot, w[i].x > 0.f ? w[i] : make_float2(0.f, 0.f));
         pre[i] = tot;
     }
     if (!(tot.x > kMinAttractionF)) return -1;
     const float2 r = ff_mul(ff_uniform(bits53), tot);
-    for (int i = 0; i < k; ++i)
-        if (ff_gt(pre[i], r)) return i;
-    for (int i = k - 1; i >= 0; --i)
-        if (w[i].x > 0.f) return i;
-    return -1;
+    int at = -1, last = -1;
+#pragma unroll
+    for (int i = 7; i >= 0; --i) {
+        if (i < k && ff_gt(pre[i], r)) at = i;
+        if (i < k && last < 0 && w[i].x > 0.f) last = i;
+    }
+    return at >= 0 ? at : last;
 }
 
 constexpr int kDescWarps = 4;
 
-// Descent counters of one level step.  The item counts rotate through three
-// slots: the step reads its input count from one, appends to the next (zeroed
-// by the step before) and zeroes the third for the step after.
-struct DescCtr {
-    const int64_t* n_in;
-    unsigned long long* n_out;
-    int64_t* n_reset;
-    unsigned long long* n_leaf;
-    unsigned long long* draws;
-    unsigned long long* overflow;     // bit 1: items, bit 2: leaf items
-};
+// The item counts of the steps rotate through DevCounts::items: step k reads its
+// input count from slot k % 3, appends to the next (zeroed by the step before) and
+// zeroes the third for the step after.
 
-// the items of both channels start at (root, root) where the root has
-// vacancies and attraction in that channel
-// Start of a selection: the root's items and the counters by one thread; no
+// Start of a selection: by one thread the counters and the items of both channels
+// at (root, root), where the root has vacancies and attraction in that channel; no
 // partner and nothing accepted yet, empty request groups (ng > 0: unless the last
 // selection left them empty), the status words of its scans.  One launch instead
 // of two and four clears (a clear of 2 us each and a gap: a selection of 4,096
@@ -162,100 +158,124 @@ __global__ void k_select_init(const int4* __restrict__ sums, const float4* __res
     for (int64_t i = i0; i < n_status; i += stride) status[i] = 0;
 }
 
-// One level step of the descent.  A warp takes four items, 8 lanes each
-// (lane i of a group for the item's axon child i): a leaf pair goes to the
-// per-element draw; a dendrite leaf is kept by every axon child with
-// vacancies; otherwise each axon child draws among the children of Y from
-// the pair table.  Items below a translated pair (candidates' attractions
-// evaluated as translations by the whole warp) follow, one at a time.
-__global__ void __launch_bounds__(kDescWarps * 32)
-k_descend(const Item* __restrict__ in, Tree tr, Exps ex,
-          const uint8_t* __restrict__ kind, const int32_t* __restrict__ pcf,
-          const float4* __restrict__ pw, uint64_t seed, StepRef stp, Item* __restrict__ out,
-          int64_t cap_out, Item* __restrict__ leaf_out, int64_t cap_leaf, DescCtr ct) {
-    const uint64_t step = stp.get();
-    __shared__ float sH[kDescWarps][48];
-    __shared__ float sb[kDescWarps][2][kMaxP * kMaxP * kMaxP];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// appends v of the lanes with `has` to list (one atomic per warp)
+__device__ __forceinline__ void append_items(bool has, const Item& v, unsigned long long* n,
+                                             Item* list, int64_t cap, unsigned long long* overflow,
+                                             unsigned long long bit) {
+    const unsigned m = __ballot_sync(0xffffffffu, has);
+    if (!m) return;
+    const int lane = threadIdx.x & 31;
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(n, (unsigned long long)__popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (!has) return;
+    const int64_t slot = (int64_t)base + __popc(m & ((1u << lane) - 1u));
+    if (slot < cap) list[slot] = v;
+    else atomicOr(overflow, bit);
+}
+
+struct DescArgs {
+    Tree tr;
+    Exps ex;
+    const uint8_t* kind;
+    const int32_t* pcf;
+    const float2* pw;            // pair q: E at 2 q, I at 2 q + 1 (hi, lo)
+    uint64_t seed;
+    StepRef stp;
+    Item* items[2];              // step k reads items[k & 1]
+    int64_t cap_out;
+    Item* leaf_out;
+    int64_t cap_leaf;
+    DevCounts* dc;
+};
+// floats of shared memory per warp: Hermite functions and two sets of coefficients
+__host__ __device__ constexpr int desc_warp_floats(int p) { return 48 + 2 * p * p * p; }
+
+// One level step of the descent by `nwarp` warps, this one `warp`.  A warp takes
+// four items, 8 lanes each (lane i of a group for the item's axon child i): a
+// leaf pair goes to the per-element draw; a dendrite leaf is kept by every axon
+// child with vacancies; otherwise each axon child draws among the children of Y
+// from the pair table.  Items below a translated pair (candidates' attractions
+// evaluated as translations by the whole warp) follow, one at a time.  Bound by
+// the chain of dependent reads (item, boxes, candidates) of the few items of a
+// step; everything that does not depend on the one before is read together.
+__device__ __forceinline__ void descend_step(const DescArgs& a, int step_k, int64_t warp,
+                                             int64_t nwarp, float* sm) {
+    const Tree& tr = a.tr;
+    const uint64_t step = a.stp.get();
+    const int lane = threadIdx.x & 31;
     const int sub = lane & 7;
+    DevCounts* dc = a.dc;
+    auto ull = [](int64_t* p) { return reinterpret_cast<unsigned long long*>(p); };
+    unsigned long long *n_out = ull(&dc->items[(step_k + 1) % 3]), *n_leaf = ull(&dc->n_leaf),
+                       *overflow = ull(&dc->overflow);
+    const Item* in = a.items[step_k & 1];
+    Item* out = a.items[(step_k + 1) & 1];
     // the count may exceed the buffer (items past it were not stored and the
     // overflow bit is set)
-    const int64_t n_in = min(*ct.n_in, cap_out);
-    if (blockIdx.x == 0 && threadIdx.x == 0) *ct.n_reset = 0;
-    const int64_t warp = (int64_t)blockIdx.x * kDescWarps + w;
-    const int64_t nwarp = (int64_t)gridDim.x * kDescWarps;
+    const int64_t n_in = min(__ldcg(&dc->items[step_k % 3]), a.cap_out);
+    if (warp == 0 && lane == 0) dc->items[(step_k + 2) % 3] = 0;
     for (int64_t k0 = 4 * warp; k0 < n_in; k0 += 4 * nwarp) {
         const int64_t k = k0 + (lane >> 3);
-        Item it = {0, 0, -1, 0};
-        bool far_item = false, drew = false;
+        Item it = {0, 0, -1, 0}, nx = {0, 0, -1, 0};
+        bool far_item = false, drew = false, leaf_pair = false, keep = false;
         if (k < n_in) {
-            it = in[k];
+            const int4 raw = __ldcg(reinterpret_cast<const int4*>(in) + k);
+            it = Item{raw.x, raw.y, raw.z, raw.w};
             const int32_t X = it.X, Y = it.Y;
             const int ch = it.ch;
-            const bool lx = tr.child_first[X] < 0, ly = tr.child_first[Y] < 0;
-            const bool split = it.q >= 0 && kind[it.q] == kSplit;
-            const int32_t cf = split ? pcf[it.q] : -1;
+            const int32_t cx = tr.child_first[X], cy = tr.child_first[Y];
+            const int nx_ch = tr.nchild[X], ny = tr.nchild[Y];
+            const uint32_t ly1 = (uint32_t)tr.level[Y] + 1u;
+            const int kd = it.q >= 0 ? a.kind[it.q] : (int)kPruned;
+            const int32_t cfq = it.q >= 0 ? a.pcf[it.q] : -1;
+            const bool lx = cx < 0, ly = cy < 0;
+            const bool split = kd == kSplit;
+            const int32_t cf = split ? cfq : -1;
             // a split pair whose children did not fit in the pair table (the
             // step is halted and redone with a larger table): nothing to read
             if (split && cf < 0) {
             } else if (lx && ly) {
                 // form_synapse: the leaf pair goes to the per-element draw
-                if (sub == 0) {
-                    const unsigned long long slot = atomicAdd(ct.n_leaf, 1ull);
-                    if ((int64_t)slot < cap_leaf) leaf_out[slot] = it;
-                    else atomicOr(ct.overflow, 4ull);
-                }
+                leaf_pair = sub == 0;
             } else if (!lx && ly) {
                 // the dendrite side is a leaf: every axon child with vacancies
                 // of this channel keeps it, without a draw
-                if (sub < tr.nchild[X]) {
-                    const int32_t xc = tr.child_first[X] + sub;
-                    const int4 sm = tr.sums[xc];
-                    bool keep = (ch ? sm.y : sm.x) > 0;
-                    if (keep && split)
-                        keep = (ch ? pw[cf + sub].z : pw[cf + sub].x) > kMinAttractionF;
-                    if (keep) {
-                        const unsigned long long slot = atomicAdd(ct.n_out, 1ull);
-                        const Item nx_it = {xc, Y, split ? cf + sub : -1, ch};
-                        if ((int64_t)slot < cap_out) out[slot] = nx_it;
-                        else atomicOr(ct.overflow, 2ull);
-                    }
+                if (sub < nx_ch) {
+                    const int4 sc = tr.sums[cx + sub];
+                    keep = (ch ? sc.y : sc.x) > 0;
+                    if (split) keep = a.pw[2 * (int64_t)(cf + sub) + ch].x > kMinAttractionF && keep;
+                    nx = Item{cx + sub, Y, split ? cf + sub : -1, ch};
                 }
             } else if (split) {
                 // a draw among the children of Y, for X itself (X a leaf) or
                 // for each axon child of X (both inner); the candidates'
                 // attractions are in the pair table
-                const int ny = tr.nchild[Y];
-                const int32_t cy = tr.child_first[Y];
-                const int nsrc = lx ? 1 : tr.nchild[X];
-                if (sub < nsrc) {
-                    const int32_t xc = lx ? X : tr.child_first[X] + sub;
-                    const int4 sm = tr.sums[xc];
-                    if (lx || (ch ? sm.y : sm.x) != 0) {
-                        float2 wk[8];
-                        for (int j = 0; j < ny; ++j) {
-                            const float4 v = pw[cf + (int64_t)sub * ny + j];
-                            wk[j] = ch ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
-                        }
-                        const uint32_t c1 = (uint32_t)(tr.level[Y] + 1) | ((uint32_t)ch << 8) |
-                                            (kTagDescend << 16);
+                if (sub < (lx ? 1 : nx_ch)) {
+                    const int32_t xc = lx ? X : cx + sub;
+                    const int4 sc = tr.sums[xc];
+                    const int64_t c0 = cf + (int64_t)sub * ny;
+                    float2 wk[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        wk[j] = j < ny ? a.pw[2 * (c0 + j) + ch] : make_float2(0.f, 0.f);
+                    if (lx || (ch ? sc.y : sc.x) != 0) {
+                        const uint32_t c1 = ly1 | ((uint32_t)ch << 8) | (kTagDescend << 16);
                         const int kk =
-                            draw_index(wk, ny, philox_bits53(seed, (uint32_t)xc, c1, step));
+                            draw_index(wk, ny, philox_bits53(a.seed, (uint32_t)xc, c1, step));
                         drew = true;
-                        if (kk >= 0) {
-                            const unsigned long long slot = atomicAdd(ct.n_out, 1ull);
-                            const Item nx_it = {xc, cy + kk, cf + sub * ny + kk, ch};
-                            if ((int64_t)slot < cap_out) out[slot] = nx_it;
-                            else atomicOr(ct.overflow, 2ull);
-                        }
+                        keep = kk >= 0;
+                        nx = Item{xc, cy + kk, (int32_t)(c0 + kk), ch};
                     }
                 }
             } else {
                 far_item = true;
             }
         }
+        append_items(leaf_pair, it, n_leaf, a.leaf_out, a.cap_leaf, overflow, 4ull);
+        append_items(keep, nx, n_out, out, a.cap_out, overflow, 2ull);
         const unsigned dm = __ballot_sync(0xffffffffu, drew);
-        if (lane == 0 && dm) atomicAdd(ct.draws, (unsigned long long)__popc(dm));
+        if (lane == 0 && dm) atomicAdd(ull(&dc->draws), (unsigned long long)__popc(dm));
         // below a translated pair: each candidate's attraction is a
         // translation the whole warp evaluates
         unsigned fm = __ballot_sync(0xffffffffu, far_item && sub == 0);
@@ -272,29 +292,58 @@ k_descend(const Item* __restrict__ in, Tree tr, Exps ex,
             for (int i = 0; i < nsrc; ++i) {
                 const int32_t xc = lx ? X : tr.child_first[X] + i;
                 if (!lx) {
-                    const int4 sm = tr.sums[xc];
-                    if ((ch ? sm.y : sm.x) == 0) continue;
+                    const int4 sc = tr.sums[xc];
+                    if ((ch ? sc.y : sc.x) == 0) continue;
+                }
+                float mine = 0.f;            // lane j: candidate j
+                for (int j = 0; j < ny; ++j) {
+                    const float v = warp_far_w(tr, a.ex, xc, cy + j, ch, sm, sm + 48,
+                                               sm + 48 + a.ex.p * a.ex.p * a.ex.p);
+                    if (lane == j) mine = v;
                 }
                 float2 wk[8];
-                for (int j = 0; j < ny; ++j)
-                    wk[j] = make_float2(
-                        warp_far_w(tr, ex, xc, cy + j, ch, sH[w], sb[w][0], sb[w][1]), 0.f);
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    wk[j] = make_float2(__shfl_sync(0xffffffffu, mine, j), 0.f);
                 if (lane == 0) {
                     const uint32_t c1 = (uint32_t)(tr.level[Y] + 1) | ((uint32_t)ch << 8) |
                                         (kTagDescend << 16);
-                    const int kk = draw_index(wk, ny, philox_bits53(seed, (uint32_t)xc, c1, step));
-                    atomicAdd(ct.draws, 1ull);
+                    const int kk = draw_index(wk, ny, philox_bits53(a.seed, (uint32_t)xc, c1, step));
+                    atomicAdd(ull(&dc->draws), 1ull);
                     if (kk >= 0) {
-                        const unsigned long long slot = atomicAdd(ct.n_out, 1ull);
-                        const Item nx_it = {xc, cy + kk, -1, ch};
-                        if ((int64_t)slot < cap_out) out[slot] = nx_it;
-                        else atomicOr(ct.overflow, 2ull);
+                        const unsigned long long slot = atomicAdd(n_out, 1ull);
+                        const Item far_nx = {xc, cy + kk, -1, ch};
+                        if ((int64_t)slot < a.cap_out) out[slot] = far_nx;
+                        else atomicOr(overflow, 2ull);
                     }
                 }
                 __syncwarp();
             }
         }
     }
+}
+
+// The first steps in one block: the items of a step are distinct (X, channel)
+// with disjoint boxes X no deeper than the step, so at most 2 * 8^k, one round of
+// 32 warps up to step 2.
+constexpr int kDescTop = 3, kDescTopWarps = 32;
+__global__ void __launch_bounds__(kDescTopWarps * 32) k_descend_top(const DescArgs a, int steps) {
+    extern __shared__ float s_desc[];
+    const int w = threadIdx.x >> 5;
+    for (int k = 0; k < steps; ++k) {
+        descend_step(a, k, w, kDescTopWarps, s_desc + w * desc_warp_floats(a.ex.p));
+        __syncthreads();
+    }
+}
+
+// Then a launch per step, with as many blocks as the step may have items for.
+// 1,000,000 neurons (serialised, cold): 82 us in eight launches whose candidates
+// lay in local memory, 64 in six; 4,096 neurons 30 in four, 22 in two.
+__global__ void __launch_bounds__(kDescWarps * 32, 8) k_descend(const DescArgs a, int step_k) {
+    extern __shared__ float s_desc[];
+    const int w = threadIdx.x >> 5;
+    descend_step(a, step_k, (int64_t)blockIdx.x * kDescWarps + w, (int64_t)gridDim.x * kDescWarps,
+                 s_desc + w * desc_warp_floats(a.ex.p));
 }
 
 // Per-element draw inside the chosen dendrite leaf, one warp per leaf pair
@@ -812,19 +861,21 @@ void select_partners(msp_ctx& c, uint64_t step, const uint8_t* type_dev, const u
     MSP_LAUNCH("select_init");
     auto ull = [](int64_t* p) { return reinterpret_cast<unsigned long long*>(p); };
     const int n_steps = c.tree_depth + 1;
-    const int gd = (int)std::max<int64_t>(1, (int64_t)c.sm_count * 16);
-    for (int k = 0; k < n_steps; ++k) {
-        DescCtr ct;
-        ct.n_in = &dc->items[k % 3];
-        ct.n_out = ull(&dc->items[(k + 1) % 3]);
-        ct.n_reset = &dc->items[(k + 2) % 3];
-        ct.n_leaf = ull(&dc->n_leaf);
-        ct.draws = ull(&dc->draws);
-        ct.overflow = ull(&dc->overflow);
-        k_descend<<<gd, kDescWarps * 32, 0, s>>>(ib[k & 1], tr, ex, c.pr_kind.get<uint8_t>(),
-                                                 c.pr_cf.get<int32_t>(), c.pr_w.get<float4>(),
-                                                 cfg.seed, stp, ib[(k + 1) & 1], cap_items, lit,
-                                                 cap_leaf, ct);
+    const DescArgs da{tr, ex, c.pr_kind.get<uint8_t>(), c.pr_cf.get<int32_t>(),
+                      c.pr_w.get<float2>(), cfg.seed, stp, {ib[0], ib[1]}, cap_items, lit, cap_leaf,
+                      dc};
+    const int top = std::min(n_steps, kDescTop);
+    const size_t warp_bytes = desc_warp_floats(cfg.p) * sizeof(float);
+    if (kDescTopWarps * warp_bytes > 48 * 1024)
+        MSP_CUDA(cudaFuncSetAttribute(k_descend_top, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(kDescTopWarps * warp_bytes)));
+    k_descend_top<<<1, kDescTopWarps * 32, kDescTopWarps * warp_bytes, s>>>(da, top);
+    MSP_LAUNCH("descend_top");
+    for (int k = top; k < n_steps; ++k) {
+        // at most two items (channels) for each of 8^k boxes, 16 a block
+        const int64_t most = std::min<int64_t>(cap_items, (int64_t)2 << std::min(3 * k, 40));
+        k_descend<<<grid_for(most, 4 * kDescWarps, (int64_t)c.sm_count * 16), kDescWarps * 32,
+                    kDescWarps * warp_bytes, s>>>(da, k);
         MSP_LAUNCH("descend");
     }
     // one warp per leaf pair, from a device work counter

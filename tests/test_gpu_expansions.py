@@ -39,3 +39,21 @@ def test_translations_match_the_oracle(oracle_mod, p, leaf, rho, n, side):
     for k in ("wE", "wI"):
         err = np.abs(t[k] - op[k])
         assert np.all(err <= 1e-4 * np.abs(op[k]) + 1e-7 * np.abs(op[k]).max()), k
+
+
+@pytest.mark.parametrize("p", [1, 4, 8])
+@pytest.mark.parametrize("leaf,rho,n,side", [(1, 0.3, 60, 1500.0), (4, 0.4, 200, 1000.0)])
+def test_descent_through_translated_pairs_matches_the_oracle(oracle_mod, p, leaf, rho, n, side):
+    w = W.uniform_cube(n, side, seed=20 + p, leaf_capacity=leaf, rho_max=rho, cutoff=4.0, p=p)
+    g = msp.MSP(w.params)
+    g.build_tree(*msp.to_device(w))
+    g.attraction()
+    sel = g.select_partners(3)
+    st = g.stats()
+    g.close()
+    o = oracle_mod.Oracle(w.params)
+    o.build_tree(*w.arrays())
+    o.attraction()
+    ro = o.select_partners(3)
+    differ = sel["partner"].cpu().numpy()[:st["n_elements"]] != ro["partner"]
+    assert st["n_far"] > 0 and np.all(ro["near_boundary"][differ])
