@@ -471,77 +471,92 @@ k_tree_level(LevelArgs a, int level, DevCounts* dc, unsigned long long* status,
 // Centroids are accumulated as weighted offsets from the box's geometric
 // centre so that single precision keeps them accurate (with frames, the
 // centre in the box's network's own frame: box_axis).  A leaf's lanes take its
-// points, an inner box's lanes its children (at most 8); a fixed butterfly
-// sums the lanes, then lane 0 writes the box's vacant-element sums and its
-// axon / dendrite centroids (offsets summed, then divided by the weight).  The
-// order of every sum is fixed whichever warp computes a box, so the results
-// are those of a level-by-level pass.  The counters are zero on entry
-// (cleared by the host before an eager build and whenever their buffer is new;
-// every complete launch leaves them zero).
-__device__ __forceinline__ void aggregate_box(int64_t i, int lane, int frame_level, float ox,
-                                              float oy, float oz, float side,
-                                              const float4* __restrict__ pts,
-                                              const uint8_t* __restrict__ level,
-                                              const uint64_t* __restrict__ prefix,
-                                              const int32_t* __restrict__ first,
-                                              const int32_t* __restrict__ count,
-                                              const int32_t* __restrict__ child_first,
-                                              const uint8_t* __restrict__ nchild,
-                                              int4* __restrict__ sums, float4* __restrict__ ca,
-                                              float4* __restrict__ cd,
-                                              int32_t* __restrict__ leaf_of) {
-    const uint64_t pre = prefix[i];
-    const int lv = (int)level[i];
-    const float bs = ldexpf(side, -lv);
-    const float g[3] = {ox + ((float)box_axis(pre, 0, lv, frame_level) + 0.5f) * bs,
-                        oy + ((float)box_axis(pre, 1, lv, frame_level) + 0.5f) * bs,
-                        oz + ((float)box_axis(pre, 2, lv, frame_level) + 0.5f) * bs};
+// points, an inner box's lanes its children (at most 8).  A fixed butterfly
+// (lane distances 16, 8, 4, 2, 1) sums the lanes: the vacant elements by the
+// warp's integer reduction, the six offset sums by halving what a lane keeps
+// while it halves the lanes (8 shuffles instead of 30), which leaves each sum in
+// a lane of its own, where it is divided by its weight.  The order of every sum
+// is fixed whichever warp computes a box, so the results are those of a
+// level-by-level pass.  The counters are zero on entry (cleared by the build
+// before an eager build and whenever their buffer is new; every complete launch
+// leaves them zero).
+//
+// Bound by the chain of arrivals (a release each) and instruction issue.
+// Serialised, cold: 1,000,000 neurons 47 -> 41 us with the halving butterfly and
+// leaf_of kept, 65,536 in leaves of at most 8: 61 -> 50 us.
+struct AggArgs {
+    int frame_level;
+    float ox, oy, oz, side;
+    const float4* pts;
+    const uint8_t* level;
+    const uint64_t* prefix;
+    const int32_t *first, *count, *parent, *child_first;
+    const uint8_t* nchild;
+    int4* sums;
+    float4 *ca, *cd;
+    int32_t* leaf_of;            // null: as they are (octree kept)
+    int32_t* arrive;
+};
+
+// cf: the box's first child (-1: a leaf), nc: its children
+__device__ __forceinline__ void aggregate_box(const AggArgs& a, int64_t i, int32_t cf, int nc,
+                                              int lane) {
+    const uint64_t pre = a.prefix[i];
+    const int lv = (int)a.level[i];
+    const float bs = ldexpf(a.side, -lv);
+    const float g[3] = {a.ox + ((float)box_axis(pre, 0, lv, a.frame_level) + 0.5f) * bs,
+                        a.oy + ((float)box_axis(pre, 1, lv, a.frame_level) + 0.5f) * bs,
+                        a.oz + ((float)box_axis(pre, 2, lv, a.frame_level) + 0.5f) * bs};
     int aE = 0, aI = 0, wE = 0, wI = 0;
     float sa[3] = {0.f, 0.f, 0.f}, sd[3] = {0.f, 0.f, 0.f};
-    const int32_t cf = child_first[i];
     if (cf < 0) {
-        const int32_t f = first[i], c = count[i];
+        const int32_t f = a.first[i], c = a.count[i];
         for (int32_t j = f + lane; j < f + c; j += 32) {
-            const float4 p = pts[j];
+            const float4 p = a.pts[j];
             const uint32_t w = __float_as_uint(p.w);
-            const int a = (int)pk_axon(w), de = (int)pk_de(w), di = (int)pk_di(w);
-            if (pk_type(w)) aI += a; else aE += a;
+            const int ax = (int)pk_axon(w), de = (int)pk_de(w), di = (int)pk_di(w);
+            if (pk_type(w)) aI += ax; else aE += ax;
             wE += de;
             wI += di;
-            const float fa = (float)a, fd = (float)(de + di);
+            const float fa = (float)ax, fd = (float)(de + di);
             const float dx = p.x - g[0], dy = p.y - g[1], dz = p.z - g[2];
             sa[0] = fmaf(fa, dx, sa[0]); sa[1] = fmaf(fa, dy, sa[1]); sa[2] = fmaf(fa, dz, sa[2]);
             sd[0] = fmaf(fd, dx, sd[0]); sd[1] = fmaf(fd, dy, sd[1]); sd[2] = fmaf(fd, dz, sd[2]);
-            leaf_of[j] = (int32_t)i;
+            if (a.leaf_of) a.leaf_of[j] = (int32_t)i;
         }
-    } else if (lane < nchild[i]) {
+    } else if (lane < nc) {
         // the children were written by other warps: read them from L2
-        const int4 sm = __ldcg(&sums[cf + lane]);
-        const float4 a4 = __ldcg(&ca[cf + lane]), d4 = __ldcg(&cd[cf + lane]);
+        const int4 sm = __ldcg(&a.sums[cf + lane]);
+        const float4 a4 = __ldcg(&a.ca[cf + lane]), d4 = __ldcg(&a.cd[cf + lane]);
         aE = sm.x; aI = sm.y; wE = sm.z; wI = sm.w;
         const float fa = (float)(sm.x + sm.y), fd = (float)(sm.z + sm.w);
         sa[0] = fa * (a4.x - g[0]); sa[1] = fa * (a4.y - g[1]); sa[2] = fa * (a4.z - g[2]);
         sd[0] = fd * (d4.x - g[0]); sd[1] = fd * (d4.y - g[1]); sd[2] = fd * (d4.z - g[2]);
     }
+    aE = __reduce_add_sync(0xffffffffu, aE);
+    aI = __reduce_add_sync(0xffffffffu, aI);
+    wE = __reduce_add_sync(0xffffffffu, wE);
+    wI = __reduce_add_sync(0xffffffffu, wI);
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+    float v[3];                       // lanes 0-15: axons, 16-31: dendrites
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        aE += __shfl_xor_sync(0xffffffffu, aE, o);
-        aI += __shfl_xor_sync(0xffffffffu, aI, o);
-        wE += __shfl_xor_sync(0xffffffffu, wE, o);
-        wI += __shfl_xor_sync(0xffffffffu, wI, o);
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            sa[d] += __shfl_xor_sync(0xffffffffu, sa[d], o);
-            sd[d] += __shfl_xor_sync(0xffffffffu, sd[d], o);
-        }
-    }
-    if (lane == 0) {
-        sums[i] = make_int4(aE, aI, wE, wI);
-        const float ta = (float)(aE + aI), td = (float)(wE + wI);
-        ca[i] = ta > 0.f ? make_float4(g[0] + sa[0] / ta, g[1] + sa[1] / ta, g[2] + sa[2] / ta, ta)
-                         : make_float4(g[0], g[1], g[2], 0.f);
-        cd[i] = td > 0.f ? make_float4(g[0] + sd[0] / td, g[1] + sd[1] / td, g[2] + sd[2] / td, td)
-                         : make_float4(g[0], g[1], g[2], 0.f);
+    for (int d = 0; d < 3; ++d)
+        v[d] = (h16 ? sd[d] : sa[d]) + __shfl_xor_sync(0xffffffffu, h16 ? sa[d] : sd[d], 16);
+    const float u0 = (h8 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, h8 ? v[0] : v[2], 8);
+    const float u1 = v[1] + __shfl_xor_sync(0xffffffffu, v[1], 8);
+    const bool one = !h8 && h4;       // axis 0: neither half, 1: h4, 2: h8
+    float x = (one ? u1 : u0) + __shfl_xor_sync(0xffffffffu, h8 || h4 ? u0 : u1, 4);
+    x += __shfl_xor_sync(0xffffffffu, x, 2);
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    // lanes 0, 4, 8 (16, 20, 24): the axes; lanes 12, 28: the weights; lane 1: sums
+    if ((lane & 3) == 0) {
+        const int q = (lane >> 2) & 3;
+        const float t = (float)(h16 ? wE + wI : aE + aI);
+        const float gq = q == 0 ? g[0] : (q == 1 ? g[1] : g[2]);
+        float* out = reinterpret_cast<float*>(h16 ? a.cd + i : a.ca + i);
+        out[q] = q == 3 ? (t > 0.f ? t : 0.f) : (t > 0.f ? gq + x / t : gq);
+    } else if (lane == 1) {
+        a.sums[i] = make_int4(aE, aI, wE, wI);
     }
 }
 
@@ -554,39 +569,41 @@ __device__ __forceinline__ int arrive_acq_rel(int32_t* p) {
 }
 
 // nodes_end: the node count (device memory); one warp per leaf
-__global__ void k_aggregate_tree(const BuildEnd end, const int64_t* __restrict__ nodes_end, int frame_level, float ox,
-                                 float oy, float oz, float side, const float4* __restrict__ pts,
-                                 const uint8_t* __restrict__ level,
-                                 const uint64_t* __restrict__ prefix,
-                                 const int32_t* __restrict__ first,
-                                 const int32_t* __restrict__ count,
-                                 const int32_t* __restrict__ parent,
-                                 const int32_t* __restrict__ child_first,
-                                 const uint8_t* __restrict__ nchild, int4* __restrict__ sums,
-                                 float4* __restrict__ ca, float4* __restrict__ cd,
-                                 int32_t* __restrict__ leaf_of, int32_t* __restrict__ arrive) {
+__global__ void k_aggregate_tree(const BuildEnd end, const int64_t* __restrict__ nodes_end,
+                                 const AggArgs a) {
     if (blockIdx.x == 0 && threadIdx.x == 0) end();
     const int64_t nn = *nodes_end;
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nn; k += nw) {
-        if (child_first[k] >= 0) continue;        // inner boxes: done by their last child's warp
+        if (a.child_first[k] >= 0) continue;      // inner boxes: done by their last child's warp
         int64_t i = k;
+        int32_t cf = -1, p = a.parent[k];
+        int nc = 0;
         for (;;) {
-            aggregate_box(i, lane, frame_level, ox, oy, oz, side, pts, level, prefix, first, count,
-                          child_first, nchild, sums, ca, cd, leaf_of);
-            const int32_t p = parent[i];
+            // the parent's place in the octree, read while the box is summed
+            int32_t pcf = 0, pp = -1;
+            int pnc = 0;
+            if (p >= 0) {
+                pcf = a.child_first[p];
+                pnc = (int)a.nchild[p];
+                pp = a.parent[p];
+            }
+            aggregate_box(a, i, cf, nc, lane);
             if (p < 0) break;
+            __syncwarp();                         // the lanes' writes before the arrival
             int last = 0;
             if (lane == 0) {
-                // lane 0 wrote the box's results
-                last = arrive_acq_rel(&arrive[p]) == (int)nchild[p] - 1;
-                if (last) arrive[p] = 0;
+                last = arrive_acq_rel(&a.arrive[p]) == pnc - 1;
+                if (last) a.arrive[p] = 0;
             }
             last = __shfl_sync(0xffffffffu, last, 0);
             if (!last) break;
             __syncwarp();                         // the lanes' reads after lane 0's acquire
             i = p;
+            cf = pcf;
+            nc = pnc;
+            p = pp;
         }
     }
 }
@@ -632,6 +649,14 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
     if (framed && n != c.frame_off_host.back())
         throw Error(MSP_ERR_INVALID_ARG, "the frames (msp_set_frames) hold a different number "
                                          "of neurons");
+    auto agg_args = [&](int32_t* lo) {
+        return AggArgs{c.frame_level, o3[0], o3[1], o3[2], cfg.side, pts,
+                       c.nd_level.get<uint8_t>(), c.nd_prefix.get<uint64_t>(),
+                       c.nd_first.get<int32_t>(), c.nd_count.get<int32_t>(),
+                       c.nd_parent.get<int32_t>(), c.nd_child_first.get<int32_t>(),
+                       c.nd_nchild.get<uint8_t>(), c.nd_sums.get<int4>(), c.nd_ca.get<float4>(),
+                       c.nd_cd.get<float4>(), lo, c.nd_arrive.get<int32_t>()};
+    };
     unsigned long long* scan_st = scan_status(c, n);
     const int64_t n_scan_st = scan_status_words(n);
 
@@ -680,11 +705,7 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
             dev_set(&dc->n_elem, 0, s);
         }
         k_aggregate_tree<<<agg_grid(c.n_nodes, c.sm_count), 128, 0, s>>>(
-            end, &dc->level_start[c.tree_levels + 1], c.frame_level, o3[0], o3[1], o3[2], cfg.side,
-            pts, c.nd_level.get<uint8_t>(), c.nd_prefix.get<uint64_t>(), c.nd_first.get<int32_t>(),
-            c.nd_count.get<int32_t>(), c.nd_parent.get<int32_t>(), c.nd_child_first.get<int32_t>(),
-            c.nd_nchild.get<uint8_t>(), c.nd_sums.get<int4>(), c.nd_ca.get<float4>(),
-            c.nd_cd.get<float4>(), leaf_of, c.nd_arrive.get<int32_t>());
+            end, &dc->level_start[c.tree_levels + 1], agg_args(nullptr));
         MSP_LAUNCH("aggregate");
         if (c.graph_mode) return;
         pull_counts(c, s);              // the one synchronisation of the build
@@ -762,9 +783,9 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
         c.nd_parent.ensure<int32_t>((size_t)cap);
         c.nd_child_first.ensure<int32_t>((size_t)cap);
         c.nd_nchild.ensure<uint8_t>((size_t)cap);
-        int4* sums = c.nd_sums.ensure<int4>((size_t)cap);
-        float4* ca = c.nd_ca.ensure<float4>((size_t)cap);
-        float4* cd = c.nd_cd.ensure<float4>((size_t)cap);
+        c.nd_sums.ensure<int4>((size_t)cap);
+        c.nd_ca.ensure<float4>((size_t)cap);
+        c.nd_cd.ensure<float4>((size_t)cap);
         // the arrival counters: cleared before an eager build and whenever
         // the buffer is new (a graph's dry run may build one level deeper than
         // the eager build and grow it); a replay finds them as the last
@@ -813,10 +834,7 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
         }
         // a4: aggregates, leaves up to the root in one launch
         k_aggregate_tree<<<agg_grid(cap, c.sm_count), 128, 0, s>>>(
-            end, &dc->level_start[L + 1], c.frame_level, o3[0], o3[1], o3[2], cfg.side, pts,
-            c.nd_level.get<uint8_t>(), c.nd_prefix.get<uint64_t>(), c.nd_first.get<int32_t>(),
-            c.nd_count.get<int32_t>(), c.nd_parent.get<int32_t>(), c.nd_child_first.get<int32_t>(),
-            c.nd_nchild.get<uint8_t>(), sums, ca, cd, leaf_of, arrive);
+            end, &dc->level_start[L + 1], agg_args(leaf_of));
         MSP_LAUNCH("aggregate");
         // inside the whole-step graph the tree of the same positions has the
         // same levels; a deeper one sets more_levels, which halts the graph
