@@ -782,12 +782,11 @@ __global__ void k_l2p(int64_t n, int64_t exp_first, int p, float inv_sigma,
 // before the sum), then a fixed butterfly over the 8 lanes.  Both orders are
 // fixed, so the table is reproducible.  sb = [first, end) of the depth's
 // entries in split; an entry is (pair, first child, child count, 0).
-__global__ void k_reduce_split(const int64_t* __restrict__ sb, const int4* __restrict__ split,
-                               float4* __restrict__ pw) {
+__device__ __forceinline__ void reduce_depth(const int64_t* __restrict__ sb,
+                                             const int4* __restrict__ split, float4* pw,
+                                             int64_t warp, int64_t nwarp) {
     const int64_t s0 = sb[0], ns = sb[1] - sb[0];
     const int lane = threadIdx.x & 31, sub = lane & 7;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
     // the loop bound is uniform across the warp (its 4 groups shuffle together)
     for (int64_t k0 = 4 * warp; k0 < ns; k0 += 4 * nwarp) {
         const int64_t k = k0 + (lane >> 3);
@@ -821,6 +820,23 @@ __global__ void k_reduce_split(const int64_t* __restrict__ sb, const int4* __res
             const float2 e = ff_two_sum(eh, ec), i = ff_two_sum(ih, ic);
             pw[q] = make_float4(e.x, e.y, i.x, i.y);
         }
+    }
+}
+__global__ void k_reduce_split(const int64_t* __restrict__ sb, const int4* __restrict__ split,
+                               float4* pw) {
+    reduce_depth(sb, split, pw, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                 ((int64_t)gridDim.x * blockDim.x) >> 5);
+}
+// The last depths (at most 64 split pairs and the root's) in one block, the others
+// with as many blocks as the depth may have pairs for: a step of two networks of
+// 21 k 1209 -> 1193 us (4 and 5 launches of 1216 blocks each before).
+constexpr int kReduceTop = 2;
+__global__ void __launch_bounds__(512) k_reduce_top(const int64_t* __restrict__ sb,
+                                                    const int4* __restrict__ split, float4* pw,
+                                                    int depths) {
+    for (int d = depths - 1; d >= 0; --d) {
+        reduce_depth(sb + d, split, pw, threadIdx.x >> 5, blockDim.x >> 5);
+        __syncthreads();
     }
 }
 
@@ -1062,10 +1078,16 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
     }
     c.nf_timed = n > 0;
     // a10: pair table, deepest pairs first
-    for (int dd = D - 1; dd >= 0; --dd) {
-        k_reduce_split<<<Gt, B, 0, s>>>(&dc->split_start[dd], split, c.pr_w.get<float4>());
+    for (int dd = D - 1; dd >= kReduceTop; --dd) {
+        // at most 64^dd pairs of this depth, four a warp
+        const int64_t pairs = std::min<int64_t>((int64_t)1 << std::min(6 * dd, 40), cap);
+        k_reduce_split<<<grid_for(8 * pairs, B, Gt), B, 0, s>>>(&dc->split_start[dd], split,
+                                                               c.pr_w.get<float4>());
         MSP_LAUNCH("reduce_split");
     }
+    k_reduce_top<<<1, 512, 0, s>>>(dc->split_start, split, c.pr_w.get<float4>(),
+                                   std::min(D, kReduceTop));
+    MSP_LAUNCH("reduce_top");
     // inside the whole-step graph the table does not grow: an overflow halts
     // the graph (checked on the device after the selection)
     if (c.graph_mode) return;
