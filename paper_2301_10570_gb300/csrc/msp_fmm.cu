@@ -580,39 +580,42 @@ k_m2l_seg(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nse
     }
 }
 
-// Order 4 (the paper's): a pass has 16 columns per channel, so half a warp takes
-// a pair and the two halves alternate over X's pairs; both channels share the
-// Hermite functions and run as the two halves of paired FMAs; the next pair's
-// coefficients are loaded while the current pair is translated.  Per pair the
-// products and sums of W(X,Y) are those of the general kernel in the same
-// order; B(X) adds the pairs of each half and then the halves.  Blocks take
-// four targets and leave (the numbers of pairs per target differ widely: a
+// Order 4 (the paper's): a pass has 16 columns per channel, so a quarter of a warp
+// takes a pair, two columns a lane, and the quarters alternate over X's pairs; both
+// channels share the Hermite functions and run as the two halves of paired FMAs;
+// the next pair's coefficients are loaded while the current pair is translated.
+// Per pair the products and sums of W(X,Y) are those of the general kernel in the
+// same order; B(X) adds the pairs of each quarter and then the quarters.  Blocks
+// take four targets and leave (the numbers of pairs per target differ widely: a
 // grid of resident blocks striding over the targets took 0.93 ms).
-// 4.9 M pairs of 65,536 neurons: 1.47 ms in the general kernel, 0.74 ms here,
-// the same 1.47 ms with unpadded rows (bank conflicts).  Bound by instruction
-// issue: 48 paired FMAs of a pair's 100, the rest Hermite functions and staging.
-__global__ void __launch_bounds__(kM2LWarps * 32)
+// 4.9 M pairs of 65,536 neurons: 1.47 ms in the general kernel, 0.72 ms here
+// (0.74 with half a warp a pair, each lane's Hermite functions for one column; 1.47
+// with unpadded rows: bank conflicts).  Bound by instruction issue: 48 paired FMAs
+// of a pair's 95 instructions, the rest Hermite functions and staging.
+__global__ void __launch_bounds__(kM2LWarps * 32, 4)
 k_m2l_seg4(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nseg_dev,
            const int32_t* __restrict__ list, int64_t exp_first, float inv_sigma,
            const int32_t* __restrict__ pX, const int32_t* __restrict__ pY,
            const float4* __restrict__ ca, const float4* __restrict__ cd,
            const float* __restrict__ A, const float* __restrict__ M, float* __restrict__ B,
            float4* __restrict__ pw) {
-    constexpr int P = 4, P3 = 64;
-    // a half's coefficients between passes: [b0][a1][a2] with rows of 20 and 4,
-    // [b0][b1][a2] with rows of 20 and 5 (16 lanes write or read 16 different
-    // pairs of banks in every pass)
-    __shared__ float2 s_t0[kM2LWarps][2][76], s_t1[kM2LWarps][2][80];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane >> 4, r = lane & 15;
-    float2* t0 = s_t0[w][half];
-    float2* t1 = s_t1[w][half];
-    const int hi = r >> 2, lo = r & 3;
-    float scale[P];
+    constexpr int P = 4, P3 = 64, QW = 88;
+    // a quarter's coefficients between passes: [b0][a1][a2] with rows of 20 and 4,
+    // [b0][b1][a2] with rows of 20 and 5, quarters 88 apart (16 lanes write or
+    // read 16 different pairs of banks in every pass)
+    __shared__ float2 s_t0[kM2LWarps][4 * QW], s_t1[kM2LWarps][4 * QW];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = lane >> 3, r = lane & 7;
+    float2* t0 = s_t0[w] + QW * quarter;
+    float2* t1 = s_t1[w] + QW * quarter;
+    const int hi = r >> 2, lo = r & 3;       // the lane's columns: (hi, lo) and (hi + 2, lo)
+    float scale[2][P];
 #pragma unroll
-    for (int b2 = 0; b2 < P; ++b2) {
-        const float f = c_inv_fact[hi] * c_inv_fact[lo] * c_inv_fact[b2];
-        scale[b2] = ((hi + lo + b2) & 1) ? -f : f;
-    }
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int b2 = 0; b2 < P; ++b2) {
+            const float f = c_inv_fact[hi + 2 * j] * c_inv_fact[lo] * c_inv_fact[b2];
+            scale[j][b2] = ((hi + lo + b2) & 1) ? -f : f;
+        }
     const int64_t nseg = *nseg_dev;
     for (int64_t sg = (int64_t)blockIdx.x * kM2LWarps + w; sg < nseg;
          sg += (int64_t)gridDim.x * kM2LWarps) {
@@ -620,32 +623,42 @@ k_m2l_seg4(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ ns
         const int32_t X = pX[list[i0]];
         const int64_t ex = X - exp_first;
         const float4 a4 = ca[X];
-        const float4 m0 = reinterpret_cast<const float4*>(M + (ex * 2) * P3)[r];
-        const float4 m1 = reinterpret_cast<const float4*>(M + (ex * 2 + 1) * P3)[r];
-        const float2 mm[P] = {make_float2(m0.x, m1.x), make_float2(m0.y, m1.y),
-                              make_float2(m0.z, m1.z), make_float2(m0.w, m1.w)};
-        float2 acc[P];
+        float2 mm[2][P], acc[2][P];
 #pragma unroll
-        for (int k = 0; k < P; ++k) acc[k] = make_float2(0.f, 0.f);
+        for (int j = 0; j < 2; ++j) {
+            const float4 m0 = reinterpret_cast<const float4*>(M + (ex * 2) * P3)[r + 8 * j];
+            const float4 m1 = reinterpret_cast<const float4*>(M + (ex * 2 + 1) * P3)[r + 8 * j];
+            mm[j][0] = make_float2(m0.x, m1.x);
+            mm[j][1] = make_float2(m0.y, m1.y);
+            mm[j][2] = make_float2(m0.z, m1.z);
+            mm[j][3] = make_float2(m0.w, m1.w);
+#pragma unroll
+            for (int k = 0; k < P; ++k) acc[j][k] = make_float2(0.f, 0.f);
+        }
         // the next pair's list entry, centre and coefficients are loaded
         // while the current pair is translated (a chain of dependent loads)
         int32_t q = 0;
         float4 d = a4;
-        float2 v[P];
+        float2 v[2][P];
         auto load = [&](int32_t i) {
 #pragma unroll
-            for (int k = 0; k < P; ++k) v[k] = make_float2(0.f, 0.f);
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int k = 0; k < P; ++k) v[j][k] = make_float2(0.f, 0.f);
             if (i >= i1) return;
             q = list[i];
             const int32_t Y = pY[q];
             d = cd[Y];
             const float* Ay = A + (Y - exp_first) * 2 * P3 + r;
 #pragma unroll
-            for (int k = 0; k < P; ++k) v[k] = make_float2(Ay[16 * k], Ay[P3 + 16 * k]);
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int k = 0; k < P; ++k)
+                    v[j][k] = make_float2(Ay[16 * k + 8 * j], Ay[P3 + 16 * k + 8 * j]);
         };
-        load(i0 + half);
-        for (int32_t ib = i0; ib < i1; ib += 2) {
-            const bool in = ib + half < i1;
+        load(i0 + quarter);
+        for (int32_t ib = i0; ib < i1; ib += 4) {
+            const bool in = ib + quarter < i1;
             const int32_t qc = q;
             float H[8];
             const float4 dc = d;
@@ -660,47 +673,70 @@ k_m2l_seg4(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ ns
             hermite_row((a4.x - dc.x) * inv_sigma, H, 2 * P - 2);
             __syncwarp();
 #pragma unroll
-            for (int o = 0; o < P; ++o) t0[20 * o + r] = apply(v, o);
-            load(ib + 2 + half);
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int o = 0; o < P; ++o) t0[20 * o + r + 8 * j] = apply(v[j], o);
+            load(ib + 4 + quarter);
             __syncwarp();
             // over a1: column (b0, a2) -> [b0][b1][a2]
             hermite_row((a4.y - dc.y) * inv_sigma, H, 2 * P - 2);
-            float2 c[P];
 #pragma unroll
-            for (int k = 0; k < P; ++k) c[k] = t0[20 * hi + 4 * k + lo];
+            for (int j = 0; j < 2; ++j) {
+                float2 c[P];
 #pragma unroll
-            for (int o = 0; o < P; ++o) t1[20 * hi + 5 * o + lo] = apply(c, o);
+                for (int k = 0; k < P; ++k) c[k] = t0[20 * (hi + 2 * j) + 4 * k + lo];
+#pragma unroll
+                for (int o = 0; o < P; ++o) t1[20 * (hi + 2 * j) + 5 * o + lo] = apply(c, o);
+            }
             __syncwarp();
             // over a2: column (b0, b1)
             hermite_row((a4.z - dc.z) * inv_sigma, H, 2 * P - 2);
+            float2 wc[2];
 #pragma unroll
-            for (int k = 0; k < P; ++k) c[k] = t1[20 * hi + 5 * lo + k];
-            float2 wc = make_float2(0.f, 0.f);
+            for (int j = 0; j < 2; ++j) {
+                float2 c[P];
 #pragma unroll
-            for (int o = 0; o < P; ++o) {
-                const float2 t = __fmul2_rn(apply(c, o), make_float2(scale[o], scale[o]));
-                acc[o] = __fadd2_rn(acc[o], t);
-                wc = __ffma2_rn(t, mm[o], wc);
+                for (int k = 0; k < P; ++k) c[k] = t1[20 * (hi + 2 * j) + 5 * lo + k];
+                wc[j] = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int o = 0; o < P; ++o) {
+                    const float2 t = __fmul2_rn(apply(c, o), make_float2(scale[j][o], scale[j][o]));
+                    acc[j][o] = __fadd2_rn(acc[j][o], t);
+                    wc[j] = __ffma2_rn(t, mm[j][o], wc[j]);
+                }
             }
+            float2 ws = __fadd2_rn(wc[0], wc[1]);
 #pragma unroll
-            for (int o = 8; o > 0; o >>= 1) {
-                wc.x += __shfl_xor_sync(0xffffffffu, wc.x, o);
-                wc.y += __shfl_xor_sync(0xffffffffu, wc.y, o);
+            for (int o = 4; o > 0; o >>= 1) {
+                ws.x += __shfl_xor_sync(0xffffffffu, ws.x, o);
+                ws.y += __shfl_xor_sync(0xffffffffu, ws.y, o);
             }
-            if (r == 0 && in) pw[qc] = make_float4(wc.x, 0.f, wc.y, 0.f);
+            if (r == 0 && in) pw[qc] = make_float4(ws.x, 0.f, ws.y, 0.f);
         }
-        // B(X) += the sum over X's far pairs (no other warp adds to B(X) here)
+        // B(X) += the sum over X's far pairs (no other warp adds to B(X) here):
+        // quarters 0, 1 write the excitatory columns, 2, 3 the inhibitory ones
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int k = 0; k < P; ++k)
+#pragma unroll
+                for (int o = 8; o < 32; o <<= 1) {
+                    acc[j][k].x += __shfl_xor_sync(0xffffffffu, acc[j][k].x, o);
+                    acc[j][k].y += __shfl_xor_sync(0xffffffffu, acc[j][k].y, o);
+                }
+        const int j = quarter & 1, ch = quarter >> 1;
+        float4* Bx = reinterpret_cast<float4*>(B + (ex * 2 + ch) * P3) + r + 8 * j;
+        float4 b = *Bx;
+        float add[P];
 #pragma unroll
         for (int k = 0; k < P; ++k) {
-            acc[k].x += __shfl_xor_sync(0xffffffffu, acc[k].x, 16);
-            acc[k].y += __shfl_xor_sync(0xffffffffu, acc[k].y, 16);
+            const float2 t = j ? acc[1][k] : acc[0][k];
+            add[k] = ch ? t.y : t.x;
         }
-        float4* Bx = reinterpret_cast<float4*>(B + (ex * 2 + half) * P3) + r;
-        float4 b = *Bx;
-        b.x += half ? acc[0].y : acc[0].x;
-        b.y += half ? acc[1].y : acc[1].x;
-        b.z += half ? acc[2].y : acc[2].x;
-        b.w += half ? acc[3].y : acc[3].x;
+        b.x += add[0];
+        b.y += add[1];
+        b.z += add[2];
+        b.w += add[3];
         *Bx = b;
     }
 }
