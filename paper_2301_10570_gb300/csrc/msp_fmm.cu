@@ -283,6 +283,7 @@ k_trav_depth(TravArgs a, int d, unsigned long long* status, int64_t timeout_bit)
     __shared__ int64_t s_tile;
     __shared__ long long s_ex[2];
     DevCounts* dc = a.dc;
+    if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
     const int64_t q0 = dc->depth_start[d], next0 = dc->depth_start[d + 1], nq = next0 - q0;
     const int64_t ntiles = (nq + kTravTile - 1) / kTravTile;
     if (ntiles == 0) {
@@ -290,7 +291,6 @@ k_trav_depth(TravArgs a, int d, unsigned long long* status, int64_t timeout_bit)
         return;
     }
     for (;;) {
-        if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
         __syncthreads();
         const int64_t t = s_tile;
         if (t >= ntiles) break;
@@ -312,7 +312,9 @@ k_trav_depth(TravArgs a, int d, unsigned long long* status, int64_t timeout_bit)
             ex[2] = s_ex[1] >> 31;
             ex[3] = s_ex[1] & m;
         });
+        if (ntiles <= gridDim.x) break;        // every block has had its one tile
         __syncthreads();
+        if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
     }
 }
 

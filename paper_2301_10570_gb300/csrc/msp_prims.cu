@@ -83,14 +83,17 @@ k_rs_pass(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin,
     __shared__ uint64_t s_key[kRsTile];
     __shared__ int32_t s_val[kRsTile];
     __shared__ uint16_t s_cnt[kRsWarps][kRsBins];   // per warp: count, then offset, of a digit
-    __shared__ int32_t s_base[kRsBins];             // where a digit starts in the output
     __shared__ int32_t s_off[kRsBins];              // where it starts in the tile
     __shared__ int32_t s_dst[kRsBins];              // output minus tile position
     __shared__ int32_t s_warp[kRsWarps];
     __shared__ int32_t s_tile;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int64_t n = n_dev ? *n_dev : n_host;
     const int bins = 1 << bits;
+    // the reads that start a pass run together: the first tile's number, the
+    // element count, the digits' totals (scanned while the keys are on their way)
+    if (t == 0) s_tile = atomicAdd(tile_ctr, 1);
+    const int32_t h0 = 2 * t < bins ? hist[2 * t] : 0, h1 = 2 * t < bins ? hist[2 * t + 1] : 0;
+    const int64_t n = n_dev ? *n_dev : n_host;
     const int ntiles = (int)((n + kRsTile - 1) / kRsTile);
     volatile unsigned long long* status = status_;
     // exclusive sums over the digits, two per thread
@@ -108,17 +111,9 @@ k_rs_pass(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin,
         __syncthreads();
         return before + inc - (a + b);
     };
-    {
-        const int32_t a = 2 * t < bins ? hist[2 * t] : 0, b = 2 * t < bins ? hist[2 * t + 1] : 0;
-        const int32_t e = digit_scan(a, b);
-        if (2 * t < bins) {
-            s_base[2 * t] = e;
-            s_base[2 * t + 1] = e + a;
-        }
-    }
+    int32_t base0 = -1;         // where digit 2 t starts in the output
     const unsigned lt = (1u << lane) - 1u;
     for (;;) {
-        if (t == 0) s_tile = atomicAdd(tile_ctr, 1);
         for (int k = t; k < kRsWarps * kRsBins / 2; k += kRsThreads)
             reinterpret_cast<uint32_t*>(&s_cnt[0][0])[k] = 0u;
         __syncthreads();
@@ -136,6 +131,7 @@ k_rs_pass(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin,
             key[r] = in ? kin[base + 32 * r] : 0ull;
             val[r] = in ? vin[base + 32 * r] : 0;
         }
+        if (base0 < 0) base0 = digit_scan(h0, h1);
 #pragma unroll
         for (int r = 0; r < kRsItems; ++r) {
             const bool in = base + 32 * r < n;
@@ -193,8 +189,8 @@ k_rs_pass(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin,
                 }
             }
             if (tile > 0) *(volatile unsigned long long*)mine = word(2, p0 + c0, p1 + c1);
-            s_dst[2 * t] = (int32_t)(s_base[2 * t] + p0 - e);
-            s_dst[2 * t + 1] = (int32_t)(s_base[2 * t + 1] + p1 - (e + c0));
+            s_dst[2 * t] = (int32_t)(base0 + p0 - e);
+            s_dst[2 * t + 1] = (int32_t)(base0 + h0 + p1 - (e + c0));
         }
         __syncthreads();
         // into digit order, then out
@@ -217,7 +213,9 @@ k_rs_pass(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin,
                 vout[o] = s_val[i];
             }
         }
+        if (ntiles <= (int)gridDim.x) break;        // every block has had its one tile
         __syncthreads();
+        if (t == 0) s_tile = atomicAdd(tile_ctr, 1);
     }
 }
 

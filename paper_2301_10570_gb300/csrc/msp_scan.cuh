@@ -116,6 +116,7 @@ k_scan_1p(In in, Out out, Fin fin, const int64_t* __restrict__ n_dev, unsigned l
     __shared__ int32_t s_v[kScanTile + kScanTile / 32];
     __shared__ long long s_tot, s_excl;
     __shared__ int64_t s_tile;
+    if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);    // while n is read
     const int64_t n = *n_dev;
     const int64_t ntiles = (n + kScanTile - 1) / kScanTile;
     if (ntiles == 0) {
@@ -123,7 +124,6 @@ k_scan_1p(In in, Out out, Fin fin, const int64_t* __restrict__ n_dev, unsigned l
         return;
     }
     for (;;) {
-        if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
         __syncthreads();
         const int64_t t = s_tile;
         __syncthreads();
@@ -175,7 +175,8 @@ k_scan_1p(In in, Out out, Fin fin, const int64_t* __restrict__ n_dev, unsigned l
             if (i < n) out(i, s_v[j + (j >> 5)], rd[k]);
         }
         if (t == ntiles - 1 && threadIdx.x == 0) fin((int64_t)(excl + agg));
-        __syncthreads();
+        if (ntiles <= gridDim.x) break;        // every block has had its one tile
+        if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
     }
 }
 

@@ -387,6 +387,7 @@ k_tree_level(LevelArgs a, int level, DevCounts* dc, unsigned long long* status,
     __shared__ long long s_excl;
     __shared__ int64_t s_tile;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (!COUNT_ONLY && threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
     const int64_t l0 = dc->level_start[level], nl = dc->level_start[level + 1] - l0;
     const int64_t next0 = l0 + nl;
     if (COUNT_ONLY) {
@@ -404,7 +405,6 @@ k_tree_level(LevelArgs a, int level, DevCounts* dc, unsigned long long* status,
         return;
     }
     for (;;) {
-        if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
         __syncthreads();
         const int64_t t = s_tile;
         if (t >= ntiles) break;
@@ -457,7 +457,9 @@ k_tree_level(LevelArgs a, int level, DevCounts* dc, unsigned long long* status,
             }
             dc->level_start[level + 2] = e;
         }
+        if (ntiles <= gridDim.x) break;        // every block has had its one tile
         __syncthreads();
+        if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
     }
 }
 
