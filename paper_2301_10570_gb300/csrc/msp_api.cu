@@ -179,7 +179,7 @@ msp_status msp_create(msp_ctx** out, const msp_config* cfg, int device) {
 msp_status msp_destroy(msp_ctx* c) {
     if (!c) return MSP_OK;
     cudaSetDevice(c->device);
-    msp::DBuf* bufs[] = {&c->keys0, &c->keys1, &c->vals0, &c->vals1, &c->perm, &c->pts,
+    msp::DBuf* bufs[] = {&c->keys0, &c->keys1, &c->vals0, &c->vals1, &c->top_cells, &c->perm, &c->pts,
                          &c->wts, &c->lw, &c->elem_off, &c->leaf_of, &c->nd_level, &c->nd_prefix,
                          &c->nd_first, &c->nd_count, &c->nd_parent, &c->nd_child_first,
                          &c->nd_nchild, &c->nd_sums, &c->nd_ca, &c->nd_cd, &c->nd_arrive, &c->pr_X, &c->pr_Y,

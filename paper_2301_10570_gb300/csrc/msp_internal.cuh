@@ -239,7 +239,7 @@ struct msp_ctx {
     msp::DBuf frame_cap, frame_g2, frame_rc2;
     // sorted points
     msp::DBuf keys0, keys1, vals0, vals1;
-    msp::DBuf perm, pts, wts, lw, elem_off, leaf_of;
+    msp::DBuf top_cells, perm, pts, wts, lw, elem_off, leaf_of;
     // octree (SoA)
     msp::DBuf nd_level, nd_prefix, nd_first, nd_count, nd_parent, nd_child_first, nd_nchild;
     msp::DBuf nd_sums, nd_ca, nd_cd;

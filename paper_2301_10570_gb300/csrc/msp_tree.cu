@@ -175,15 +175,28 @@ __device__ __forceinline__ void put_weights(int64_t j, uint8_t vde, uint8_t vdi,
     lw[j] = make_float2(vde ? log2f((float)vde) : -INFINITY, vdi ? log2f((float)vdi) : -INFINITY);
 }
 
+// the octree's first levels in one block (k_tree_top), and the cells of the last
+constexpr int kTopLevels = 4;
+constexpr int kTopCells = 1 << (3 * kTopLevels);
+
+// points and weights into sorted order; and where the cells of level kTopLevels
+// start: cells[i] = the first point of a cell >= i, i in [0, kTopCells]
 __global__ void k_gather(const int32_t* __restrict__ order, int64_t n, const float* __restrict__ x,
                          const float* __restrict__ y, const float* __restrict__ z,
                          const uint8_t* __restrict__ type, const uint8_t* __restrict__ va,
                          const uint8_t* __restrict__ vde, const uint8_t* __restrict__ vdi,
                          int32_t* __restrict__ perm, float4* __restrict__ pts,
-                         float2* __restrict__ wts, float2* __restrict__ lw) {
+                         float2* __restrict__ wts, float2* __restrict__ lw,
+                         const uint64_t* __restrict__ keys, int32_t* __restrict__ cells) {
+    constexpr int kShift = 3 * (kMortonBits - kTopLevels);
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
          j += (int64_t)gridDim.x * blockDim.x) {
         const int32_t i = order[j];
+        const int cell = (int)(keys[j] >> kShift) & (kTopCells - 1);
+        const int prev = j > 0 ? (int)(keys[j - 1] >> kShift) & (kTopCells - 1) : -1;
+        for (int k = prev + 1; k <= cell; ++k) cells[k] = (int32_t)j;
+        if (j == n - 1)
+            for (int k = cell + 1; k <= kTopCells; ++k) cells[k] = (int32_t)n;
         perm[j] = i;
         pts[j] = make_float4(x[i], y[i], z[i],
                              __uint_as_float(pack_counts(type[i], va[i], vde[i], vdi[i])));
@@ -300,14 +313,20 @@ __device__ __forceinline__ void emit_children(const LevelArgs& a, int64_t i, int
     }
 }
 
-// The root and the levels below it down to level `levels` (at most kTopLevels:
-// one round of at most 64 boxes per level) by one block, a block barrier
-// between levels instead of a launch each.  (A fourth level, four rounds of
-// dependent reads on one SM, took longer than a launch over several.)
-constexpr int kTopLevels = 3;
+// The root and the levels below it down to level `levels` (at most kTopLevels) by
+// one block, a block barrier between levels instead of a launch each.  A box's
+// octants are looked up in cells, where the cells of level kTopLevels start in the
+// keys (k_gather finds them on its way).  Bound by the chain of barriers and of
+// reads of what the level above wrote.  262,144 / 21,013 neurons (serialised,
+// cold), down to level 4: 33 + 14 / 25 + 11 us with a search per box and level,
+// three levels here and the fourth a launch; 12 / 10 us now.
+constexpr int kTopRounds = (1 << (3 * (kTopLevels - 1))) / 128;   // of 128 boxes
 
-__global__ void __launch_bounds__(1024) k_tree_top(LevelArgs a, int levels, DevCounts* dc) {
-    __shared__ int s_off[32];
+__global__ void __launch_bounds__(1024) k_tree_top(LevelArgs a, int levels,
+                                                   const int32_t* __restrict__ cells,
+                                                   DevCounts* dc) {
+    __shared__ int32_t s_b[kTopCells + 1];
+    __shared__ int s_off[32 * kTopRounds];
     __shared__ int s_tot;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
@@ -323,49 +342,72 @@ __global__ void __launch_bounds__(1024) k_tree_top(LevelArgs a, int levels, DevC
         a.child_first[0] = -1;
         a.nchild[0] = 0;
     }
+    // (inside [0, n] also after a sort whose wait gave up, which the host reports)
+    if (a.n > 0)
+        for (int i = threadIdx.x; i <= kTopCells; i += 1024)
+            s_b[i] = (int32_t)min((uint32_t)cells[i], (uint32_t)a.n);
     int64_t l0 = 0, nl = 1;
     for (int l = 0; l < levels; ++l) {
         __syncthreads();
         const int64_t next0 = l0 + nl;
-        int64_t run = 0;
-        for (int64_t base = 0; base < nl; base += 128) {
-            const int64_t k = base + 4 * w + (lane >> 3), i = l0 + k;
-            const bool valid = k < nl;
-            int32_t start, end;
-            octant_split(a, valid, i, l, start, end);
-            const unsigned m = __ballot_sync(0xffffffffu, end > start);
-            if (lane == 0) s_off[w] = __popc(m);
-            __syncthreads();
-            if (w == 0) {
-                const int v = s_off[lane];
-                int inc = v;
+        int32_t start[kTopRounds], end[kTopRounds];
+        unsigned m[kTopRounds];
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int u = __shfl_up_sync(0xffffffffu, inc, o);
-                    if (lane >= o) inc += u;
-                }
-                s_off[lane] = inc - v;
-                if (lane == 31) s_tot = inc;
+        for (int r = 0; r < kTopRounds; ++r) {
+            const int64_t k = 128 * r + 4 * w + (lane >> 3), i = l0 + k;
+            start[r] = end[r] = 0;              // of octant lane & 7
+            if (k < nl && splits(a, i, l, a.count[i])) {
+                const int sh = 3 * (kTopLevels - l - 1);
+                const int cell = (int)(a.prefix[i] << 3) + (lane & 7);
+                start[r] = s_b[cell << sh];
+                end[r] = s_b[(cell + 1) << sh];
             }
-            __syncthreads();
-            const int64_t at = next0 + run + s_off[w];
-            const unsigned grp = (m >> (lane & ~7)) & 0xffu;
-            const bool fits = next0 + run + s_tot <= a.node_cap;
-            if (valid && grp && fits)
-                emit_children(a, i, l, grp, at + __popc(m & ((1u << (lane & ~7)) - 1u)),
-                              at + __popc(m & ((1u << lane) - 1u)), start, end);
-            // the node arrays could not hold the level (a bound that cannot
-            // be exceeded; guarded all the same)
-            if (!fits && threadIdx.x == 0) {
-                dc->overflow |= 16;
-                dc->need_nodes = next0 + run + s_tot;
-            }
-            if (fits) run += s_tot;
-            __syncthreads();
+            m[r] = __ballot_sync(0xffffffffu, end[r] > start[r]);
+            if (lane == 0) s_off[32 * r + w] = __popc(m[r]);
         }
-        if (threadIdx.x == 0) dc->level_start[l + 2] = next0 + run;
+        __syncthreads();
+        if (w == 0) {
+            int v[kTopRounds], sum = 0;
+#pragma unroll
+            for (int r = 0; r < kTopRounds; ++r) {
+                v[r] = s_off[kTopRounds * lane + r];
+                sum += v[r];
+            }
+            int inc = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += u;
+            }
+            int run = inc - sum;
+#pragma unroll
+            for (int r = 0; r < kTopRounds; ++r) {
+                s_off[kTopRounds * lane + r] = run;
+                run += v[r];
+            }
+            if (lane == 31) s_tot = inc;
+        }
+        __syncthreads();
+        // the node arrays could not hold the level (a bound that cannot be
+        // exceeded; guarded all the same)
+        const bool fits = next0 + s_tot <= a.node_cap;
+        if (!fits && threadIdx.x == 0) {
+            dc->overflow |= 16;
+            dc->need_nodes = next0 + s_tot;
+        }
+#pragma unroll
+        for (int r = 0; r < kTopRounds; ++r) {
+            const int64_t k = 128 * r + 4 * w + (lane >> 3);
+            const int64_t at = next0 + s_off[32 * r + w];
+            const unsigned grp = (m[r] >> (lane & ~7)) & 0xffu;
+            if (k < nl && grp && fits)
+                emit_children(a, l0 + k, l, grp, at + __popc(m[r] & ((1u << (lane & ~7)) - 1u)),
+                              at + __popc(m[r] & ((1u << lane) - 1u)), start[r], end[r]);
+        }
+        const int64_t made = fits ? s_tot : 0;
+        if (threadIdx.x == 0) dc->level_start[l + 2] = next0 + made;
         l0 = next0;
-        nl = run;
+        nl = made;
     }
 }
 
@@ -642,6 +684,7 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
     float2* lw = c.lw.ensure<float2>(nn);
     int32_t* eoff = c.elem_off.ensure<int32_t>(nn + 1);
     int32_t* leaf_of = c.leaf_of.ensure<int32_t>(nn);
+    int32_t* cells = c.top_cells.ensure<int32_t>(kTopCells + 1);
     const int B = 256;
     const int G = grid_for(n, B, (int64_t)c.sm_count * 16);
     // box centres: in the domain's frame, or (frames) in each network's own
@@ -738,7 +781,7 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
             MSP_LAUNCH("morton");
         }
         radix_sort_dev(c, k0, v0, k1, v1, nullptr, n, 3 * kMortonBits, s);
-        k_gather<<<G, B, 0, s>>>(v0, n, x, y, z, type, va, vde, vdi, perm, pts, wts, lw);
+        k_gather<<<G, B, 0, s>>>(v0, n, x, y, z, type, va, vde, vdi, perm, pts, wts, lw, k0, cells);
         MSP_LAUNCH("gather");
         // element offsets: exclusive prefix of the vacant axonal counts
         scan_launch(c, ScanU8{va}, ScanStore{eoff}, ScanTotalAfter{&dc->n_elem, eoff, &dc->n},
@@ -820,7 +863,7 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
         for (int l = top; l < L; ++l) nw += words(l);
         unsigned long long* st = c.lv_status.ensure<unsigned long long>((size_t)std::max<int64_t>(nw, 1));
         if (nw > 0) MSP_CUDA(cudaMemsetAsync(st, 0, (size_t)nw * sizeof(unsigned long long), s));
-        k_tree_top<<<1, 1024, 0, s>>>(la, top, dc);
+        k_tree_top<<<1, 1024, 0, s>>>(la, top, cells, dc);
         MSP_LAUNCH("tree_top");
         for (int l = top; l < L; ++l) {
             const int64_t tiles = words(l) - 1;
