@@ -607,7 +607,16 @@ msp_status msp_export_expansions(msp_ctx* c, float* A, float* M, float* B, int64
         if (!c->attraction_done) throw msp::Error(MSP_ERR_NOT_BUILT, "no attraction");
         MSP_CUDA(cudaDeviceSynchronize());
         size_t m = (size_t)c->exp_nodes * 2 * c->cfg.p * c->cfg.p * c->cfg.p * sizeof(float);
-        if (A && m) MSP_CUDA(cudaMemcpy(A, c->expA.p, m, cudaMemcpyDeviceToHost));
+        if (A && m) {
+            // on the device a coefficient's channels lie side by side
+            const size_t p3 = (size_t)c->cfg.p * c->cfg.p * c->cfg.p;
+            std::vector<float> a(m / sizeof(float));
+            MSP_CUDA(cudaMemcpy(a.data(), c->expA.p, m, cudaMemcpyDeviceToHost));
+            for (size_t e = 0; e < (size_t)c->exp_nodes; ++e)
+                for (size_t i = 0; i < p3; ++i)
+                    for (size_t ch = 0; ch < 2; ++ch)
+                        A[(e * 2 + ch) * p3 + i] = a[(e * p3 + i) * 2 + ch];
+        }
         if (M && m) MSP_CUDA(cudaMemcpy(M, c->expM.p, m, cudaMemcpyDeviceToHost));
         if (B && m) MSP_CUDA(cudaMemcpy(B, c->expB.p, m, cudaMemcpyDeviceToHost));
         if (first_node) *first_node = c->exp_first;

@@ -320,7 +320,9 @@ k_trav_depth(TravArgs a, int d, unsigned long long* status, int64_t timeout_bit)
 
 // ---------------------------------------------------------------------------
 // a6: Hermite coefficients of the dendritic weights (Eq. 7) and axon moments
-// M_beta = sum_t a_t ((t - c_A)/sigma)^beta, per channel, one block per box
+// M_beta = sum_t a_t ((t - c_A)/sigma)^beta, per channel, one block per box.
+// A holds a coefficient's two channels side by side (the translations read them as
+// one 8-byte pair), M and B channel after channel.
 // ---------------------------------------------------------------------------
 constexpr int kP2MThreads = 128;
 constexpr int kP2MChunk = 32;
@@ -393,7 +395,7 @@ k_p2m(int64_t first_node, float inv_sigma, const float4* __restrict__ pts,
         if (idx >= 4 * P3) continue;
         const int which = idx / P3, a = idx % P3;
         if (which < 2)
-            A[(e * 2 + which) * P3 + a] = acc[r] * c_inv_fact[a / P2] *
+            A[(e * P3 + a) * 2 + which] = acc[r] * c_inv_fact[a / P2] *
                                           c_inv_fact[(a / P) % P] * c_inv_fact[a % P];
         else
             M[(e * 2 + which - 2) * P3 + a] = acc[r];
@@ -485,7 +487,7 @@ k_m2l_seg(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nse
 #pragma unroll
             for (int k = 0; k < NA; ++k) {
                 const int e = lane + 32 * k;
-                if (e < 2 * P3) s0[e] = an[k];
+                if (e < 2 * P3) s0[(e & 1) * P3 + (e >> 1)] = an[k];
             }
             if (i + 1 < i1) {
                 qn = list[i + 1];
@@ -590,10 +592,10 @@ k_m2l_seg(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nse
 // same order; B(X) adds the pairs of each quarter and then the quarters.  Blocks
 // take four targets and leave (the numbers of pairs per target differ widely: a
 // grid of resident blocks striding over the targets took 0.93 ms).
-// 4.9 M pairs of 65,536 neurons: 1.47 ms in the general kernel, 0.72 ms here
-// (0.74 with half a warp a pair, each lane's Hermite functions for one column; 1.47
-// with unpadded rows: bank conflicts).  Bound by instruction issue: 48 paired FMAs
-// of a pair's 95 instructions, the rest Hermite functions and staging.
+// 4.9 M pairs of 65,536 neurons: 1.47 ms in the general kernel, 0.67 ms here (0.72
+// with the channels' coefficients read one by one, 0.74 with half a warp a pair,
+// 1.47 with unpadded rows: bank conflicts).  Bound by instruction issue: 48 paired
+// FMAs of a pair's 90 instructions, the rest Hermite functions and staging.
 __global__ void __launch_bounds__(kM2LWarps * 32, 4)
 k_m2l_seg4(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nseg_dev,
            const int32_t* __restrict__ list, int64_t exp_first, float inv_sigma,
@@ -651,12 +653,12 @@ k_m2l_seg4(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ ns
             q = list[i];
             const int32_t Y = pY[q];
             d = cd[Y];
-            const float* Ay = A + (Y - exp_first) * 2 * P3 + r;
+            const float2* Ay = reinterpret_cast<const float2*>(A) + (Y - exp_first) * P3 + r;
 #pragma unroll
             for (int j = 0; j < 2; ++j)
 #pragma unroll
                 for (int k = 0; k < P; ++k)
-                    v[j][k] = make_float2(Ay[16 * k + 8 * j], Ay[P3 + 16 * k + 8 * j]);
+                    v[j][k] = Ay[16 * k + 8 * j];
         };
         load(i0 + quarter);
         for (int32_t ib = i0; ib < i1; ib += 4) {

@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kGemmThreads) k_m2l_gemm(GemmArgs a) {
             float v = 0.f;
             if (pi < npair) {
                 const int64_t ey = a.pY[sq[pi]] - a.exp_first;
-                v = a.A[(ey * 2 + ch) * p3 + al];
+                v = a.A[(ey * p3 + al) * 2 + ch];
             }
             As[i] = v;
         }

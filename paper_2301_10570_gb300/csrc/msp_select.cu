@@ -57,9 +57,9 @@ __device__ float warp_far_w(const Tree& tr, const Exps& ex, int32_t X, int32_t Y
         if (2 * p - 2 >= 1) h[1] = 2.f * x * h0;
         for (int k = 1; k < 2 * p - 2; ++k) h[k + 1] = 2.f * x * h[k] - 2.f * (float)k * h[k - 1];
     }
-    const float* Ag = ex.A + ((int64_t)(Y - ex.first) * 2 + ch) * p3;
+    const float* Ag = ex.A + (int64_t)(Y - ex.first) * p3 * 2 + ch;
     const float* Mg = ex.M + ((int64_t)(X - ex.first) * 2 + ch) * p3;
-    for (int i = lane; i < p3; i += 32) b0[i] = Ag[i];
+    for (int i = lane; i < p3; i += 32) b0[i] = Ag[2 * i];
     __syncwarp();
     for (int o = lane; o < p3; o += 32) {
         int c0 = o / p2, r = o - c0 * p2;
