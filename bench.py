@@ -49,9 +49,10 @@ FP32_PER_SM_CLK = 128
 FP32_PER_INTERACTION = 8
 # algorithmic DRAM bytes of one near-field launch: per neuron its packed point
 # (16 B) and log-weights (8 B) read once and u (4 B) written; per near-field
-# pair its source range (8 B), list entry (4 B) and W slot (8 B)
+# pair its source range (8 B), list entry (4 B), W slot (8 B) and pair table
+# entry (16 B)
 NF_BYTES_PER_NEURON = 28
-NF_BYTES_PER_PAIR = 20
+NF_BYTES_PER_PAIR = 36
 # the fastest plan with translated pairs found for the 1M clustered network
 # (profiles/autotune_clustered_1m.md): timed beside the headline
 FMM_TRANSLATED_PLAN = dict(leaf_capacity=64, cutoff=3.5, rho_max=0.35, p=6, m2l_min_pairs=256)

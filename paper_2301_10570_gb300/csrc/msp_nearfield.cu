@@ -19,8 +19,8 @@
 // The per-target sums of the warps are added in a fixed order, so u is
 // reproducible run to run.  Per pair, the warp reduces the box-pair
 // attraction W(X,Y) = sum_t a_t sum_s w_s K(t,s) of each channel in single
-// precision into a per-pair slot; a second kernel widens it into the double
-// precision pair table.
+// precision into a per-pair slot; when its segment is complete the block writes
+// the slots to the double-FP32 pair table.
 //
 // Arithmetic.  With k = log2(e)/sigma^2 and hats denoting sqrt(k)(position-c)
 // for the geometric centre c of X,
@@ -74,7 +74,7 @@ struct NFArgs {
     float2* w32;                 // per near-field pair (list order): W of E and I
     unsigned long long* work;
     const uint8_t* small;        // segments that k_near_small takes, or null: none
-    float4* pw;                  // the pair table (k_near_small's results)
+    float4* pw;                  // the pair table
 };
 
 __device__ __forceinline__ void nf_add_u(const NFArgs& a, int32_t t, float v) {
