@@ -592,9 +592,10 @@ k_m2l_seg(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nse
 // same order; B(X) adds the pairs of each quarter and then the quarters.  Blocks
 // take four targets and leave (the numbers of pairs per target differ widely: a
 // grid of resident blocks striding over the targets took 0.93 ms).
-// 4.9 M pairs of 65,536 neurons: 1.47 ms in the general kernel, 0.67 ms here (0.72
-// with the channels' coefficients read one by one, 0.74 with half a warp a pair,
-// 1.47 with unpadded rows: bank conflicts).  Bound by instruction issue: 48 paired
+// 4.9 M pairs of 65,536 neurons: 1.47 ms in the general kernel, 0.58 ms here (0.67
+// with list entry, source box and coefficients read one pair ahead, 0.72 with the
+// channels' coefficients read one by one too, 0.74 with half a warp a pair, 1.47
+// with unpadded rows: bank conflicts).  Bound by instruction issue: 48 paired
 // FMAs of a pair's 90 instructions, the rest Hermite functions and staging.
 __global__ void __launch_bounds__(kM2LWarps * 32, 4)
 k_m2l_seg4(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ nseg_dev,
@@ -639,19 +640,20 @@ k_m2l_seg4(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ ns
 #pragma unroll
             for (int k = 0; k < P; ++k) acc[j][k] = make_float2(0.f, 0.f);
         }
-        // the next pair's list entry, centre and coefficients are loaded
-        // while the current pair is translated (a chain of dependent loads)
-        int32_t q = 0;
+        // the next pair's centre and coefficients are loaded while the current
+        // pair is translated, its source box a pair earlier and the list entry
+        // two (a chain of dependent reads longer than a pair's work)
+        auto entry = [&](int32_t i) { return (uint32_t)i < (uint32_t)i1 ? list[i] : -1; };
+        auto source = [&](int32_t q) { return q >= 0 ? pY[q] : -1; };
+        int32_t q = entry(i0 + quarter), q1 = entry(i0 + 4 + quarter), q2 = entry(i0 + 8 + quarter);
         float4 d = a4;
         float2 v[2][P];
-        auto load = [&](int32_t i) {
+        auto load = [&](int32_t Y) {
 #pragma unroll
             for (int j = 0; j < 2; ++j)
 #pragma unroll
                 for (int k = 0; k < P; ++k) v[j][k] = make_float2(0.f, 0.f);
-            if (i >= i1) return;
-            q = list[i];
-            const int32_t Y = pY[q];
+            if (Y < 0) return;
             d = cd[Y];
             const float2* Ay = reinterpret_cast<const float2*>(A) + (Y - exp_first) * P3 + r;
 #pragma unroll
@@ -660,9 +662,10 @@ k_m2l_seg4(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ ns
                 for (int k = 0; k < P; ++k)
                     v[j][k] = Ay[16 * k + 8 * j];
         };
-        load(i0 + quarter);
-        for (int32_t ib = i0; ib < i1; ib += 4) {
-            const bool in = ib + quarter < i1;
+        load(source(q));
+        int32_t y1 = source(q1);
+        for (int32_t ib = i0; (uint32_t)ib < (uint32_t)i1; ib += 4) {
+            const bool in = q >= 0;
             const int32_t qc = q;
             float H[8];
             const float4 dc = d;
@@ -680,7 +683,11 @@ k_m2l_seg4(const int32_t* __restrict__ seg_first, const int64_t* __restrict__ ns
             for (int j = 0; j < 2; ++j)
 #pragma unroll
                 for (int o = 0; o < P; ++o) t0[20 * o + r + 8 * j] = apply(v[j], o);
-            load(ib + 4 + quarter);
+            load(y1);
+            q = q1;
+            y1 = source(q2);
+            q1 = q2;
+            q2 = entry(ib + 12 + quarter);
             __syncwarp();
             // over a1: column (b0, a2) -> [b0][b1][a2]
             hermite_row((a4.y - dc.y) * inv_sigma, H, 2 * P - 2);
