@@ -596,10 +596,12 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : (NW == 8 ? 3 : 1)) k_ne
 // the general kernel does (source pair by source pair, group by group), so it
 // is the same bit for bit.  Bound by the latency of the points' reads.  65,536
 // neurons with translated pairs (4.2 M near-field pairs of 2.6 points a leaf):
-// 1020 us and 58 for the pair slots in the general kernel, 234 us here and 14 in
-// the general kernel for the few segments that are not small.
+// 1020 us and 58 for the pair slots in the general kernel, 183 us here and 14 in
+// the general kernel for the few segments that are not small.  64 registers and 32
+// warps per SM in spite of 124 bytes of spills: 1070 us a step, 1100 with 72 or 79
+// registers, 1087 with 48; blocks of 8 warps striding over the segments 1128.
 constexpr int kNFSmall = 8;
-constexpr int kNFSmallWarps = 8;
+constexpr int kNFSmallWarps = 4;
 
 template <int R>
 __device__ __forceinline__ void nf_small_segment(const NFArgs& a, const int32_t* tl, int nt, int g,
@@ -710,7 +712,7 @@ __device__ __forceinline__ void nf_small_segment(const NFArgs& a, const int32_t*
     }
 }
 
-__global__ void __launch_bounds__(kNFSmallWarps * 32, 3) k_near_small(NFArgs a) {
+__global__ void __launch_bounds__(kNFSmallWarps * 32, 8) k_near_small(NFArgs a) {
     __shared__ int32_t s_tl[kNFSmallWarps][kNFSmall + 4];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nseg = *a.nseg;
@@ -813,7 +815,6 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
     if (nseg_cap <= 0 || nlist_cap <= 0) return;
     const msp_config& cfg = c.cfg;
     float2* w32 = c.nf_w32.ensure<float2>((size_t)nlist_cap);
-    const int gl = (int)std::max<int64_t>(1, (int64_t)c.sm_count * 8);
     // small leaves: most segments go to k_near_small
     int max_cap = cfg.leaf_capacity;
     if (c.frame_level > 0 && c.frame_plans)
@@ -864,7 +865,9 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
     a.small = small;
     a.pw = c.pr_w.get<float4>();
     if (small) {
-        k_near_small<<<gl, kNFSmallWarps * 32, 0, s>>>(a);
+        // a warp per segment, handed out by the hardware
+        const int64_t blocks = (nseg_cap + kNFSmallWarps - 1) / kNFSmallWarps;
+        k_near_small<<<(int)std::min<int64_t>(blocks, 1 << 30), kNFSmallWarps * 32, 0, s>>>(a);
         MSP_LAUNCH("near_small");
     }
     // one block per segment (blocks past the device count return at once), or
