@@ -155,8 +155,9 @@ msp_status msp_destroy(msp_ctx *ctx);
  * The inputs are read during the call's stream work only; the context keeps
  * its own sorted copy.  The octree depends on the positions only: when n and
  * the positions equal those of the context's last build (a checksum of every
- * coordinate's bits, read back: one more synchronisation), the sorted order
- * and the octree are kept and only the counts and aggregates are refreshed.
+ * coordinate's bits, read back: one more synchronisation unless the last build
+ * kept them too), the sorted order and the octree are kept and only the counts
+ * and aggregates are refreshed.
  * Synchronous (the per-level node counts are read back).  n may be 0.  Errors: MSP_ERR_INVALID_ARG (n < 0, n > 2^31-2, null
  * pointer with n > 0, a position outside [origin, origin + side) or not
  * finite: the boxes of the tree must contain their points), MSP_ERR_OOM
