@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "msp_hostdev.cuh"
 #include "msp_scan.cuh"
 
 namespace msp {
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(kTravTile) k_trav_top(TravArgs a, int64_t n, i
         if (nq == 0) {
             if (threadIdx.x == 0) trav_empty(dc, d);
         } else {
-            trav_tile(a, d, 0, q0, nq, next0, true, [](const int*, long long (&ex)[4]) {
+            trav_tile(a, d, 0, q0, nq, next0, true, [](const int (&)[4], long long (&ex)[4]) {
                 ex[0] = ex[1] = ex[2] = ex[3] = 0;
                 __syncthreads();
             });
@@ -276,12 +277,12 @@ __global__ void __launch_bounds__(kTravTile) k_trav_top(TravArgs a, int64_t n, i
     }
 }
 
-// one depth; status: a tile counter and two words per tile (children and
-// split pairs, near-field and far pairs, 31 bits each), zero on entry
+// one depth; status: a tile counter and kTravWords words per tile (trav_pack),
+// zero on entry
 __global__ void __launch_bounds__(kTravTile)
 k_trav_depth(TravArgs a, int d, unsigned long long* status, int64_t timeout_bit) {
     __shared__ int64_t s_tile;
-    __shared__ long long s_ex[2];
+    __shared__ long long s_ex[kTravWords];
     DevCounts* dc = a.dc;
     if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
     const int64_t q0 = dc->depth_start[d], next0 = dc->depth_start[d + 1], nq = next0 - q0;
@@ -294,23 +295,21 @@ k_trav_depth(TravArgs a, int d, unsigned long long* status, int64_t timeout_bit)
         __syncthreads();
         const int64_t t = s_tile;
         if (t >= ntiles) break;
-        trav_tile(a, d, t, q0, nq, next0, t == ntiles - 1, [&](const int* tot, long long (&ex)[4]) {
+        trav_tile(a, d, t, q0, nq, next0, t == ntiles - 1,
+                  [&](const int (&tot)[4], long long (&ex)[4]) {
+            long long e[kTravWords];
             if (threadIdx.x < 32) {
-                const long long own[2] = {(long long)tot[0] << 31 | tot[1],
-                                          (long long)tot[2] << 31 | tot[3]};
-                long long e[2];
-                look_back<2>(status + 1, t, own, e, &dc->overflow, timeout_bit, kSpinLimit);
-                if (threadIdx.x == 0) {
-                    s_ex[0] = e[0];
-                    s_ex[1] = e[1];
-                }
+                long long own[kTravWords];
+                trav_pack(tot, own);
+                look_back<kTravWords>(status + 1, t, own, e, &dc->overflow, timeout_bit, kSpinLimit);
+                if (threadIdx.x == 0)
+#pragma unroll
+                    for (int k = 0; k < kTravWords; ++k) s_ex[k] = e[k];
             }
             __syncthreads();
-            const long long m = (1ll << 31) - 1;
-            ex[0] = s_ex[0] >> 31;
-            ex[1] = s_ex[0] & m;
-            ex[2] = s_ex[1] >> 31;
-            ex[3] = s_ex[1] & m;
+#pragma unroll
+            for (int k = 0; k < kTravWords; ++k) e[k] = s_ex[k];
+            trav_unpack(e, ex);
         });
         if (ntiles <= gridDim.x) break;        // every block has had its one tile
         __syncthreads();
@@ -1009,7 +1008,7 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
     };
     const int dtop = std::min(D, kTopDepths);
     int64_t nw = 0;
-    for (int d = dtop; d < D; ++d) nw += 1 + 2 * tiles_at(d);
+    for (int d = dtop; d < D; ++d) nw += 1 + kTravWords * tiles_at(d);
     unsigned long long* st = c.tv_status.ensure<unsigned long long>((size_t)std::max<int64_t>(nw, 1));
     if (nw > 0) MSP_CUDA(cudaMemsetAsync(st, 0, (size_t)nw * sizeof(unsigned long long), s));
     k_trav_top<<<1, kTravTile, 0, s>>>(ta, n, dtop);
@@ -1019,7 +1018,7 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
         k_trav_depth<<<(unsigned)std::min<int64_t>(tiles, (int64_t)c.sm_count * 6), kTravTile, 0, s>>>(
             ta, d, st, kScanTimeoutBit);
         MSP_LAUNCH("trav_depth");
-        st += 1 + 2 * tiles;
+        st += 1 + kTravWords * tiles;
     }
     // the near-field list grouped by target leaf (at most one segment per box)
     radix_sort_dev(c, pk0, pv0, pk1, pv1, &dc->n_p2p, cap, xbits, s);

@@ -1,0 +1,36 @@
+// msp_hostdev.cuh -- arithmetic of the kernels that is also run on the host by
+// the tests: plain C++ without CUDA headers.
+#pragma once
+
+#include <cstdint>
+
+#ifdef __CUDACC__
+#define MSP_HD __host__ __device__ __forceinline__
+#else
+#define MSP_HD inline
+#endif
+
+namespace msp {
+
+// What a traversal tile counts (children, split, near-field and far pairs) as
+// the words of its look-back, which adds them modulo 2^62.  The pairs of a
+// depth lie in the pair table (at most 2^31 - 1), so two of their counts share a
+// word; a depth's children may be 64 times as many and have a word of their own:
+// their number has to be exact beyond the table too, or the depths that do not
+// fit would not be seen.
+constexpr int kTravWords = 3;
+
+MSP_HD void trav_pack(const int (&tot)[4], long long (&w)[kTravWords]) {
+    w[0] = tot[0];
+    w[1] = (long long)tot[1] << 31 | tot[2];
+    w[2] = tot[3];
+}
+
+MSP_HD void trav_unpack(const long long (&w)[kTravWords], long long (&ex)[4]) {
+    ex[0] = w[0];
+    ex[1] = w[1] >> 31;
+    ex[2] = w[1] & ((1ll << 31) - 1);
+    ex[3] = w[2];
+}
+
+}  // namespace msp
