@@ -87,8 +87,7 @@ struct BuildEnd {
     DevCounts* dc;
     bool graph;              // otherwise nothing to do (the host looks)
     // octree kept: the positions must be those of the build that made it
-    // (checksum ref) and the arrays that build's (stamp gen), or the step halts;
-    // octree built anew: no capture holds the stamp it leaves
+    // (checksum ref) and the arrays that build's (stamp gen), or the step halts
     bool keep;
     uint64_t ref, gen;
     // more elements than the selection's buffers hold leave the step with no
@@ -96,8 +95,7 @@ struct BuildEnd {
     int64_t elem_cap;
     __device__ void operator()() const {
         if (!graph) return;
-        if (!keep) dc->tree_gen = ~0ull;
-        else if (dc->pos_sum != ref || dc->tree_gen != gen) dc->bad_pos = 1;
+        if (keep && (dc->pos_sum != ref || dc->tree_gen != gen)) dc->bad_pos = 1;
         if (dc->n_elem > elem_cap) {
             dc->halt |= kHaltElements;
             dc->n_elem = 0;
@@ -105,12 +103,20 @@ struct BuildEnd {
     }
 };
 
+// The first kernel of a build that makes the octree anew, and the last moment at
+// which the arrays of the one before are whole: no capture holds the stamp left
+// here, and a build that fails later on leaves it.
+__device__ __forceinline__ void drop_stamp(DevCounts* dc) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) dc->tree_gen = ~0ull;
+}
+
 // keys; a position outside [origin, origin + side) or not finite is counted
 // (the build then fails: the tree's boxes must contain their points)
 __global__ void k_morton(const float* __restrict__ x, const float* __restrict__ y,
                          const float* __restrict__ z, int64_t n, float ox, float oy, float oz,
                          float side, float scale, uint64_t* __restrict__ keys,
-                         int32_t* __restrict__ vals, int64_t* __restrict__ bad) {
+                         int32_t* __restrict__ vals, DevCounts* dc) {
+    drop_stamp(dc);
     bool any_bad = false;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -123,7 +129,7 @@ __global__ void k_morton(const float* __restrict__ x, const float* __restrict__ 
         vals[i] = (int32_t)i;
     }
     if (__any_sync(0xffffffffu, any_bad) && (threadIdx.x & 31) == 0)
-        atomicAdd(reinterpret_cast<unsigned long long*>(bad), 1ull);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&dc->bad_pos), 1ull);
 }
 
 // Keys of independent networks in local frames.  Neuron i belongs to the
@@ -138,7 +144,8 @@ __global__ void k_morton_frames(const float* __restrict__ x, const float* __rest
                                 const float* __restrict__ z, int64_t n,
                                 const int64_t* __restrict__ off, int64_t nf, int L0, float cs,
                                 float scale, uint64_t* __restrict__ keys,
-                                int32_t* __restrict__ vals, int64_t* __restrict__ bad) {
+                                int32_t* __restrict__ vals, DevCounts* dc) {
+    drop_stamp(dc);
     const int sh = kMortonBits - L0;
     const uint32_t qmax = (1u << sh) - 1u;
     const int64_t G = 1ll << (L0 - 1);
@@ -161,7 +168,7 @@ __global__ void k_morton_frames(const float* __restrict__ x, const float* __rest
         vals[i] = (int32_t)i;
     }
     if (__any_sync(0xffffffffu, any_bad) && (threadIdx.x & 31) == 0)
-        atomicAdd(reinterpret_cast<unsigned long long*>(bad), 1ull);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&dc->bad_pos), 1ull);
 }
 
 __device__ __forceinline__ uint32_t pack_counts(uint8_t type, uint8_t va, uint8_t vde, uint8_t vdi) {
@@ -776,11 +783,11 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
             k_morton_frames<<<G, B, 0, s>>>(x, y, z, n, c.frame_off.get<int64_t>(),
                                             (int64_t)c.frame_off_host.size() - 1, c.frame_level,
                                             ldexpf(cfg.side, -c.frame_level), c.morton_scale, mk,
-                                            mv, &dc->bad_pos);
+                                            mv, dc);
             MSP_LAUNCH("morton_frames");
         } else {
             k_morton<<<G, B, 0, s>>>(x, y, z, n, cfg.origin[0], cfg.origin[1], cfg.origin[2],
-                                     cfg.side, c.morton_scale, mk, mv, &dc->bad_pos);
+                                     cfg.side, c.morton_scale, mk, mv, dc);
             MSP_LAUNCH("morton");
         }
         radix_sort_dev(c, k0, v0, k1, v1, nullptr, n, 3 * kMortonBits, s);
