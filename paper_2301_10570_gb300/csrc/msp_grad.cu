@@ -454,6 +454,18 @@ void attraction_grad(msp_ctx& c, const uint8_t* type, const uint8_t* va, const u
     const int2* src = c.nf_src.get<int2>();
     const float4* pts = c.pts.get<float4>();
     const int nb = (int)std::min<int64_t>(std::max<int64_t>(c.n_nodes, 1), 1 << 30);
+    // every input is gathered before an output is written: an output may be g
+    const bool adjoint = gE || gI;
+    const int32_t* off = nullptr;
+    float4* pt = nullptr;
+    float* pg = nullptr;
+    if (adjoint) {
+        off = ps_offsets(c, fl, s);
+        pt = c.gr_pt.ensure<float4>((size_t)n);
+        pg = c.gr_tmp.ensure<float>((size_t)n);
+        k_grad_pack<<<G, B, 0, s>>>(n, fl, off, perm, pts, g, pt, pg);
+        MSP_LAUNCH("grad_pack");
+    }
     if (u || dud) {
         if (u) MSP_CUDA(cudaMemsetAsync(u, 0, (size_t)n * sizeof(float), s));
         if (dud) MSP_CUDA(cudaMemsetAsync(dud, 0, (size_t)n * sizeof(float), s));
@@ -461,14 +473,9 @@ void attraction_grad(msp_ctx& c, const uint8_t* type, const uint8_t* va, const u
                                                     ncount, pts, wt, fl, perm, sqk, dscale, u, dud);
         MSP_LAUNCH("grad_forward");
     }
-    if (gE || gI) {
+    if (adjoint) {
         if (gE) MSP_CUDA(cudaMemsetAsync(gE, 0, (size_t)n * sizeof(float), s));
         if (gI) MSP_CUDA(cudaMemsetAsync(gI, 0, (size_t)n * sizeof(float), s));
-        const int32_t* off = ps_offsets(c, fl, s);
-        float4* pt = c.gr_pt.ensure<float4>((size_t)n);
-        float* pg = c.gr_tmp.ensure<float>((size_t)n);
-        k_grad_pack<<<G, B, 0, s>>>(n, fl, off, perm, pts, g, pt, pg);
-        MSP_LAUNCH("grad_pack");
         k_grad_adjoint<<<nb, kPsWarps * 32, 0, s>>>(segf, &dc->nseg, order, list, pX, src, nfirst,
                                                     ncount, n, pts, PsPacked{pt, off}, pg, perm,
                                                     sqk, gE, gI);
