@@ -586,7 +586,8 @@ msp_status msp_philox(int64_t n, const uint32_t *ctr, const uint32_t *key, uint3
  *   x,y,z,type,vac_*     device inputs as for msp_build_tree (caller order)
  *   sigma                kernel width
  *   u                    device output, n floats: u(t) of the neuron's own
- *                        channel if vac_axon > 0, else 0
+ *                        channel if vac_axon > 0, else 0; it may lie over
+ *                        an input (one launch more, which copies the inputs)
  *   stream               cudaStream_t as void* (NULL = legacy default stream)
  * It allocates nothing and needs no context.  Its scratch is one fixed
  * file-scope device array of MSP_NOALLOC_MAX_N * 24 bytes that every GPU

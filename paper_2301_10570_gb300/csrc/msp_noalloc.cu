@@ -27,8 +27,9 @@ static_assert(kNaPtsBytes + kNaListBytes +
               "the scratch holds the packed copy, the target lists, their counts and the boxes");
 
 // The scratch: the packed neurons (float4), the target lists (int32), their
-// counts and the source tiles' boxes of up to MSP_NOALLOC_MAX_N neurons.  Shared by every call; everything in it is rewritten before it is
-// read, so nothing left by an earlier call is ever used.
+// counts and the source tiles' boxes of up to MSP_NOALLOC_MAX_N neurons.  Shared
+// by every call; everything in it is rewritten before it is read, so nothing left
+// by an earlier call is ever used.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaBytes];
 
 // Device address of g_noalloc_scratch, looked up once per device and CUDA
@@ -94,6 +95,18 @@ bool on_device(const void* p, int dev) {
     return (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) && a.device == dev;
 }
 
+// the packed copy of the caller's arrays, for calls whose u lies over one of them
+__global__ void k_dir_pack(int64_t n, msp::DirRaw src, float4* __restrict__ pts) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < n) pts[i] = src.get(i);
+}
+
+// whether [a, a + na) and [b, b + nb) have a byte in common
+bool meets(const void* a, int64_t na, const void* b, int64_t nb) {
+    const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
+    return pa < pb + (uintptr_t)nb && pb < pa + (uintptr_t)na;
+}
+
 }  // namespace
 
 extern "C" msp_status msp_direct_noalloc(int64_t n, const float* x, const float* y, const float* z,
@@ -135,17 +148,30 @@ extern "C" msp_status msp_direct_noalloc(int64_t n, const float* x, const float*
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const float k2 = (float)(1.4426950408889634 / (sigma * sigma));
     const msp::DirRaw src{x, y, z, type, vac_axon, vac_dend_e, vac_dend_i};
-    int launches = 1;
-    if (n <= msp::kDirSmallN) {
-        msp::k_dir_small<false><<<(unsigned)((n + 31) / 32), msp::kDirSmallWarps * 32, 0, s>>>(
-            n, src, k2, nullptr, 0, nullptr, u);
+    unsigned char* sc = static_cast<unsigned char*>(base);
+    float4* P = reinterpret_cast<float4*>(sc);
+    int32_t* list = reinterpret_cast<int32_t*>(sc + kNaPtsBytes);
+    const msp::DirScratch t(reinterpret_cast<int32_t*>(sc + kNaPtsBytes + kNaListBytes), n);
+    // u may lie over an input: every input is packed first then, since the
+    // kernels read them while they write u
+    const bool over = meets(u, n * 4, x, n * 4) || meets(u, n * 4, y, n * 4) ||
+                      meets(u, n * 4, z, n * 4) || meets(u, n * 4, type, n) ||
+                      meets(u, n * 4, vac_axon, n) || meets(u, n * 4, vac_dend_e, n) ||
+                      meets(u, n * 4, vac_dend_i, n);
+    const unsigned small = (unsigned)((n + 31) / 32), threads = msp::kDirSmallWarps * 32;
+    int launches = n <= msp::kDirSmallN ? 1 : 3;
+    if (over) {
+        ++launches;
+        k_dir_pack<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, src, P);
+        const msp::DirPacked packed{P};
+        if (n <= msp::kDirSmallN)
+            msp::k_dir_small<false><<<small, threads, 0, s>>>(n, packed, k2, nullptr, 0, nullptr, u);
+        else
+            msp::dir_launch_tiles<false>(n, packed, nullptr, P, list, t, k2, nullptr, 0, nullptr, u, s);
+    } else if (n <= msp::kDirSmallN) {
+        msp::k_dir_small<false><<<small, threads, 0, s>>>(n, src, k2, nullptr, 0, nullptr, u);
     } else {
-        unsigned char* sc = static_cast<unsigned char*>(base);
-        float4* P = reinterpret_cast<float4*>(sc);
-        int32_t* list = reinterpret_cast<int32_t*>(sc + kNaPtsBytes);
-        const msp::DirScratch t(reinterpret_cast<int32_t*>(sc + kNaPtsBytes + kNaListBytes), n);
         msp::dir_launch_tiles<false>(n, src, P, P, list, t, k2, nullptr, 0, nullptr, u, s);
-        launches = 3;
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) {

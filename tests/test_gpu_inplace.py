@@ -33,3 +33,32 @@ def test_derivatives_written_over_g(shared):
     for k in want:
         assert torch.equal(got[k], want[k]), k
     ctx.close()
+
+
+# one block, the largest size of the one-launch kernel and the next, both sides of
+# the change of targets per lane
+@pytest.mark.parametrize("n", [31, 1021, 8192, 8193, 40_001])
+@pytest.mark.parametrize("over", ["x", "z", "between"])
+def test_all_pairs_written_over_the_positions(n, over):
+    w = W.uniform_cube(n, 625.0 * n ** (1 / 3), seed=n)
+    w.vac_axon[::5] = 0
+    pos, t, a, e, i = msp.to_device(w)
+    want = msp.direct_noalloc(pos, t, a, e, i, w.params["sigma"])
+    work = pos.clone()
+    flat = work.view(-1)
+    out = {"x": work[0], "z": work[2], "between": flat[n // 2:n // 2 + n]}[over]
+    got = msp.direct_noalloc(work, t, a, e, i, w.params["sigma"], out=out)
+    assert got.data_ptr() == out.data_ptr() and torch.equal(got, want)
+
+
+def test_all_pairs_written_over_the_counts():
+    n = 3001
+    w = W.uniform_cube(n, 9000.0, seed=5)
+    pos, t, a, e, i = msp.to_device(w)
+    want = msp.direct_noalloc(pos, t, a, e, i, w.params["sigma"])
+    room = torch.empty(n, dtype=torch.float32, device="cuda")
+    counts = room.view(torch.uint8)[:4 * n].view(4, n)      # the four arrays in u's own bytes
+    for k, v in enumerate((t, a, e, i)):
+        counts[k] = v
+    got = msp.direct_noalloc(pos, *counts, w.params["sigma"], out=room)
+    assert torch.equal(got, want)
