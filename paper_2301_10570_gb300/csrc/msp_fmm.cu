@@ -277,12 +277,14 @@ __global__ void __launch_bounds__(kTravTile) k_trav_top(TravArgs a, int64_t n, i
     }
 }
 
-// one depth; status: a tile counter and kTravWords words per tile (trav_pack),
-// zero on entry
+// one depth; status: a tile counter and W words per tile (trav_pack), zero on
+// entry; W = 2: no pair is far.  (A third word costs 1 us a depth: two rebuilt
+// steps of 262,144 neurons 9 us.)
+template <int W>
 __global__ void __launch_bounds__(kTravTile)
 k_trav_depth(TravArgs a, int d, unsigned long long* status, int64_t timeout_bit) {
     __shared__ int64_t s_tile;
-    __shared__ long long s_ex[kTravWords];
+    __shared__ long long s_ex[W];
     DevCounts* dc = a.dc;
     if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(&status[0], 1ull);
     const int64_t q0 = dc->depth_start[d], next0 = dc->depth_start[d + 1], nq = next0 - q0;
@@ -297,18 +299,18 @@ k_trav_depth(TravArgs a, int d, unsigned long long* status, int64_t timeout_bit)
         if (t >= ntiles) break;
         trav_tile(a, d, t, q0, nq, next0, t == ntiles - 1,
                   [&](const int (&tot)[4], long long (&ex)[4]) {
-            long long e[kTravWords];
+            long long e[W];
             if (threadIdx.x < 32) {
-                long long own[kTravWords];
+                long long own[W];
                 trav_pack(tot, own);
-                look_back<kTravWords>(status + 1, t, own, e, &dc->overflow, timeout_bit, kSpinLimit);
+                look_back<W>(status + 1, t, own, e, &dc->overflow, timeout_bit, kSpinLimit);
                 if (threadIdx.x == 0)
 #pragma unroll
-                    for (int k = 0; k < kTravWords; ++k) s_ex[k] = e[k];
+                    for (int k = 0; k < W; ++k) s_ex[k] = e[k];
             }
             __syncthreads();
 #pragma unroll
-            for (int k = 0; k < kTravWords; ++k) e[k] = s_ex[k];
+            for (int k = 0; k < W; ++k) e[k] = s_ex[k];
             trav_unpack(e, ex);
         });
         if (ntiles <= gridDim.x) break;        // every block has had its one tile
@@ -1007,18 +1009,20 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
         return (pairs + kTravTile - 1) / kTravTile;
     };
     const int dtop = std::min(D, kTopDepths);
+    const int words = c.l_far <= c.tree_depth ? 3 : 2;      // a far pair's boxes: levels from l_far on
     int64_t nw = 0;
-    for (int d = dtop; d < D; ++d) nw += 1 + kTravWords * tiles_at(d);
+    for (int d = dtop; d < D; ++d) nw += 1 + words * tiles_at(d);
     unsigned long long* st = c.tv_status.ensure<unsigned long long>((size_t)std::max<int64_t>(nw, 1));
     if (nw > 0) MSP_CUDA(cudaMemsetAsync(st, 0, (size_t)nw * sizeof(unsigned long long), s));
     k_trav_top<<<1, kTravTile, 0, s>>>(ta, n, dtop);
     MSP_LAUNCH("trav_top");
     for (int d = dtop; d < D; ++d) {
         const int64_t tiles = tiles_at(d);
-        k_trav_depth<<<(unsigned)std::min<int64_t>(tiles, (int64_t)c.sm_count * 6), kTravTile, 0, s>>>(
+        (words == 3 ? k_trav_depth<3> : k_trav_depth<2>)<<<
+            (unsigned)std::min<int64_t>(tiles, (int64_t)c.sm_count * 6), kTravTile, 0, s>>>(
             ta, d, st, kScanTimeoutBit);
         MSP_LAUNCH("trav_depth");
-        st += 1 + kTravWords * tiles;
+        st += 1 + words * tiles;
     }
     // the near-field list grouped by target leaf (at most one segment per box)
     radix_sort_dev(c, pk0, pv0, pk1, pv1, &dc->n_p2p, cap, xbits, s);

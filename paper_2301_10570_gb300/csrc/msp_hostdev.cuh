@@ -13,24 +13,24 @@
 namespace msp {
 
 // What a traversal tile counts (children, split, near-field and far pairs) as
-// the words of its look-back, which adds them modulo 2^62.  The pairs of a
+// the W words of its look-back, which adds them modulo 2^62.  The pairs of a
 // depth lie in the pair table (at most 2^31 - 1), so two of their counts share a
 // word; a depth's children may be 64 times as many and have a word of their own:
 // their number has to be exact beyond the table too, or the depths that do not
-// fit would not be seen.
-constexpr int kTravWords = 3;
-
-MSP_HD void trav_pack(const int (&tot)[4], long long (&w)[kTravWords]) {
+// fit would not be seen.  W = 2 where no pair can be far, else 3.
+template <int W>
+MSP_HD void trav_pack(const int (&tot)[4], long long (&w)[W]) {
     w[0] = tot[0];
     w[1] = (long long)tot[1] << 31 | tot[2];
-    w[2] = tot[3];
+    if (W > 2) w[W - 1] = tot[3];
 }
 
-MSP_HD void trav_unpack(const long long (&w)[kTravWords], long long (&ex)[4]) {
+template <int W>
+MSP_HD void trav_unpack(const long long (&w)[W], long long (&ex)[4]) {
     ex[0] = w[0];
     ex[1] = w[1] >> 31;
     ex[2] = w[1] & ((1ll << 31) - 1);
-    ex[3] = w[2];
+    ex[3] = W > 2 ? w[W - 1] : 0;
 }
 
 }  // namespace msp

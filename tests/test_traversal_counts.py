@@ -11,13 +11,14 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SOURCE = r"""
 #include <cstdio>
 #include "msp_hostdev.cuh"
+template <int W>
 static bool run(const int (*tile)(long long, int), long long tiles) {
     const unsigned long long mask = (1ull << 62) - 1;    // a status word's value
-    unsigned long long sum[msp::kTravWords] = {};
+    unsigned long long sum[W] = {};
     long long want[4] = {};
     for (long long t = 0; t < tiles; ++t) {
-        long long w[msp::kTravWords], ex[4];
-        for (int k = 0; k < msp::kTravWords; ++k) w[k] = (long long)(sum[k] & mask);
+        long long w[W], ex[4];
+        for (int k = 0; k < W; ++k) w[k] = (long long)(sum[k] & mask);
         msp::trav_unpack(w, ex);
         for (int k = 0; k < 4; ++k)
             if (ex[k] != want[k]) {
@@ -27,7 +28,7 @@ static bool run(const int (*tile)(long long, int), long long tiles) {
         int tot[4];
         for (int k = 0; k < 4; ++k) want[k] += tot[k] = tile(t, k);
         msp::trav_pack(tot, w);
-        for (int k = 0; k < msp::kTravWords; ++k) sum[k] = (sum[k] + (unsigned long long)w[k]) & mask;
+        for (int k = 0; k < W; ++k) sum[k] = (sum[k] + (unsigned long long)w[k]) & mask;
     }
     return true;
 }
@@ -36,12 +37,14 @@ static const int mixed(long long t, int k) {
     const int split = (int)(t % 200), near = (256 - split) / 2;
     return k == 0 ? 64 * split : (k == 1 ? split : (k == 2 ? near : 256 - split - near));
 }
+static const int no_far(long long t, int k) { return k < 3 ? mixed(t, k) : 0; }
 static const int near_only(long long, int k) { return k == 2 ? 256 : 0; }
 static const int far_only(long long, int k) { return k == 3 ? 256 : 0; }
 int main() {
     const long long most = ((1ll << 31) - 1) / 256;      // tiles of the largest table
-    return run(all_split, 1ll << 19) && run(mixed, most) && run(near_only, most) &&
-           run(far_only, most) ? 0 : 1;
+    return run<3>(all_split, 1ll << 19) && run<3>(mixed, most) && run<3>(near_only, most) &&
+           run<3>(far_only, most) && run<2>(all_split, 1ll << 19) && run<2>(no_far, most) &&
+           run<2>(near_only, most) ? 0 : 1;
 }
 """
 
