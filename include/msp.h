@@ -256,6 +256,13 @@ msp_status msp_commit_synapses(msp_ctx *ctx, const int64_t *n_syn_dev, int64_t c
  * gave up as designed (any other status is a failure); the context stays
  * usable.  Synchronises. */
 msp_status msp_selftest_bounded_wait(msp_ctx *ctx, void *stream);
+/* The same for one kind of wait, without looking at the outcome: 0 the scan's
+ * (also that of the octree levels, the traversal and the compaction), 1 the
+ * sort's, 2 the barrier between the steps of msp_neuron_steps.  The wait runs
+ * out on the device and the next call that synchronises (msp_build_tree,
+ * msp_attraction, msp_select_partners, msp_update_synapses,
+ * msp_append_synapses) returns MSP_ERR_TIMEOUT, once.  Asynchronous. */
+msp_status msp_selftest_wait(msp_ctx *ctx, int which, void *stream);
 
 /* ---- The neuron side of the model (Section 3.1, Table 1) -------------------
  * The Model of Structural Plasticity's neurons produce the vacant elements

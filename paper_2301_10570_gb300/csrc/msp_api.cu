@@ -35,6 +35,8 @@ void attraction_grad(msp_ctx& c, const uint8_t* type, const uint8_t* va, const u
                      const uint8_t* vdi, const float* g, float* u, float* dud, float* gE,
                      float* gI, cudaStream_t s);
 void scan_wait_selftest(msp_ctx& c, cudaStream_t s);
+void sort_wait_selftest(msp_ctx& c, cudaStream_t s);
+void barrier_wait_selftest(msp_ctx& c, cudaStream_t s);
 void length_loss(msp_ctx& c, const uint8_t* type, const uint8_t* va, const float* we,
                  const float* wi, double target, double* out4, float* gE, float* gI,
                  cudaStream_t s);
@@ -294,7 +296,19 @@ msp_status msp_commit_synapses(msp_ctx* c, const int64_t* n_syn, int64_t capacit
 }
 
 msp_status msp_selftest_bounded_wait(msp_ctx* c, void* stream) {
-    return guarded(c, [&] { msp::scan_wait_selftest(*c, as_stream(stream)); });
+    return guarded(c, [&] {
+        msp::scan_wait_selftest(*c, as_stream(stream));
+        msp::pull_counts(*c, as_stream(stream));
+    });
+}
+
+msp_status msp_selftest_wait(msp_ctx* c, int which, void* stream) {
+    return guarded(c, [&] {
+        require(which >= 0 && which <= 2, "no such wait");
+        (which == 0 ? msp::scan_wait_selftest
+                    : (which == 1 ? msp::sort_wait_selftest : msp::barrier_wait_selftest))(
+            *c, as_stream(stream));
+    });
 }
 
 msp_status msp_neuron_steps(msp_ctx* c, int64_t n, uint64_t first_step, int n_steps,

@@ -338,7 +338,7 @@ k_neuron_step(int64_t n, int vec4, uint64_t seed, uint64_t step,
 // to the last, and only the input counts travel through memory.  One
 // cooperative block per SM; a step ends with a grid-wide barrier (the spikes of
 // step k are step k + 1's input), whose waiting time holds the next step's
-// random draws.  A barrier wait of more than kSpinLimit polls sets timeout_bit
+// random draws.  A barrier wait of more than SPINS polls sets timeout_bit
 // in *overflow and every later wait is skipped: the kernel always ends (the
 // counts are then wrong, and the next synchronising call reports it).
 //
@@ -368,7 +368,7 @@ struct NrRun {
 constexpr int kNrGroupBytes = 6 * 16 + 8 + 8;
 constexpr int kNrMaxGroups = 220 * 1024 / kNrGroupBytes;
 
-template <bool FAST>
+template <bool FAST, int SPINS>
 __global__ void __launch_bounds__(1024, 1) k_neuron_run(NrRun a) {
     extern __shared__ float4 nr_sm[];
     __shared__ int s_dead, s_nsp[2];
@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(1024, 1) k_neuron_run(NrRun a) {
             const unsigned int goal = (unsigned int)(st + 1) * gridDim.x;
             volatile unsigned int* b = a.barrier;
             int spin = 0;
-            while (*b < goal && spin < kSpinLimit) ++spin;
+            while (*b < goal && spin < SPINS) ++spin;
             if (*b < goal) {
                 s_dead = 1;
                 atomicOr(reinterpret_cast<unsigned long long*>(a.overflow),
@@ -520,13 +520,17 @@ __global__ void __launch_bounds__(1024, 1) k_neuron_run(NrRun a) {
 // and the list compacted through a copy, 0.29 ms now (the synchronisation of
 // the check included).
 // ---------------------------------------------------------------------------
+constexpr unsigned long long kBadWait = 1ull << 40;
+
 // bound synapses per group; counts the edges naming a neuron outside [0, n),
-// and an edge count above the capacity
+// and an edge count above the capacity; kBadWait more where a wait before gave up
 __global__ void k_bound(const int64_t* __restrict__ n_edges, int64_t cap, int64_t n,
                         const int32_t* __restrict__ pre, const int32_t* __restrict__ post,
                         const uint8_t* __restrict__ typ, int32_t* __restrict__ bound,
-                        unsigned long long* __restrict__ bad) {
+                        unsigned long long* __restrict__ bad, const int64_t* __restrict__ overflow,
+                        int64_t timeout_bit) {
     const int64_t m0 = *n_edges;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && (*overflow & timeout_bit)) atomicAdd(bad, kBadWait);
     if (blockIdx.x == 0 && threadIdx.x == 0 && (m0 < 0 || m0 > cap)) atomicAdd(bad, 1ull);
     const int64_t m = min(max(m0, (int64_t)0), cap);
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
@@ -850,7 +854,8 @@ void neuron_steps(msp_ctx& c, int64_t n, uint64_t first_step, int n_steps,
         const bool fast = nr_fast(mp, r.fast);
         MSP_CUDA(cudaMemsetAsync(r.barrier, 0, sizeof(int64_t), s));
         const size_t smem = (size_t)per * kNrGroupBytes;
-        const void* kernel = fast ? (const void*)k_neuron_run<true> : (const void*)k_neuron_run<false>;
+        const void* kernel = fast ? (const void*)k_neuron_run<true, kSpinLimit>
+                                  : (const void*)k_neuron_run<false, kSpinLimit>;
         if (smem > 48 * 1024)
             MSP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)smem));
@@ -869,6 +874,48 @@ void neuron_steps(msp_ctx& c, int64_t n, uint64_t first_step, int n_steps,
                                           spiked);
         MSP_LAUNCH("neuron_step");
     }
+}
+
+// The barrier's bounded wait, exercised: the arrivals start one below zero, so the
+// one block's own arrival does not complete the first step; it waits at most
+// kSelftestSpins polls, records the timeout bit and goes on to the end.
+void barrier_wait_selftest(msp_ctx& c, cudaStream_t s) {
+    const int64_t n = 256;
+    const int groups = (int)n / 4;
+    NrRun r = {};
+    r.n4 = groups;
+    r.n = n;
+    r.per = groups;
+    r.n_steps = 3;
+    r.mp.x0 = r.mp.eps = 0.5f;
+    r.mp.tau_x = 5.0f;
+    r.mp.eta_axon = r.mp.eta_dend = 0.25f;
+    const size_t ints = (size_t)4 * n;               // input counts, edge starts and numbers
+    int32_t* zero = c.nr_inp.ensure<int32_t>(ints);
+    MSP_CUDA(cudaMemsetAsync(zero, 0, ints * sizeof(int32_t), s));
+    r.inp0 = zero;
+    r.inp1 = zero + n;
+    r.off = zero + 2 * n;
+    r.deg = zero + 3 * n;
+    r.targets = r.off;                               // no edges: not read
+    float* state = c.nr_key0.ensure<float>((size_t)6 * n);
+    MSP_CUDA(cudaMemsetAsync(state, 0, (size_t)6 * n * sizeof(float), s));
+    r.x = state;
+    r.ca = state + n;
+    r.za = state + 2 * n;
+    r.ze = state + 3 * n;
+    r.zi = state + 4 * n;
+    r.refr = reinterpret_cast<uint8_t*>(state + 5 * n);
+    r.spiked = r.refr + n;
+    int64_t* cnt = c.nr_cnt.ensure<int64_t>(4);
+    r.barrier = reinterpret_cast<unsigned int*>(cnt + 3);
+    MSP_CUDA(cudaMemsetAsync(r.barrier, 0xff, sizeof(int64_t), s));
+    r.overflow = &dcounts(c)->overflow;
+    r.timeout_bit = kScanTimeoutBit;
+    void* args[] = {&r};
+    MSP_CUDA(cudaLaunchCooperativeKernel((const void*)k_neuron_run<false, kSelftestSpins>, dim3(1),
+                                         dim3(groups), args, (size_t)groups * kNrGroupBytes, s));
+    MSP_LAUNCH("barrier_wait_selftest");
 }
 
 void update_synapses(msp_ctx& c, int64_t n, uint64_t step, const float* za, const float* ze,
@@ -893,15 +940,18 @@ void update_synapses(msp_ctx& c, int64_t n, uint64_t step, const float* za, cons
     int64_t* cnt = c.nr_upd.ensure<int64_t>(8);
     const int ge = (int)c.sm_count * 8;
     const int gn = grid_for(n, 256, (int64_t)c.sm_count * 16);
-    // the edges must name neurons in [0, n) and fit the capacity
+    // the edges must name neurons in [0, n) and fit the capacity; a wait of the
+    // steps before that gave up is reported here, before the edges change
     MSP_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int64_t), s));
     MSP_CUDA(cudaMemsetAsync(bound, 0, (size_t)3 * n * sizeof(int32_t), s));
     k_bound<<<ge, 256, 0, s>>>(n_edges, cap, n, pre, post, typ, bound,
-                               reinterpret_cast<unsigned long long*>(cnt));
+                               reinterpret_cast<unsigned long long*>(cnt), &dcounts(c)->overflow,
+                               kScanTimeoutBit);
     MSP_LAUNCH("bound");
     int64_t bad = 0;
     MSP_CUDA(cudaMemcpyAsync(&bad, cnt, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     MSP_CUDA(cudaStreamSynchronize(s));
+    if ((unsigned long long)bad >= kBadWait) pull_counts(c, s);      // throws
     if (bad) throw Error(MSP_ERR_INVALID_ARG, "an edge names a neuron outside [0, n), or the "
                                               "edge count exceeds the capacity");
     MSP_CUDA(cudaMemsetAsync(del, 0, ecap, s));

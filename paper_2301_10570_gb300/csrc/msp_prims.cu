@@ -72,8 +72,9 @@ k_rs_hist(const uint64_t* __restrict__ keys, int64_t n_host, const int64_t* __re
 }
 
 // One pass.  tile_ctr hands out the tiles in order (zero on entry), so every
-// tile's predecessors have started; a wait of more than kSpinLimit polls gives
+// tile's predecessors have started; a wait of more than SPINS polls gives
 // up, counts the tile as 0 and sets timeout_bit in *overflow.
+template <int SPINS>
 __global__ void __launch_bounds__(kRsThreads, 3)
 k_rs_pass(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin,
           uint64_t* __restrict__ kout, int32_t* __restrict__ vout, int64_t n_host,
@@ -176,7 +177,7 @@ k_rs_pass(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin,
                 for (int k = 0; k < kRsLook; ++k) {
                     if (done) continue;
                     int spin = 0;
-                    while ((v[k] >> 62) == 0 && spin < kSpinLimit) {
+                    while ((v[k] >> 62) == 0 && spin < SPINS) {
                         ++spin;
                         v[k] = status[(int64_t)(j - k) * (bins / 2) + t];
                     }
@@ -244,10 +245,11 @@ void scan_dev(msp_ctx& c, const int32_t* in, int32_t* out, const int64_t* n_dev,
     scan_launch(c, ScanI32{in}, ScanStore{out}, ScanTotal{total_dst}, n_dev, n_cap, s);
 }
 
-// The scan's bounded wait, exercised: the tile counter starts at 1, so tile
-// 0 is never taken and its status never published; the tiles after it wait
-// on it at most `spin_limit` polls, give up, record the timeout bit and
-// finish.  pull_counts then reports MSP_ERR_TIMEOUT.
+// The bounded waits of the scan and of the sort, exercised: the tile counter
+// starts at 1, so tile 0 is never taken and its status never published; the tiles
+// after it wait on it at most kSelftestSpins polls, give up, record the timeout
+// bit and finish.  The next pull_counts then reports MSP_ERR_TIMEOUT.  (The look-back
+// of the octree levels, the traversal depths and the compaction is the scan's.)
 void scan_wait_selftest(msp_ctx& c, cudaStream_t s) {
     const int64_t n = 3 * (int64_t)kScanTile;
     int32_t* in = c.cnt.ensure<int32_t>((size_t)n);
@@ -259,9 +261,27 @@ void scan_wait_selftest(msp_ctx& c, cudaStream_t s) {
     dev_set(reinterpret_cast<int64_t*>(status), 1, s);       // tile 0 is skipped
     dev_set(nd, n, s);
     k_scan_1p<<<3, kScanThreads, 0, s>>>(ScanI32{in}, ScanStore{out}, ScanTotal{nd + 1}, nd, status,
-                                         &dcounts(c)->overflow, kScanTimeoutBit, 1 << 12);
+                                         &dcounts(c)->overflow, kScanTimeoutBit, kSelftestSpins);
     MSP_LAUNCH("scan_wait_selftest");
-    pull_counts(c, s);
+}
+
+void sort_wait_selftest(msp_ctx& c, cudaStream_t s) {
+    const int64_t n = 3 * (int64_t)kRsTile;
+    const int bits = 8, bins = 1 << bits;
+    uint64_t* key[2] = {c.rq_key0.ensure<uint64_t>((size_t)n), c.keys1.ensure<uint64_t>((size_t)n)};
+    int32_t* val[2] = {c.rq_val0.ensure<int32_t>((size_t)n), c.vals1.ensure<int32_t>((size_t)n)};
+    int32_t* hist = c.rs_hist.ensure<int32_t>((size_t)kRsMaxPasses * (kRsBins + 1));
+    unsigned long long* status = c.rs_status.ensure<unsigned long long>((size_t)(3 * bins / 2));
+    MSP_CUDA(cudaMemsetAsync(key[0], 0, (size_t)n * sizeof(uint64_t), s));
+    MSP_CUDA(cudaMemsetAsync(val[0], 0, (size_t)n * sizeof(int32_t), s));
+    MSP_CUDA(cudaMemsetAsync(hist, 0, (size_t)(bins + 2) * sizeof(int32_t), s));
+    k_rs_hist<<<3, kRsThreads, 0, s>>>(key[0], n, nullptr, 1, bits, hist, status, 3 * bins / 2);
+    MSP_LAUNCH("rs_hist");
+    // the tile counter (hist[bins], with the zero above it) starts at 1
+    dev_set(reinterpret_cast<int64_t*>(hist + bins), 1, s);
+    k_rs_pass<kSelftestSpins><<<3, kRsThreads, 0, s>>>(key[0], val[0], key[1], val[1], n, nullptr, 0, bits, hist,
+                                       hist + bins, status, &dcounts(c)->overflow, kScanTimeoutBit);
+    MSP_LAUNCH("sort_wait_selftest");
 }
 
 static int rs_passes(int64_t n_cap, int bits) {
@@ -297,7 +317,7 @@ void radix_sort_dev(msp_ctx& c, uint64_t* keys, int32_t* vals, uint64_t* keys_tm
     MSP_LAUNCH("rs_hist");
     const int g = (int)std::min<int64_t>(tiles_cap, (int64_t)c.sm_count * 3);
     for (int ps = 0; ps < passes; ++ps) {
-        k_rs_pass<<<g, kRsThreads, 0, s>>>(ka, va, kb, vb, n_cap, n_dev, ps * per, per,
+        k_rs_pass<kSpinLimit><<<g, kRsThreads, 0, s>>>(ka, va, kb, vb, n_cap, n_dev, ps * per, per,
                                            hist + ps * bins, ctr + ps, status + ps * stride,
                                            &dcounts(c)->overflow, kScanTimeoutBit);
         MSP_LAUNCH("rs_pass");

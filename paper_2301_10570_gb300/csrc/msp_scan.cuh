@@ -22,6 +22,7 @@ constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;
 constexpr unsigned long long kValMask = (1ull << 62) - 1;
 constexpr int kSpinLimit = 1 << 22;
+constexpr int kSelftestSpins = 1 << 12;      // of the waits that are made to run out
 
 __device__ __forceinline__ long long warp_incl_scan(long long v) {
     int lane = threadIdx.x & 31;

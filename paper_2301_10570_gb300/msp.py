@@ -34,7 +34,7 @@ EXPORTED = ("msp_create", "msp_destroy", "msp_build_tree", "msp_attraction", "ms
             "msp_set_pair_capacity", "msp_batch_layout", "msp_attraction_grad",
             "msp_set_workspace_limit", "msp_workspace_bytes", "msp_neuron_steps",
             "msp_update_synapses", "msp_append_synapses", "msp_selftest_bounded_wait",
-            "msp_philox", "msp_step_graph_set_full_build", "msp_length_loss",
+            "msp_selftest_wait", "msp_philox", "msp_step_graph_set_full_build", "msp_length_loss",
             "msp_set_sigma", "msp_set_frames")
 MAX_VACANCY = 5         # the vacancy walk's bound on every vacant count
 NOALLOC_MAX_N = 65536   # MSP_NOALLOC_MAX_N of include/msp.h
@@ -152,6 +152,8 @@ def load(path: str = LIB_PATH):
         L.msp_update_synapses.argtypes = [vp, i64, u64] + [vp] * 7 + [i64] + [vp] * 3 + [vp]
         L.msp_append_synapses.argtypes = [vp, vp, i64] + [vp] * 7 + [i64, vp]
         L.msp_selftest_bounded_wait.argtypes = [vp, vp]
+        L.msp_selftest_wait.argtypes = [vp, C.c_int, vp]
+        L.msp_selftest_wait.restype = C.c_int
         L.msp_philox.argtypes = [i64, vp, vp, vp, vp]
         L.msp_philox.restype = C.c_int
         L.msp_step_graph_set_full_build.argtypes = [vp, C.c_int]
@@ -375,6 +377,11 @@ class MSP:
         """Runs the device scan with a predecessor that never publishes; the
         bounded wait gives up: raises MSPError with code 4 (MSP_ERR_TIMEOUT)."""
         _check(load().msp_selftest_bounded_wait(self._h, _stream(stream)))
+
+    def selftest_wait(self, which: int, stream=None):
+        """Lets the wait of the scan (0), the sort (1) or the neuron steps' barrier
+        (2) run out; the next synchronising call raises MSP_ERR_TIMEOUT."""
+        _check(load().msp_selftest_wait(self._h, int(which), _stream(stream)))
 
     # -- the neuron side of the model (Section 3.1) ------------------------------
     def neuron_steps(self, first_step, n_steps, params, edges, state, stream=None):
