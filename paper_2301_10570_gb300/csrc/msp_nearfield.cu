@@ -35,6 +35,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "msp_hostdev.cuh"
 #include "msp_internal.cuh"
 
 namespace msp {
@@ -447,10 +448,8 @@ __device__ __forceinline__ void nf_targets(const NFArgs& a, int nt, int nreal, i
             const int slot = tg.slot0 + r;
             const int32_t t = slot < nt ? tl[slot] : -1;
             if (t >= 0) {
-                float sacc = sm.red[0][slot];
-#pragma unroll
-                for (int k = 1; k < NW; ++k) sacc += sm.red[k][slot];
-                nf_add_u(a, t, sacc * sm.scale[slot]);
+                const float sum = sum_totals<NW>([&](int k) { return sm.red[k][slot]; });
+                nf_add_u(a, t, sum * sm.scale[slot]);
             }
         }
     }
