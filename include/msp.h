@@ -263,6 +263,10 @@ msp_status msp_selftest_bounded_wait(msp_ctx *ctx, void *stream);
  * msp_attraction, msp_select_partners, msp_update_synapses,
  * msp_append_synapses) returns MSP_ERR_TIMEOUT, once.  Asynchronous. */
 msp_status msp_selftest_wait(msp_ctx *ctx, int which, void *stream);
+/* With refuse != 0 the context's cooperative launches (several steps of
+ * msp_neuron_steps in one launch) act as if the device had refused them, which
+ * must not change a result: the steps are launched one by one. */
+msp_status msp_selftest_refuse_cooperative(msp_ctx *ctx, int refuse);
 
 /* ---- The neuron side of the model (Section 3.1, Table 1) -------------------
  * The Model of Structural Plasticity's neurons produce the vacant elements

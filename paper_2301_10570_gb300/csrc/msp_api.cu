@@ -311,6 +311,10 @@ msp_status msp_selftest_wait(msp_ctx* c, int which, void* stream) {
     });
 }
 
+msp_status msp_selftest_refuse_cooperative(msp_ctx* c, int refuse) {
+    return guarded(c, [&] { c->refuse_cooperative = refuse != 0; });
+}
+
 msp_status msp_neuron_steps(msp_ctx* c, int64_t n, uint64_t first_step, int n_steps,
                             const msp_neuron_params* params, const int64_t* n_edges,
                             int64_t capacity, const int32_t* pre, const int32_t* post, float* x,

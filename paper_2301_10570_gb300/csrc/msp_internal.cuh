@@ -256,6 +256,7 @@ struct msp_ctx {
     // neuron side (msp_neuron.cu): input counts, outgoing-edge lists; bound
     // synapses, excess and starts per group, deletion sort keys and flags
     msp::DBuf nr_inp, nr_bout, nr_xout, nr_sout, nr_pos, nr_cnt;
+    bool refuse_cooperative = false;     // self-test: cooperative launches fail as too large
     msp::DBuf nr_bin, nr_xin, nr_sin, nr_key0, nr_key1, nr_val0, nr_val1, nr_del, nr_upd;
     // geometric expansion centres and the grouped translations (msp_m2l_gemm.cu)
     int gm_smem_set = 0;   // dynamic shared memory opted in for the grouped translations

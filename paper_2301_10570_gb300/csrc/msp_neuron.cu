@@ -860,10 +860,19 @@ void neuron_steps(msp_ctx& c, int64_t n, uint64_t first_step, int n_steps,
             MSP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)smem));
         void* args[] = {&r};
-        MSP_CUDA(cudaLaunchCooperativeKernel(kernel, dim3((unsigned)blocks), dim3((unsigned)T), args,
-                                             smem, s));
-        MSP_LAUNCH("neuron_run");
-        return;
+        // refused where the process may not have a block on every SM that the
+        // device reports: the steps then go one by one
+        const cudaError_t e =
+            c.refuse_cooperative
+                ? cudaErrorCooperativeLaunchTooLarge
+                : cudaLaunchCooperativeKernel(kernel, dim3((unsigned)blocks), dim3((unsigned)T), args,
+                                              smem, s);
+        if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) {
+            cuda_check(e, "cudaLaunchCooperativeKernel");
+            MSP_LAUNCH("neuron_run");
+            return;
+        }
+        (void)cudaGetLastError();
     }
     const int gv = grid_for(vec4 ? (n + 3) / 4 : n, 256, (int64_t)c.sm_count * 16);
     for (int k = 0; k < n_steps; ++k) {

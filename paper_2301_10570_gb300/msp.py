@@ -34,8 +34,9 @@ EXPORTED = ("msp_create", "msp_destroy", "msp_build_tree", "msp_attraction", "ms
             "msp_set_pair_capacity", "msp_batch_layout", "msp_attraction_grad",
             "msp_set_workspace_limit", "msp_workspace_bytes", "msp_neuron_steps",
             "msp_update_synapses", "msp_append_synapses", "msp_selftest_bounded_wait",
-            "msp_selftest_wait", "msp_philox", "msp_step_graph_set_full_build", "msp_length_loss",
-            "msp_set_sigma", "msp_set_frames")
+            "msp_selftest_wait", "msp_selftest_refuse_cooperative", "msp_philox",
+            "msp_step_graph_set_full_build", "msp_length_loss", "msp_set_sigma",
+            "msp_set_frames")
 MAX_VACANCY = 5         # the vacancy walk's bound on every vacant count
 NOALLOC_MAX_N = 65536   # MSP_NOALLOC_MAX_N of include/msp.h
 
@@ -154,6 +155,8 @@ def load(path: str = LIB_PATH):
         L.msp_selftest_bounded_wait.argtypes = [vp, vp]
         L.msp_selftest_wait.argtypes = [vp, C.c_int, vp]
         L.msp_selftest_wait.restype = C.c_int
+        L.msp_selftest_refuse_cooperative.argtypes = [vp, C.c_int]
+        L.msp_selftest_refuse_cooperative.restype = C.c_int
         L.msp_philox.argtypes = [i64, vp, vp, vp, vp]
         L.msp_philox.restype = C.c_int
         L.msp_step_graph_set_full_build.argtypes = [vp, C.c_int]
@@ -382,6 +385,10 @@ class MSP:
         """Lets the wait of the scan (0), the sort (1) or the neuron steps' barrier
         (2) run out; the next synchronising call raises MSP_ERR_TIMEOUT."""
         _check(load().msp_selftest_wait(self._h, int(which), _stream(stream)))
+
+    def selftest_refuse_cooperative(self, refuse: bool):
+        """Lets this context's cooperative launches act as refused by the device."""
+        _check(load().msp_selftest_refuse_cooperative(self._h, 1 if refuse else 0))
 
     # -- the neuron side of the model (Section 3.1) ------------------------------
     def neuron_steps(self, first_step, n_steps, params, edges, state, stream=None):
