@@ -259,7 +259,6 @@ struct msp_ctx {
     bool refuse_cooperative = false;     // self-test: cooperative launches fail as too large
     msp::DBuf nr_bin, nr_xin, nr_sin, nr_key0, nr_key1, nr_val0, nr_val1, nr_del, nr_upd;
     // geometric expansion centres and the grouped translations (msp_m2l_gemm.cu)
-    int gm_smem_set = 0;   // dynamic shared memory opted in for the grouped translations
     msp::DBuf nd_gc, gm_key0, gm_key1, gm_q, gm_q1, gm_flag, gm_gid, gm_gstart, gm_ntile,
         gm_toff, gm_tiles, gm_cnt;
     // derivatives (msp_grad.cu)
@@ -374,6 +373,17 @@ bool radix_from_tmp(int64_t n_cap, int bits);
 void radix_sort_dev(msp_ctx& c, uint64_t* keys, int32_t* vals, uint64_t* keys_tmp,
                     int32_t* vals_tmp, const int64_t* n_dev, int64_t n_cap, int bits,
                     cudaStream_t s);
+// Before a launch with `bytes` of dynamic shared memory: lets the kernel have
+// `most` (the largest that any of its launches asks for) if that is above the
+// default.  The limit belongs to the kernel on the device, not to the context, and a
+// smaller one would fail another context's launch between its limit and its
+// launch: always the same value, which never shrinks.
+template <class Kernel>
+inline void allow_shared(Kernel kernel, size_t bytes, size_t most) {
+    if (bytes > 48 * 1024)
+        MSP_CUDA(cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel),
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+}
 // small device-side bookkeeping (msp_prims.cu)
 void dev_set(int64_t* dst, int64_t v, cudaStream_t s);
 // device counts of a context and their host mirror (synchronous)

@@ -274,6 +274,15 @@ void geo_centres(msp_ctx& c, cudaStream_t s) {
 
 bool m2l_gemm_fits(int p) { return p <= kGemmMaxP; }
 
+// four rows a thread hold the operator up to this order
+constexpr int kGemmSmallP = 4;
+
+static size_t gemm_smem(int p) {
+    const size_t p3 = (size_t)p * p * p, PB = p <= kGemmSmallP ? 64 : 128, ncol = 2 * kGemmTile;
+    return sizeof(float) * (p3 * PB + p3 * ncol + PB * ncol + 48) + sizeof(int32_t) * kGemmTile +
+           sizeof(float) * ncol;
+}
+
 // Translations of the far pairs far_q[0, *nfar) grouped by offset.  On return
 // the far pairs are in key order in c.gm_q and *first_fallback (device)
 // holds the position from which the caller translates pair by pair.
@@ -309,18 +318,10 @@ const int32_t* m2l_gemm(msp_ctx& c, const int32_t* far_q, const int64_t* nfar, i
     scan_dev(c, ntile, toff, cnt, cap, cnt + 1, s);
     k_tile_list<<<ge, 256, 0, s>>>(gstart, ntile, toff, cnt, tiles);
     MSP_LAUNCH("tile_list");
-    const int p = c.cfg.p, p3 = p * p * p;
-    const int RM = p3 <= 64 ? 4 : 8;
-    const size_t PB = 16 * (size_t)RM, ncol = 2 * kGemmTile;
-    const size_t smem = sizeof(float) * ((size_t)p3 * PB + (size_t)p3 * ncol + PB * ncol + 48) +
-                        sizeof(int32_t) * kGemmTile + sizeof(float) * ncol;
-    if (smem > 48 * 1024 && (int)smem > c.gm_smem_set) {
-        MSP_CUDA(cudaFuncSetAttribute(k_m2l_gemm<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
-        MSP_CUDA(cudaFuncSetAttribute(k_m2l_gemm<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
-        c.gm_smem_set = (int)smem;
-    }
+    const int p = c.cfg.p;
+    const size_t smem = gemm_smem(p);
+    allow_shared(p <= kGemmSmallP ? k_m2l_gemm<4> : k_m2l_gemm<8>, smem,
+                 gemm_smem(p <= kGemmSmallP ? kGemmSmallP : kGemmMaxP));
     GemmArgs a;
     a.tiles = tiles;
     a.ntiles = cnt + 1;
@@ -339,8 +340,8 @@ const int32_t* m2l_gemm(msp_ctx& c, const int32_t* far_q, const int64_t* nfar, i
     a.p = p;
     a.half_box_over_sigma_l0 = (float)(0.5 * (double)c.cfg.side / c.cfg.sigma);
     const int grid = (int)c.sm_count * (smem <= 64 * 1024 ? 3 : 1);
-    if (RM == 4) k_m2l_gemm<4><<<grid, kGemmThreads, smem, s>>>(a);
-    else         k_m2l_gemm<8><<<grid, kGemmThreads, smem, s>>>(a);
+    if (p <= kGemmSmallP) k_m2l_gemm<4><<<grid, kGemmThreads, smem, s>>>(a);
+    else                  k_m2l_gemm<8><<<grid, kGemmThreads, smem, s>>>(a);
     MSP_LAUNCH("m2l_gemm");
     *first_fallback = cnt + 2;
     return v0;

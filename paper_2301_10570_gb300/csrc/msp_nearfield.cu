@@ -874,9 +874,7 @@ void launch_near_field(msp_ctx& c, const int32_t* seg_first, const int64_t* nseg
     const int64_t segs = small ? std::min<int64_t>(nseg_cap, 7 * (int64_t)c.sm_count) : nseg_cap;
     const int grid = (int)std::min<int64_t>(segs, 1 << 30);
     auto launch = [&](auto kernel, int nw, size_t smem) {
-        if (smem > 48 * 1024)
-            MSP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem));
+        allow_shared(kernel, smem, smem);
         kernel<<<grid, nw * 32, smem, s>>>(a);
     };
     // Warps per segment by the number of boxes (a bound on the segments): 4

@@ -856,9 +856,7 @@ void neuron_steps(msp_ctx& c, int64_t n, uint64_t first_step, int n_steps,
         const size_t smem = (size_t)per * kNrGroupBytes;
         const void* kernel = fast ? (const void*)k_neuron_run<true, kSpinLimit>
                                   : (const void*)k_neuron_run<false, kSpinLimit>;
-        if (smem > 48 * 1024)
-            MSP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem));
+        allow_shared(kernel, smem, (size_t)kNrMaxGroups * kNrGroupBytes);
         void* args[] = {&r};
         // refused where the process may not have a block on every SM that the
         // device reports: the steps then go one by one

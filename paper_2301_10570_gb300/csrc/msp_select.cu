@@ -866,9 +866,8 @@ void select_partners(msp_ctx& c, uint64_t step, const uint8_t* type_dev, const u
                       dc};
     const int top = std::min(n_steps, kDescTop);
     const size_t warp_bytes = desc_warp_floats(cfg.p) * sizeof(float);
-    if (kDescTopWarps * warp_bytes > 48 * 1024)
-        MSP_CUDA(cudaFuncSetAttribute(k_descend_top, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(kDescTopWarps * warp_bytes)));
+    allow_shared(k_descend_top, kDescTopWarps * warp_bytes,
+                 kDescTopWarps * desc_warp_floats(kMaxP) * sizeof(float));
     k_descend_top<<<1, kDescTopWarps * 32, kDescTopWarps * warp_bytes, s>>>(da, top);
     MSP_LAUNCH("descend_top");
     for (int k = top; k < n_steps; ++k) {
