@@ -370,6 +370,7 @@ void scan_dev(msp_ctx& c, const int32_t* in, int32_t* out, const int64_t* n_dev,
 // (keys, vals); the input is read from there, or from (keys_tmp, vals_tmp)
 // when radix_from_tmp says so (an odd number of passes).
 bool radix_from_tmp(int64_t n_cap, int bits);
+void radix_reserve(msp_ctx& c, int64_t n_cap, int bits);      // its scratch, ahead of the call
 void radix_sort_dev(msp_ctx& c, uint64_t* keys, int32_t* vals, uint64_t* keys_tmp,
                     int32_t* vals_tmp, const int64_t* n_dev, int64_t n_cap, int bits,
                     cudaStream_t s);

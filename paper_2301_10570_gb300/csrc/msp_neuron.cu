@@ -934,17 +934,36 @@ void update_synapses(msp_ctx& c, int64_t n, uint64_t step, const float* za, cons
     int32_t* bound = c.nr_bin.ensure<int32_t>((size_t)3 * n);
     int32_t* excess = c.nr_xin.ensure<int32_t>((size_t)3 * n);
     int32_t* start = c.nr_sin.ensure<int32_t>((size_t)3 * n);
-    // both sides' entries in one sort (one side at a time where they could
-    // exceed the sort's 2^31)
-    const int sides = cap < (1ll << 30) ? 2 : 1;
-    const int64_t ncap = sides * (int64_t)ecap;
-    uint64_t* k0 = c.nr_key0.ensure<uint64_t>((size_t)ncap);
-    uint64_t* k1 = c.nr_key1.ensure<uint64_t>((size_t)ncap);
-    int32_t* v0 = c.nr_val0.ensure<int32_t>((size_t)ncap);
-    int32_t* v1 = c.nr_val1.ensure<int32_t>((size_t)ncap);
     uint8_t* del = c.nr_del.ensure<uint8_t>(ecap);
     // bad edges, edges, groups, entries, kept entries
     int64_t* cnt = c.nr_upd.ensure<int64_t>(8);
+    // both sides' entries in one sort; one side at a time where they could exceed
+    // the sort's 2^31, or where the memory or its limit does not hold both (60
+    // bytes an edge, 31 for one side; 42 were enough for a sort per side and a
+    // copy of the list)
+    const int bits = 32 + bits_for_neuron(3 * n);
+    int sides = cap < (1ll << 30) ? 2 : 1;
+    auto reserve = [&] {
+        const size_t ncap = sides * ecap;
+        c.nr_key0.ensure<uint64_t>(ncap);
+        c.nr_key1.ensure<uint64_t>(ncap);
+        c.nr_val0.ensure<int32_t>(ncap);
+        c.nr_val1.ensure<int32_t>(ncap);
+        radix_reserve(c, (int64_t)ncap, bits);
+        scan_status(c, std::max<int64_t>((int64_t)ncap, 3 * n));
+    };
+    try {
+        reserve();
+    } catch (const Error& e) {
+        if (sides == 1 || e.code != MSP_ERR_OOM) throw;
+        (void)cudaGetLastError();
+        for (DBuf* b : {&c.nr_key0, &c.nr_key1, &c.nr_val0, &c.nr_val1, &c.rs_status}) b->release();
+        sides = 1;
+        reserve();
+    }
+    const int64_t ncap = sides * (int64_t)ecap;
+    uint64_t *k0 = c.nr_key0.get<uint64_t>(), *k1 = c.nr_key1.get<uint64_t>();
+    int32_t *v0 = c.nr_val0.get<int32_t>(), *v1 = c.nr_val1.get<int32_t>();
     const int ge = (int)c.sm_count * 8;
     const int gn = grid_for(n, 256, (int64_t)c.sm_count * 16);
     // the edges must name neurons in [0, n) and fit the capacity; a wait of the
@@ -967,7 +986,6 @@ void update_synapses(msp_ctx& c, int64_t n, uint64_t step, const float* za, cons
     MSP_LAUNCH("excess");
     scan_launch(c, ScanOverfull{bound, excess}, ScanStore{start}, ScanTotal{nullptr}, cnt + 2, 3 * n,
                 s);
-    const int bits = 32 + bits_for_neuron(3 * n);
     const bool odd = radix_from_tmp(ncap, bits);
     for (int side0 = 0; side0 < 2; side0 += sides) {
         const DelEntries in{cnt + 1, n, side0, pre, post, typ, excess};

@@ -288,6 +288,20 @@ static int rs_passes(int64_t n_cap, int bits) {
     return n_cap <= 1 || bits <= 0 ? 0 : (bits + kRsMaxBits - 1) / kRsMaxBits;
 }
 
+// bits of a digit, status words of a pass
+static int rs_digit(int passes, int bits) { return (bits + passes - 1) / passes; }
+static int64_t rs_stride(int64_t n_cap, int per) {
+    return (n_cap + kRsTile - 1) / kRsTile * ((1 << per) / 2);
+}
+
+void radix_reserve(msp_ctx& c, int64_t n_cap, int bits) {
+    const int passes = rs_passes(n_cap, bits);
+    if (passes == 0) return;
+    c.rs_hist.ensure<int32_t>((size_t)kRsMaxPasses * (kRsBins + 1));
+    c.rs_status.ensure<unsigned long long>(
+        (size_t)(passes * rs_stride(n_cap, rs_digit(passes, bits))));
+}
+
 bool radix_from_tmp(int64_t n_cap, int bits) { return (rs_passes(n_cap, bits) & 1) != 0; }
 
 void radix_sort_dev(msp_ctx& c, uint64_t* keys, int32_t* vals, uint64_t* keys_tmp,
@@ -295,15 +309,14 @@ void radix_sort_dev(msp_ctx& c, uint64_t* keys, int32_t* vals, uint64_t* keys_tm
                     cudaStream_t s) {
     const int passes = rs_passes(n_cap, bits);
     if (passes == 0) return;
-    const int per = (bits + passes - 1) / passes, bins = 1 << per;
-    const int64_t tiles_cap = (n_cap + kRsTile - 1) / kRsTile;
+    radix_reserve(c, n_cap, bits);
+    const int per = rs_digit(passes, bits), bins = 1 << per;
+    const int64_t tiles_cap = (n_cap + kRsTile - 1) / kRsTile, stride = rs_stride(n_cap, per);
     // digit counts and tile counters (cleared here), status words (cleared
     // by the counting kernel, as many as the elements need)
-    int32_t* hist = c.rs_hist.ensure<int32_t>((size_t)kRsMaxPasses * (kRsBins + 1));
+    int32_t* hist = c.rs_hist.get<int32_t>();
     int32_t* ctr = hist + passes * bins;
-    const int64_t stride = tiles_cap * (bins / 2);
-    unsigned long long* status =
-        c.rs_status.ensure<unsigned long long>((size_t)(passes * stride));
+    unsigned long long* status = c.rs_status.get<unsigned long long>();
     MSP_CUDA(cudaMemsetAsync(hist, 0, (size_t)passes * (bins + 1) * sizeof(int32_t), s));
     uint64_t *ka = keys, *kb = keys_tmp;
     int32_t *va = vals, *vb = vals_tmp;
