@@ -172,7 +172,7 @@ def load(path: str = LIB_PATH):
             getattr(L, name).restype = C.c_int
         for name in ("msp_step_graph_capture", "msp_step_graph_launch", "msp_step_graph_finish",
                      "msp_set_pair_capacity", "msp_batch_layout", "msp_attraction_grad",
-            "msp_set_workspace_limit", "msp_workspace_bytes", "msp_neuron_steps",
+            "msp_set_workspace_limit", "msp_neuron_steps",
             "msp_update_synapses", "msp_append_synapses", "msp_selftest_bounded_wait"):
             getattr(L, name).restype = C.c_int
         for name in ("msp_create", "msp_destroy", "msp_build_tree", "msp_attraction",
