@@ -46,9 +46,6 @@ __global__ void k_graph_init(DevCounts* dc, uint64_t step, int64_t halt) {
     dc->interactions_run = 0;
 }
 
-// a step without neurons has no selection to end it
-__global__ void k_graph_end(DevCounts* dc, GraphEnd end) { end(dc); }
-
 // graph mode for the dry run and the capture, with the graph's options
 struct GraphModeScope {
     msp_ctx& c;
@@ -66,16 +63,11 @@ struct GraphModeScope {
 
 // one step in graph mode on the stream (captured or, for the dry run, eager)
 void record_step(msp_ctx& c, const msp_ctx::GraphArgs& g, cudaStream_t s) {
-    DevCounts* dc = dcounts(c);
     if (g.walk) vacancy_walk(c, g.n, 0, g.va, g.vde, g.vdi, s);
     build_tree(c, g.n, g.x, g.y, g.z, g.type, g.va, g.vde, g.vdi, s);
     attraction(c, g.u, s);
     select_partners(c, 0, g.type, g.va, g.vde, g.vdi, g.partner, g.pre, g.post, g.styp, g.n_syn,
                     s);
-    if (g.elem_cap <= 0) {
-        k_graph_end<<<1, 1, 0, s>>>(dc, c.graph_end);
-        MSP_LAUNCH("graph_end");
-    }
     if (g.commit)
         commit_synapses(c, g.n_syn, g.capacity, g.pre, g.post, g.styp, g.va, g.vde, g.vdi, s);
 }
@@ -95,6 +87,9 @@ void capture(msp_ctx& c, msp_ctx::StepGraph& G, const msp_ctx::GraphArgs& args, 
     if (!c.tree_built || !c.attraction_done || c.n != args.n)
         throw Error(MSP_ERR_NOT_BUILT,
                     "build the tree of these positions and run the attraction once first");
+    // the last scan of the selection ends a step: there is one
+    if (args.n <= 0 || args.elem_cap <= 0)
+        throw Error(MSP_ERR_INVALID_ARG, "a step graph needs neurons and room for elements");
     release(G);
     DevCounts* dc = dcounts(c);
     {
