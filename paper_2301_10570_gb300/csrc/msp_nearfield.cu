@@ -589,8 +589,9 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : (NW == 8 ? 3 : 1)) k_ne
 // plans with translated pairs, leaf capacity 8).  A pair is then 10 evaluations
 // or so, and a warp per pair spends nearly all its time on staging, shuffles
 // and the pair's W.  Here a warp takes a segment and its lanes take pairs: the
-// targets of X form g <= 3 groups of R slots, as in the general kernel, and a
-// pair is g neighbouring lanes, each evaluating its group against Y's points
+// targets of X form g <= 4 groups of R slots, as in the general kernel (four where
+// seven targets of one channel meet one of the other), and a pair is g
+// neighbouring lanes, each evaluating its group against Y's points
 // read straight from memory.  W(X,Y) adds the same terms in the same order as
 // the general kernel does (source pair by source pair, group by group), so it
 // is the same bit for bit.  Bound by the latency of the points' reads.  65,536
