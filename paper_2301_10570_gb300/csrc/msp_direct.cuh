@@ -18,6 +18,7 @@
 // target per lane, scalar FP32 and every pair evaluated, 1.00 ms now.
 #pragma once
 
+#include "msp_hostdev.cuh"
 #include "msp_internal.cuh"
 
 namespace msp {
@@ -435,9 +436,7 @@ k_dir_tiles(int64_t n, const float4* __restrict__ pts, const int32_t* __restrict
     for (int r = 0; r < R; ++r) red[w][32 * r + lane] = __fsub_rn(acc[r], comp[r]);
     __syncthreads();
     for (int slot = threadIdx.x; slot < m; slot += NW * 32) {
-        float v = red[0][slot];
-#pragma unroll
-        for (int k = 1; k < NW; ++k) v += red[k][slot];
+        const float v = sum_totals<NW>([&](int k) { return red[k][slot]; });
         const int32_t t = ch ? list[n - 1 - (first + slot)] : list[first + slot];
         u[perm ? perm[t] : t] = v;
     }
