@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "msp_hostdev.cuh"
 #include "msp_pairsum.cuh"
 
 namespace msp {
@@ -454,18 +455,22 @@ void attraction_grad(msp_ctx& c, const uint8_t* type, const uint8_t* va, const u
     const int2* src = c.nf_src.get<int2>();
     const float4* pts = c.pts.get<float4>();
     const int nb = (int)std::min<int64_t>(std::max<int64_t>(c.n_nodes, 1), 1 << 30);
-    // every input is gathered before an output is written: an output may be g
     const bool adjoint = gE || gI;
     const int32_t* off = nullptr;
     float4* pt = nullptr;
     float* pg = nullptr;
-    if (adjoint) {
+    auto pack = [&] {
         off = ps_offsets(c, fl, s);
         pt = c.gr_pt.ensure<float4>((size_t)n);
         pg = c.gr_tmp.ensure<float>((size_t)n);
         k_grad_pack<<<G, B, 0, s>>>(n, fl, off, perm, pts, g, pt, pg);
         MSP_LAUNCH("grad_pack");
-    }
+    };
+    // an output may lie over g: g is gathered before any is written then (else
+    // while the forward sums run, so that a first call's allocations overlap them)
+    bool over = false;
+    for (const float* o : {u, dud, gE, gI}) over |= o && adjoint && meets(o, 4 * n, g, 4 * n);
+    if (over) pack();
     if (u || dud) {
         if (u) MSP_CUDA(cudaMemsetAsync(u, 0, (size_t)n * sizeof(float), s));
         if (dud) MSP_CUDA(cudaMemsetAsync(dud, 0, (size_t)n * sizeof(float), s));
@@ -474,6 +479,7 @@ void attraction_grad(msp_ctx& c, const uint8_t* type, const uint8_t* va, const u
         MSP_LAUNCH("grad_forward");
     }
     if (adjoint) {
+        if (!over) pack();
         if (gE) MSP_CUDA(cudaMemsetAsync(gE, 0, (size_t)n * sizeof(float), s));
         if (gI) MSP_CUDA(cudaMemsetAsync(gI, 0, (size_t)n * sizeof(float), s));
         k_grad_adjoint<<<nb, kPsWarps * 32, 0, s>>>(segf, &dc->nseg, order, list, pX, src, nfirst,

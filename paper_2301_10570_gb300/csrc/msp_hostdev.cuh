@@ -1,5 +1,5 @@
-// msp_hostdev.cuh -- arithmetic of the kernels that is also run on the host by
-// the tests: plain C++ without CUDA headers.
+// msp_hostdev.cuh -- arithmetic that host and kernels share, or that the tests run
+// on the host: plain C++ without CUDA headers.
 #pragma once
 
 #include <cstdint>
@@ -11,6 +11,12 @@
 #endif
 
 namespace msp {
+
+// whether the bytes [a, a + na) and [b, b + nb) meet
+inline bool meets(const void* a, int64_t na, const void* b, int64_t nb) {
+    const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
+    return pa < pb + (uintptr_t)nb && pb < pa + (uintptr_t)na;
+}
 
 // What a traversal tile counts (children, split, near-field and far pairs) as
 // the W words of its look-back, which adds them modulo 2^62.  The pairs of a

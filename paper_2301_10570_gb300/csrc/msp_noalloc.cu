@@ -101,12 +101,6 @@ __global__ void k_dir_pack(int64_t n, msp::DirRaw src, float4* __restrict__ pts)
     if (i < n) pts[i] = src.get(i);
 }
 
-// whether [a, a + na) and [b, b + nb) have a byte in common
-bool meets(const void* a, int64_t na, const void* b, int64_t nb) {
-    const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
-    return pa < pb + (uintptr_t)nb && pb < pa + (uintptr_t)na;
-}
-
 }  // namespace
 
 extern "C" msp_status msp_direct_noalloc(int64_t n, const float* x, const float* y, const float* z,
@@ -154,6 +148,7 @@ extern "C" msp_status msp_direct_noalloc(int64_t n, const float* x, const float*
     const msp::DirScratch t(reinterpret_cast<int32_t*>(sc + kNaPtsBytes + kNaListBytes), n);
     // u may lie over an input: every input is packed first then, since the
     // kernels read them while they write u
+    using msp::meets;
     const bool over = meets(u, n * 4, x, n * 4) || meets(u, n * 4, y, n * 4) ||
                       meets(u, n * 4, z, n * 4) || meets(u, n * 4, type, n) ||
                       meets(u, n * 4, vac_axon, n) || meets(u, n * 4, vac_dend_e, n) ||
