@@ -1101,10 +1101,10 @@ void attraction(msp_ctx& c, float* u_dev, cudaStream_t s) {
         switch (p) {
             MSP_M2L_CASE(1) MSP_M2L_CASE(2) MSP_M2L_CASE(3)
             case 4:
-                k_m2l_seg4<<<(unsigned)((c.exp_nodes + kM2LWarps - 1) / kM2LWarps), kM2LWarps * 32, 0, s>>>(mseg, &dc->m2l_nseg, mv0, c.exp_first,
-                                                         inv_sigma, c.pr_X.get<int32_t>(),
-                                                         c.pr_Y.get<int32_t>(), eca, ecd, eA, eM, eB,
-                                                         c.pr_w.get<float4>());
+                k_m2l_seg4<<<(unsigned)((c.exp_nodes + kM2LWarps - 1) / kM2LWarps), kM2LWarps * 32,
+                             0, s>>>(mseg, &dc->m2l_nseg, mv0, c.exp_first, inv_sigma,
+                                     c.pr_X.get<int32_t>(), c.pr_Y.get<int32_t>(), eca, ecd, eA, eM,
+                                     eB, c.pr_w.get<float4>());
                 break;
             MSP_M2L_CASE(5) MSP_M2L_CASE(6) MSP_M2L_CASE(7) MSP_M2L_CASE(8)
             default: throw Error(MSP_ERR_INVALID_ARG, "expansion order out of range");

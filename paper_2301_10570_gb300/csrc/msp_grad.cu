@@ -6,10 +6,10 @@
 //   dL/dw^T_s = sum_{t != s, a_t > 0, T(t) = T} g_t K(t,s)   for L = sum_t g_t u(t)
 // summed over the near-field leaf pairs of the last attraction (a plan
 // without translated pairs), at counts the caller passes (the tree's own
-// counts only chose the pairs).  The forward sums run one block per target
-// leaf over the pair list sorted by target leaf; the transposed sums regroup
-// the same pairs by source leaf (a radix sort), one block per source leaf;
-// both stage the partner leaves' points in shared memory.
+// counts only chose the pairs).  Both directions run one block per leaf over its
+// segment of the pair list sorted by target leaf: the near-field pairs are
+// symmetric (msp_pairsum.cuh), so the segment names the leaf's partners as
+// sources and as targets; the partners' points are staged in shared memory.
 // Every sum has a fixed order: the results are reproducible.  The distance
 // is formed as a difference (no expanded form), in single precision.
 #include <algorithm>

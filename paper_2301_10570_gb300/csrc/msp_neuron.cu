@@ -819,7 +819,8 @@ void neuron_steps(msp_ctx& c, int64_t n, uint64_t first_step, int n_steps,
                      al(calcium, 16) && al(za, 16) && al(ze, 16) && al(zi, 16) && al(refr, 4) &&
                      al(spiked, 4);
     // several steps in one launch while the state fits the chip's shared
-    // memory (1.3 M neurons): one block per SM (fewer for small networks), the
+    // memory (four neurons to a group, kNrMaxGroups groups an SM: 1.22 M neurons on
+    // 152 SMs): one block per SM (fewer for small networks), the
     // groups spread evenly over the blocks
     const int64_t n4 = n / 4;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(c.sm_count, n4 / 64));

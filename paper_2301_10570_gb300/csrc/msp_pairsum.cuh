@@ -210,8 +210,8 @@ __device__ __forceinline__ void ps_stage_fwd(PsFwdStage& st, const float4* __res
     st.I[slot] = make_float4(z.x, z.y, w0.y, w1.y);
 }
 
-// Transposed staging: the targets of one channel, packed (msp_grad.cu:
-// transposed_points) as {x, y, z, sorted index}; difference form: A = (-x0,
+// Transposed staging: the targets of one channel, packed (PsPacked, filled by
+// k_grad_pack and k_len_pack) as {x, y, z, sorted index}; difference form: A = (-x0,
 // -x1, -y0, -y1), B = (-z0, -z1, ..); D: the sorted indices (own leaf only).
 struct PsAdjStage {
     float4 A[kPsPairs], B[kPsPairs];

@@ -7,19 +7,21 @@ namespace msp {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Stable LSD radix sort, one kernel per digit.  A first kernel counts the
-// digits of every pass in one reading of the keys; then each pass reads,
-// ranks and writes its tiles once: a tile publishes its digit counts, looks
-// back over its predecessors' (as the scan above, eight tiles per step), and
-// so knows where each of its digits goes without a histogram per tile, its
-// scan and a second reading of the keys.  The tile is put in digit order in
-// shared memory first, so that the writes of a digit are contiguous.  Bound by
-// latency below some 100,000 keys (a pass is one chain of tile number, loads,
-// ranks, look-back and stores, about 9 us cold) and by the look-back and the
-// scattered writes above.  The sorts of a rebuilt step at 262,144 neurons (63,
-// 13 and 16 bits): 275 us in 60 launches with a histogram, three scan kernels
-// and a scatter per 8-bit digit, 157 us in 14 launches now (serialised, cold);
-// the step 822 -> 732 us.  Nine bits a digit: 7 passes for a Morton key.
+// Stable LSD radix sort, one kernel per digit, the published single-pass scheme
+// (Adinets and Merrill, "Onesweep: A Faster Least Significant Digit Radix Sort for
+// GPUs", 2022; the look-back of Merrill and Garland, "Single-pass Parallel Prefix
+// Scan with Decoupled Look-back", 2016).  A first kernel counts the digits of every
+// pass in one reading of the keys; then each pass reads, ranks and writes its tiles
+// once: a tile publishes its digit counts, looks back over its predecessors' (as the
+// scan of msp_scan.cuh, eight tiles per step), and so knows where each of its digits
+// goes without a histogram per tile, its scan and a second reading of the keys.
+// The tile is put in digit order in shared memory first, so that the writes of a
+// digit are contiguous.  Bound by latency below some 100,000 keys (a pass is one
+// chain of tile number, loads, ranks, look-back and stores, about 9 us cold) and by
+// the look-back and the scattered writes above.  The sorts of a rebuilt step at
+// 262,144 neurons (63, 13 and 16 bits): 275 us in 60 launches with a histogram,
+// three scan kernels and a scatter per 8-bit digit, 157 us in 14 launches now
+// (serialised, cold); the step 822 -> 732 us.  Nine bits a digit: 7 passes for a Morton key.
 // ---------------------------------------------------------------------------
 constexpr int kRsThreads = 256;
 constexpr int kRsItems = 8;
