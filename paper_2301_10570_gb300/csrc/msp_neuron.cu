@@ -338,7 +338,8 @@ k_neuron_step(int64_t n, int vec4, uint64_t seed, uint64_t step,
 // to the last, and only the input counts travel through memory.  One
 // cooperative block per SM; a step ends with a grid-wide barrier (the spikes of
 // step k are step k + 1's input), whose waiting time holds the next step's
-// random draws.  A barrier wait of more than SPINS polls sets timeout_bit
+// random draws.  A barrier wait of more than SPINS polls (and four for each edge of
+// the network, whose numbers per neuron have no bound) sets timeout_bit
 // in *overflow and every later wait is skipped: the kernel always ends (the
 // counts are then wrong, and the next synchronising call reports it).
 //
@@ -355,6 +356,8 @@ struct NrRun {
     msp_neuron_params mp;
     int32_t *inp0, *inp1;       // input counts of even and odd steps
     const int32_t *off, *deg, *targets;
+    const int64_t* n_edges;     // of the caller's list, at most cap (null: none)
+    int64_t cap;
     float *x, *ca, *za, *ze, *zi;
     uint8_t *refr, *spiked;
     unsigned int* barrier;      // arrivals, zero on entry
@@ -367,6 +370,16 @@ struct NrRun {
 // of spiking neurons for each
 constexpr int kNrGroupBytes = 6 * 16 + 8 + 8;
 constexpr int kNrMaxGroups = 220 * 1024 / kNrGroupBytes;
+
+// A spiking neuron's edges are one thread's work (60 ns an edge; a poll takes
+// longer): four polls more for each edge of the network.  Whether the arrivals
+// reached the goal.  (Out of line: inside the kernel it made a step 1 % slower.)
+__device__ __noinline__ bool nr_wait_longer(volatile unsigned int* arrivals, unsigned int goal,
+                                            const int64_t* n_edges, int64_t cap) {
+    int64_t more = n_edges ? 4 * min(max(*n_edges, (int64_t)0), cap) : 0;
+    while (*arrivals < goal && more > 0) --more;
+    return *arrivals >= goal;
+}
 
 template <bool FAST, int SPINS>
 __global__ void __launch_bounds__(1024, 1) k_neuron_run(NrRun a) {
@@ -492,7 +505,7 @@ __global__ void __launch_bounds__(1024, 1) k_neuron_run(NrRun a) {
             volatile unsigned int* b = a.barrier;
             int spin = 0;
             while (*b < goal && spin < SPINS) ++spin;
-            if (*b < goal) {
+            if (*b < goal && !nr_wait_longer(b, goal, a.n_edges, a.cap)) {
                 s_dead = 1;
                 atomicOr(reinterpret_cast<unsigned long long*>(a.overflow),
                          (unsigned long long)a.timeout_bit);
@@ -842,6 +855,8 @@ void neuron_steps(msp_ctx& c, int64_t n, uint64_t first_step, int n_steps,
         r.off = off;
         r.deg = deg;
         r.targets = targets;
+        r.n_edges = n_edges;
+        r.cap = cap;
         r.x = x;
         r.ca = calcium;
         r.za = za;

@@ -44,3 +44,30 @@ def test_refused_launch_goes_step_by_step(n):
     for s in states[1:]:
         for k, v in s.items():
             assert torch.equal(v, states[0][k]), k
+
+
+def test_a_hub_of_many_edges_is_waited_for():
+    # a neuron that spikes in every step with ten million outgoing edges: its
+    # block is busy with them for half a second a step while the others wait
+    n, m = 1024, 10_000_000
+    post = torch.arange(m, device="cuda", dtype=torch.int32) % n
+    edges = msp.edge_list(m, pre=torch.full_like(post, 5), post=post,
+                          type_=torch.zeros(m, dtype=torch.uint8))
+    first = {k: torch.zeros(n, device="cuda") for k in ("x", "calcium", "z_axon", "z_dend_e",
+                                                        "z_dend_i")}
+    first["x"][5] = 1e6
+    first.update({k: torch.zeros(n, dtype=torch.uint8, device="cuda")
+                  for k in ("refractory", "spiked")})
+    params = msp.neuron_params(input_per_spike=1e-9, refractory=0, tau_x=1e9)
+    w = W.uniform_cube(100, 1000.0, seed=1)
+    g = msp.MSP(w.params)
+    once, by_one = ({k: v.clone() for k, v in first.items()} for _ in range(2))
+    g.neuron_steps(0, 3, params, edges, once)
+    g.build_tree(*msp.to_device(w))          # synchronises: reports a wait that gave up
+    for k in range(3):
+        g.neuron_steps(k, 1, params, edges, by_one)
+    torch.cuda.synchronize()
+    g.close()
+    assert int(once["spiked"][5]) == 1
+    for k, v in once.items():
+        assert torch.equal(v, by_one[k]), k
