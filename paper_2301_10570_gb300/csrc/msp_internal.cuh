@@ -297,8 +297,9 @@ struct msp_ctx {
     int64_t graph_elem_cap = 0;                // element capacity in graph mode
     bool graph_full_build = false;             // graph mode rebuilds the whole octree
     msp::GraphEnd graph_end;                   // the end of a step in graph mode
-    // every eager build stamps a new tree generation (also in device memory);
-    // a replay that reuses the octree checks the stamp it was captured with
+    // every eager build that makes the octree anew, also one that fails, stamps a
+    // new tree generation (in device memory too); a replay that reuses the octree
+    // checks the stamp it was captured with
     uint64_t tree_gen = 0;
     struct GraphArgs {
         const float *x = nullptr, *y = nullptr, *z = nullptr;

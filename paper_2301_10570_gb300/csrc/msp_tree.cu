@@ -104,10 +104,10 @@ struct BuildEnd {
 };
 
 // The first kernel of a build that makes the octree anew, and the last moment at
-// which the arrays of the one before are whole: no capture holds the stamp left
-// here, and a build that fails later on leaves it.
-__device__ __forceinline__ void drop_stamp(DevCounts* dc) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) dc->tree_gen = ~0ull;
+// which the arrays of the one before are whole: the build's own stamp, which no
+// capture holds yet and which a build that fails later on leaves too.
+__device__ __forceinline__ void put_stamp(DevCounts* dc, uint64_t stamp) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) dc->tree_gen = stamp;
 }
 
 // keys; a position outside [origin, origin + side) or not finite is counted
@@ -115,8 +115,8 @@ __device__ __forceinline__ void drop_stamp(DevCounts* dc) {
 __global__ void k_morton(const float* __restrict__ x, const float* __restrict__ y,
                          const float* __restrict__ z, int64_t n, float ox, float oy, float oz,
                          float side, float scale, uint64_t* __restrict__ keys,
-                         int32_t* __restrict__ vals, DevCounts* dc) {
-    drop_stamp(dc);
+                         int32_t* __restrict__ vals, DevCounts* dc, uint64_t stamp) {
+    put_stamp(dc, stamp);
     bool any_bad = false;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -144,8 +144,8 @@ __global__ void k_morton_frames(const float* __restrict__ x, const float* __rest
                                 const float* __restrict__ z, int64_t n,
                                 const int64_t* __restrict__ off, int64_t nf, int L0, float cs,
                                 float scale, uint64_t* __restrict__ keys,
-                                int32_t* __restrict__ vals, DevCounts* dc) {
-    drop_stamp(dc);
+                                int32_t* __restrict__ vals, DevCounts* dc, uint64_t stamp) {
+    put_stamp(dc, stamp);
     const int sh = kMortonBits - L0;
     const uint32_t qmax = (1u << sh) - 1u;
     const int64_t G = 1ll << (L0 - 1);
@@ -775,6 +775,9 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
         }
         // the positions changed after all (dc->pos_sum is their checksum)
     }
+    // every eager build that gets here has a stamp of its own, a replay one that
+    // no capture and no eager build holds
+    const uint64_t stamp = c.graph_mode ? ~0ull : ++c.tree_gen;
     if (!c.graph_mode) c.lists_valid = false;
 
     // a1 + a2: keys, stable sort, gather into Morton order
@@ -786,11 +789,11 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
             k_morton_frames<<<G, B, 0, s>>>(x, y, z, n, c.frame_off.get<int64_t>(),
                                             (int64_t)c.frame_off_host.size() - 1, c.frame_level,
                                             ldexpf(cfg.side, -c.frame_level), c.morton_scale, mk,
-                                            mv, dc);
+                                            mv, dc, stamp);
             MSP_LAUNCH("morton_frames");
         } else {
             k_morton<<<G, B, 0, s>>>(x, y, z, n, cfg.origin[0], cfg.origin[1], cfg.origin[2],
-                                     cfg.side, c.morton_scale, mk, mv, dc);
+                                     cfg.side, c.morton_scale, mk, mv, dc, stamp);
             MSP_LAUNCH("morton");
         }
         radix_sort_dev(c, k0, v0, k1, v1, nullptr, n, 3 * kMortonBits, s);
@@ -801,6 +804,7 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
                     &dc->n, n, s, keep ? nullptr : scan_st);
     } else {
         dev_set(&dc->n_elem, 0, s);
+        dev_set(reinterpret_cast<int64_t*>(&dc->tree_gen), (int64_t)stamp, s);
     }
 
     // a3: level-synchronous octree; the level sizes stay in device memory.
@@ -921,8 +925,6 @@ void build_tree(msp_ctx& c, int64_t n, const float* x, const float* y, const flo
     c.n_elem = hc.n_elem;
     c.tree_levels = L;
     c.pos_sum_ref = hc.pos_sum;
-    c.tree_gen += 1;
-    dev_set(reinterpret_cast<int64_t*>(&dc->tree_gen), (int64_t)c.tree_gen, s);
     c.tree_built = true;
 }
 
